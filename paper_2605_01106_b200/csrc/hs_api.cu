@@ -99,6 +99,7 @@ struct Derived {
     int nslot, log_w;         // state slots per (layer, sequence); floats of one logged update (rollback by replay)
     int literal;              // the draft model keeps its own state: a ring of Tm + 1 draft slots, a second set of conv buffers
     int64_t state_elems;
+    int pf_rows;              // activation rows of a prompt pass (a multiple of 128)
 };
 
 Derived derive(const hs_config &c) {
@@ -124,13 +125,19 @@ Derived derive(const hs_config &c) {
     while (chunk > 32 && (int64_t)c.max_batch * c.kvh * ((c.kv_capacity + chunk - 1) / chunk) < 296) chunk >>= 1;
     v.att_chunk = chunk;
     v.att_nch = (c.kv_capacity + chunk - 1) / chunk;
+    // a prompt pass never carries more rows than all caches hold together
+    v.pf_rows = (int)((std::min<int64_t>(HS_PREFILL_ROWS, (int64_t)c.max_batch * c.kv_capacity) + 127) / 128 * 128);
     return v;
 }
+
+// rows per plane of the packed activation operands
+int64_t tc_rows_max(const Derived &v) { return std::max<int64_t>(gemm_tc_rows(v.R), gemm_tc_rows(v.pf_rows)); }
 
 // layout of the work buffer; base may be null to only measure
 struct WorkLayout {
     int64_t kv_len, slot, cand, g, margin, n_acc, emitted, stage_n, stage_next, status, counters, am_counters, dslot;
-    int64_t rope, h, zx, gbuf, obuf, abuf, logits, dlogits, att_acc, att_ml, am_part, xb, xb_h, xb_a, ssbuf, total;
+    int64_t rope, h, zx, gbuf, obuf, abuf, logits, dlogits, att_acc, att_ml, am_part, xb, xb_h, xb_a, ssbuf;
+    int64_t pf_rowtab, pf_segtab, pf_list, pf_xbc, pf_dtv, pf_hfin, pf_q, total;
 };
 
 WorkLayout work_layout(const hs_config &c, const Derived &v) {
@@ -143,10 +150,13 @@ WorkLayout work_layout(const hs_config &c, const Derived &v) {
     w.status = take(4); w.counters = take((int64_t)4 * v.B * c.kvh); w.am_counters = take((int64_t)4 * v.R);
     w.dslot = take(4 * v.B);
     w.rope = take((int64_t)c.kv_capacity * (c.hd / 2) * 8);
-    w.h = take((int64_t)4 * 2 * HS_H_PARTS * v.R * c.d);
-    w.zx = take((int64_t)4 * v.R * v.in_rows_max);
-    w.gbuf = take((int64_t)4 * v.R * v.gw);
-    w.obuf = take((int64_t)4 * v.R * c.qh * c.hd);
+    // activations of a pass: B * (max_k + 1) rows of a verify pass (its residual stream in up to HS_H_PARTS parts), or the
+    // rows of a prompt pass
+    const int64_t pr = std::max<int64_t>(v.R, v.pf_rows);
+    w.h = take((int64_t)4 * 2 * std::max<int64_t>((int64_t)HS_H_PARTS * v.R, v.pf_rows) * c.d);
+    w.zx = take(4 * pr * v.in_rows_max);
+    w.gbuf = take(4 * pr * v.gw);
+    w.obuf = take(4 * pr * c.qh * c.hd);
     w.abuf = take((int64_t)4 * v.R * c.ff);
     w.logits = take((int64_t)4 * v.R * c.V);
     w.dlogits = take((int64_t)4 * v.B * std::max(c.max_k, 1) * c.V);
@@ -155,14 +165,21 @@ WorkLayout work_layout(const hs_config &c, const Derived &v) {
     w.am_part = take((int64_t)16 * v.R * HS_ARGMAX_CHUNKS);
     {   // packed bf16 activation operand of the many-row projection kernel: [2][rows][widest reduction]
         const int64_t kmax = std::max<int64_t>(std::max<int64_t>(c.d, c.ff), (int64_t)v.gw + c.qh * c.hd);
-        const int64_t pr = gemm_tc_rows(v.R);
-        w.xb = take((int64_t)2 * 2 * pr * kmax);
+        const int64_t tr = tc_rows_max(v);
+        w.xb = take((int64_t)2 * 2 * tr * kmax);
         // the same for the residual stream and the MLP activations, written by the producing projection's epilogue,
         // and the partial sums of squares (one per 128 model dimensions) of the residual stream's rows
-        w.xb_h = take((int64_t)2 * 2 * pr * c.d);
-        w.xb_a = take((int64_t)2 * 2 * pr * c.ff);
-        w.ssbuf = take((int64_t)4 * pr * ((c.d + 127) / 128));
+        w.xb_h = take((int64_t)2 * 2 * tr * c.d);
+        w.xb_a = take((int64_t)2 * 2 * tr * c.ff);
+        w.ssbuf = take((int64_t)4 * tr * ((c.d + 127) / 128));
     }
+    w.pf_rowtab = take((int64_t)16 * v.pf_rows);
+    w.pf_segtab = take((int64_t)16 * v.B);
+    w.pf_list = take((int64_t)8 * (v.R + v.B));
+    w.pf_xbc = take((int64_t)4 * v.pf_rows * v.convd);
+    w.pf_dtv = take((int64_t)4 * v.pf_rows * 2 * std::max(c.H, c.gh));
+    w.pf_hfin = take((int64_t)4 * (v.R + v.B) * c.d);
+    w.pf_q = take((int64_t)2 * 2 * v.pf_rows * c.qh * c.hd);
     w.total = off;
     return w;
 }
@@ -493,6 +510,163 @@ int enqueue_accept(hs_model *m, int k, int b0, int nb, const int32_t *fn, const 
     return HS_OK;
 }
 
+// One pass of the full model over the rows in pf_rowtab / pf_segtab (prompt positions; see PfPrepArgs).  The projections
+// hand each other packed operands as in a tcgen05 verify pass; the residual stream ends in hbuf[*cur_out].
+int prefill_pass(hs_model *m, int rows, int nseg, int max_seg, int *cur_out) {
+    const hs_config &c = m->c;
+    cudaStream_t s = m->stream;
+    const int d = c.d, ss_parts = (d + 127) / 128;
+    const int64_t q_plane = (int64_t)m->pf_rows * c.qh * c.hd;
+    int32_t *st_w = m->ctrl.status;
+    int cur = 0;
+    PROF(HS_PROF_EMBED, 0, launch_pf_embed(m->embed, d, c.V, m->pf_rowtab, rows, m->hbuf[0], st_w, s), "prefill embed");
+    ++m->launches;
+    for (int l = 0; l < c.L; ++l) {
+        const HsLayer &ly = m->layers[l];
+        const bool attn = ly.type != HS_LAYER_GDN, rec = ly.type != HS_LAYER_ATT, par = ly.type == HS_LAYER_PAR;
+        GemvArgs ga{};
+        ga.W0 = ly.W_in; ga.ldw0 = d; ga.K0 = d; ga.x0 = m->hbuf[cur]; ga.ldx0 = d; ga.xparts = 1;
+        ga.norm_w = ly.norm1; ga.eps = c.eps; ga.O = ly.in_rows_full; ga.out = m->zx; ga.ldo = m->in_rows_max;
+        ga.nrows = rows; ga.epi = EPI_STORE; ga.early_trigger = 1; ga.xb = m->xb; ga.xb_rows = m->xb_rows;
+        if (l > 0) { ga.pk_in = m->xb_h; ga.ss_in = m->ssbuf; ga.ss_parts = ss_parts; }
+        PROF(HS_PROF_GEMV, gemv_bytes(ga), launch_gemm_tc(ga, st_w, s, &m->launches, nullptr), "prefill in_proj");
+        PfPrepArgs pa{};
+        pa.rows = m->pf_rowtab; pa.nrows = rows; pa.zx = m->zx; pa.in_ld = m->in_rows_max; pa.kv_len = m->ctrl.kv_len; pa.cap = c.kv_capacity; pa.status = st_w;
+        const size_t lrB = rec ? (size_t)ly.rl * m->B : 0;
+        float *win = rec ? m->cw + lrB * 3 * m->convd : nullptr;
+        if (rec) {
+            pa.nconv = (m->convd + 255) / 256; pa.convd = m->convd; pa.conv_off = par ? m->di : 0;
+            pa.conv_w = ly.conv_w; pa.conv_b = ly.conv_b; pa.win = win; pa.xbc = m->pf_xbc; pa.dtv = m->pf_dtv;
+            if (par) { pa.heads = c.H; pa.dt_off = m->di + m->convd; pa.A_log = ly.A_log; pa.dt_bias = ly.dt_bias; }
+            else { pa.heads = c.gh; pa.dt_off = 2 * c.gh * c.gdk + 2 * c.gh * c.gdv; }
+        }
+        const size_t per_layer = (size_t)m->B * c.kvh * c.kv_capacity * c.hd;
+        if (attn) {
+            pa.qh = c.qh; pa.kvh = c.kvh; pa.hd = c.hd; pa.q_off = par ? ly.in_rows_draft : 0;
+            pa.k_off = pa.q_off + c.qh * c.hd; pa.v_off = pa.k_off + c.kvh * c.hd; pa.rope = m->rope;
+            pa.q = m->pf_q; pa.q_plane = q_plane; pa.Kc = m->Kc + ly.al * per_layer; pa.Vc = m->Vc + ly.al * per_layer;
+        }
+        PROF(HS_PROF_MIXER, 0, launch_pf_prep(pa, s), "prefill prep");
+        ++m->launches;
+        if (rec) {
+            PfScanArgs sa{};
+            sa.segs = m->pf_segtab; sa.nseg = nseg; sa.zx = m->zx; sa.in_ld = m->in_rows_max; sa.conv_off = pa.conv_off;
+            sa.xbc = m->pf_xbc; sa.convd = m->convd; sa.di = m->di; sa.dtv = m->pf_dtv; sa.heads = pa.heads;
+            sa.P = par ? c.P : c.gdv; sa.N = par ? c.N : c.gdk; sa.D = ly.D; sa.onorm = ly.gnorm; sa.eps = c.eps;
+            sa.state = m->snap + lrB * m->nslot * m->state_elems; sa.state_elems = m->state_elems; sa.nslot = m->nslot; sa.slot = m->ctrl.slot;
+            sa.win = win; sa.g = m->gbuf; sa.gw = m->gw; sa.status = st_w;
+            PROF(HS_PROF_MIXER, 0, par ? launch_pf_ssm(sa, s) : launch_pf_gdn(sa, s), "prefill scan");
+            ++m->launches;
+        }
+        if (attn) {
+            PfAttnArgs aa{};
+            aa.segs = m->pf_segtab; aa.nseg = nseg; aa.max_seg = max_seg; aa.q = m->pf_q; aa.q_plane = q_plane;
+            aa.Kc = pa.Kc; aa.Vc = pa.Vc; aa.kv_len = m->ctrl.kv_len; aa.qh = c.qh; aa.kvh = c.kvh; aa.hd = c.hd; aa.cap = c.kv_capacity; aa.o = m->obuf;
+            PROF(HS_PROF_ATTN, 0, launch_pf_attn(aa, s), "prefill attention");
+            ++m->launches;
+        }
+        GemvArgs go{};
+        go.O = d; go.out = m->hbuf[cur ^ 1]; go.ldo = d; go.max_oparts = 1; go.resid = m->hbuf[cur]; go.rparts = 1;
+        go.nrows = rows; go.epi = EPI_RESID; go.xparts = 1; go.early_trigger = 1; go.xb = m->xb; go.xb_rows = m->xb_rows;
+        if (rec) {
+            go.W0 = ly.W_out; go.ldw0 = m->gw; go.K0 = m->gw; go.x0 = m->gbuf; go.ldx0 = m->gw;
+            if (par) {
+                go.norm_w = ly.gnorm; go.eps = c.eps;
+                go.W1 = ly.W_o; go.ldw1 = c.qh * c.hd; go.K1 = c.qh * c.hd; go.x1 = m->obuf; go.ldx1 = c.qh * c.hd;
+            }
+        } else { go.W0 = ly.W_o; go.ldw0 = c.qh * c.hd; go.K0 = c.qh * c.hd; go.x0 = m->obuf; go.ldx0 = c.qh * c.hd; }
+        go.pk_out = m->xb_h; go.pk_ld = d; go.pk_nw = ly.norm2; go.ss_out = m->ssbuf;
+        PROF(HS_PROF_GEMV, gemv_bytes(go), launch_gemm_tc(go, st_w, s, &m->launches, nullptr), "prefill out_proj");
+        cur ^= 1;
+        GemvArgs gu{};
+        gu.W0 = ly.W_gu; gu.ldw0 = d; gu.K0 = d; gu.O = 2 * c.ff; gu.out = nullptr; gu.ldo = c.ff; gu.nrows = rows; gu.epi = EPI_SWIGLU;
+        gu.eps = c.eps; gu.early_trigger = 1; gu.pk_in = m->xb_h; gu.ss_in = m->ssbuf; gu.ss_parts = ss_parts; gu.pk_out = m->xb_a; gu.pk_ld = c.ff;
+        PROF(HS_PROF_GEMV, gemv_bytes(gu), launch_gemm_tc(gu, st_w, s, &m->launches, nullptr), "prefill gate_up");
+        GemvArgs dn{};
+        dn.W0 = ly.W_down; dn.ldw0 = c.ff; dn.K0 = c.ff; dn.O = d; dn.out = m->hbuf[cur ^ 1]; dn.ldo = d; dn.max_oparts = 1;
+        dn.resid = m->hbuf[cur]; dn.rparts = 1; dn.nrows = rows; dn.epi = EPI_RESID; dn.early_trigger = 1; dn.pk_in = m->xb_a;
+        dn.pk_out = m->xb_h; dn.pk_ld = d; dn.pk_nw = l + 1 < c.L ? m->layers[l + 1].norm1 : m->final_norm; dn.ss_out = m->ssbuf;
+        PROF(HS_PROF_GEMV, gemv_bytes(dn), launch_gemm_tc(dn, st_w, s, &m->launches, nullptr), "prefill down");
+        cur ^= 1;
+    }
+    PROF(HS_PROF_EMBED, 0, launch_pf_advance(m->pf_segtab, nseg, m->ctrl.kv_len, m->ctrl.slot, s), "prefill advance");
+    ++m->launches;
+    *cur_out = cur;
+    return HS_OK;
+}
+
+// LM head and greedy choice over hidden rows x [nb][T] of sequences b0 .. b0 + nb - 1; the choice after a sequence's last
+// row becomes its pending token
+int prefill_head(hs_model *m, const float *x, int T, int b0, int nb) {
+    const hs_config &c = m->c;
+    GemvArgs lm{};
+    lm.W0 = m->lm_head; lm.ldw0 = c.d; lm.K0 = c.d; lm.x0 = x; lm.ldx0 = c.d; lm.xparts = 1; lm.norm_w = m->final_norm; lm.eps = c.eps;
+    lm.O = c.V; lm.out = m->logits; lm.ldo = c.V; lm.nrows = nb * T; lm.epi = EPI_STORE; lm.early_trigger = 1; lm.xb = m->xb; lm.xb_rows = m->xb_rows;
+    PROF(HS_PROF_GEMV, gemv_bytes(lm), launch_gemv(lm, m->ctrl.status, m->stream, &m->launches, nullptr), "prefill lm_head");
+    PROF(HS_PROF_ARGMAX, 0, launch_argmax(m->logits, c.V, T, b0, nb, m->Tm, m->ctrl.g, 0, m->ctrl.margin, m->am_part, m->ctrl.am_counters, m->stream), "prefill argmax");
+    PROF(HS_PROF_ARGMAX, 0, launch_pf_pending(m->ctrl.g, m->ctrl.cand, m->Tm, T, b0, nb, m->stream), "prefill pending");
+    m->launches += 2;
+    m->last_rows = nb * T;
+    return HS_OK;
+}
+
+// Prompts in passes of up to pf_rows positions over all sequences.  What a caller finds afterwards is what a chain of
+// verify passes over chunks of Tm positions leaves: the committed state in the slot of the last chunk's last position,
+// and as logits those of the last chunk of the sequences that chain would have finished with.
+int prefill_wide(hs_model *m, const int32_t *tokens_host, const int32_t *lens_host, int batch) {
+    const int Tm = m->Tm, d = m->c.d, R = m->B * Tm;
+    cudaStream_t s = m->stream;
+    std::vector<int64_t> start(batch);
+    std::vector<int> done(batch, 0);
+    int64_t left = 0;
+    for (int b = 0; b < batch; ++b) { start[b] = left; left += lens_host[b]; }
+    auto chunk = [&](int b) { return (lens_host[b] - 1) / Tm; };               // a sequence's last chunk and its positions
+    auto last_T = [&](int b) { return (lens_host[b] - 1) % Tm + 1; };
+    int hi = 0, lo;
+    for (int b = 1; b < batch; ++b) if (chunk(b) >= chunk(hi)) hi = b;
+    for (lo = hi; lo > 0 && chunk(lo - 1) == chunk(hi) && last_T(lo - 1) == last_T(hi); --lo) {}
+    const int Tl = last_T(hi), nrun = hi - lo + 1;
+    const bool others = nrun < batch;
+    // pf_hfin: the run's last chunks [nrun][Tl], and from row R on the last position of every sequence
+    std::vector<std::vector<int4>> tabs;          // alive until the final synchronisation
+    std::vector<std::vector<int2>> lists;
+    // segments are whole chunks (a prompt's last chunk is never cut)
+    const int budget = m->pf_rows / Tm * Tm;
+    while (left > 0) {
+        std::vector<int4> rows, segs;
+        std::vector<int2> list;
+        int max_seg = 0;
+        for (int b = 0; b < batch; ++b) {
+            const int n = std::min(lens_host[b] - done[b], (budget - (int)rows.size()) / Tm * Tm), row0 = (int)rows.size();
+            if (n <= 0) continue;
+            segs.push_back(make_int4(b, row0, n, m->log_w ? 0 : last_T(b) - 1));
+            for (int i = 0; i < n; ++i) rows.push_back(make_int4(tokens_host[start[b] + done[b] + i], b, i, 0));
+            done[b] += n; left -= n; max_seg = std::max(max_seg, n);
+            if (done[b] < lens_host[b]) continue;
+            if (others) list.push_back(make_int2(row0 + n - 1, R + b));
+            if (b >= lo && b <= hi) for (int i = 0; i < Tl; ++i) list.push_back(make_int2(row0 + n - Tl + i, (b - lo) * Tl + i));
+        }
+        CK(cudaMemcpyAsync(m->pf_rowtab, rows.data(), sizeof(int4) * rows.size(), cudaMemcpyHostToDevice, s), "prefill rows");
+        CK(cudaMemcpyAsync(m->pf_segtab, segs.data(), sizeof(int4) * segs.size(), cudaMemcpyHostToDevice, s), "prefill segments");
+        if (!list.empty()) CK(cudaMemcpyAsync(m->pf_list, list.data(), sizeof(int2) * list.size(), cudaMemcpyHostToDevice, s), "prefill rows kept");
+        int cur = 0;
+        const int rc = prefill_pass(m, (int)rows.size(), (int)segs.size(), max_seg, &cur);
+        if (rc) return rc;
+        if (!list.empty()) {
+            PROF(HS_PROF_EMBED, 0, launch_pf_gather(m->pf_list, (int)list.size(), m->hbuf[cur], d, m->pf_hfin, s), "prefill gather");
+            ++m->launches;
+        }
+        tabs.push_back(std::move(rows)); tabs.push_back(std::move(segs)); lists.push_back(std::move(list));
+    }
+    if (others) { const int rc = prefill_head(m, m->pf_hfin + (size_t)R * d, 1, 0, batch); if (rc) return rc; }
+    const int rc = prefill_head(m, m->pf_hfin, Tl, lo, nrun);
+    if (rc) return rc;
+    for (int b = 0; b < batch; ++b) m->kv_upper[b] += lens_host[b];
+    CK(cudaStreamSynchronize(s), "prefill sync");           // the tables and the caller's tokens were read by now
+    m->batch = batch; m->phase = 0;
+    return hs_device_status(m);
+}
+
 // Run `body` directly, or (HS_FLAG_GRAPHS) capture it once per key and replay the graph.
 template <class F>
 int run_maybe_graph(hs_model *m, uint64_t key, F body) {
@@ -606,10 +780,12 @@ static int init_model(hs_model *m, const hs_config *cfg, const hs_buffers *bufs,
     m->ctrl.status = (int32_t *)(w + wl.status); m->ctrl.counters = (int32_t *)(w + wl.counters); m->ctrl.am_counters = (int32_t *)(w + wl.am_counters);
     m->ctrl.dslot = (int32_t *)(w + wl.dslot);
     m->rope = (float2 *)(w + wl.rope);
-    m->hbuf[0] = (float *)(w + wl.h); m->hbuf[1] = m->hbuf[0] + (size_t)HS_H_PARTS * v.R * c.d; m->zx = (float *)(w + wl.zx); m->gbuf = (float *)(w + wl.gbuf);
+    m->hbuf[0] = (float *)(w + wl.h); m->hbuf[1] = m->hbuf[0] + std::max<size_t>((size_t)HS_H_PARTS * v.R, v.pf_rows) * c.d; m->zx = (float *)(w + wl.zx); m->gbuf = (float *)(w + wl.gbuf);
     m->obuf = (float *)(w + wl.obuf); m->abuf = (float *)(w + wl.abuf); m->logits = (float *)(w + wl.logits); m->dlogits = (float *)(w + wl.dlogits);
     m->tau = 0.f; m->u_draft = m->u_accept = m->u_final = nullptr;
-    m->att_acc = (float *)(w + wl.att_acc); m->att_ml = (float *)(w + wl.att_ml); m->am_part = w + wl.am_part; m->xb = (__nv_bfloat16 *)(w + wl.xb); m->xb_rows = gemm_tc_rows(v.R);
+    m->att_acc = (float *)(w + wl.att_acc); m->att_ml = (float *)(w + wl.att_ml); m->am_part = w + wl.am_part; m->xb = (__nv_bfloat16 *)(w + wl.xb); m->xb_rows = tc_rows_max(v);
+    m->pf_rows = v.pf_rows; m->pf_rowtab = (int4 *)(w + wl.pf_rowtab); m->pf_segtab = (int4 *)(w + wl.pf_segtab); m->pf_list = (int2 *)(w + wl.pf_list);
+    m->pf_xbc = (float *)(w + wl.pf_xbc); m->pf_dtv = (float *)(w + wl.pf_dtv); m->pf_hfin = (float *)(w + wl.pf_hfin); m->pf_q = (__nv_bfloat16 *)(w + wl.pf_q);
     m->xb_h = (__nv_bfloat16 *)(w + wl.xb_h); m->xb_a = (__nv_bfloat16 *)(w + wl.xb_a); m->ssbuf = (float *)(w + wl.ssbuf);
     // the tcgen05 kernel's fixed cost (operand packing, tensor-memory set-up, epilogue out of tensor memory) pays from
     // 7 activation rows on, from 4 where the weight matrices are large (measured: model widths 1024 and 2560)
@@ -627,6 +803,7 @@ static int init_model(hs_model *m, const hs_config *cfg, const hs_buffers *bufs,
     m->ulog = m->log_w ? m->snap + (size_t)v.n_rl * v.B * v.nslot * v.state_elems : nullptr;
     CK(configure_gemv(), "configure gemv");
     CK(configure_attn(), "configure attention");
+    CK(configure_prefill(), "configure prefill");
     if (configure_gemm_tc() != cudaSuccess) { g_hs_gemm_tc = false; cudaGetLastError(); }   // falls back to several 16-row launches
     if (g_hs_tensor_maps && c.hd % 64 == 0) {     // tensor maps of every attention layer's cache (streaming attention form)
         const size_t per_layer = (size_t)v.B * c.kvh * c.kv_capacity * c.hd;
@@ -681,6 +858,14 @@ int hs_prefill(hs_model *m, const int32_t *tokens_host, const int32_t *lens_host
             if (tokens_host[off + p] < 0 || tokens_host[off + p] >= m->c.V) return fail(m, HS_ERR_INVALID_ARG, "prompt token id outside [0, V)");
         off += lens_host[b];
     }
+    int longest = 0;
+    for (int b = 0; b < batch; ++b) longest = std::max(longest, lens_host[b]);
+    // Prompts longer than one verify pass: passes of many positions (their activations do not fit the verify-pass
+    // kernels' registers, the projections need the tcgen05 path).  The literal draft state also runs the draft model
+    // over the prompt and stays on verify-sized passes.  Measured, chunks of max_k + 1 positions against wide passes: 512
+    // tokens on the 0.5B-class hybrid 103.4 -> 14.0 ms, 2048 tokens on the 3B-class one 1371 -> 80.4 ms, four ragged prompts
+    // (2.3 k tokens) on the sequential one 229 -> 28.6 ms.  A prompt of at most one chunk is one verify pass either way.
+    if (longest > m->Tm && g_hs_gemm_tc && !m->literal) return prefill_wide(m, tokens_host, lens_host, batch);
     // Chunk c covers prompt positions [c * Tm, (c + 1) * Tm) of every sequence that reaches that far; neighbouring
     // sequences with the same number of tokens in the chunk go out as one verify pass with every candidate accepted.
     // Nothing waits on the host between chunks (the token slices and accept lengths are staged by the copies).

@@ -13,6 +13,7 @@
 #define HS_MAX_T (HS_MAX_K + 1)
 #define HS_H_PARTS 4          // a projection may leave the residual stream as up to 4 partial sums
 #define HS_ARGMAX_CHUNKS 32    // CTAs that share one logits row in the argmax
+#define HS_PREFILL_ROWS 2048   // most prompt positions of one pass (all sequences together)
 #define HS_MAX_GT 48          // (q heads per kv head) * (k+1) upper bound of the attention kernel
 
 // ---------------------------------------------------------------------------------------------
@@ -78,6 +79,9 @@ struct hs_model {
     std::vector<CUtensorMap> kmaps, vmaps;   // per attention layer (streaming attention form)
     int tc_min_rows_auto;                 // the automatic row threshold of the tcgen05 kernel for this model
     __nv_bfloat16 *xb_h, *xb_a; float *ssbuf;   // packed residual stream / MLP activations handed from projection to projection, row statistics
+    // prompt path: activation rows per pass (0: prompts go through verify passes), row / segment / gather tables, conv
+    // outputs, per-head dt and decay, query planes, hidden rows of the prompts' last positions
+    int pf_rows; int4 *pf_rowtab, *pf_segtab; int2 *pf_list; float *pf_xbc, *pf_dtv, *pf_hfin; __nv_bfloat16 *pf_q;
     void *am_part;             // argmax partials [B*Tm][HS_ARGMAX_CHUNKS] x 16 bytes
     // conv buffers
     float *cw, *hist, *dcw;
@@ -278,3 +282,42 @@ cudaError_t launch_sample(const float *logits, int64_t row_stride, int V, int Tm
 cudaError_t launch_spec_accept(const float *dlogits, int64_t d_seq_stride, const float *vlogits, const int32_t *cand,
                                const float *u_acc, const float *u_final, int u_stride, int32_t *n_out, int32_t *next_out,
                                int V, int Tm, int k, int b0, int nb, float tau, cudaStream_t s);
+
+// ---- prompt path (kernels_prefill.cu) ----------------------------------------------------------------------
+// A pass over many prompt positions: `rows` [nrows] = {token, sequence, index within the segment, -}; `segs`
+// [nseg] = {sequence, first row, rows, state slot that receives the final state}.  Rows of a segment are consecutive
+// positions kv_len[sequence] + index; a sequence has at most one segment per pass.
+struct PfPrepArgs {
+    const int4 *rows; int nrows;
+    const float *zx; int in_ld;
+    int nconv, convd, conv_off; const float *conv_w, *conv_b, *win; float *xbc;      // nconv: 256-channel chunks (0: no conv)
+    int heads, dt_off; const float *A_log, *dt_bias; float *dtv;                     // dtv [nrows][2][heads]; A_log NULL: DeltaNet gates
+    int qh, kvh, hd, q_off, k_off, v_off, cap; const float2 *rope;                   // qh = 0: no attention
+    __nv_bfloat16 *q; int64_t q_plane;                                               // head plane; the remainder plane follows q_plane elements on
+    __nv_bfloat16 *Kc, *Vc; const int32_t *kv_len;
+    int32_t *status;
+};
+struct PfScanArgs {
+    const int4 *segs; int nseg;
+    const float *zx; int in_ld, conv_off;
+    const float *xbc; int convd, di; const float *dtv; int heads, P, N;              // DeltaNet: P = value dim, N = key dim
+    const float *D; const float *onorm; float eps;
+    float *state; int64_t state_elems; int nslot; const int32_t *slot;
+    float *win; float *g; int gw;
+    int32_t *status;
+};
+struct PfAttnArgs {
+    const int4 *segs; int nseg, max_seg;                                             // max_seg: longest segment
+    const __nv_bfloat16 *q; int64_t q_plane;
+    const __nv_bfloat16 *Kc, *Vc; const int32_t *kv_len; int qh, kvh, hd, cap;
+    float *o;
+};
+cudaError_t configure_prefill();
+cudaError_t launch_pf_embed(const __nv_bfloat16 *E, int d, int V, const int4 *rows, int nrows, float *h, int32_t *status, cudaStream_t s);
+cudaError_t launch_pf_prep(const PfPrepArgs &a, cudaStream_t s);
+cudaError_t launch_pf_ssm(const PfScanArgs &a, cudaStream_t s);
+cudaError_t launch_pf_gdn(const PfScanArgs &a, cudaStream_t s);
+cudaError_t launch_pf_attn(const PfAttnArgs &a, cudaStream_t s);
+cudaError_t launch_pf_gather(const int2 *list, int n, const float *h, int d, float *out, cudaStream_t s);
+cudaError_t launch_pf_advance(const int4 *segs, int nseg, int32_t *kv_len, int32_t *slot, cudaStream_t s);
+cudaError_t launch_pf_pending(const int32_t *g, int32_t *cand, int Tm, int T, int b0, int nb, cudaStream_t s);

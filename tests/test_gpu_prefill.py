@@ -1,0 +1,73 @@
+"""Prompts longer than one verify pass: the wide prefill path against the CPU oracle at the sizes where it can go wrong
+(edges of the 8-position scan tiles, the 16-row conv tiles, the 64-position attention tiles; prompts of one to three
+positions beyond a conv window; a batch that needs more than one pass; a prompt appended to a context)."""
+import numpy as np
+import pytest
+
+import hs_inputs as hi
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = {
+    "par64": hi.CONFIGS["cfg1_tiny"],
+    "par128": hi.CONFIGS["cfg1_tiny"].replace(N=128, hd=128),
+    "par256": hi.CONFIGS["cfg1_tiny"].replace(N=256, H=12, qh=6, kvh=2, hd=128),
+    "seq": hi.CONFIGS["test_seq"],
+    "seq32": hi.CONFIGS["test_seq"].replace(gdv=32, gh=8, hd=128),
+}
+
+
+@pytest.fixture(scope="module")
+def env():
+    import oracle
+    from paper_2605_01106_b200 import build, binding
+    build.build()
+    import harness
+    return dict(oracle=oracle, hs=binding, harness=harness)
+
+
+@pytest.mark.parametrize("name,lens,max_k,flags", [
+    ("par64", [65, 1, 16, 129, 7], 4, 0),
+    ("par64", [1500, 2, 700, 33], 8, 2),          # two passes; rollback by replay
+    ("par128", [64, 63, 130], 2, 1),
+    ("par256", [17, 50], 4, 0),
+    ("seq", [72, 3, 9, 128, 40], 4, 0),
+    ("seq", [1100, 1100], 8, 2),
+    ("seq32", [66, 31], 8, 1),
+])
+def test_wide_prefill_matches_oracle(env, name, lens, max_k, flags):
+    s = SHAPES[name]
+    blob, table = hi.make_weights(s, 0, "jitter")
+    cap = max(lens) + 64
+    eng = env["hs"].Engine(s, blob, max_batch=len(lens), max_k=max_k, kv_capacity=cap, flags=flags)
+    model = env["oracle"].Model(s, blob, table, cap)
+    prompts = [hi.make_prompt(s.V, n, seq=40 + b) for b, n in enumerate(lens)]
+    seqs = [model.new_seq() for _ in lens]
+    for q, p in zip(seqs, prompts):
+        q.prefill(p)
+    eng.prefill(prompts)
+    env["harness"].compare_states(eng, seqs, s, kv_rows=None)
+    rep = env["harness"].run_rounds(eng, seqs, s, max_k, 2, forced=[hi.forced_accept(max_k, 2, seq=b) for b in range(len(lens))])
+    # the next turn of a conversation: prompts appended behind what every sequence holds
+    more = [hi.make_prompt(s.V, 11 + 2 * b, seq=80 + b) for b in range(len(lens))]
+    for q, p in zip(seqs, more):
+        q.prefill(p)
+    eng.prefill(more)
+    env["harness"].compare_states(eng, seqs, s, rep)
+    assert eng.device_status() == 0
+
+
+def test_logits_after_prefill(env):
+    # get_logits after a prefill: the positions of the prompt's last chunk of max_k + 1
+    s = SHAPES["par64"]
+    blob, table = hi.make_weights(s, 0, "jitter")
+    eng = env["hs"].Engine(s, blob, max_batch=1, max_k=4, kv_capacity=96)
+    model = env["oracle"].Model(s, blob, table, 96)
+    prompt = hi.make_prompt(s.V, 48, seq=5)
+    eng.prefill([prompt])
+    got = eng.get_logits(3)                       # 48 = 9 * 5 + 3
+    for i in range(3):
+        q = model.new_seq()
+        q.prefill(prompt[:45])
+        want = q.round(2, cand_in=np.asarray(prompt[45:48], np.int32), forced_n=2, want_logits=True)["logits"][i]
+        assert np.abs(got[i] - want).max() <= env["harness"].LOGIT_TOL
