@@ -137,7 +137,7 @@ int64_t tc_rows_max(const Derived &v) { return std::max<int64_t>(gemm_tc_rows(v.
 struct WorkLayout {
     int64_t kv_len, slot, cand, g, margin, n_acc, emitted, stage_n, stage_next, status, counters, am_counters, dslot;
     int64_t rope, h, zx, gbuf, obuf, abuf, logits, dlogits, att_acc, att_ml, am_part, xb, xb_h, xb_a, ssbuf;
-    int64_t pf_rowtab, pf_segtab, pf_list, pf_xbc, pf_dtv, pf_hfin, pf_q, total;
+    int64_t pf_rowtab, pf_segtab, pf_list, pf_xbc, pf_dtv, pf_hfin, pf_q, pf_rec, total;
 };
 
 WorkLayout work_layout(const hs_config &c, const Derived &v) {
@@ -179,6 +179,7 @@ WorkLayout work_layout(const hs_config &c, const Derived &v) {
     w.pf_xbc = take((int64_t)4 * v.pf_rows * v.convd);
     w.pf_dtv = take((int64_t)4 * v.pf_rows * 2 * std::max(c.H, c.gh));
     w.pf_hfin = take((int64_t)4 * (v.R + v.B) * c.d);
+    w.pf_rec = take(4 * pf_record_floats(v.pf_rows, v.B, c.arch == HS_ARCH_PARALLEL ? c.H : c.gh, c.arch != HS_ARCH_PARALLEL));
     w.pf_q = take((int64_t)2 * 2 * v.pf_rows * c.qh * c.hd);
     w.total = off;
     return w;
@@ -527,7 +528,7 @@ int prefill_pass(hs_model *m, int rows, int nseg, int max_seg, int *cur_out) {
         GemvArgs ga{};
         ga.W0 = ly.W_in; ga.ldw0 = d; ga.K0 = d; ga.x0 = m->hbuf[cur]; ga.ldx0 = d; ga.xparts = 1;
         ga.norm_w = ly.norm1; ga.eps = c.eps; ga.O = ly.in_rows_full; ga.out = m->zx; ga.ldo = m->in_rows_max;
-        ga.nrows = rows; ga.epi = EPI_STORE; ga.early_trigger = 1; ga.xb = m->xb; ga.xb_rows = m->xb_rows;
+        ga.nrows = rows; ga.epi = EPI_STORE; ga.early_trigger = 0; ga.xb = m->xb; ga.xb_rows = m->xb_rows;
         if (l > 0) { ga.pk_in = m->xb_h; ga.ss_in = m->ssbuf; ga.ss_parts = ss_parts; }
         PROF(HS_PROF_GEMV, gemv_bytes(ga), launch_gemm_tc(ga, st_w, s, &m->launches, nullptr), "prefill in_proj");
         PfPrepArgs pa{};
@@ -550,13 +551,12 @@ int prefill_pass(hs_model *m, int rows, int nseg, int max_seg, int *cur_out) {
         ++m->launches;
         if (rec) {
             PfScanArgs sa{};
-            sa.segs = m->pf_segtab; sa.nseg = nseg; sa.zx = m->zx; sa.in_ld = m->in_rows_max; sa.conv_off = pa.conv_off;
+            sa.segs = m->pf_segtab; sa.nseg = nseg; sa.max_seg = max_seg; sa.nrows = rows; sa.rec = m->pf_rec; sa.xbc_rw = m->pf_xbc; sa.zx = m->zx; sa.in_ld = m->in_rows_max; sa.conv_off = pa.conv_off;
             sa.xbc = m->pf_xbc; sa.convd = m->convd; sa.di = m->di; sa.dtv = m->pf_dtv; sa.heads = pa.heads;
             sa.P = par ? c.P : c.gdv; sa.N = par ? c.N : c.gdk; sa.D = ly.D; sa.onorm = ly.gnorm; sa.eps = c.eps;
             sa.state = m->snap + lrB * m->nslot * m->state_elems; sa.state_elems = m->state_elems; sa.nslot = m->nslot; sa.slot = m->ctrl.slot;
             sa.win = win; sa.g = m->gbuf; sa.gw = m->gw; sa.status = st_w;
-            PROF(HS_PROF_MIXER, 0, par ? launch_pf_ssm(sa, s) : launch_pf_gdn(sa, s), "prefill scan");
-            ++m->launches;
+            PROF(HS_PROF_MIXER, 0, par ? launch_pf_ssm(sa, s, &m->launches) : launch_pf_gdn(sa, s, &m->launches), "prefill scan");
         }
         if (attn) {
             PfAttnArgs aa{};
@@ -567,7 +567,7 @@ int prefill_pass(hs_model *m, int rows, int nseg, int max_seg, int *cur_out) {
         }
         GemvArgs go{};
         go.O = d; go.out = m->hbuf[cur ^ 1]; go.ldo = d; go.max_oparts = 1; go.resid = m->hbuf[cur]; go.rparts = 1;
-        go.nrows = rows; go.epi = EPI_RESID; go.xparts = 1; go.early_trigger = 1; go.xb = m->xb; go.xb_rows = m->xb_rows;
+        go.nrows = rows; go.epi = EPI_RESID; go.xparts = 1; go.early_trigger = 0; go.xb = m->xb; go.xb_rows = m->xb_rows;
         if (rec) {
             go.W0 = ly.W_out; go.ldw0 = m->gw; go.K0 = m->gw; go.x0 = m->gbuf; go.ldx0 = m->gw;
             if (par) {
@@ -580,11 +580,11 @@ int prefill_pass(hs_model *m, int rows, int nseg, int max_seg, int *cur_out) {
         cur ^= 1;
         GemvArgs gu{};
         gu.W0 = ly.W_gu; gu.ldw0 = d; gu.K0 = d; gu.O = 2 * c.ff; gu.out = nullptr; gu.ldo = c.ff; gu.nrows = rows; gu.epi = EPI_SWIGLU;
-        gu.eps = c.eps; gu.early_trigger = 1; gu.pk_in = m->xb_h; gu.ss_in = m->ssbuf; gu.ss_parts = ss_parts; gu.pk_out = m->xb_a; gu.pk_ld = c.ff;
+        gu.eps = c.eps; gu.early_trigger = 0; gu.pk_in = m->xb_h; gu.ss_in = m->ssbuf; gu.ss_parts = ss_parts; gu.pk_out = m->xb_a; gu.pk_ld = c.ff;
         PROF(HS_PROF_GEMV, gemv_bytes(gu), launch_gemm_tc(gu, st_w, s, &m->launches, nullptr), "prefill gate_up");
         GemvArgs dn{};
         dn.W0 = ly.W_down; dn.ldw0 = c.ff; dn.K0 = c.ff; dn.O = d; dn.out = m->hbuf[cur ^ 1]; dn.ldo = d; dn.max_oparts = 1;
-        dn.resid = m->hbuf[cur]; dn.rparts = 1; dn.nrows = rows; dn.epi = EPI_RESID; dn.early_trigger = 1; dn.pk_in = m->xb_a;
+        dn.resid = m->hbuf[cur]; dn.rparts = 1; dn.nrows = rows; dn.epi = EPI_RESID; dn.early_trigger = 0; dn.pk_in = m->xb_a;
         dn.pk_out = m->xb_h; dn.pk_ld = d; dn.pk_nw = l + 1 < c.L ? m->layers[l + 1].norm1 : m->final_norm; dn.ss_out = m->ssbuf;
         PROF(HS_PROF_GEMV, gemv_bytes(dn), launch_gemm_tc(dn, st_w, s, &m->launches, nullptr), "prefill down");
         cur ^= 1;
@@ -785,7 +785,7 @@ static int init_model(hs_model *m, const hs_config *cfg, const hs_buffers *bufs,
     m->tau = 0.f; m->u_draft = m->u_accept = m->u_final = nullptr;
     m->att_acc = (float *)(w + wl.att_acc); m->att_ml = (float *)(w + wl.att_ml); m->am_part = w + wl.am_part; m->xb = (__nv_bfloat16 *)(w + wl.xb); m->xb_rows = tc_rows_max(v);
     m->pf_rows = v.pf_rows; m->pf_rowtab = (int4 *)(w + wl.pf_rowtab); m->pf_segtab = (int4 *)(w + wl.pf_segtab); m->pf_list = (int2 *)(w + wl.pf_list);
-    m->pf_xbc = (float *)(w + wl.pf_xbc); m->pf_dtv = (float *)(w + wl.pf_dtv); m->pf_hfin = (float *)(w + wl.pf_hfin); m->pf_q = (__nv_bfloat16 *)(w + wl.pf_q);
+    m->pf_xbc = (float *)(w + wl.pf_xbc); m->pf_dtv = (float *)(w + wl.pf_dtv); m->pf_hfin = (float *)(w + wl.pf_hfin); m->pf_rec = (float *)(w + wl.pf_rec); m->pf_q = (__nv_bfloat16 *)(w + wl.pf_q);
     m->xb_h = (__nv_bfloat16 *)(w + wl.xb_h); m->xb_a = (__nv_bfloat16 *)(w + wl.xb_a); m->ssbuf = (float *)(w + wl.ssbuf);
     // the tcgen05 kernel's fixed cost (operand packing, tensor-memory set-up, epilogue out of tensor memory) pays from
     // 7 activation rows on, from 4 where the weight matrices are large (measured: model widths 1024 and 2560)

@@ -13,7 +13,7 @@
 #define HS_MAX_T (HS_MAX_K + 1)
 #define HS_H_PARTS 4          // a projection may leave the residual stream as up to 4 partial sums
 #define HS_ARGMAX_CHUNKS 32    // CTAs that share one logits row in the argmax
-#define HS_PREFILL_ROWS 2048   // most prompt positions of one pass (all sequences together)
+#define HS_PREFILL_ROWS 2176   // most prompt positions of one pass, all sequences together (17 * 128: a 2048-token prompt in chunks of any size fits)
 #define HS_MAX_GT 48          // (q heads per kv head) * (k+1) upper bound of the attention kernel
 
 // ---------------------------------------------------------------------------------------------
@@ -81,7 +81,7 @@ struct hs_model {
     __nv_bfloat16 *xb_h, *xb_a; float *ssbuf;   // packed residual stream / MLP activations handed from projection to projection, row statistics
     // prompt path: activation rows per pass (0: prompts go through verify passes), row / segment / gather tables, conv
     // outputs, per-head dt and decay, query planes, hidden rows of the prompts' last positions
-    int pf_rows; int4 *pf_rowtab, *pf_segtab; int2 *pf_list; float *pf_xbc, *pf_dtv, *pf_hfin; __nv_bfloat16 *pf_q;
+    int pf_rows; int4 *pf_rowtab, *pf_segtab; int2 *pf_list; float *pf_xbc, *pf_dtv, *pf_hfin, *pf_rec; __nv_bfloat16 *pf_q;
     void *am_part;             // argmax partials [B*Tm][HS_ARGMAX_CHUNKS] x 16 bytes
     // conv buffers
     float *cw, *hist, *dcw;
@@ -298,8 +298,10 @@ struct PfPrepArgs {
     int32_t *status;
 };
 struct PfScanArgs {
-    const int4 *segs; int nseg;
+    const int4 *segs; int nseg, max_seg, nrows;
     const float *zx; int in_ld, conv_off;
+    float *rec;                                                                      // tile records (pf_record_floats)
+    float *xbc_rw;                                                                   // DeltaNet: q and k are normalised in place
     const float *xbc; int convd, di; const float *dtv; int heads, P, N;              // DeltaNet: P = value dim, N = key dim
     const float *D; const float *onorm; float eps;
     float *state; int64_t state_elems; int nslot; const int32_t *slot;
@@ -313,10 +315,11 @@ struct PfAttnArgs {
     float *o;
 };
 cudaError_t configure_prefill();
+int64_t pf_record_floats(int rows, int segs, int heads, bool gdn);   // scratch of the scans
 cudaError_t launch_pf_embed(const __nv_bfloat16 *E, int d, int V, const int4 *rows, int nrows, float *h, int32_t *status, cudaStream_t s);
 cudaError_t launch_pf_prep(const PfPrepArgs &a, cudaStream_t s);
-cudaError_t launch_pf_ssm(const PfScanArgs &a, cudaStream_t s);
-cudaError_t launch_pf_gdn(const PfScanArgs &a, cudaStream_t s);
+cudaError_t launch_pf_ssm(const PfScanArgs &a, cudaStream_t s, int64_t *launches);
+cudaError_t launch_pf_gdn(const PfScanArgs &a, cudaStream_t s, int64_t *launches);
 cudaError_t launch_pf_attn(const PfAttnArgs &a, cudaStream_t s);
 cudaError_t launch_pf_gather(const int2 *list, int n, const float *h, int d, float *out, cudaStream_t s);
 cudaError_t launch_pf_advance(const int4 *segs, int nseg, int32_t *kv_len, int32_t *slot, cudaStream_t s);

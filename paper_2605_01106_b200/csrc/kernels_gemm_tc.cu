@@ -133,6 +133,7 @@ struct TcArgs {
     // ss_out[weight-row tile][rpad] of the results.  nullptr: not wanted.
     __nv_bfloat16 *pk_out; int pk_ld; const float *pk_nw; float *ss_out;
     const void *pf_ptr; long long pf_bytes;     // weights of the next projection, pulled into L2 before the wait
+    int early_trigger;          // let the next kernel start before this one has waited (else when its accumulators are complete)
     int off_rx, off_misc;       // shared-memory carve-up behind the stages (bytes from the aligned base)
 };
 
@@ -268,7 +269,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
     const int m0 = blockIdx.y * TC_BM, n0h = blockIdx.z * BNH;
     const int nk = a.nk0 + a.nk1, NS = a.ns;
     const int kb0 = (int)((long long)q * nk / S), kb1 = (int)((long long)(q + 1) * nk / S), nkl = kb1 - kb0;
-    pdl_trigger();
+    if (a.early_trigger) pdl_trigger();
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
         mbar_init(&done_bar, 1);
@@ -373,6 +374,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
     float res[8];
     if (EPI == EPI_RESID) tc_load_resid(a, res, n0h + first, nact - first, row);
     const bool ok = mbar_wait(&done_bar, 0) && !failed_s;
+    if (!a.early_trigger) pdl_trigger();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t taddr = tmem_d + ((uint32_t)((warp & 3) * 32) << 16);
     if (!ok && tid == 0) atomicCAS(a.status, 0, (int)HS_ERR_TIMEOUT);
@@ -603,6 +605,7 @@ cudaError_t launch_gemm_tc(const GemvArgs &a, int32_t *status, cudaStream_t s, i
     }
     t.pf_ptr = a.pf_ptr; t.pf_bytes = a.pf_ptr ? (long long)a.pf_bytes : 0;
     t.off_rx = (int)((size_t)ns * stage); t.off_misc = (int)((size_t)ns * stage + rx_bytes);
+    t.early_trigger = a.early_trigger;
     if (oparts) *oparts = 1;
     if (launches) ++*launches;
     const dim3 grid(S, mtiles, ntiles);

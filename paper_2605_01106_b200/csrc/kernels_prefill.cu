@@ -4,12 +4,14 @@
 // ("segment") per sequence.  The projections are plain dense contractions at that size (kernels_gemm_tc.cu); here are
 //   pf_prep_kernel   causal conv + SiLU of the recurrent channels, dt / decay of every head, RoPE of q and k, and the
 //                    append of the new K and V rows to the cache - everything that is local to a position
-//   pf_ssm_kernel    the Mamba-2 recurrence over the whole segment, state rows resident in registers
-//   pf_gdn_kernel    the gated delta rule over the whole segment
+//   pf_gram_kernel, pf_ssm_kernel                          the Mamba-2 recurrence over the whole segment
+//   pf_gdn_gram_kernel, pf_gdn_kernel, pf_gdn_out_kernel   the gated delta rule over the whole segment, output norm and gate
 //   pf_attn_kernel   causal attention of the segment's positions over the cache (which already holds the new rows)
 //   pf_embed_kernel, pf_gather_kernel, pf_advance_kernel, pf_pending_kernel   gathers and control words
 // The verify-pass kernels are built for at most nine positions (one trip to L2, everything in registers); their cost
 // per position is that of streaming all weights once per nine tokens, which is what this path removes.
+// Every kernel of this path lets its successor start when its own work is done, not earlier: blocks that wait hold
+// the registers and shared memory that the blocks still to come need (14.0 -> 9.6 ms for 512 tokens on the 0.5B-class hybrid).
 // fp32 values keep their precision throughout: the recurrences run in fp32, attention splits queries and probabilities
 // into a bf16 head and a bf16 remainder (exact to 2^-17), keys and values enter as the bf16 the cache holds.
 #include "hs_internal.h"
@@ -20,9 +22,6 @@ using namespace hsd;
 
 __device__ __forceinline__ void cp16(void *dst_smem, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem_u32(dst_smem)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp4(void *dst_smem, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(smem_u32(dst_smem)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -72,16 +71,16 @@ __global__ void pf_embed_kernel(const __nv_bfloat16 *E, int d, int V, const int4
 }
 
 // ---- position-local work ------------------------------------------------------------------------------------
-// grid = (row tiles of PREP_ROWS, conv chunks of 256 channels + one slot for the heads and the attention rows).
-// A conv thread owns one channel and walks the rows of the tile with its three previous raw inputs in registers, so a
-// raw value is read once per tile (plus the three rows before it).
+// grid = (row tiles of PREP_ROWS, roles): `nconv` chunks of 256 conv channels, one block for dt / decay of every head,
+// then chunks of 256 (rotation) pairs of the q | k | v rows.  A thread owns one channel or pair and walks the rows of
+// the tile; the loads of all rows are issued before the first is used.  (One block for all heads and pairs of a tile:
+// 41 us at 512 rows of the 0.5B-class hybrid; split: 16 us.)
 constexpr int PREP_ROWS = 16;
 
 __global__ void __launch_bounds__(256) pf_prep_kernel(const PfPrepArgs a) {
     __shared__ int4 info[PREP_ROWS];
     __shared__ int base[PREP_ROWS];               // position of the row in its sequence, -1: outside the cache
     const int r0 = blockIdx.x * PREP_ROWS, nr = min(PREP_ROWS, a.nrows - r0), tid = threadIdx.x;
-    pdl_trigger();
     pdl_wait();
     if (tid < nr) {
         info[tid] = __ldcg(a.rows + r0 + tid);
@@ -90,8 +89,9 @@ __global__ void __launch_bounds__(256) pf_prep_kernel(const PfPrepArgs a) {
         if (p < 0 || p >= a.cap) { base[tid] = -1; atomicCAS(a.status, 0, p < 0 ? (int)HS_ERR_DEVICE : (int)HS_ERR_CAPACITY); }
     }
     __syncthreads();
-    if ((int)blockIdx.y < a.nconv) {
-        const int c = blockIdx.y * 256 + tid;
+    int role = blockIdx.y;
+    if (role < a.nconv) {
+        const int c = role * 256 + tid;
         if (c >= a.convd) return;
         const float4 tap = *reinterpret_cast<const float4 *>(a.conv_w + 4 * c);
         const float bias = a.conv_b[c];
@@ -122,50 +122,52 @@ __global__ void __launch_bounds__(256) pf_prep_kernel(const PfPrepArgs a) {
         }
         return;
     }
-    // dt and decay of every head (Mamba-2), or the decay / write-strength gates (DeltaNet)
-    for (int idx = tid; idx < nr * a.heads; idx += 256) {
-        const int i = idx / a.heads, h = idx - i * a.heads;
-        const float *row = a.zx + (size_t)(r0 + i) * a.in_ld + a.dt_off;
-        float u, v;
-        if (a.A_log) {
-            u = softplus_f(__ldcg(row + h) + a.dt_bias[h]);
-            v = expf(-u * expf(a.A_log[h]));
-        } else { u = sigmoid_f(__ldcg(row + h)); v = sigmoid_f(__ldcg(row + a.heads + h)); }
-        float *out = a.dtv + (size_t)(r0 + i) * 2 * a.heads;
-        out[h] = u; out[a.heads + h] = v;
-    }
-    if (a.qh == 0) return;
-    // q: rotated, scaled, split into bf16 head and remainder; k: rotated and v: rounded to bf16 and appended
-    const int hp = a.hd / 2, nq = a.qh * hp, nk = a.kvh * hp, per = nq + 2 * nk;
-    const float scale = rsqrtf((float)a.hd);
-    for (int idx = tid; idx < nr * per; idx += 256) {
-        const int i = idx / per, j = idx - i * per, pos = base[i];
-        if (pos < 0) continue;
-        const float *row = a.zx + (size_t)(r0 + i) * a.in_ld;
-        if (j < nq + nk) {
-            const bool isq = j < nq;
-            const int jj = isq ? j : j - nq, h = jj / hp, e = jj - h * hp;
-            const float *s = row + (isq ? a.q_off : a.k_off) + h * a.hd + e;
-            const float x0 = __ldcg(s), x1 = __ldcg(s + hp);
-            const float2 cs = a.rope[(size_t)pos * hp + e];
-            const float y0 = x0 * cs.x - x1 * cs.y, y1 = x1 * cs.x + x0 * cs.y;
-            if (isq) {
-                const float v0 = y0 * scale, v1 = y1 * scale;
-                const __nv_bfloat16 h0 = __float2bfloat16_rn(v0), h1 = __float2bfloat16_rn(v1);
-                __nv_bfloat16 *q = a.q + (size_t)(r0 + i) * a.qh * a.hd + h * a.hd + e;
-                q[0] = h0; q[hp] = h1;
-                q += a.q_plane;
-                q[0] = __float2bfloat16_rn(v0 - __bfloat162float(h0)); q[hp] = __float2bfloat16_rn(v1 - __bfloat162float(h1));
-            } else {
-                __nv_bfloat16 *k = a.Kc + (((size_t)info[i].y * a.kvh + h) * a.cap + pos) * a.hd + e;
-                k[0] = __float2bfloat16_rn(y0); k[hp] = __float2bfloat16_rn(y1);
-            }
-        } else {
-            const int jj = j - nq - nk, h = jj / hp, e = jj - h * hp;
-            const float *s = row + a.v_off + h * a.hd + 2 * e;
-            __nv_bfloat16 *v = a.Vc + (((size_t)info[i].y * a.kvh + h) * a.cap + pos) * a.hd + 2 * e;
-            *reinterpret_cast<uint32_t *>(v) = pack_bf16x2(__ldcg(s), __ldcg(s + 1));
+    role -= a.nconv;
+    if (a.heads && role-- == 0) {
+        // dt and decay of every head (Mamba-2), or the decay / write-strength gates (DeltaNet)
+        for (int idx = tid; idx < nr * a.heads; idx += 256) {
+            const int i = idx / a.heads, h = idx - i * a.heads;
+            const float *row = a.zx + (size_t)(r0 + i) * a.in_ld + a.dt_off;
+            float u, v;
+            if (a.A_log) {
+                u = softplus_f(__ldcg(row + h) + a.dt_bias[h]);
+                v = expf(-u * expf(a.A_log[h]));
+            } else { u = sigmoid_f(__ldcg(row + h)); v = sigmoid_f(__ldcg(row + a.heads + h)); }
+            float *out = a.dtv + (size_t)(r0 + i) * 2 * a.heads;
+            out[h] = u; out[a.heads + h] = v;
         }
+        return;
+    }
+    // q: rotated, scaled, split into bf16 head and remainder; k: rotated and v: rounded to bf16 and appended
+    const int hp = a.hd / 2, nq = a.qh * hp, nk = a.kvh * hp;
+    const int j = role * 256 + tid;
+    if (j >= nq + 2 * nk) return;
+    const bool isq = j < nq, isv = j >= nq + nk;
+    const int jj = isq ? j : isv ? j - nq - nk : j - nq, h = jj / hp, e = jj - h * hp;
+    const float *src = a.zx + (size_t)r0 * a.in_ld + (isq ? a.q_off : isv ? a.v_off : a.k_off) + h * a.hd + (isv ? 2 * e : e);
+    const int step = isv ? 1 : hp;                // the pair: (e, e + hd / 2) for a rotation, two neighbours for v
+    const float scale = isq ? rsqrtf((float)a.hd) : 1.f;
+    float x0[PREP_ROWS], x1[PREP_ROWS];
+#pragma unroll
+    for (int i = 0; i < PREP_ROWS; ++i) {
+        x0[i] = i < nr ? __ldcg(src + (size_t)i * a.in_ld) : 0.f;
+        x1[i] = i < nr ? __ldcg(src + (size_t)i * a.in_ld + step) : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < PREP_ROWS; ++i) {
+        const int pos = i < nr ? base[i] : -1;
+        if (pos < 0) continue;
+        const size_t crow = (((size_t)info[i].y * a.kvh + h) * a.cap + pos) * a.hd;
+        if (isv) { *reinterpret_cast<uint32_t *>(a.Vc + crow + 2 * e) = pack_bf16x2(x0[i], x1[i]); continue; }
+        const float2 cs = a.rope[(size_t)pos * hp + e];
+        const float y0 = (x0[i] * cs.x - x1[i] * cs.y) * scale, y1 = (x1[i] * cs.x + x0[i] * cs.y) * scale;
+        const __nv_bfloat16 h0 = __float2bfloat16_rn(y0), h1 = __float2bfloat16_rn(y1);
+        if (isq) {
+            __nv_bfloat16 *q = a.q + (size_t)(r0 + i) * a.qh * a.hd + h * a.hd + e;
+            q[0] = h0; q[hp] = h1;
+            q += a.q_plane;
+            q[0] = __float2bfloat16_rn(y0 - __bfloat162float(h0)); q[hp] = __float2bfloat16_rn(y1 - __bfloat162float(h1));
+        } else { a.Kc[crow + e] = h0; a.Kc[crow + e + hp] = h1; }
     }
 }
 
@@ -178,147 +180,111 @@ __device__ __forceinline__ void shift_window(const PfScanArgs &a, int b, int row
                                            : __ldcg(a.zx + (size_t)(row0 + n + j - 3) * a.in_ld + a.conv_off + c);
 }
 
-// ---- Mamba-2 recurrence -------------------------------------------------------------------------------------
-// grid = (strips of 16 state rows, heads, segments), four warps of four rows.  A lane holds EPL = N / 32 state values
-// of each of its warp's rows in registers for the whole segment; B, C, x, z and the decays of eight positions at a
-// time arrive through a ring of shared-memory stages (asynchronous copies).  The outputs of eight positions x four
-// rows are 32 partial sums per lane: one transposing reduction leaves lane l with the total of (position l / 4,
-// row l % 4), which that lane gates and stores.  Bound by the issue of its own instructions (packed fp32 pairs).
-constexpr int SC_POS = 8, SC_STAGES = 4, SC_THREADS = 128, SC_ROWS = 16;
-__host__ __device__ constexpr int sc_stage_floats(int N) { return SC_POS * (2 * N + 2 * SC_ROWS + 4); }
-
-template <int EPL>
-__global__ void __launch_bounds__(SC_THREADS) pf_ssm_kernel(const PfScanArgs a) {
-    constexpr int N = 32 * EPL, VW = EPL < 4 ? EPL : 4, NVEC = EPL / VW, NP = EPL / 2;
-    constexpr int STG = sc_stage_floats(N), CB = N / 4, PER = 2 * CB + 8;      // 16-byte pieces of one position
-    extern __shared__ __align__(16) float sm[];
-    const int p0 = blockIdx.x * SC_ROWS, h = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    pdl_trigger();
-    pdl_wait();
-    const int4 sg = __ldcg(a.segs + blockIdx.z);
-    const int b = sg.x, row0 = sg.y, n = sg.z, slot_out = sg.w;
-    const int slot_in = a.nslot == 1 ? 0 : __ldcg(a.slot + b);
-    if ((unsigned)slot_in >= (unsigned)a.nslot || (unsigned)slot_out >= (unsigned)a.nslot) {
-        if (tid == 0) atomicCAS(a.status, 0, (int)HS_ERR_DEVICE);
-        return;
-    }
-    float *base = a.state + (size_t)b * a.nslot * a.state_elems + ((size_t)h * a.P + p0 + warp * 4) * N;
-    const float *sin_ = base + (size_t)slot_in * a.state_elems;
-    f2 s[4][NP];
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int v = 0; v < NVEC; ++v) {
-            const float *src = sin_ + r * N + v * (32 * VW) + lane * VW;
-            if (VW == 4) { const float4 t = __ldcg(reinterpret_cast<const float4 *>(src)); s[r][2 * v] = pk2(t.x, t.y); s[r][2 * v + NP / NVEC - 1] = pk2(t.z, t.w); }
-            else { const float2 t = __ldcg(reinterpret_cast<const float2 *>(src)); s[r][0] = pk2(t.x, t.y); }
-        }
-    const int ntile = (n + SC_POS - 1) / SC_POS;
-    auto fetch = [&](int t) {
-        if (t < ntile) {
-            float *st = sm + (size_t)(t % SC_STAGES) * STG;
-            const int cnt = min(SC_POS, n - t * SC_POS);
-            for (int idx = tid; idx < cnt * PER; idx += SC_THREADS) {
-                const int i = idx / PER, j = idx - i * PER;
-                const size_t row = (size_t)(row0 + t * SC_POS + i);
-                const float *xr = a.xbc + row * a.convd;
-                if (j < CB) cp16(st + i * N + 4 * j, xr + a.di + 4 * j);
-                else if (j < 2 * CB) cp16(st + SC_POS * N + i * N + 4 * (j - CB), xr + a.di + N + 4 * (j - CB));
-                else if (j < 2 * CB + 4) cp16(st + 2 * SC_POS * N + i * SC_ROWS + 4 * (j - 2 * CB), xr + h * a.P + p0 + 4 * (j - 2 * CB));
-                else cp16(st + 2 * SC_POS * N + SC_POS * SC_ROWS + i * SC_ROWS + 4 * (j - 2 * CB - 4), a.zx + row * a.in_ld + h * a.P + p0 + 4 * (j - 2 * CB - 4));
-            }
-            if (tid < 2 * cnt) {
-                const int i = tid >> 1, w = tid & 1;
-                cp4(st + 2 * SC_POS * N + 2 * SC_POS * SC_ROWS + 4 * i + w, a.dtv + (size_t)(row0 + t * SC_POS + i) * 2 * a.heads + w * a.heads + h);
-            }
-        }
-        cp_commit();
-    };
-    const float Dh = a.D[h];
-#pragma unroll
-    for (int t = 0; t < SC_STAGES - 1; ++t) fetch(t);
-#pragma unroll 1
-    for (int t = 0; t < ntile; ++t) {
-        cp_wait<SC_STAGES - 2>();
-        __syncthreads();                  // stage t complete; everybody is done with the stage that is refilled now
-        fetch(t + SC_STAGES - 1);
-        const float *st = sm + (size_t)(t % SC_STAGES) * STG;
-        const float *Bs = st, *Cs = st + SC_POS * N, *xs = st + 2 * SC_POS * N, *zs = xs + SC_POS * SC_ROWS, *dd = zs + SC_POS * SC_ROWS;
-        const int cnt = min(SC_POS, n - t * SC_POS);
-        float acc[32];
-#pragma unroll
-        for (int i = 0; i < SC_POS; ++i) {
-            if (i < cnt) {
-                f2 Bv[NP], Cv[NP];
-#pragma unroll
-                for (int v = 0; v < NVEC; ++v) {
-                    if (VW == 4) {
-                        const float4 x = *reinterpret_cast<const float4 *>(Bs + i * N + v * 128 + lane * 4), y = *reinterpret_cast<const float4 *>(Cs + i * N + v * 128 + lane * 4);
-                        Bv[2 * v] = pk2(x.x, x.y); Bv[2 * v + NP / NVEC - 1] = pk2(x.z, x.w);
-                        Cv[2 * v] = pk2(y.x, y.y); Cv[2 * v + NP / NVEC - 1] = pk2(y.z, y.w);
-                    } else {
-                        const float2 x = *reinterpret_cast<const float2 *>(Bs + i * N + lane * 2), y = *reinterpret_cast<const float2 *>(Cs + i * N + lane * 2);
-                        Bv[0] = pk2(x.x, x.y); Cv[0] = pk2(y.x, y.y);
-                    }
-                }
-                const float2 dt = *reinterpret_cast<const float2 *>(dd + 4 * i);       // dt, decay
-                const float4 xv = *reinterpret_cast<const float4 *>(xs + i * SC_ROWS + warp * 4);
-                const f2 dec = pk2(dt.y, dt.y);
-                const float xr[4] = {xv.x, xv.y, xv.z, xv.w};
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const float dx = dt.x * xr[r];
-                    const f2 dtx = pk2(dx, dx);
-                    f2 y = 0ull;
-#pragma unroll
-                    for (int e = 0; e < NP; ++e) {
-                        s[r][e] = fma2(dec, s[r][e], mul2(dtx, Bv[e]));
-                        y = e ? fma2(s[r][e], Cv[e], y) : mul2(s[r][e], Cv[e]);
-                    }
-                    float lo, hi;
-                    up2(y, lo, hi);
-                    acc[i * 4 + r] = lo + hi;
-                }
-            } else {
-#pragma unroll
-                for (int r = 0; r < 4; ++r) acc[i * 4 + r] = 0.f;
-            }
-        }
-        const float y = xreduce<32>(acc, lane);
-        const int i = lane >> 2, rr = warp * 4 + (lane & 3);
-        if (i < cnt)
-            a.g[(size_t)(row0 + t * SC_POS + i) * a.gw + h * a.P + p0 + rr] = (y + Dh * xs[i * SC_ROWS + rr]) * silu_f(zs[i * SC_ROWS + rr]);
-    }
-    cp_wait<0>();
-    float *sout = base + (size_t)slot_out * a.state_elems;
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int v = 0; v < NVEC; ++v) {
-            float *p = sout + r * N + v * (32 * VW) + lane * VW;
-            float x0, x1, x2, x3;
-            up2(s[r][VW == 4 ? 2 * v : 0], x0, x1);
-            if (VW == 4) { up2(s[r][2 * v + NP / NVEC - 1], x2, x3); *reinterpret_cast<float4 *>(p) = make_float4(x0, x1, x2, x3); }
-            else *reinterpret_cast<float2 *>(p) = make_float2(x0, x1);
-        }
-    if (tid < SC_ROWS) shift_window(a, b, row0, n, h * a.P + p0 + tid);
-    if (blockIdx.x == 0 && h == 0)
-        for (int c = tid; c < 2 * N; c += SC_THREADS) shift_window(a, b, row0, n, a.di + c);
+// ---- recurrences in tiles of eight positions ------------------------------------------------------------------
+// Unrolled over a tile of eight positions a linear recurrence needs the state only twice: for the eight products of
+// the OLD state with the tile's read vectors, and for one update with the tile's eight outer products.  What couples
+// the positions of a tile is small and shared by all state rows - products of the tile's vectors with each other times
+// the decays between them - so it is computed once per tile (pf_gram / pf_gdn_gram) into a record that the scan reads:
+//   Mamba-2   y_i = P_i (C_i . S) + sum_{j<=i} M_ij x_j + D x_i ,   S <- P_7 S + sum_j (E_j x_j) B_j^T
+//             P_i = prod_{u<=i} a_u ,  M_ij = (C_i . B_j) dt_j prod_{j<u<=i} a_u ,  E_j = dt_j prod_{j<u<=7} a_u
+//   DeltaNet  u_i = beta_i v_i - beta_i P_i (S k_i) - sum_{j<i} MK_ij u_j   (per value row, solved in order)
+//             o_i = P_i (S q_i) + sum_{j<=i} MQ_ij u_j ,            S <- P_7 S + sum_j (E_j u_j) k_j^T
+//             MK_ij = beta_i (k_i . k_j) prod_{j<u<=i} alpha_u ,  MQ_ij = (q_i . k_j) prod.. ,  E_j = prod_{j<u<=7} alpha_u
+// Against one position at a time: 17 instead of 24 multiply-adds per state element and tile, no serial chain but the
+// eight-term solve, and one reduction over lanes per (row, position) of which 32 go together.  All of it in fp32.
+// Positions beyond the end of a segment have decay 1 and E_j = 0.
+// The tiles arrive through a ring of shared-memory stages: a producer warp issues the bulk copies of a whole tile (one
+// lane per piece), the consumer warps only wait for bytes and hand stages back - no block-wide barrier in the loop.
+constexpr int SC_POS = 8, SC_MAXSTAGES = 6;
+constexpr int REC_SSM = 80;       // M[8][8] P[8] E[8]
+constexpr int REC_GDN = 152;      // MK[8][8] MQ[8][8] P[8] E[8] beta[8]
+// record slot of tile t of segment number s that starts at row0: tiles of different segments never share one
+__device__ __forceinline__ int rec_slot(int row0, int s, int t) { return row0 / SC_POS + s + t; }
+__device__ __forceinline__ void bulk_tile(void *dst_smem, const void *src, uint32_t bytes, uint64_t *bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 :: "r"(smem_u32(dst_smem)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(bar)) : "memory");
 }
 
-// ---- gated delta rule ---------------------------------------------------------------------------------------
-// grid = (heads, segments); two lanes per value row, each with 32 of the 64 key columns in registers.  The dependent
-// chain of a position is one dot product (S k), one shuffle, the update; S q and the output norm hang off it.
-constexpr int GD_POS = 8, GD_STAGES = 3, GD_THREADS = 128;
-constexpr int GD_STG = GD_POS * (4 * 64 + 4);
-
-__global__ void __launch_bounds__(GD_THREADS) pf_gdn_kernel(const PfScanArgs a) {
-    extern __shared__ __align__(16) float sm[];
-    __shared__ float os[GD_POS][64];
-    const int h = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int dv = a.P, nk = a.heads * 64, nv = a.heads * dv;
-    pdl_trigger();
+// grid = (tiles, segments), eight warps: warp i takes position i of the tile
+template <int EPL>
+__global__ void __launch_bounds__(256) pf_gram_kernel(const PfScanArgs a) {
+    constexpr int N = 32 * EPL;
+    __shared__ float G[SC_POS][SC_POS];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, t = blockIdx.x;
     pdl_wait();
+    const int4 sg = __ldcg(a.segs + blockIdx.y);
+    const int row0 = sg.y, cnt = min(SC_POS, sg.z - t * SC_POS);
+    if (cnt <= 0) return;
+    if (warp < cnt) {
+        const float *x = a.xbc + (size_t)(row0 + t * SC_POS) * a.convd + a.di;
+        float c[EPL], b[SC_POS][EPL];
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) c[e] = __ldcg(x + (size_t)warp * a.convd + N + e * 32 + lane);
+#pragma unroll
+        for (int j = 0; j < SC_POS; ++j)
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) b[j][e] = j <= warp ? __ldcg(x + (size_t)j * a.convd + e * 32 + lane) : 0.f;
+        float d[SC_POS];
+#pragma unroll
+        for (int j = 0; j < SC_POS; ++j) {
+            d[j] = 0.f;
+#pragma unroll
+            for (int e = 0; e < EPL; ++e) d[j] = fmaf(c[e], b[j][e], d[j]);
+        }
+        const float g = xreduce<SC_POS>(d, lane);            // lanes 4 j .. 4 j + 3 hold C_i . B_j
+        if ((lane & 3) == 0) G[warp][lane >> 2] = g;
+    }
+    __syncthreads();
+    float *rec = a.rec + (size_t)rec_slot(row0, blockIdx.y, t) * a.heads * REC_SSM;
+    for (int idx = tid; idx < a.heads * SC_POS; idx += 256) {
+        const int i = idx / a.heads, h = idx - i * a.heads;
+        const float *dv = a.dtv + (size_t)(row0 + t * SC_POS) * 2 * a.heads + h;
+        float dt[SC_POS], dec[SC_POS];
+#pragma unroll
+        for (int j = 0; j < SC_POS; ++j) {
+            dt[j] = j < cnt ? __ldcg(dv + (size_t)j * 2 * a.heads) : 0.f;
+            dec[j] = j < cnt ? __ldcg(dv + (size_t)j * 2 * a.heads + a.heads) : 1.f;
+        }
+        float m[SC_POS], prod = 1.f, tail = 1.f, ei = 0.f;
+#pragma unroll
+        for (int j = SC_POS - 1; j >= 0; --j) {
+            m[j] = 0.f;
+            if (j <= i) { m[j] = i < cnt ? G[i][j] * prod * dt[j] : 0.f; prod *= dec[j]; }
+            if (j == i) ei = tail * dt[j];
+            tail *= dec[j];
+        }
+        float4 *out = reinterpret_cast<float4 *>(rec + (size_t)h * REC_SSM + i * SC_POS);
+        out[0] = make_float4(m[0], m[1], m[2], m[3]); out[1] = make_float4(m[4], m[5], m[6], m[7]);
+        rec[(size_t)h * REC_SSM + 64 + i] = prod; rec[(size_t)h * REC_SSM + 72 + i] = ei;
+    }
+    pdl_trigger();
+}
+
+// The Mamba-2 scan.  grid = (strips of 8 * RW state rows, segments); eight consumer warps and one producer warp.  A warp
+// owns RW rows of the [heads * P][N] state (they may belong to two heads) for the whole segment, lane l holding N / 32
+// values of each.  RW is the smallest that leaves at most one block per SM (see launch_ssm_n).
+// Bound by latency within a tile at few rows, by the fp32 pipes at many.
+constexpr int SC_WARPS = 8, SC_THREADS = (SC_WARPS + 1) * 32;
+__host__ __device__ constexpr int sc_stage_floats(int N, int RW) { return SC_POS * (2 * N + 2 * SC_WARPS * RW) + 4 * REC_SSM; }
+
+template <int EPL, int RW>
+__global__ void __launch_bounds__(SC_THREADS) pf_ssm_kernel(const PfScanArgs a, const int stages) {
+    constexpr int N = 32 * EPL, VW = EPL < 4 ? EPL : 4, NVEC = EPL / VW, NP = EPL / 2, PPV = NP / NVEC;
+    constexpr int CR = SC_WARPS * RW, STG = sc_stage_floats(N, RW), RWP = (RW + 1) & ~1;
+    extern __shared__ __align__(128) float sm[];
+    __shared__ __align__(16) float2 es[SC_WARPS][SC_POS + 1][RWP];             // per warp: E_j x_j of its rows, then P_7; each twice
+    __shared__ __align__(8) uint64_t full[SC_MAXSTAGES], empty[SC_MAXSTAGES];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int R0 = blockIdx.x * CR, Rw = R0 + warp * RW;                       // first row of the block / of the warp
+    // positions a last tile does not have keep whatever a stage holds: finite values (their coefficients are zero)
+    for (int i = tid; i < stages * STG / 4; i += SC_THREADS) reinterpret_cast<float4 *>(sm)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (tid < stages) { mbar_init(&full[tid], 1); mbar_init(&empty[tid], SC_WARPS); mbar_fence_init(); }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    pdl_wait();
+    __syncthreads();
     const int4 sg = __ldcg(a.segs + blockIdx.y);
     const int b = sg.x, row0 = sg.y, n = sg.z, slot_out = sg.w;
     const int slot_in = a.nslot == 1 ? 0 : __ldcg(a.slot + b);
@@ -326,115 +292,379 @@ __global__ void __launch_bounds__(GD_THREADS) pf_gdn_kernel(const PfScanArgs a) 
         if (tid == 0) atomicCAS(a.status, 0, (int)HS_ERR_DEVICE);
         return;
     }
-    float *base = a.state + (size_t)b * a.nslot * a.state_elems + (size_t)h * dv * 64;
-    const int vr = tid >> 1, half = tid & 1;          // value row, half of the key columns
-    const bool live = vr < dv;
-    f2 s[16];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {                     // columns half * 4 + 8 e .. + 3: both lanes of a row read 32 bytes in a row
-        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (live) t = __ldcg(reinterpret_cast<const float4 *>(base + (size_t)slot_in * a.state_elems + (size_t)vr * 64 + 8 * e + 4 * half));
-        s[2 * e] = pk2(t.x, t.y); s[2 * e + 1] = pk2(t.z, t.w);
-    }
-    const int ntile = (n + GD_POS - 1) / GD_POS, vpc = dv / 4, PER = 32 + 2 * vpc;
-    auto fetch = [&](int t) {
-        if (t < ntile) {
-            float *st = sm + (size_t)(t % GD_STAGES) * GD_STG;      // q[8][64] k[8][64] v[8][64] z[8][64] ab[8][4]
-            const int cnt = min(GD_POS, n - t * GD_POS);
-            for (int idx = tid; idx < cnt * PER; idx += GD_THREADS) {
-                const int i = idx / PER, j = idx - i * PER;
-                const size_t row = (size_t)(row0 + t * GD_POS + i);
-                const float *xr = a.xbc + row * a.convd;
-                if (j < 16) cp16(st + i * 64 + 4 * j, xr + h * 64 + 4 * j);
-                else if (j < 32) cp16(st + 512 + i * 64 + 4 * (j - 16), xr + nk + h * 64 + 4 * (j - 16));
-                else if (j < 32 + vpc) cp16(st + 1024 + i * 64 + 4 * (j - 32), xr + 2 * nk + h * dv + 4 * (j - 32));
-                else cp16(st + 1536 + i * 64 + 4 * (j - 32 - vpc), a.zx + row * a.in_ld + 2 * nk + nv + h * dv + 4 * (j - 32 - vpc));
-            }
-            if (tid < 2 * cnt) {
-                const int i = tid >> 1, w = tid & 1;
-                cp4(st + 2048 + 4 * i + w, a.dtv + (size_t)(row0 + t * GD_POS + i) * 2 * a.heads + w * a.heads + h);
-            }
+    const int ntile = (n + SC_POS - 1) / SC_POS;
+    const int h0 = R0 / a.P, nh = (min(R0 + CR, a.di) - 1) / a.P - h0 + 1;     // heads of the block's rows (at most 4)
+    bool ok = true;
+    if (warp == SC_WARPS) {
+        // ---- producer: lane 0..7 B | C of a position, 8..15 its x, 16..23 its z, 24 the record
+        const uint32_t xbytes = (uint32_t)min(CR, a.di - R0) * 4, rbytes = (uint32_t)nh * REC_SSM * 4;
+        const int i = lane & 7, kind = lane >> 3;
+        const float *src = kind == 0 ? a.xbc + (size_t)(row0 + i) * a.convd + a.di : kind == 1 ? a.xbc + (size_t)(row0 + i) * a.convd + R0
+                         : kind == 2 ? a.zx + (size_t)(row0 + i) * a.in_ld + R0 : a.rec + ((size_t)rec_slot(row0, blockIdx.y, 0) * a.heads + h0) * REC_SSM;
+        const size_t step = kind < 2 ? (size_t)SC_POS * a.convd : kind == 2 ? (size_t)SC_POS * a.in_ld : (size_t)a.heads * REC_SSM;
+        const int dst = kind == 0 ? i * 2 * N : kind == 1 ? SC_POS * 2 * N + i * CR : kind == 2 ? SC_POS * (2 * N + CR) + i * CR : SC_POS * (2 * N + 2 * CR);
+        const uint32_t bytes = kind == 0 ? 2 * N * 4 : kind < 3 ? xbytes : rbytes;
+        int s = 0; uint32_t ph = 0;
+        for (int t = 0; t < ntile; ++t) {
+            if (!__all_sync(0xffffffffu, mbar_wait_n(&empty[s], ph ^ 1u, 1 << 20))) { ok = false; break; }
+            const int cnt = min(SC_POS, n - t * SC_POS);
+            if (lane == 0) mbar_expect_tx(&full[s], (uint32_t)cnt * (2 * N * 4 + 2 * xbytes) + rbytes);
+            __syncwarp();
+            if (kind < 3 ? i < cnt : lane == 24) bulk_tile(sm + (size_t)s * STG + dst, src, bytes, &full[s]);
+            src += step;
+            if (++s == stages) { s = 0; ph ^= 1u; }
         }
-        cp_commit();
-    };
+    } else {
+        float *base = a.state + (size_t)b * a.nslot * a.state_elems;
+        f2 st[RW][NP];
 #pragma unroll
-    for (int t = 0; t < GD_STAGES - 1; ++t) fetch(t);
+        for (int r = 0; r < RW; ++r)
+#pragma unroll
+            for (int v = 0; v < NVEC; ++v) {
+                const float *src = base + (size_t)slot_in * a.state_elems + (size_t)(Rw + r) * N + v * (32 * VW) + lane * VW;
+                float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (Rw + r < a.di) {
+                    if (VW == 4) x = __ldcg(reinterpret_cast<const float4 *>(src));
+                    else { const float2 y = __ldcg(reinterpret_cast<const float2 *>(src)); x.x = y.x; x.y = y.y; }
+                }
+                st[r][v * PPV] = pk2(x.x, x.y);
+                if (VW == 4) st[r][v * PPV + PPV - 1] = pk2(x.z, x.w);
+            }
+        // rows of the warp are finished in groups of 4, 2 and 1: eight positions x four rows are one transposing reduction
+        constexpr int GA = RW >= 4 ? 4 : RW >= 2 ? 2 : 1, GB = RW - GA;         // GB: 0, 1 or 2
+        struct Out { int i, col, row, head; float D; bool live; };
+        auto outputs = [&](int r_lo, int G) {
+            const int lpv = 32 / (SC_POS * G), v = lane / lpv;
+            Out o; o.i = v / G; const int r = r_lo + v % G;
+            o.col = warp * RW + r; o.row = Rw + r; o.live = lane % lpv == 0 && o.row < a.di;
+            const int hd = min(o.row, a.di - 1) / a.P; o.head = (hd - h0) * REC_SSM; o.D = a.D[hd];
+            return o;
+        };
+        const Out oa = outputs(0, GA), ob = outputs(GA, GB ? GB : 1);
+        // coefficient lanes: value (j, r) of the update
+        constexpr int NQ = (SC_POS * RW + 31) / 32;
+        int e_head[NQ], e_j[NQ], e_r[NQ];
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const int idx = lane + 32 * q;
+            e_j[q] = idx / RW; e_r[q] = idx - e_j[q] * RW;
+            e_head[q] = (min(Rw + e_r[q], a.di - 1) / a.P - h0) * REC_SSM;
+        }
+        const int p_head = (min(Rw + min(lane, RW - 1), a.di - 1) / a.P - h0) * REC_SSM;
+        int s = 0; uint32_t ph = 0;
 #pragma unroll 1
-    for (int t = 0; t < ntile; ++t) {
-        cp_wait<GD_STAGES - 2>();
-        __syncthreads();
-        fetch(t + GD_STAGES - 1);
-        float *st = sm + (size_t)(t % GD_STAGES) * GD_STG;
-        const int cnt = min(GD_POS, n - t * GD_POS);
-        // q and k of the tile's positions are L2-normalised in place: a warp takes four of the sixteen vectors
+        for (int t = 0; t < ntile; ++t) {
+            if (!__all_sync(0xffffffffu, mbar_wait_n(&full[s], ph, 1 << 20))) { ok = false; break; }
+            const float *sg_ = sm + (size_t)s * STG;
+            const float *xs = sg_ + SC_POS * 2 * N, *zs = xs + SC_POS * CR, *rs = zs + SC_POS * CR;
+            const int cnt = min(SC_POS, n - t * SC_POS);
+            // coefficients of the update, each stored as a pair (rows beyond the state: x is zero there)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int vec = warp * 4 + u;
-            if ((vec & 7) < cnt) {
-                float2 *p = reinterpret_cast<float2 *>(st + (vec >> 3) * 512 + (vec & 7) * 64) + lane;
-                float2 x = *p;
-                const float inv = rsqrtf(warp_sum(x.x * x.x + x.y * x.y) + 1e-6f);
-                x.x *= inv; x.y *= inv;
-                *p = x;
+            for (int q = 0; q < NQ; ++q)
+                if (lane + 32 * q < SC_POS * RW) {
+                    const float v = rs[e_head[q] + 72 + e_j[q]] * xs[e_j[q] * CR + warp * RW + e_r[q]];
+                    es[warp][e_j[q]][e_r[q]] = make_float2(v, v);
+                }
+            if (lane < RW) { const float v = rs[p_head + 71]; es[warp][SC_POS][lane] = make_float2(v, v); }
+            // products of the old state with C of every position
+            float va[SC_POS * GA], vb[SC_POS * (GB ? GB : 1)];
+#pragma unroll
+            for (int i = 0; i < SC_POS; ++i) {
+                f2 Cv[NP];
+#pragma unroll
+                for (int v = 0; v < NVEC; ++v) {
+                    const float *p = sg_ + i * 2 * N + N + v * (32 * VW) + lane * VW;
+                    if (VW == 4) { const float4 x = *reinterpret_cast<const float4 *>(p); Cv[v * PPV] = pk2(x.x, x.y); Cv[v * PPV + PPV - 1] = pk2(x.z, x.w); }
+                    else { const float2 x = *reinterpret_cast<const float2 *>(p); Cv[0] = pk2(x.x, x.y); }
+                }
+#pragma unroll
+                for (int r = 0; r < RW; ++r) {
+                    f2 y = mul2(st[r][0], Cv[0]);
+#pragma unroll
+                    for (int e = 1; e < NP; ++e) y = fma2(st[r][e], Cv[e], y);
+                    float lo, hi;
+                    up2(y, lo, hi);
+                    if (r < GA) va[i * GA + (r < GA ? r : 0)] = lo + hi;
+                    else vb[i * (GB ? GB : 1) + (r >= GA ? r - GA : 0)] = lo + hi;
+                }
             }
+            __syncwarp();                 // es complete
+            // S <- P_7 S + sum_j e_j B_j
+#pragma unroll
+            for (int r = 0; r < RW; ++r) {
+                const f2 p7 = *reinterpret_cast<const f2 *>(&es[warp][SC_POS][r]);
+#pragma unroll
+                for (int e = 0; e < NP; ++e) st[r][e] = mul2(p7, st[r][e]);
+            }
+#pragma unroll
+            for (int j = 0; j < SC_POS; ++j) {
+                f2 Bv[NP];
+#pragma unroll
+                for (int v = 0; v < NVEC; ++v) {
+                    const float *p = sg_ + j * 2 * N + v * (32 * VW) + lane * VW;
+                    if (VW == 4) { const float4 x = *reinterpret_cast<const float4 *>(p); Bv[v * PPV] = pk2(x.x, x.y); Bv[v * PPV + PPV - 1] = pk2(x.z, x.w); }
+                    else { const float2 x = *reinterpret_cast<const float2 *>(p); Bv[0] = pk2(x.x, x.y); }
+                }
+#pragma unroll
+                for (int r = 0; r < RW; ++r) {
+                    const f2 ee = *reinterpret_cast<const f2 *>(&es[warp][j][r]);
+#pragma unroll
+                    for (int e = 0; e < NP; ++e) st[r][e] = fma2(ee, Bv[e], st[r][e]);
+                }
+            }
+            // outputs: reduce over lanes, add what the tile's own positions contribute, gate
+            auto finish = [&](float tot, const Out &o) {
+                if (!o.live || o.i >= cnt) return;
+                const float4 ma = *reinterpret_cast<const float4 *>(rs + o.head + o.i * SC_POS), mb = *reinterpret_cast<const float4 *>(rs + o.head + o.i * SC_POS + 4);
+                const float *xc = xs + o.col;
+                float y = rs[o.head + 64 + o.i] * tot + o.D * xc[o.i * CR], w = ma.x * xc[0];
+                y = fmaf(ma.y, xc[CR], y); w = fmaf(ma.z, xc[2 * CR], w); y = fmaf(ma.w, xc[3 * CR], y);
+                w = fmaf(mb.x, xc[4 * CR], w); y = fmaf(mb.y, xc[5 * CR], y); w = fmaf(mb.z, xc[6 * CR], w); y = fmaf(mb.w, xc[7 * CR], y);
+                a.g[(size_t)(row0 + t * SC_POS + o.i) * a.gw + o.row] = (y + w) * silu_f(zs[o.i * CR + o.col]);
+            };
+            finish(xreduce<SC_POS * GA>(va, lane), oa);
+            if (GB) finish(xreduce<SC_POS * (GB ? GB : 1)>(vb, lane), ob);
+            __syncwarp();                 // es may be overwritten
+            if (lane == 0) mbar_arrive(&empty[s]);
+            if (++s == stages) { s = 0; ph ^= 1u; }
         }
-        __syncthreads();
-#pragma unroll 1
-        for (int i = 0; i < cnt; ++i) {
-            const float *q = st + i * 64 + 4 * half, *k = st + 512 + i * 64 + 4 * half;
-            const float alpha = st[2048 + 4 * i], beta = st[2048 + 4 * i + 1];
-            const float v = live ? st[1024 + i * 64 + vr] : 0.f;
-            f2 kv[16];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const float4 x = *reinterpret_cast<const float4 *>(k + 8 * e);
-                kv[2 * e] = pk2(x.x, x.y); kv[2 * e + 1] = pk2(x.z, x.w);
-            }
-            f2 d0 = mul2(s[0], kv[0]), d1 = mul2(s[1], kv[1]), d2 = mul2(s[2], kv[2]), d3 = mul2(s[3], kv[3]);
+        for (int r = 0; r < RW; ++r)
 #pragma unroll
-            for (int e = 4; e < 16; e += 4) {
-                d0 = fma2(s[e], kv[e], d0); d1 = fma2(s[e + 1], kv[e + 1], d1);
-                d2 = fma2(s[e + 2], kv[e + 2], d2); d3 = fma2(s[e + 3], kv[e + 3], d3);
+            for (int v = 0; v < NVEC; ++v) {
+                float *p = base + (size_t)slot_out * a.state_elems + (size_t)(Rw + r) * N + v * (32 * VW) + lane * VW;
+                float x0, x1, x2, x3;
+                up2(st[r][v * PPV], x0, x1);
+                if (Rw + r < a.di) {
+                    if (VW == 4) { up2(st[r][v * PPV + PPV - 1], x2, x3); *reinterpret_cast<float4 *>(p) = make_float4(x0, x1, x2, x3); }
+                    else *reinterpret_cast<float2 *>(p) = make_float2(x0, x1);
+                }
             }
-            float x0, x1, x2, x3, x4, x5, x6, x7;
-            up2(d0, x0, x1); up2(d1, x2, x3); up2(d2, x4, x5); up2(d3, x6, x7);
-            float dot = ((x0 + x1) + (x2 + x3)) + ((x4 + x5) + (x6 + x7));
-            dot += __shfl_xor_sync(0xffffffffu, dot, 1);
-            const float u = beta * (v - alpha * dot);
-            const f2 uu = pk2(u, u), aa = pk2(alpha, alpha);
-            f2 o0 = 0ull, o1 = 0ull;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const float4 x = *reinterpret_cast<const float4 *>(q + 8 * e);
-                s[2 * e] = fma2(aa, s[2 * e], mul2(uu, kv[2 * e]));
-                s[2 * e + 1] = fma2(aa, s[2 * e + 1], mul2(uu, kv[2 * e + 1]));
-                o0 = fma2(s[2 * e], pk2(x.x, x.y), o0); o1 = fma2(s[2 * e + 1], pk2(x.z, x.w), o1);
-            }
-            up2(o0, x0, x1); up2(o1, x2, x3);
-            float o = (x0 + x1) + (x2 + x3);
-            o += __shfl_xor_sync(0xffffffffu, o, 1);
-            if (live && half == 0) os[i][vr] = o * 0.125f;          // 1 / sqrt(64)
-        }
-        __syncthreads();
-        // per-head RMSNorm over dv, then the output gate silu(z)
-        for (int i = warp; i < cnt; i += GD_THREADS / 32) {
-            float ss = 0.f;
-            for (int j = lane; j < dv; j += 32) ss = fmaf(os[i][j], os[i][j], ss);
-            const float rstd = rsqrtf(warp_sum(ss) / (float)dv + a.eps);
-            for (int j = lane; j < dv; j += 32)
-                a.g[(size_t)(row0 + t * GD_POS + i) * a.gw + h * dv + j] = os[i][j] * rstd * a.onorm[j] * silu_f(st[1536 + i * 64 + j]);
-        }
     }
-    cp_wait<0>();
-    if (live)
+    if (!ok && lane == 0) atomicCAS(a.status, 0, (int)HS_ERR_TIMEOUT);          // a copy never landed
+    if (tid < CR && R0 + tid < a.di) shift_window(a, b, row0, n, R0 + tid);
+    if (blockIdx.x == 0)
+        for (int c = tid; c < 2 * N; c += SC_THREADS) shift_window(a, b, row0, n, a.di + c);
+    pdl_trigger();
+}
+
+// DeltaNet: q and k of a tile L2-normalised (in place), the tile's record.  grid = (tiles, heads, segments), warp = position
+__global__ void __launch_bounds__(256) pf_gdn_gram_kernel(const PfScanArgs a) {
+    __shared__ float qs[SC_POS][68], ks[SC_POS][68];
+    const int tid = threadIdx.x, i = tid >> 5, lane = tid & 31, t = blockIdx.x, h = blockIdx.y;
+    pdl_wait();
+    const int4 sg = __ldcg(a.segs + blockIdx.z);
+    const int row0 = sg.y, cnt = min(SC_POS, sg.z - t * SC_POS);
+    if (cnt <= 0) return;
+    float alpha[SC_POS], beta = 0.f;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            float x0, x1, x2, x3;
-            up2(s[2 * e], x0, x1); up2(s[2 * e + 1], x2, x3);
-            *reinterpret_cast<float4 *>(base + (size_t)slot_out * a.state_elems + (size_t)vr * 64 + 8 * e + 4 * half) = make_float4(x0, x1, x2, x3);
+    for (int j = 0; j < SC_POS; ++j) alpha[j] = j < cnt ? __ldcg(a.dtv + (size_t)(row0 + t * SC_POS + j) * 2 * a.heads + h) : 1.f;
+    if (i < cnt) {
+        beta = __ldcg(a.dtv + (size_t)(row0 + t * SC_POS + i) * 2 * a.heads + a.heads + h);
+        float2 *q = reinterpret_cast<float2 *>(a.xbc_rw + (size_t)(row0 + t * SC_POS + i) * a.convd + h * 64) + lane;
+        float2 *k = q + a.heads * 32;
+        float2 x = __ldcg(q), y = __ldcg(k);
+        const float iq = rsqrtf(warp_sum(x.x * x.x + x.y * x.y) + 1e-6f), ik = rsqrtf(warp_sum(y.x * y.x + y.y * y.y) + 1e-6f);
+        x.x *= iq; x.y *= iq; y.x *= ik; y.y *= ik;
+        *q = x; *k = y;
+        qs[i][2 * lane] = x.x; qs[i][2 * lane + 1] = x.y; ks[i][2 * lane] = y.x; ks[i][2 * lane + 1] = y.y;
+    }
+    __syncthreads();
+    // lane = (position j, quarter of the key columns)
+    const int j = lane >> 2, c0 = (lane & 3) * 16;
+    float kk = 0.f, qk = 0.f;
+    if (i < cnt && j <= i)
+#pragma unroll
+        for (int c = 0; c < 16; ++c) { kk = fmaf(ks[i][c0 + c], ks[j][c0 + c], kk); qk = fmaf(qs[i][c0 + c], ks[j][c0 + c], qk); }
+    kk += __shfl_xor_sync(0xffffffffu, kk, 1); qk += __shfl_xor_sync(0xffffffffu, qk, 1);
+    kk += __shfl_xor_sync(0xffffffffu, kk, 2); qk += __shfl_xor_sync(0xffffffffu, qk, 2);
+    float dij = 1.f, pi = 1.f, ej = i < cnt ? 1.f : 0.f;
+#pragma unroll
+    for (int u = 0; u < SC_POS; ++u) {
+        if (u > j && u <= i) dij *= alpha[u];
+        if (u <= i) pi *= alpha[u]; else ej *= alpha[u];
+    }
+    float *rec = a.rec + ((size_t)rec_slot(row0, blockIdx.z, t) * a.heads + h) * REC_GDN;
+    if ((lane & 3) == 0) {
+        rec[i * SC_POS + j] = j < i ? beta * kk * dij : 0.f;
+        rec[64 + i * SC_POS + j] = j <= i ? qk * dij : 0.f;
+    }
+    if (lane == 0) { rec[128 + i] = pi; rec[136 + i] = ej; rec[144 + i] = beta; }
+    pdl_trigger();
+}
+
+// The delta rule.  grid = (strips of 16 * RT value rows, heads, segments), four consumer warps and one producer warp; eight
+// lanes share RT rows (columns 4 c .. 4 c + 3 and 32 + 4 c .. of lane c), the tile's k vectors stay in registers between
+// the products and the update.  Every lane of a row gathers the eight right-hand sides and solves for the u_i itself:
+// one exchange instead of eight.
+constexpr int GD_STG = SC_POS * (128 + 32) + REC_GDN, GD_STAGES = 4, GD_WARPS = 4, GD_THREADS = (GD_WARPS + 1) * 32;
+
+template <int RT>
+__global__ void __launch_bounds__(GD_THREADS) pf_gdn_kernel(const PfScanArgs a) {
+    __shared__ __align__(128) float sm[GD_STAGES * GD_STG];
+    __shared__ __align__(8) uint64_t full[GD_STAGES], empty[GD_STAGES];
+    const int h = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, cl = lane & 7;
+    const int dv = a.P, nk = a.heads * 64, v0 = blockIdx.x * 16 * RT, vr = warp * 4 * RT + (lane >> 3) * RT;    // this thread's first row of the strip
+    for (int i = tid; i < GD_STAGES * GD_STG / 4; i += GD_THREADS) reinterpret_cast<float4 *>(sm)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (tid < GD_STAGES) { mbar_init(&full[tid], 1); mbar_init(&empty[tid], GD_WARPS); mbar_fence_init(); }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    pdl_wait();
+    __syncthreads();
+    const int4 sg = __ldcg(a.segs + blockIdx.z);
+    const int b = sg.x, row0 = sg.y, n = sg.z, slot_out = sg.w;
+    const int slot_in = a.nslot == 1 ? 0 : __ldcg(a.slot + b);
+    if ((unsigned)slot_in >= (unsigned)a.nslot || (unsigned)slot_out >= (unsigned)a.nslot) {
+        if (tid == 0) atomicCAS(a.status, 0, (int)HS_ERR_DEVICE);
+        return;
+    }
+    const int ntile = (n + SC_POS - 1) / SC_POS;
+    bool ok = true;
+    if (warp == GD_WARPS) {
+        // ---- producer: stage = q[8][64] k[8][64] v[8][32] record; lane 0..7 q, 8..15 k, 16..23 v, 24 the record
+        const int i = lane & 7, kind = lane >> 3;
+        const float *xr = a.xbc + (size_t)(row0 + i) * a.convd;
+        const float *src = kind == 0 ? xr + h * 64 : kind == 1 ? xr + nk + h * 64 : kind == 2 ? xr + 2 * nk + h * dv + v0
+                         : a.rec + ((size_t)rec_slot(row0, blockIdx.z, 0) * a.heads + h) * REC_GDN;
+        const size_t step = kind < 3 ? (size_t)SC_POS * a.convd : (size_t)a.heads * REC_GDN;
+        const int dst = kind < 2 ? kind * 512 + i * 64 : kind == 2 ? 1024 + i * 32 : SC_POS * 160;
+        const uint32_t bytes = kind < 2 ? 256 : kind == 2 ? 64 * RT : REC_GDN * 4;
+        int s = 0; uint32_t ph = 0;
+        for (int t = 0; t < ntile; ++t) {
+            if (!__all_sync(0xffffffffu, mbar_wait_n(&empty[s], ph ^ 1u, 1 << 20))) { ok = false; break; }
+            const int cnt = min(SC_POS, n - t * SC_POS);
+            if (lane == 0) mbar_expect_tx(&full[s], (uint32_t)cnt * (512 + 64 * RT) + REC_GDN * 4);
+            __syncwarp();
+            if (kind < 3 ? i < cnt : lane == 24) bulk_tile(sm + (size_t)s * GD_STG + dst, src, bytes, &full[s]);
+            src += step;
+            if (++s == GD_STAGES) { s = 0; ph ^= 1u; }
         }
-    for (int c = tid; c < 128 + dv; c += GD_THREADS)
-        shift_window(a, b, row0, n, c < 64 ? h * 64 + c : c < 128 ? nk + h * 64 + (c - 64) : 2 * nk + h * dv + (c - 128));
+    } else {
+        float *base = a.state + (size_t)b * a.nslot * a.state_elems + ((size_t)h * dv + v0 + vr) * 64 + 4 * cl;
+        f2 s[RT][4];
+#pragma unroll
+        for (int r = 0; r < RT; ++r)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float4 x = __ldcg(reinterpret_cast<const float4 *>(base + (size_t)slot_in * a.state_elems + r * 64 + 32 * e));
+                s[r][2 * e] = pk2(x.x, x.y); s[r][2 * e + 1] = pk2(x.z, x.w);
+            }
+        int sl = 0; uint32_t ph = 0;
+#pragma unroll 1
+        for (int t = 0; t < ntile; ++t) {
+            if (!__all_sync(0xffffffffu, mbar_wait_n(&full[sl], ph, 1 << 20))) { ok = false; break; }
+            const float *st = sm + (size_t)sl * GD_STG, *rs = st + SC_POS * 160;
+            const int cnt = min(SC_POS, n - t * SC_POS);
+            f2 kv[SC_POS][4];
+            float dk[RT][SC_POS], dq[RT][SC_POS];
+#pragma unroll
+            for (int i = 0; i < SC_POS; ++i) {
+                f2 qv[4];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float4 x = *reinterpret_cast<const float4 *>(st + 512 + i * 64 + 32 * e + 4 * cl), y = *reinterpret_cast<const float4 *>(st + i * 64 + 32 * e + 4 * cl);
+                    kv[i][2 * e] = pk2(x.x, x.y); kv[i][2 * e + 1] = pk2(x.z, x.w);
+                    qv[2 * e] = pk2(y.x, y.y); qv[2 * e + 1] = pk2(y.z, y.w);
+                }
+#pragma unroll
+                for (int r = 0; r < RT; ++r) {
+                    float lo, hi;
+                    up2(fma2(s[r][3], kv[i][3], fma2(s[r][2], kv[i][2], fma2(s[r][1], kv[i][1], mul2(s[r][0], kv[i][0])))), lo, hi);
+                    dk[r][i] = lo + hi;
+                    up2(fma2(s[r][3], qv[3], fma2(s[r][2], qv[2], fma2(s[r][1], qv[1], mul2(s[r][0], qv[0])))), lo, hi);
+                    dq[r][i] = lo + hi;
+                }
+            }
+            // transposing sums over the eight lanes of a row: lane c ends with position c
+            auto xred8 = [&](float (&v)[SC_POS]) {
+#pragma unroll
+                for (int off = 4; off >= 1; off >>= 1) {
+                    const bool up = (cl & off) != 0;
+#pragma unroll
+                    for (int q = 0; q < off; ++q) {
+                        const float keep = up ? v[q + off] : v[q], send = up ? v[q] : v[q + off];
+                        v[q] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+                    }
+                }
+                return v[0];
+            };
+            const float Pc = rs[128 + cl], bc = rs[144 + cl];
+            float u[RT][SC_POS], qo[RT];
+#pragma unroll
+            for (int r = 0; r < RT; ++r) {
+                const float sk = xred8(dk[r]);
+                qo[r] = Pc * xred8(dq[r]);
+                const float w = bc * (st[1024 + cl * 32 + vr + r] - Pc * sk);
+#pragma unroll
+                for (int i = 0; i < SC_POS; ++i) u[r][i] = __shfl_sync(0xffffffffu, w, (lane & 24) + i);
+            }
+#pragma unroll
+            for (int i = 1; i < SC_POS; ++i) {
+                const float4 ma = *reinterpret_cast<const float4 *>(rs + i * SC_POS), mb = *reinterpret_cast<const float4 *>(rs + i * SC_POS + 4);
+                const float mr[8] = {ma.x, ma.y, ma.z, ma.w, mb.x, mb.y, mb.z, mb.w};
+#pragma unroll
+                for (int r = 0; r < RT; ++r)
+#pragma unroll
+                    for (int j = 0; j < i; ++j) u[r][i] = fmaf(-mr[j], u[r][j], u[r][i]);
+            }
+            const float4 ma = *reinterpret_cast<const float4 *>(rs + 64 + cl * SC_POS), mb = *reinterpret_cast<const float4 *>(rs + 64 + cl * SC_POS + 4);
+            const float4 ea = *reinterpret_cast<const float4 *>(rs + 136), eb = *reinterpret_cast<const float4 *>(rs + 140);
+            const float p7 = rs[135], ee[8] = {ea.x, ea.y, ea.z, ea.w, eb.x, eb.y, eb.z, eb.w};
+            __syncwarp();                 // the stage has been read
+            if (lane == 0) mbar_arrive(&empty[sl]);
+            if (++sl == GD_STAGES) { sl = 0; ph ^= 1u; }
+            const f2 pp = pk2(p7, p7);
+#pragma unroll
+            for (int r = 0; r < RT; ++r) {
+                float o = qo[r];
+                o = fmaf(ma.x, u[r][0], o); o = fmaf(ma.y, u[r][1], o); o = fmaf(ma.z, u[r][2], o); o = fmaf(ma.w, u[r][3], o);
+                o = fmaf(mb.x, u[r][4], o); o = fmaf(mb.y, u[r][5], o); o = fmaf(mb.z, u[r][6], o); o = fmaf(mb.w, u[r][7], o);
+                if (cl < cnt) a.g[(size_t)(row0 + t * SC_POS + cl) * a.gw + h * dv + v0 + vr + r] = o * 0.125f;      // 1 / sqrt(64)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) s[r][e] = mul2(pp, s[r][e]);
+#pragma unroll
+                for (int j = 0; j < SC_POS; ++j) {
+                    const float c = ee[j] * u[r][j];
+                    const f2 cc = pk2(c, c);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) s[r][e] = fma2(cc, kv[j][e], s[r][e]);
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < RT; ++r)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float x0, x1, x2, x3;
+                up2(s[r][2 * e], x0, x1); up2(s[r][2 * e + 1], x2, x3);
+                *reinterpret_cast<float4 *>(base + (size_t)slot_out * a.state_elems + r * 64 + 32 * e) = make_float4(x0, x1, x2, x3);
+            }
+    }
+    if (!ok && lane == 0) atomicCAS(a.status, 0, (int)HS_ERR_TIMEOUT);
+    if (tid < 16 * RT) shift_window(a, b, row0, n, 2 * nk + h * dv + v0 + tid);
+    if (blockIdx.x == 0 && tid < 128) shift_window(a, b, row0, n, tid < 64 ? h * 64 + tid : nk + h * 64 + (tid - 64));
+    pdl_trigger();
+}
+
+// per-head RMSNorm over the dv outputs, then the gate silu(z), in place; a warp per (row, head)
+__global__ void __launch_bounds__(256) pf_gdn_out_kernel(const PfScanArgs a) {
+    const int h = blockIdx.y * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, dv = a.P;
+    pdl_wait();
+    if (h >= a.heads) return;
+    float *o = a.g + (size_t)blockIdx.x * a.gw + h * dv;
+    const float *z = a.zx + (size_t)blockIdx.x * a.in_ld + a.heads * (128 + dv) + h * dv;
+    float x[2], zz[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int j = lane + 32 * q;
+        x[q] = j < dv ? __ldcg(o + j) : 0.f; zz[q] = j < dv ? __ldcg(z + j) : 0.f;
+    }
+    const float rstd = rsqrtf(warp_sum(x[0] * x[0] + x[1] * x[1]) / (float)dv + a.eps);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int j = lane + 32 * q;
+        if (j < dv) o[j] = x[q] * rstd * a.onorm[j] * silu_f(zz[q]);
+    }
+    pdl_trigger();
 }
 
 // ---- attention ----------------------------------------------------------------------------------------------
@@ -449,7 +679,6 @@ __global__ void __launch_bounds__(PA_THREADS) pf_attn_kernel(const PfAttnArgs a)
     extern __shared__ __align__(16) unsigned char smraw[];
     __nv_bfloat16 *K_s = reinterpret_cast<__nv_bfloat16 *>(smraw), *V_s = K_s + 2 * PA_K * KS;      // [2][PA_K][KS] each
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g8 = lane >> 2, t4 = lane & 3;
-    pdl_trigger();
     pdl_wait();
     const int4 sg = __ldcg(a.segs + blockIdx.z);
     const int b = sg.x, row0 = sg.y, n = sg.z, qt = gridDim.x - 1 - blockIdx.x, h = blockIdx.y;
@@ -577,6 +806,7 @@ __global__ void __launch_bounds__(PA_THREADS) pf_attn_kernel(const PfAttnArgs a)
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) *reinterpret_cast<float2 *>(o + nt * 8) = make_float2(O[nt][2 * r] * inv, O[nt][2 * r + 1] * inv);
     }
+    pdl_trigger();
 }
 
 // ---- gathers and control words ------------------------------------------------------------------------------
@@ -611,18 +841,43 @@ cudaError_t allow_smem(K kernel, size_t bytes) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
     return e;
 }
-constexpr size_t ssm_smem(int N) { return (size_t)SC_STAGES * sc_stage_floats(N) * 4; }
-constexpr size_t GDN_SMEM = (size_t)GD_STAGES * GD_STG * 4;
 constexpr size_t pa_smem(int hd) { return (size_t)4 * PA_K * (hd + 8) * 2; }
+
+template <int EPL, int RW>
+cudaError_t launch_scan(const PfScanArgs &a, cudaStream_t s) {
+    constexpr size_t stage = (size_t)sc_stage_floats(32 * EPL, RW) * 4, alone = 116 * 1024;
+    static bool configured = false;
+    if (!configured) {
+        const cudaError_t e = allow_smem(pf_ssm_kernel<EPL, RW>, 6 * stage > alone ? 6 * stage : alone);
+        if (e != cudaSuccess) return e;
+        configured = true;
+    }
+    const dim3 grid((a.di + SC_WARPS * RW - 1) / (SC_WARPS * RW), a.nseg);
+    // at most one block per SM: ask for more than half of its shared memory, or the scheduler puts two on some SMs while
+    // others idle (3B-class, 2048 positions: 780 instead of 530 us with the first form of this kernel)
+    const bool spread = (int64_t)grid.x * grid.y <= 148;
+    const int stages = spread ? 6 : 4;
+    const size_t smem = spread && stages * stage < alone ? alone : stages * stage;
+    return launch_pdl(pf_ssm_kernel<EPL, RW>, grid, dim3(SC_THREADS), smem, s, a, stages);
+}
+template <int EPL>
+cudaError_t launch_ssm_n(const PfScanArgs &a, cudaStream_t s) {
+    const cudaError_t e = launch_pdl(pf_gram_kernel<EPL>, dim3((a.max_seg + SC_POS - 1) / SC_POS, a.nseg), dim3(256), 0, s, a);
+    if (e != cudaSuccess) return e;
+    // rows per warp: the fewest that leave at most one block on each of the 148 SMs (the time of a tile grows with them)
+    const int64_t rows = (int64_t)a.di * a.nseg;
+    if (rows <= 148 * 8) return launch_scan<EPL, 1>(a, s);
+    if (rows <= 148 * 16) return launch_scan<EPL, 2>(a, s);
+    if (rows <= 148 * 24) return launch_scan<EPL, 3>(a, s);
+    return launch_scan<EPL, 5>(a, s);
+}
 
 }  // namespace
 
+int64_t pf_record_floats(int rows, int segs, int heads, bool gdn) { return (int64_t)(rows / SC_POS + 1 + segs) * heads * (gdn ? REC_GDN : REC_SSM); }
+
 cudaError_t configure_prefill() {
-    cudaError_t e = allow_smem(pf_ssm_kernel<2>, ssm_smem(64));
-    if (e == cudaSuccess) e = allow_smem(pf_ssm_kernel<4>, ssm_smem(128));
-    if (e == cudaSuccess) e = allow_smem(pf_ssm_kernel<8>, ssm_smem(256));
-    if (e == cudaSuccess) e = allow_smem(pf_gdn_kernel, GDN_SMEM);
-    if (e == cudaSuccess) e = allow_smem(pf_attn_kernel<64>, pa_smem(64));
+    cudaError_t e = allow_smem(pf_attn_kernel<64>, pa_smem(64));
     if (e == cudaSuccess) e = allow_smem(pf_attn_kernel<128>, pa_smem(128));
     return e;
 }
@@ -633,18 +888,27 @@ cudaError_t launch_pf_embed(const __nv_bfloat16 *E, int d, int V, const int4 *ro
     return cudaGetLastError();
 }
 cudaError_t launch_pf_prep(const PfPrepArgs &a, cudaStream_t s) {
-    return launch_pdl(pf_prep_kernel, dim3((a.nrows + PREP_ROWS - 1) / PREP_ROWS, a.nconv + 1), dim3(256), 0, s, a);
+    const int pairs = (a.qh + 2 * a.kvh) * a.hd / 2;
+    return launch_pdl(pf_prep_kernel, dim3((a.nrows + PREP_ROWS - 1) / PREP_ROWS, a.nconv + (a.heads ? 1 : 0) + (a.qh ? (pairs + 255) / 256 : 0)), dim3(256), 0, s, a);
 }
-cudaError_t launch_pf_ssm(const PfScanArgs &a, cudaStream_t s) {
-    const dim3 grid(a.P / SC_ROWS, a.heads, a.nseg), block(SC_THREADS);
-    if (a.N == 64) return launch_pdl(pf_ssm_kernel<2>, grid, block, ssm_smem(64), s, a);
-    if (a.N == 128) return launch_pdl(pf_ssm_kernel<4>, grid, block, ssm_smem(128), s, a);
-    if (a.N == 256) return launch_pdl(pf_ssm_kernel<8>, grid, block, ssm_smem(256), s, a);
+cudaError_t launch_pf_ssm(const PfScanArgs &a, cudaStream_t s, int64_t *launches) {
+    *launches += 2;
+    if (a.N == 64) return launch_ssm_n<2>(a, s);
+    if (a.N == 128) return launch_ssm_n<4>(a, s);
+    if (a.N == 256) return launch_ssm_n<8>(a, s);
     return cudaErrorInvalidValue;
 }
-cudaError_t launch_pf_gdn(const PfScanArgs &a, cudaStream_t s) {
-    if (a.P > 64 || (a.P & 3)) return cudaErrorInvalidValue;
-    return launch_pdl(pf_gdn_kernel, dim3(a.heads, a.nseg), dim3(GD_THREADS), GDN_SMEM, s, a);
+cudaError_t launch_pf_gdn(const PfScanArgs &a, cudaStream_t s, int64_t *launches) {
+    if (a.P > 64 || (a.P & 15)) return cudaErrorInvalidValue;
+    *launches += 3;
+    cudaError_t e = launch_pdl(pf_gdn_gram_kernel, dim3((a.max_seg + SC_POS - 1) / SC_POS, a.heads, a.nseg), dim3(256), 0, s, a);
+    if (e != cudaSuccess) return e;
+    // two rows per lane group halve the blocks: where 16-row strips would leave several on every SM
+    if (a.P % 32 == 0 && (int64_t)(a.P / 16) * a.heads * a.nseg > 2 * 148)
+        e = launch_pdl(pf_gdn_kernel<2>, dim3(a.P / 32, a.heads, a.nseg), dim3(GD_THREADS), 0, s, a);
+    else e = launch_pdl(pf_gdn_kernel<1>, dim3(a.P / 16, a.heads, a.nseg), dim3(GD_THREADS), 0, s, a);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(pf_gdn_out_kernel, dim3(a.nrows, (a.heads + 7) / 8), dim3(256), 0, s, a);
 }
 cudaError_t launch_pf_attn(const PfAttnArgs &a, cudaStream_t s) {
     const dim3 grid((a.max_seg + PA_Q - 1) / PA_Q, a.qh, a.nseg), block(PA_THREADS);
