@@ -804,6 +804,7 @@ static int init_model(hs_model *m, const hs_config *cfg, const hs_buffers *bufs,
     CK(configure_gemv(), "configure gemv");
     CK(configure_attn(), "configure attention");
     CK(configure_prefill(), "configure prefill");
+    CK(configure_gemm_wide(), "configure wide projections");
     if (configure_gemm_tc() != cudaSuccess) { g_hs_gemm_tc = false; cudaGetLastError(); }   // falls back to several 16-row launches
     if (g_hs_tensor_maps && c.hd % 64 == 0) {     // tensor maps of every attention layer's cache (streaming attention form)
         const size_t per_layer = (size_t)v.B * c.kvh * c.kv_capacity * c.hd;

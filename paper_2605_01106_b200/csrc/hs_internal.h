@@ -176,6 +176,13 @@ extern int g_hs_tc_min_rows;      // projections with at least this many activat
 cudaError_t configure_gemm_tc();
 int gemm_tc_rows(int nrows);
 cudaError_t launch_gemm_tc(const GemvArgs &a, int32_t *status, cudaStream_t s, int64_t *launches, int *oparts);
+// activation operand packed for the tcgen05 kernels ([2][rpad][K0 + K1] at a.xb)
+cudaError_t launch_pack(const GemvArgs &a, int rpad, cudaStream_t s, int64_t *launches);
+cudaError_t hs_make_tile_map(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_rows);
+// hundreds of activation rows: persistent two-CTA tiles (kernels_gemm_wide.cu)
+bool gemm_wide_applies(int nrows, int O);
+cudaError_t configure_gemm_wide();
+cudaError_t launch_gemm_wide(const GemvArgs &a, int32_t *status, cudaStream_t s, int64_t *launches, int *oparts);
 cudaError_t configure_attn();
 
 // serial = true: launched in plain stream order (without the programmatic attribute); see model_pass

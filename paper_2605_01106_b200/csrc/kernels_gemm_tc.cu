@@ -17,6 +17,7 @@
 // once and the result does not depend on timing.
 #include "hs_internal.h"
 #include "hs_device.cuh"
+#include "gemm_tc_common.cuh"
 #include <cuda.h>
 #include <cstdio>
 #include <cstdlib>
@@ -24,8 +25,6 @@
 namespace {
 using namespace hsd;
 
-constexpr int TC_BM = 128;          // weight rows per CTA
-constexpr int TC_BK = 64;           // K columns per stage: one 128-byte swizzle atom of bf16
 constexpr int TC_THREADS = 256;    // two warps per tensor-memory lane quarter: each takes half of the columns in the epilogue
 constexpr int TC_MAXSTAGES = 8;
 
@@ -116,134 +115,6 @@ __global__ void __launch_bounds__(256) pack_kernel(const PackArgs a) {
 }
 
 // ---- the contraction ---------------------------------------------------------------------------------------
-struct TcArgs {
-    int O, nk0, nk1;            // output rows; 64-column K blocks of segment 0 / 1
-    int nrows, rpad, bnh;       // activation rows, rows per plane of the packed operand, rows per plane per CTA
-    int ns;                     // shared-memory stages (at most TC_MAXSTAGES)
-    int rb;                     // K split: activation rows of a tile each rank finishes (a power of two >= 4, rb * S >= bnh)
-    float *out; int ldo;
-    const float *resid; int rparts; int64_t rpstride;
-    int32_t *status;
-    // The packed operand may come without the 1/rms factor of its RMSNorm (a projection epilogue wrote it, see
-    // pk_out): then ss_in[p * rpad + r], p < ss_parts, are partial sums of squares of activation row r and the
-    // factor rsqrt(sum * inv_k + eps) is applied to the finished sums of that row.
-    const float *ss_in; int ss_parts; float inv_k, eps;
-    // Packed output for the projection that consumes this one's result: bf16 head | remainder planes
-    // [2][rpad][pk_ld] of (result * pk_nw[output row]), and (residual epilogue) the partial sums of squares
-    // ss_out[weight-row tile][rpad] of the results.  nullptr: not wanted.
-    __nv_bfloat16 *pk_out; int pk_ld; const float *pk_nw; float *ss_out;
-    const void *pf_ptr; long long pf_bytes;     // weights of the next projection, pulled into L2 before the wait
-    int early_trigger;          // let the next kernel start before this one has waited (else when its accumulators are complete)
-    int off_rx, off_misc;       // shared-memory carve-up behind the stages (bytes from the aligned base)
-};
-
-__device__ __forceinline__ void tma_load_2d(void *dst_smem, const CUtensorMap *map, int x, int y, uint64_t *bar) {
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                 :: "r"(smem_u32(dst_smem)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar)) : "memory");
-}
-// the same for a weight tile: streamed once per step, so marked evict-first in L2
-__device__ __forceinline__ void tma_load_2d_stream(void *dst_smem, const CUtensorMap *map, int x, int y, uint64_t *bar) {
-    uint64_t pol;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;"
-                 :: "r"(smem_u32(dst_smem)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar)), "l"(pol) : "memory");
-}
-// shared-memory operand descriptor: K-major rows of 128 bytes, 128-byte swizzle, 8-row groups 1024 bytes apart
-__device__ __forceinline__ uint64_t umma_desc(uint32_t smem_addr) {
-    const uint32_t lo = ((smem_addr >> 4) & 0x3fffu) | (1u << 16);
-    const uint32_t hi = (1024u >> 4) | (1u << 14) | (2u << 29);
-    return ((uint64_t)hi << 32) | lo;
-}
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %6, %7, %8}, p;\n\t}"
-                 :: "r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(0u), "r"(0u), "r"(0u), "r"(0u) : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint64_t *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr));
-}
-__device__ __forceinline__ void split_bf16(float x, __nv_bfloat16 &h, __nv_bfloat16 &l) {
-    h = __float2bfloat16_rn(x);
-    l = __float2bfloat16_rn(x - __bfloat162float(h));
-}
-
-// Residual of eight consecutive activation rows r0..r0+7 of weight row `row` (parts added in order); the loads
-// are issued early, so that their trip to L2 hides behind the wait that precedes the epilogue proper.
-__device__ __forceinline__ void tc_load_resid(const TcArgs &a, float (&res)[8], int r0, int nvalid, int row) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) res[j] = 0.f;
-    if (row >= a.O) return;
-    const size_t oi = (size_t)r0 * a.ldo + row;
-    for (int p = 0; p < a.rparts; ++p) {
-        const float *rp = a.resid + (size_t)p * a.rpstride + oi;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) if (j < nvalid) res[j] += __ldcg(rp + (size_t)j * a.ldo);
-    }
-}
-
-// Epilogue for eight consecutive activation rows r0..r0+7 (indices inside the launch) of weight row `row`
-// (v[j] = the finished sum of row r0 + j, 1/rms already applied); nvalid of them exist.  Every lane of the warp
-// calls it (the SwiGLU pairing and the sums of squares shuffle).  res: the residual (tc_load_resid); nw: weight
-// folded into the packed output.  Returns (residual epilogue with statistics) the warp's sum of squares of row
-// r0 + lane / 4.
-template <int EPI>
-__device__ __forceinline__ float tc_finish8(const TcArgs &a, float (&v)[8], const float (&res)[8], int r0, int nvalid, int row, float nw, int lane) {
-    if (EPI == EPI_SWIGLU) {
-        // weight rows come in (gate, up) pairs held by neighbouring lanes.  The even lane finishes the even
-        // columns of the pair, the odd lane the odd ones, so both lanes work and each evaluates one SiLU per two
-        // columns: lanes swap what the other needs (even sends its gate of column j + 1, odd its up of column j).
-        const bool odd = row & 1;
-        const bool st = (row | 1) < a.O;
-#pragma unroll
-        for (int j = 0; j < 8; j += 2) {
-            const float got = __shfl_xor_sync(0xffffffffu, odd ? v[j] : v[j + 1], 1);
-            const float gate = odd ? got : v[j], up = odd ? v[j + 1] : got;
-            const int jj = j + (odd ? 1 : 0);
-            if (st && jj < nvalid) {
-                const float r = silu_f(gate) * up;
-                if (a.pk_out) {
-                    __nv_bfloat16 h, l;
-                    split_bf16(r, h, l);
-                    __nv_bfloat16 *p = a.pk_out + (size_t)(r0 + jj) * a.pk_ld + (row >> 1);
-                    p[0] = h; p[(size_t)a.rpad * a.pk_ld] = l;
-                } else {
-                    a.out[(size_t)(r0 + jj) * a.ldo + (row >> 1)] = r;
-                }
-            }
-        }
-        return 0.f;
-    } else {
-        const bool st = row < a.O;
-        if (EPI == EPI_RESID)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] += res[j];
-        float *p = a.out + (size_t)r0 * a.ldo + row;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) if (st && j < nvalid) p[(size_t)j * a.ldo] = v[j];
-        if (EPI == EPI_RESID && a.pk_out) {
-            __nv_bfloat16 *ph = a.pk_out + (size_t)r0 * a.pk_ld + row;
-            const size_t plane = (size_t)a.rpad * a.pk_ld;
-            float ssq[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const bool live = st && j < nvalid;
-                if (live) {
-                    __nv_bfloat16 h, l;
-                    split_bf16(v[j] * nw, h, l);
-                    ph[(size_t)j * a.pk_ld] = h; ph[(size_t)j * a.pk_ld + plane] = l;
-                }
-                ssq[j] = live ? v[j] * v[j] : 0.f;
-            }
-            return xreduce<8>(ssq, lane);           // lanes 4 j .. 4 j + 3 hold the total of row r0 + j
-        }
-        return 0.f;
-    }
-}
-
 // BN: N of the MMA = 2 * bnh (head columns, then remainder columns).  EPI: the epilogue, fixed at compile time.
 template <int BN, int EPI>
 __global__ void __launch_bounds__(TC_THREADS, 2)
@@ -489,6 +360,9 @@ cudaError_t launch_tc_epi(int epi, const CUtensorMap &mA0, const CUtensorMap &mA
 bool g_hs_gemm_tc = true;
 bool g_hs_tensor_maps = false;
 
+cudaError_t hs_make_tile_map(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_rows) {
+    return make_map(map, base, rows, cols, ld, box_rows);
+}
 // K or V cache of one layer as a 2-D bf16 tensor [rows][hd]: boxes of 64 columns x 128 rows, 128-byte swizzle
 cudaError_t hs_make_kv_tensor_map(CUtensorMap *map, const void *base, uint64_t rows, int hd) {
     if (hd % 64) return cudaErrorInvalidValue;
@@ -528,9 +402,16 @@ cudaError_t configure_gemm_tc() {
 static int tc_bnh(int nrows) { int b = 16; while (b < 128 && b < nrows) b <<= 1; return b; }
 int gemm_tc_rows(int nrows) { const int b = tc_bnh(nrows); return (nrows + b - 1) / b * b; }
 
+cudaError_t launch_pack(const GemvArgs &a, int rpad, cudaStream_t s, int64_t *launches) {
+    const PackArgs p{a.x0, a.ldx0, a.K0, a.xparts, a.xpstride, a.norm_w, a.eps, a.x1, a.ldx1, a.K1, a.xb, a.nrows, rpad};
+    if (launches) ++*launches;
+    return launch_pdl(pack_kernel, dim3(rpad), dim3(256), 0, s, p);
+}
+
 cudaError_t launch_gemm_tc(const GemvArgs &a, int32_t *status, cudaStream_t s, int64_t *launches, int *oparts) {
     if ((!a.xb && !a.pk_in) || (a.K0 & 63) || (a.K1 & 63) || a.nrows < 1) return cudaErrorInvalidValue;
     const int Kt = a.K0 + a.K1;
+    if (gemm_wide_applies(a.nrows, a.O)) return launch_gemm_wide(a, status, s, launches, oparts);
     const int mtiles = (a.O + TC_BM - 1) / TC_BM, nk = Kt / TC_BK;
     // Rows per plane per CTA.  The packed operand is laid out for the largest tile (rpad rows per plane); a small
     // weight matrix is cheap to read again from L2, so its activation rows are cut into more, smaller tiles, which
@@ -584,10 +465,8 @@ cudaError_t launch_gemm_tc(const GemvArgs &a, int32_t *status, cudaStream_t s, i
     const __nv_bfloat16 *xb = a.pk_in;
     if (!xb) {
         if ((int64_t)rpad > a.xb_rows) return cudaErrorInvalidValue;
-        PackArgs p{a.x0, a.ldx0, a.K0, a.xparts, a.xpstride, a.norm_w, a.eps, a.x1, a.ldx1, a.K1, a.xb, a.nrows, rpad};
-        cudaError_t e = launch_pdl(pack_kernel, dim3(rpad), dim3(256), 0, s, p);
+        const cudaError_t e = launch_pack(a, rpad, s, launches);
         if (e != cudaSuccess) return e;
-        if (launches) ++*launches;
         xb = a.xb;
     }
     CUtensorMap mA0, mA1, mB;
