@@ -263,6 +263,8 @@ struct AttnArgs {
 };
 cudaError_t launch_attn(const AttnArgs &a, cudaStream_t s);
 extern bool g_hs_tensor_maps;   // the driver's tensor-map encoder was found (configure_gemm_tc)
+// fp32 tensor [rows][cols], row stride ld elements, boxes of box_cols x box_rows, no swizzle; outside reads zero
+cudaError_t hs_make_f32_map(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_cols, uint32_t box_rows);
 cudaError_t hs_make_kv_tensor_map(CUtensorMap *map, const void *base, uint64_t rows, int hd);
 // mixer + attention of a parallel block in one launch (verify pass); *fused = false: not applicable, nothing launched
 cudaError_t launch_ssm_attn(const SsmArgs &sa, const AttnArgs &a, cudaStream_t s, bool *fused);

@@ -193,8 +193,9 @@ __device__ __forceinline__ void shift_window(const PfScanArgs &a, int b, int row
 // Against one position at a time: 17 instead of 24 multiply-adds per state element and tile, no serial chain but the
 // eight-term solve, and one reduction over lanes per (row, position) of which 32 go together.  All of it in fp32.
 // Positions beyond the end of a segment have decay 1 and E_j = 0.
-// The tiles arrive through a ring of shared-memory stages: a producer warp issues the bulk copies of a whole tile (one
-// lane per piece), the consumer warps only wait for bytes and hand stages back - no block-wide barrier in the loop.
+// The tiles arrive through a ring of shared-memory stages: a producer thread issues a tile's four or five copies (tensor
+// copies of eight rows; one bulk copy per row and piece, 25 a tile, took 1900 cycles to issue and set the pace), the
+// consumer warps only wait for bytes and hand stages back - no block-wide barrier in the loop.
 constexpr int SC_POS = 8, SC_MAXSTAGES = 6;
 constexpr int REC_SSM = 80;       // M[8][8] P[8] E[8]
 constexpr int REC_GDN = 152;      // MK[8][8] MQ[8][8] P[8] E[8] beta[8]
@@ -203,6 +204,10 @@ __device__ __forceinline__ int rec_slot(int row0, int s, int t) { return row0 / 
 __device__ __forceinline__ void bulk_tile(void *dst_smem, const void *src, uint32_t bytes, uint64_t *bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  :: "r"(smem_u32(dst_smem)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void tensor_tile(void *dst_smem, const CUtensorMap *map, int x, int y, uint64_t *bar) {
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                 :: "r"(smem_u32(dst_smem)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar)) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(bar)) : "memory");
@@ -271,18 +276,19 @@ constexpr int SC_WARPS = 8, SC_THREADS = (SC_WARPS + 1) * 32;
 __host__ __device__ constexpr int sc_stage_floats(int N, int RW) { return SC_POS * (2 * N + 2 * SC_WARPS * RW) + 4 * REC_SSM; }
 
 template <int EPL, int RW>
-__global__ void __launch_bounds__(SC_THREADS) pf_ssm_kernel(const PfScanArgs a, const int stages) {
+__global__ void __launch_bounds__(SC_THREADS)
+pf_ssm_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mBC, const __grid_constant__ CUtensorMap mX,
+              const __grid_constant__ CUtensorMap mZ, const int stages) {
     constexpr int N = 32 * EPL, VW = EPL < 4 ? EPL : 4, NVEC = EPL / VW, NP = EPL / 2, PPV = NP / NVEC;
     constexpr int CR = SC_WARPS * RW, STG = sc_stage_floats(N, RW), RWP = (RW + 1) & ~1;
-    extern __shared__ __align__(128) float sm[];
+    constexpr int BCW = 2 * N < 256 ? 2 * N : 256;                             // columns of one B | C copy
+    extern __shared__ __align__(128) float sm_raw[];
+    float *sm = sm_raw + ((128u - (smem_u32(sm_raw) & 127u)) & 127u) / 4;
     __shared__ __align__(16) float2 es[SC_WARPS][SC_POS + 1][RWP];             // per warp: E_j x_j of its rows, then P_7; each twice
     __shared__ __align__(8) uint64_t full[SC_MAXSTAGES], empty[SC_MAXSTAGES];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int R0 = blockIdx.x * CR, Rw = R0 + warp * RW;                       // first row of the block / of the warp
-    // positions a last tile does not have keep whatever a stage holds: finite values (their coefficients are zero)
-    for (int i = tid; i < stages * STG / 4; i += SC_THREADS) reinterpret_cast<float4 *>(sm)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (tid < stages) { mbar_init(&full[tid], 1); mbar_init(&empty[tid], SC_WARPS); mbar_fence_init(); }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     pdl_wait();
     __syncthreads();
     const int4 sg = __ldcg(a.segs + blockIdx.y);
@@ -296,23 +302,25 @@ __global__ void __launch_bounds__(SC_THREADS) pf_ssm_kernel(const PfScanArgs a, 
     const int h0 = R0 / a.P, nh = (min(R0 + CR, a.di) - 1) / a.P - h0 + 1;     // heads of the block's rows (at most 4)
     bool ok = true;
     if (warp == SC_WARPS) {
-        // ---- producer: lane 0..7 B | C of a position, 8..15 its x, 16..23 its z, 24 the record
-        const uint32_t xbytes = (uint32_t)min(CR, a.di - R0) * 4, rbytes = (uint32_t)nh * REC_SSM * 4;
-        const int i = lane & 7, kind = lane >> 3;
-        const float *src = kind == 0 ? a.xbc + (size_t)(row0 + i) * a.convd + a.di : kind == 1 ? a.xbc + (size_t)(row0 + i) * a.convd + R0
-                         : kind == 2 ? a.zx + (size_t)(row0 + i) * a.in_ld + R0 : a.rec + ((size_t)rec_slot(row0, blockIdx.y, 0) * a.heads + h0) * REC_SSM;
-        const size_t step = kind < 2 ? (size_t)SC_POS * a.convd : kind == 2 ? (size_t)SC_POS * a.in_ld : (size_t)a.heads * REC_SSM;
-        const int dst = kind == 0 ? i * 2 * N : kind == 1 ? SC_POS * 2 * N + i * CR : kind == 2 ? SC_POS * (2 * N + CR) + i * CR : SC_POS * (2 * N + 2 * CR);
-        const uint32_t bytes = kind == 0 ? 2 * N * 4 : kind < 3 ? xbytes : rbytes;
-        int s = 0; uint32_t ph = 0;
-        for (int t = 0; t < ntile; ++t) {
-            if (!__all_sync(0xffffffffu, mbar_wait_n(&empty[s], ph ^ 1u, 1 << 20))) { ok = false; break; }
-            const int cnt = min(SC_POS, n - t * SC_POS);
-            if (lane == 0) mbar_expect_tx(&full[s], (uint32_t)cnt * (2 * N * 4 + 2 * xbytes) + rbytes);
-            __syncwarp();
-            if (kind < 3 ? i < cnt : lane == 24) bulk_tile(sm + (size_t)s * STG + dst, src, bytes, &full[s]);
-            src += step;
-            if (++s == stages) { s = 0; ph ^= 1u; }
+        // ---- producer.  Rows behind a segment's end belong to the next one or lie outside the tensor (zero): finite
+        // values with zero coefficients
+        if (lane == 0) {
+            const float *rec = a.rec + ((size_t)rec_slot(row0, blockIdx.y, 0) * a.heads + h0) * REC_SSM;
+            const uint32_t rbytes = (uint32_t)nh * REC_SSM * 4;
+            int s = 0; uint32_t ph = 0;
+            for (int t = 0; t < ntile; ++t) {
+                if (!mbar_wait_n(&empty[s], ph ^ 1u, 1 << 20)) { ok = false; break; }
+                float *dst = sm + (size_t)s * STG;
+                const int y = row0 + t * SC_POS;
+                mbar_expect_tx(&full[s], (uint32_t)SC_POS * (2 * N + 2 * CR) * 4 + rbytes);
+#pragma unroll
+                for (int q = 0; q < 2 * N / BCW; ++q) tensor_tile(dst + q * SC_POS * BCW, &mBC, a.di + q * BCW, y, &full[s]);
+                tensor_tile(dst + SC_POS * 2 * N, &mX, R0, y, &full[s]);
+                tensor_tile(dst + SC_POS * (2 * N + CR), &mZ, R0, y, &full[s]);
+                bulk_tile(dst + SC_POS * (2 * N + 2 * CR), rec, rbytes, &full[s]);
+                rec += (size_t)a.heads * REC_SSM;
+                if (++s == stages) { s = 0; ph ^= 1u; }
+            }
         }
     } else {
         float *base = a.state + (size_t)b * a.nslot * a.state_elems;
@@ -358,7 +366,9 @@ __global__ void __launch_bounds__(SC_THREADS) pf_ssm_kernel(const PfScanArgs a, 
             const float *sg_ = sm + (size_t)s * STG;
             const float *xs = sg_ + SC_POS * 2 * N, *zs = xs + SC_POS * CR, *rs = zs + SC_POS * CR;
             const int cnt = min(SC_POS, n - t * SC_POS);
-            // coefficients of the update, each stored as a pair (rows beyond the state: x is zero there)
+            // position i of B (which = 0) or C (1): with N = 256 they are two copies, else one of 2 N columns
+            auto vec = [&](int i, int which) { return sg_ + (2 * N > 256 ? which * SC_POS * N + i * N : i * 2 * N + which * N) + lane * VW; };
+            // coefficients of the update, each stored as a pair
 #pragma unroll
             for (int q = 0; q < NQ; ++q)
                 if (lane + 32 * q < SC_POS * RW) {
@@ -373,7 +383,7 @@ __global__ void __launch_bounds__(SC_THREADS) pf_ssm_kernel(const PfScanArgs a, 
                 f2 Cv[NP];
 #pragma unroll
                 for (int v = 0; v < NVEC; ++v) {
-                    const float *p = sg_ + i * 2 * N + N + v * (32 * VW) + lane * VW;
+                    const float *p = vec(i, 1) + v * (32 * VW);
                     if (VW == 4) { const float4 x = *reinterpret_cast<const float4 *>(p); Cv[v * PPV] = pk2(x.x, x.y); Cv[v * PPV + PPV - 1] = pk2(x.z, x.w); }
                     else { const float2 x = *reinterpret_cast<const float2 *>(p); Cv[0] = pk2(x.x, x.y); }
                 }
@@ -401,7 +411,7 @@ __global__ void __launch_bounds__(SC_THREADS) pf_ssm_kernel(const PfScanArgs a, 
                 f2 Bv[NP];
 #pragma unroll
                 for (int v = 0; v < NVEC; ++v) {
-                    const float *p = sg_ + j * 2 * N + v * (32 * VW) + lane * VW;
+                    const float *p = vec(j, 0) + v * (32 * VW);
                     if (VW == 4) { const float4 x = *reinterpret_cast<const float4 *>(p); Bv[v * PPV] = pk2(x.x, x.y); Bv[v * PPV + PPV - 1] = pk2(x.z, x.w); }
                     else { const float2 x = *reinterpret_cast<const float2 *>(p); Bv[0] = pk2(x.x, x.y); }
                 }
@@ -497,17 +507,16 @@ __global__ void __launch_bounds__(256) pf_gdn_gram_kernel(const PfScanArgs a) {
 // lanes share RT rows (columns 4 c .. 4 c + 3 and 32 + 4 c .. of lane c), the tile's k vectors stay in registers between
 // the products and the update.  Every lane of a row gathers the eight right-hand sides and solves for the u_i itself:
 // one exchange instead of eight.
-constexpr int GD_STG = SC_POS * (128 + 32) + REC_GDN, GD_STAGES = 4, GD_WARPS = 4, GD_THREADS = (GD_WARPS + 1) * 32;
+constexpr int GD_STG = (SC_POS * (128 + 32) + REC_GDN + 31) / 32 * 32, GD_STAGES = 4, GD_WARPS = 4, GD_THREADS = (GD_WARPS + 1) * 32;
 
 template <int RT>
-__global__ void __launch_bounds__(GD_THREADS) pf_gdn_kernel(const PfScanArgs a) {
+__global__ void __launch_bounds__(GD_THREADS)
+pf_gdn_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mQK, const __grid_constant__ CUtensorMap mV) {
     __shared__ __align__(128) float sm[GD_STAGES * GD_STG];
     __shared__ __align__(8) uint64_t full[GD_STAGES], empty[GD_STAGES];
     const int h = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, cl = lane & 7;
     const int dv = a.P, nk = a.heads * 64, v0 = blockIdx.x * 16 * RT, vr = warp * 4 * RT + (lane >> 3) * RT;    // this thread's first row of the strip
-    for (int i = tid; i < GD_STAGES * GD_STG / 4; i += GD_THREADS) reinterpret_cast<float4 *>(sm)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (tid < GD_STAGES) { mbar_init(&full[tid], 1); mbar_init(&empty[tid], GD_WARPS); mbar_fence_init(); }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     pdl_wait();
     __syncthreads();
     const int4 sg = __ldcg(a.segs + blockIdx.z);
@@ -520,23 +529,22 @@ __global__ void __launch_bounds__(GD_THREADS) pf_gdn_kernel(const PfScanArgs a) 
     const int ntile = (n + SC_POS - 1) / SC_POS;
     bool ok = true;
     if (warp == GD_WARPS) {
-        // ---- producer: stage = q[8][64] k[8][64] v[8][32] record; lane 0..7 q, 8..15 k, 16..23 v, 24 the record
-        const int i = lane & 7, kind = lane >> 3;
-        const float *xr = a.xbc + (size_t)(row0 + i) * a.convd;
-        const float *src = kind == 0 ? xr + h * 64 : kind == 1 ? xr + nk + h * 64 : kind == 2 ? xr + 2 * nk + h * dv + v0
-                         : a.rec + ((size_t)rec_slot(row0, blockIdx.z, 0) * a.heads + h) * REC_GDN;
-        const size_t step = kind < 3 ? (size_t)SC_POS * a.convd : (size_t)a.heads * REC_GDN;
-        const int dst = kind < 2 ? kind * 512 + i * 64 : kind == 2 ? 1024 + i * 32 : SC_POS * 160;
-        const uint32_t bytes = kind < 2 ? 256 : kind == 2 ? 64 * RT : REC_GDN * 4;
-        int s = 0; uint32_t ph = 0;
-        for (int t = 0; t < ntile; ++t) {
-            if (!__all_sync(0xffffffffu, mbar_wait_n(&empty[s], ph ^ 1u, 1 << 20))) { ok = false; break; }
-            const int cnt = min(SC_POS, n - t * SC_POS);
-            if (lane == 0) mbar_expect_tx(&full[s], (uint32_t)cnt * (512 + 64 * RT) + REC_GDN * 4);
-            __syncwarp();
-            if (kind < 3 ? i < cnt : lane == 24) bulk_tile(sm + (size_t)s * GD_STG + dst, src, bytes, &full[s]);
-            src += step;
-            if (++s == GD_STAGES) { s = 0; ph ^= 1u; }
+        // ---- producer: stage = q[8][64] k[8][64] v[8][16 RT] record
+        if (lane == 0) {
+            const float *rec = a.rec + ((size_t)rec_slot(row0, blockIdx.z, 0) * a.heads + h) * REC_GDN;
+            int s = 0; uint32_t ph = 0;
+            for (int t = 0; t < ntile; ++t) {
+                if (!mbar_wait_n(&empty[s], ph ^ 1u, 1 << 20)) { ok = false; break; }
+                float *dst = sm + (size_t)s * GD_STG;
+                const int y = row0 + t * SC_POS;
+                mbar_expect_tx(&full[s], SC_POS * (128 + 16 * RT) * 4 + REC_GDN * 4);
+                tensor_tile(dst, &mQK, h * 64, y, &full[s]);
+                tensor_tile(dst + 512, &mQK, nk + h * 64, y, &full[s]);
+                tensor_tile(dst + 1024, &mV, 2 * nk + h * dv + v0, y, &full[s]);
+                bulk_tile(dst + SC_POS * 160, rec, REC_GDN * 4, &full[s]);
+                rec += (size_t)a.heads * REC_GDN;
+                if (++s == GD_STAGES) { s = 0; ph ^= 1u; }
+            }
         }
     } else {
         float *base = a.state + (size_t)b * a.nslot * a.state_elems + ((size_t)h * dv + v0 + vr) * 64 + 4 * cl;
@@ -593,7 +601,7 @@ __global__ void __launch_bounds__(GD_THREADS) pf_gdn_kernel(const PfScanArgs a) 
             for (int r = 0; r < RT; ++r) {
                 const float sk = xred8(dk[r]);
                 qo[r] = Pc * xred8(dq[r]);
-                const float w = bc * (st[1024 + cl * 32 + vr + r] - Pc * sk);
+                const float w = bc * (st[1024 + cl * 16 * RT + vr + r] - Pc * sk);
 #pragma unroll
                 for (int i = 0; i < SC_POS; ++i) u[r][i] = __shfl_sync(0xffffffffu, w, (lane & 24) + i);
             }
@@ -848,7 +856,7 @@ cudaError_t launch_scan(const PfScanArgs &a, cudaStream_t s) {
     constexpr size_t stage = (size_t)sc_stage_floats(32 * EPL, RW) * 4, alone = 116 * 1024;
     static bool configured = false;
     if (!configured) {
-        const cudaError_t e = allow_smem(pf_ssm_kernel<EPL, RW>, 6 * stage > alone ? 6 * stage : alone);
+        const cudaError_t e = allow_smem(pf_ssm_kernel<EPL, RW>, 6 * stage + 128 > alone ? 6 * stage + 128 : alone);
         if (e != cudaSuccess) return e;
         configured = true;
     }
@@ -857,8 +865,14 @@ cudaError_t launch_scan(const PfScanArgs &a, cudaStream_t s) {
     // others idle (3B-class, 2048 positions: 780 instead of 530 us with the first form of this kernel)
     const bool spread = (int64_t)grid.x * grid.y <= 148;
     const int stages = spread ? 6 : 4;
-    const size_t smem = spread && stages * stage < alone ? alone : stages * stage;
-    return launch_pdl(pf_ssm_kernel<EPL, RW>, grid, dim3(SC_THREADS), smem, s, a, stages);
+    const size_t smem = spread && stages * stage + 128 < alone ? alone : stages * stage + 128;
+    constexpr int N = 32 * EPL;
+    CUtensorMap mBC, mX, mZ;
+    cudaError_t e = hs_make_f32_map(&mBC, a.xbc, a.nrows, a.convd, a.convd, 2 * N < 256 ? 2 * N : 256, SC_POS);
+    if (e == cudaSuccess) e = hs_make_f32_map(&mX, a.xbc, a.nrows, a.convd, a.convd, SC_WARPS * RW, SC_POS);
+    if (e == cudaSuccess) e = hs_make_f32_map(&mZ, a.zx, a.nrows, a.di, a.in_ld, SC_WARPS * RW, SC_POS);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(pf_ssm_kernel<EPL, RW>, grid, dim3(SC_THREADS), smem, s, a, mBC, mX, mZ, stages);
 }
 template <int EPL>
 cudaError_t launch_ssm_n(const PfScanArgs &a, cudaStream_t s) {
@@ -904,9 +918,13 @@ cudaError_t launch_pf_gdn(const PfScanArgs &a, cudaStream_t s, int64_t *launches
     cudaError_t e = launch_pdl(pf_gdn_gram_kernel, dim3((a.max_seg + SC_POS - 1) / SC_POS, a.heads, a.nseg), dim3(256), 0, s, a);
     if (e != cudaSuccess) return e;
     // two rows per lane group halve the blocks: where 16-row strips would leave several on every SM
-    if (a.P % 32 == 0 && (int64_t)(a.P / 16) * a.heads * a.nseg > 2 * 148)
-        e = launch_pdl(pf_gdn_kernel<2>, dim3(a.P / 32, a.heads, a.nseg), dim3(GD_THREADS), 0, s, a);
-    else e = launch_pdl(pf_gdn_kernel<1>, dim3(a.P / 16, a.heads, a.nseg), dim3(GD_THREADS), 0, s, a);
+    const int RT = a.P % 32 == 0 && (int64_t)(a.P / 16) * a.heads * a.nseg > 2 * 148 ? 2 : 1;
+    CUtensorMap mQK, mV;
+    e = hs_make_f32_map(&mQK, a.xbc, a.nrows, a.convd, a.convd, 64, SC_POS);
+    if (e == cudaSuccess) e = hs_make_f32_map(&mV, a.xbc, a.nrows, a.convd, a.convd, 16 * RT, SC_POS);
+    if (e != cudaSuccess) return e;
+    const dim3 grid(a.P / (16 * RT), a.heads, a.nseg);
+    e = RT == 2 ? launch_pdl(pf_gdn_kernel<2>, grid, dim3(GD_THREADS), 0, s, a, mQK, mV) : launch_pdl(pf_gdn_kernel<1>, grid, dim3(GD_THREADS), 0, s, a, mQK, mV);
     if (e != cudaSuccess) return e;
     return launch_pdl(pf_gdn_out_kernel, dim3(a.nrows, (a.heads + 7) / 8), dim3(256), 0, s, a);
 }
