@@ -136,7 +136,7 @@ int64_t tc_rows_max(const Derived &v) { return std::max<int64_t>(gemm_tc_rows(v.
 // layout of the work buffer; base may be null to only measure
 struct WorkLayout {
     int64_t kv_len, slot, cand, g, margin, n_acc, emitted, stage_n, stage_next, status, counters, am_counters, dslot;
-    int64_t rope, h, zx, gbuf, obuf, abuf, logits, dlogits, att_acc, att_ml, am_part, xb, xb_h, xb_a, ssbuf;
+    int64_t rope, h, zx, gbuf, obuf, abuf, logits, dlogits, dstat, att_acc, att_ml, am_part, xb, xb_h, xb_a, ssbuf;
     int64_t pf_rowtab, pf_segtab, pf_list, pf_xbc, pf_dtv, pf_hfin, pf_q, pf_rec, total;
 };
 
@@ -160,6 +160,7 @@ WorkLayout work_layout(const hs_config &c, const Derived &v) {
     w.abuf = take((int64_t)4 * v.R * c.ff);
     w.logits = take((int64_t)4 * v.R * c.V);
     w.dlogits = take((int64_t)4 * v.B * std::max(c.max_k, 1) * c.V);
+    w.dstat = take((int64_t)8 * v.B * std::max(c.max_k, 1));
     w.att_acc = take((int64_t)4 * v.B * c.kvh * v.att_nch * HS_MAX_GT * c.hd);
     w.att_ml = take((int64_t)4 * v.B * c.kvh * v.att_nch * HS_MAX_GT * 2);
     w.am_part = take((int64_t)16 * v.R * HS_ARGMAX_CHUNKS);
@@ -474,7 +475,7 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
     if (tc_pass && h_packed) { lm.pk_in = m->xb_h; lm.ss_in = m->ssbuf; lm.ss_parts = ss_parts; }
     PROF(HS_PROF_GEMV, gemv_bytes(lm), launch_gemv(lm, st_w, s, &m->launches, nullptr), "lm_head");
     if (sampled) PROF(HS_PROF_ARGMAX, 0, launch_sample(m->dlogits + (size_t)step * c.V, dstride, c.V, m->Tm, b0, nb, m->tau, m->u_draft, c.max_k, step,
-                                                       m->ctrl.cand, step + 1, s), "draft draw");
+                                                       m->ctrl.cand, step + 1, m->dstat, std::max(c.max_k, 1), s), "draft draw");
     else if (draft) PROF(HS_PROF_ARGMAX, 0, launch_argmax(m->logits, c.V, 1, b0, nb, m->Tm, m->ctrl.cand, step + 1, nullptr, m->am_part, m->ctrl.am_counters, s), "argmax");
     else PROF(HS_PROF_ARGMAX, 0, launch_argmax(m->logits, c.V, T, b0, nb, m->Tm, m->ctrl.g, 0, m->ctrl.margin, m->am_part, m->ctrl.am_counters, s), "argmax");
     ++m->launches;
@@ -781,7 +782,7 @@ static int init_model(hs_model *m, const hs_config *cfg, const hs_buffers *bufs,
     m->ctrl.dslot = (int32_t *)(w + wl.dslot);
     m->rope = (float2 *)(w + wl.rope);
     m->hbuf[0] = (float *)(w + wl.h); m->hbuf[1] = m->hbuf[0] + std::max<size_t>((size_t)HS_H_PARTS * v.R, v.pf_rows) * c.d; m->zx = (float *)(w + wl.zx); m->gbuf = (float *)(w + wl.gbuf);
-    m->obuf = (float *)(w + wl.obuf); m->abuf = (float *)(w + wl.abuf); m->logits = (float *)(w + wl.logits); m->dlogits = (float *)(w + wl.dlogits);
+    m->obuf = (float *)(w + wl.obuf); m->abuf = (float *)(w + wl.abuf); m->logits = (float *)(w + wl.logits); m->dlogits = (float *)(w + wl.dlogits); m->dstat = (float2 *)(w + wl.dstat);
     m->tau = 0.f; m->u_draft = m->u_accept = m->u_final = nullptr;
     m->att_acc = (float *)(w + wl.att_acc); m->att_ml = (float *)(w + wl.att_ml); m->am_part = w + wl.am_part; m->xb = (__nv_bfloat16 *)(w + wl.xb); m->xb_rows = tc_rows_max(v);
     m->pf_rows = v.pf_rows; m->pf_rowtab = (int4 *)(w + wl.pf_rowtab); m->pf_segtab = (int4 *)(w + wl.pf_segtab); m->pf_list = (int2 *)(w + wl.pf_list);
@@ -958,7 +959,7 @@ int hs_accept_rollback(hs_model *m, const int32_t *forced_n_dev, const int32_t *
     if (m->tau > 0.f && !forced_n_dev) {
         // Eq. 6: the accept length and the correction / bonus token are drawn on the device, then applied like forced ones
         if (!m->sampled_draft && k > 0) return fail(m, HS_ERR_ORDER, "sampling needs the draft distributions of this round: hs_draft at the same temperature, or forced accept lengths");
-        PROF(HS_PROF_ACCEPT, 0, launch_spec_accept(m->dlogits, (int64_t)std::max(m->c.max_k, 1) * m->c.V, m->logits, m->ctrl.cand, m->u_accept, m->u_final,
+        PROF(HS_PROF_ACCEPT, 0, launch_spec_accept(m->dlogits, (int64_t)std::max(m->c.max_k, 1) * m->c.V, m->dstat, std::max(m->c.max_k, 1), m->logits, m->ctrl.cand, m->u_accept, m->u_final,
                                                    m->c.max_k, m->ctrl.stage_n, m->ctrl.stage_next, m->c.V, m->Tm, k, 0, nb, m->tau, m->stream), "sampled accept");
         ++m->launches;
         forced_n_dev = m->ctrl.stage_n;

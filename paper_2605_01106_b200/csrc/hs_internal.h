@@ -72,6 +72,7 @@ struct hs_model {
     float *hbuf[2];            // residual stream, ping-pong; each [HS_H_PARTS][B*Tm][d] partial sums
     float *zx, *gbuf, *obuf, *abuf, *logits;
     float *dlogits;            // [B][max(max_k,1)][V] logits of the draft steps (kept for Eq. 6)
+    float2 *dstat;             // [B][max(max_k,1)] (max, sum of exponentials) of those rows, from the draws
     float tau;                 // sampling temperature; 0: greedy
     const float *u_draft, *u_accept, *u_final;   // DEVICE uniforms of the round: [B][max_k], [B][max_k], [B]
     float *att_acc, *att_ml;
@@ -287,8 +288,8 @@ cudaError_t launch_accept(const AcceptArgs &a, cudaStream_t s);
 cudaError_t launch_wait_probe(int32_t *status, int polls, cudaStream_t s);
 // speculative sampling (Eq. 6): a draft draw from softmax(logits / tau), and the accept / correction / bonus decision
 cudaError_t launch_sample(const float *logits, int64_t row_stride, int V, int Tm, int b0, int nb, float tau,
-                          const float *u, int u_stride, int u_col, int32_t *tok_out, int tok_col, cudaStream_t s);
-cudaError_t launch_spec_accept(const float *dlogits, int64_t d_seq_stride, const float *vlogits, const int32_t *cand,
+                          const float *u, int u_stride, int u_col, int32_t *tok_out, int tok_col, float2 *stat, int stat_stride, cudaStream_t s);
+cudaError_t launch_spec_accept(const float *dlogits, int64_t d_seq_stride, const float2 *stat, int stat_stride, const float *vlogits, const int32_t *cand,
                                const float *u_acc, const float *u_final, int u_stride, int32_t *n_out, int32_t *next_out,
                                int V, int Tm, int k, int b0, int nb, float tau, cudaStream_t s);
 

@@ -174,71 +174,155 @@ __global__ void accept_kernel(AcceptArgs a) {
 }
 
 // ------------------------------------------------------------------------------------------------
-// Speculative sampling at temperature > 0 (paper Sec. 3.3, Eq. 6).  One block per sequence; a logits row is
-// walked in per-thread contiguous segments so that every sum has a fixed order (reproducible draws).
-constexpr int SP_THREADS = 1024;
+// Speculative sampling at temperature > 0 (paper Sec. 3.3, Eq. 6).  One cluster of eight CTAs per sequence: each takes a
+// contiguous eighth of the vocabulary and the CTAs exchange row maxima, sums and segment totals through distributed shared
+// memory (one barrier per exchange).  Every sum has a fixed order, so draws are reproducible.
+// Bound by latency: two or three sweeps over a logits row that sits in L2.  (One block of 1024 threads per sequence, each
+// thread walking a contiguous segment and adding up all 1024 segment totals by itself, took 150-400 us a row at 32768 ids.)
+constexpr int SP_CL = 8, SP_THREADS = 512, SP_WARPS = SP_THREADS / 32;
+constexpr int SP_BLOCKS = 1024;            // blocks of 32 * m ids a CTA's share is divided into, at most
 
-struct RowStat { float mx, Z; };
-
-// max and sum of exp((l - max) / tau) of one row; every thread returns the same values
-__device__ __forceinline__ RowStat sp_row_stat(const float *row, int V, float inv_tau, float *red_s) {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    float mx = -INFINITY;
-    for (int j = tid; j < V; j += SP_THREADS) mx = fmaxf(mx, __ldcg(row + j));
-    mx = warp_max(mx);
-    __syncthreads();
-    if (lane == 0) red_s[warp] = mx;
-    __syncthreads();
-    mx = red_s[0];
-    for (int w = 1; w < SP_THREADS / 32; ++w) mx = fmaxf(mx, red_s[w]);
-    float z = 0.f;
-    for (int j = tid; j < V; j += SP_THREADS) z += expf((__ldcg(row + j) - mx) * inv_tau);
-    z = warp_sum(z);
-    __syncthreads();
-    if (lane == 0) red_s[warp] = z;
-    __syncthreads();
-    z = 0.f;
-    for (int w = 0; w < SP_THREADS / 32; ++w) z += red_s[w];
-    return RowStat{mx, z};
+// A CTA's share of the vocabulary: ids [lo, hi), block i = ids lo + i * 32 m .., one warp per block
+struct SpShare { int lo, hi, m, nblk, rank; };
+__device__ __forceinline__ SpShare sp_share(int V) {
+    SpShare s;
+    s.rank = (int)(blockIdx.x % SP_CL);
+    const int per = ((V + SP_CL - 1) / SP_CL + 31) & ~31;
+    s.lo = min(V, s.rank * per); s.hi = min(V, s.lo + per);
+    s.m = (per / 32 + SP_BLOCKS - 1) / SP_BLOCKS;
+    s.nblk = (s.hi - s.lo + 32 * s.m - 1) / (32 * s.m);
+    return s;
 }
 
-// Inverse-CDF draw from the unnormalised weights wf(j) >= 0: the smallest j whose cumulative weight exceeds u * total.
-// Thread t owns the contiguous segment [t * S, (t + 1) * S); segment sums are scanned in thread order.  Returns the
-// index (the same in every thread), or -1 if the total is not positive.
-template <class WF>
-__device__ __forceinline__ int sp_draw(WF wf, int V, float u, float *seg_s, int *pick_s) {
-    const int tid = threadIdx.x;
-    const int S = (V + SP_THREADS - 1) / SP_THREADS, j0 = tid * S, j1 = min(V, j0 + S);
-    float seg = 0.f;
-    for (int j = j0; j < j1; ++j) seg += wf(j);
-    __syncthreads();
-    seg_s[tid] = seg;
-    if (tid == 0) { pick_s[0] = 0x7fffffff; pick_s[1] = 0; }
-    __syncthreads();
-    // exclusive prefix of this thread's segment and the total: plain ordered sums (1024 adds, once per draw)
-    float excl = 0.f, tot = 0.f;
-    for (int i = 0; i < SP_THREADS; ++i) { const float v = seg_s[i]; if (i < tid) excl += v; tot += v; }
-    if (!(tot > 0.f)) return -1;
-    const float t = u * tot;
-    if (seg > 0.f && excl + seg > t) atomicMin(pick_s, tid);       // the first segment that reaches past the threshold
-    __syncthreads();
-    int owner = *pick_s;
-    __syncthreads();
-    if (owner == 0x7fffffff) {                                     // u * total rounded up to the total: the last positive segment
-        if (seg > 0.f) atomicMax(pick_s + 1, tid);
-        __syncthreads();
-        owner = pick_s[1];
+struct SpSmem {
+    float red[SP_WARPS][HS_MAX_T], gat[3][SP_CL][HS_MAX_T], blk[SP_BLOCKS];
+    int n;
+};
+// every rank's v[0 .. cnt) (in shared memory, complete) to every rank: g[rank][i]
+__device__ __forceinline__ void sp_gather(float (*g)[HS_MAX_T], const float *v, int cnt, int rank) {
+    for (int i = threadIdx.x; i < SP_CL * cnt; i += SP_THREADS) {
+        const int dest = i / cnt, k = i - dest * cnt;
+        dsmem_st_f32(dsmem_addr(smem_u32(&g[rank][k]), (uint32_t)dest), v[k]);
     }
-    if (tid == owner) {
-        float c = excl; int pick = -1, lastpos = j0;
-        for (int j = j0; j < j1; ++j) {
-            const float w = wf(j);
-            if (w > 0.f) { lastpos = j; c += w; if (c > t) { pick = j; break; } }
+    cluster_arrive(); cluster_wait();
+}
+
+// maximum and sum of exp((l - max) / tau) of `rows` logits rows (V floats apart): afterwards gat[0] and gat[1] hold every rank's
+// local maxima and sums, sp_max / sp_sum combine them in rank order
+__device__ __forceinline__ float sp_max(const SpSmem &s, int i) {
+    float m = s.gat[0][0][i];
+#pragma unroll
+    for (int r = 1; r < SP_CL; ++r) m = fmaxf(m, s.gat[0][r][i]);
+    return m;
+}
+__device__ __forceinline__ float sp_sum(const SpSmem &s, int i) {
+    float z = 0.f;
+#pragma unroll
+    for (int r = 0; r < SP_CL; ++r) z += s.gat[1][r][i];
+    return z;
+}
+__device__ __forceinline__ void sp_row_stats(SpSmem &s, const SpShare &sh, const float *row, int rows, int V, float inv_tau) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int i = 0; i < rows; ++i) {
+            const float *r = row + (size_t)i * V;
+            const float mx = pass ? sp_max(s, i) : 0.f;
+            float v = pass ? 0.f : -INFINITY;
+#pragma unroll 8
+            for (int j = sh.lo + tid; j < sh.hi; j += SP_THREADS) {
+                const float l = __ldcg(r + j);
+                v = pass ? v + expf((l - mx) * inv_tau) : fmaxf(v, l);
+            }
+            v = pass ? warp_sum(v) : warp_max(v);
+            if (lane == 0) s.red[warp][i] = v;
         }
-        pick_s[2] = pick >= 0 ? pick : lastpos;
+        __syncthreads();
+        if (tid < rows) {
+            float v = s.red[0][tid];
+            for (int w = 1; w < SP_WARPS; ++w) v = pass ? v + s.red[w][tid] : fmaxf(v, s.red[w][tid]);
+            s.red[0][tid] = v;
+        }
+        __syncthreads();
+        sp_gather(s.gat[pass], s.red[0], rows, sh.rank);
+    }
+}
+
+// Inverse-CDF draw from the unnormalised weights wf(j) >= 0: the smallest j whose cumulative weight exceeds u * total (the
+// last positive one if rounding lets none exceed it).  *out is written by one thread of the cluster.  Returns false, in
+// every thread, if the total is not positive.  Uses gat[2] slot `slot`: two draws of one launch take different ones.
+template <class WF>
+__device__ __forceinline__ bool sp_draw(SpSmem &s, const SpShare &sh, WF wf, float u, int slot, int32_t *out) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    __syncthreads();
+#pragma unroll 4
+    for (int b = warp; b < sh.nblk; b += SP_WARPS) {
+        float v = 0.f;
+        for (int q = 0; q < sh.m; ++q) {
+            const int j = sh.lo + (b * sh.m + q) * 32 + lane;
+            if (j < sh.hi) v += wf(j);
+        }
+        v = warp_sum(v);
+        if (lane == 0) s.blk[b] = v;
     }
     __syncthreads();
-    return pick_s[2];
+    // warp 0: lane l adds up blocks [l * per, (l + 1) * per), exclusive prefix over the lanes
+    const int per = (sh.nblk + 31) / 32, b0 = min(lane * per, sh.nblk), b1 = min(b0 + per, sh.nblk);
+    float seg = 0.f, incl = 0.f;
+    if (warp == 0) {
+        for (int b = b0; b < b1; ++b) seg += s.blk[b];
+        incl = seg;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const float x = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += x; }
+        const float total = __shfl_sync(0xffffffffu, incl, 31);
+        if (lane < SP_CL) dsmem_st_f32(dsmem_addr(smem_u32(&s.gat[2][sh.rank][slot]), (uint32_t)lane), total);
+    }
+    cluster_arrive(); cluster_wait();
+    float tot = 0.f, before = 0.f;
+    int owner = -1, lastpos = -1;
+    for (int r = 0; r < SP_CL; ++r) tot += s.gat[2][r][slot];
+    if (!(tot > 0.f)) return false;
+    const float t = u * tot;
+    float cum = 0.f;
+    for (int r = 0; r < SP_CL; ++r) {
+        const float v = s.gat[2][r][slot];
+        if (v > 0.f) {
+            if (owner < 0 && cum + v > t) { owner = r; before = cum; }
+            lastpos = r;
+        }
+        cum += v;
+    }
+    const bool any = owner >= 0;                  // none: u * total rounded up to the total - the last positive id
+    if (!any) owner = lastpos;
+    if (owner != sh.rank || warp != 0) return true;
+    // the block, then the id inside it
+    float c = before + (incl - seg), base = 0.f;
+    int blk = -1, last = -1;
+    for (int b = b0; b < b1; ++b) {
+        const float v = s.blk[b];
+        if (v > 0.f) {
+            if (any && blk < 0 && c + v > t) { blk = b; base = c; }
+            last = b;
+        }
+        c += v;
+    }
+    const unsigned hit = __ballot_sync(0xffffffffu, blk >= 0), pos = __ballot_sync(0xffffffffu, last >= 0);
+    const int src = hit ? __ffs(hit) - 1 : 31 - __clz(pos);
+    blk = __shfl_sync(0xffffffffu, hit ? blk : last, src);
+    base = __shfl_sync(0xffffffffu, base, src);
+    int pick = -1, lastid = -1;
+    for (int q = 0; q < sh.m && pick < 0; ++q) {
+        const int j = sh.lo + (blk * sh.m + q) * 32 + lane;
+        const float w = j < sh.hi ? wf(j) : 0.f;
+        float in = w;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const float x = __shfl_up_sync(0xffffffffu, in, o); if (lane >= o) in += x; }
+        const unsigned over = __ballot_sync(0xffffffffu, hit && w > 0.f && base + in > t), p = __ballot_sync(0xffffffffu, w > 0.f);
+        if (p) lastid = j - lane + 31 - __clz(p);
+        if (over) pick = j - lane + __ffs(over) - 1;
+        base += __shfl_sync(0xffffffffu, in, 31);
+    }
+    if (lane == 0) *out = pick >= 0 ? pick : lastid;
+    return true;
 }
 
 struct SampleArgs {
@@ -246,25 +330,30 @@ struct SampleArgs {
     int V, Tm, b0; float inv_tau;
     const float *u; int u_stride, u_col;       // uniform of sequence b at u[b * u_stride + u_col]
     int32_t *tok_out; int tok_col;             // cand[b][tok_col]
+    float2 *stat; int stat_stride;             // (max, sum) of the row, kept for the acceptance test: stat[b * stat_stride + u_col]
 };
 
 // draft step: token ~ softmax(logits / tau)
 __global__ void __launch_bounds__(SP_THREADS) sample_kernel(const SampleArgs a) {
-    __shared__ float red_s[SP_THREADS / 32], seg_s[SP_THREADS];
-    __shared__ int pick_s[4];
-    const int b = a.b0 + blockIdx.x;
+    __shared__ SpSmem s;
+    const int b = a.b0 + blockIdx.x / SP_CL;
+    const SpShare sh = sp_share(a.V);
     pdl_trigger();
+    cluster_arrive();
     pdl_wait();
+    cluster_wait();                              // every rank runs: its shared memory may be written
     const float *row = a.logits + (size_t)b * a.row_stride;
-    const RowStat st = sp_row_stat(row, a.V, a.inv_tau, red_s);
-    const float u = __ldcg(a.u + (size_t)b * a.u_stride + a.u_col);
-    int tok = sp_draw([&](int j) { return expf((__ldcg(row + j) - st.mx) * a.inv_tau); }, a.V, u, seg_s, pick_s);
-    if (tok < 0) tok = 0;
-    if (threadIdx.x == 0) a.tok_out[b * a.Tm + a.tok_col] = tok;
+    sp_row_stats(s, sh, row, 1, a.V, a.inv_tau);
+    const float mx = sp_max(s, 0);
+    int32_t *tok = a.tok_out + b * a.Tm + a.tok_col;
+    if (sh.rank == 0 && threadIdx.x == 0) a.stat[(size_t)b * a.stat_stride + a.u_col] = make_float2(mx, sp_sum(s, 0));
+    if (!sp_draw(s, sh, [&](int j) { return expf((__ldcg(row + j) - mx) * a.inv_tau); }, __ldcg(a.u + (size_t)b * a.u_stride + a.u_col), 0, tok) &&
+        sh.rank == 0 && threadIdx.x == 0) *tok = 0;
 }
 
 struct SpecAcceptArgs {
     const float *dlogits; int64_t d_seq_stride;     // draft logits: row i of sequence b at dlogits + b * d_seq_stride + i * V
+    const float2 *stat; int stat_stride;            // (max, sum) of those rows, from sample_kernel
     const float *vlogits;                           // verify logits: row (b - b0) * T + i, V floats each
     const int32_t *cand;                            // [B][Tm]
     const float *u_acc, *u_final; int u_stride;     // u_acc[b * u_stride + i], u_final[b]
@@ -275,42 +364,47 @@ struct SpecAcceptArgs {
 // Eq. 6 for one sequence: accept draft i+1 iff u_i < P_H(x) / P_S(x); at the first rejection draw the correction from
 // the positive part of P_H - P_S, after k acceptances draw the bonus token from P_H.
 __global__ void __launch_bounds__(SP_THREADS) spec_accept_kernel(const SpecAcceptArgs a) {
-    __shared__ float red_s[SP_THREADS / 32], seg_s[SP_THREADS];
-    __shared__ int pick_s[4];
-    const int lb = blockIdx.x, b = a.b0 + lb, T = a.k + 1;
+    __shared__ SpSmem s;
+    const int lb = blockIdx.x / SP_CL, b = a.b0 + lb, T = a.k + 1;
+    const SpShare sh = sp_share(a.V);
     pdl_trigger();
+    cluster_arrive();
     pdl_wait();
+    cluster_wait();
     const float *drow = a.dlogits + (size_t)b * a.d_seq_stride, *vrow = a.vlogits + (size_t)lb * T * a.V;
-    int n = 0;
-    RowStat sS{0.f, 1.f}, sH{0.f, 1.f};
-    for (; n < a.k; ++n) {
-        sS = sp_row_stat(drow + (size_t)n * a.V, a.V, a.inv_tau, red_s);
-        sH = sp_row_stat(vrow + (size_t)n * a.V, a.V, a.inv_tau, red_s);
-        const int x = __ldcg(a.cand + b * a.Tm + n + 1);
-        const float pS = expf((__ldcg(drow + (size_t)n * a.V + x) - sS.mx) * a.inv_tau) / sS.Z;
-        const float pH = expf((__ldcg(vrow + (size_t)n * a.V + x) - sH.mx) * a.inv_tau) / sH.Z;
-        const float ratio = pS > 0.f ? pH / pS : 1.f;
-        if (!(ratio >= 1.f) && !(__ldcg(a.u_acc + (size_t)b * a.u_stride + n) < ratio)) break;      // rejected
+    const float2 *stat = a.stat + (size_t)b * a.stat_stride;
+    sp_row_stats(s, sh, vrow, T, a.V, a.inv_tau);       // every position's P_H at once
+    if (threadIdx.x < 32) {
+        // lane i: would draft i + 1 be accepted?
+        const int i = threadIdx.x;
+        bool reject = false;
+        if (i < a.k) {
+            const int x = __ldcg(a.cand + b * a.Tm + i + 1);
+            const float2 sS = __ldcg(stat + i);
+            const float pS = expf((__ldcg(drow + (size_t)i * a.V + x) - sS.x) * a.inv_tau) / sS.y;
+            const float pH = expf((__ldcg(vrow + (size_t)i * a.V + x) - sp_max(s, i)) * a.inv_tau) / sp_sum(s, i);
+            const float ratio = pS > 0.f ? pH / pS : 1.f;
+            reject = !(ratio >= 1.f) && !(__ldcg(a.u_acc + (size_t)b * a.u_stride + i) < ratio);
+        }
+        const unsigned r = __ballot_sync(0xffffffffu, reject);
+        if (i == 0) s.n = r ? __ffs(r) - 1 : a.k;
     }
-    const float uf = __ldcg(a.u_final + b);
-    int tok;
+    __syncthreads();
+    const int n = s.n;
+    const float uf = __ldcg(a.u_final + b), mH = sp_max(s, n), iH = 1.f / sp_sum(s, n);
+    const float *vr = vrow + (size_t)n * a.V;
+    bool done = false;
     if (n < a.k) {
-        const float *dr = drow + (size_t)n * a.V, *vr = vrow + (size_t)n * a.V;
-        const float iS = 1.f / sS.Z, iH = 1.f / sH.Z;
-        tok = sp_draw([&](int j) {
-            const float d = expf((__ldcg(vr + j) - sH.mx) * a.inv_tau) * iH - expf((__ldcg(dr + j) - sS.mx) * a.inv_tau) * iS;
-            return d > 0.f ? d : 0.f; }, a.V, uf, seg_s, pick_s);
-    } else {
-        sH = sp_row_stat(vrow + (size_t)a.k * a.V, a.V, a.inv_tau, red_s);
-        tok = -1;
+        const float *dr = drow + (size_t)n * a.V;
+        const float2 sS = __ldcg(stat + n);
+        const float iS = 1.f / sS.y;
+        done = sp_draw(s, sh, [&](int j) {
+            const float d = expf((__ldcg(vr + j) - mH) * a.inv_tau) * iH - expf((__ldcg(dr + j) - sS.x) * a.inv_tau) * iS;
+            return d > 0.f ? d : 0.f; }, uf, 0, a.next_out + b);
     }
-    if (tok < 0) {                                   // bonus draw, or an empty residual: draw from P_H of that position
-        const float *vr = vrow + (size_t)n * a.V;
-        if (n < a.k) sH = sp_row_stat(vr, a.V, a.inv_tau, red_s);
-        tok = sp_draw([&](int j) { return expf((__ldcg(vr + j) - sH.mx) * a.inv_tau); }, a.V, uf, seg_s, pick_s);
-        if (tok < 0) tok = 0;
-    }
-    if (threadIdx.x == 0) { a.n_out[b] = n; a.next_out[b] = tok; }
+    if (!done)                                       // bonus draw, or an empty residual: draw from P_H of that position
+        done = sp_draw(s, sh, [&](int j) { return expf((__ldcg(vr + j) - mH) * a.inv_tau); }, uf, 1, a.next_out + b);
+    if (sh.rank == 0 && threadIdx.x == 0) { a.n_out[b] = n; if (!done) a.next_out[b] = 0; }
 }
 
 // Self-test of the bounded wait every copy-fed kernel uses: one warp arms an mbarrier for bytes that no copy
@@ -329,16 +423,16 @@ __global__ void wait_probe_kernel(int32_t *status, int polls) {
 }  // namespace
 
 cudaError_t launch_sample(const float *logits, int64_t row_stride, int V, int Tm, int b0, int nb, float tau,
-                          const float *u, int u_stride, int u_col, int32_t *tok_out, int tok_col, cudaStream_t s) {
-    SampleArgs a{logits, row_stride, V, Tm, b0, 1.0f / tau, u, u_stride, u_col, tok_out, tok_col};
-    return launch_pdl(sample_kernel, dim3(nb), dim3(SP_THREADS), 0, s, a);
+                          const float *u, int u_stride, int u_col, int32_t *tok_out, int tok_col, float2 *stat, int stat_stride, cudaStream_t s) {
+    SampleArgs a{logits, row_stride, V, Tm, b0, 1.0f / tau, u, u_stride, u_col, tok_out, tok_col, stat, stat_stride};
+    return launch_pdl_cluster(sample_kernel, dim3(nb * SP_CL), dim3(SP_THREADS), 0, s, SP_CL, a);
 }
 
-cudaError_t launch_spec_accept(const float *dlogits, int64_t d_seq_stride, const float *vlogits, const int32_t *cand,
+cudaError_t launch_spec_accept(const float *dlogits, int64_t d_seq_stride, const float2 *stat, int stat_stride, const float *vlogits, const int32_t *cand,
                                const float *u_acc, const float *u_final, int u_stride, int32_t *n_out, int32_t *next_out,
                                int V, int Tm, int k, int b0, int nb, float tau, cudaStream_t s) {
-    SpecAcceptArgs a{dlogits, d_seq_stride, vlogits, cand, u_acc, u_final, u_stride, n_out, next_out, V, Tm, k, b0, 1.0f / tau};
-    return launch_pdl(spec_accept_kernel, dim3(nb), dim3(SP_THREADS), 0, s, a);
+    SpecAcceptArgs a{dlogits, d_seq_stride, stat, stat_stride, vlogits, cand, u_acc, u_final, u_stride, n_out, next_out, V, Tm, k, b0, 1.0f / tau};
+    return launch_pdl_cluster(spec_accept_kernel, dim3(nb * SP_CL), dim3(SP_THREADS), 0, s, SP_CL, a);
 }
 
 cudaError_t launch_wait_probe(int32_t *status, int polls, cudaStream_t s) {
