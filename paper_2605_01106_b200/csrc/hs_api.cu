@@ -242,7 +242,11 @@ AttnGeom attn_geom(const hs_model *m, int Tq, int T, int b0, int nb) {
         const int limit = m->c.arch == HS_ARCH_PARALLEL ? 128 : 256;
         int ck = 32;
         while (ck < limit && 8 * ck < maxlen + T) ck += 32;
-        if (g_hs_attn_small && (m->c.qh / m->c.kvh) * Tq <= 16 && 8 * ck >= maxlen + T) return AttnGeom{ck, 1, 1, 0};
+        // more than 16 query rows are several clusters per KV head, up to about two thirds of the SMs (verify pass, general form ->
+        // this: sequential hybrid at 5 / 9 rows and 1024 / 2000 keys 0.93 / 1.25 -> 0.80 / 1.02 ms, 0.5B-class at 5 / 9 / 15 rows
+        // 1.50 / 1.74 / 2.05 -> 1.47 / 1.67 / 2.00 ms; with 144 CTAs, 27 rows, 2.50 -> 2.56 ms)
+        const int tiles = ((m->c.qh / m->c.kvh) * Tq + 15) / 16;
+        if (g_hs_attn_small && (tiles == 1 || nb * m->c.kvh * tiles * 8 <= 96) && 8 * ck >= maxlen + T) return AttnGeom{ck, 1, 1, 0};
     }
     int want = 32;
     while (want < 128 && 8 * want < maxlen + T) want += 32;

@@ -518,8 +518,9 @@ __device__ __forceinline__ void attn_body(const AttnArgs &a, const int split, co
 
 
 // ------------------------------------------------------------------------------------------------
-// Short caches and few query rows (G*T <= 16, the whole cache within one cluster of eight CTAs): the
-// latency-lean form.  A CTA holds its whole key range (up to 256 cached keys plus the new rows) in shared
+// Short caches and few query rows (the whole cache within one cluster of eight CTAs): the latency-lean form.  A cluster takes
+// 16 of the G * T query rows of a KV head; more rows are several clusters, each reading the key range for itself (from L2).
+// A CTA holds its whole key range (up to 256 cached keys plus the new rows) in shared
 // memory, fetched before the dependency wait.  After the queries are staged there is no block-wide
 // synchronisation any more: every warp takes 16 keys at a time, computes the scores on the tensor cores,
 // keeps the probabilities in registers (the accumulator layout of the score tile is the operand layout of
@@ -544,9 +545,11 @@ __host__ __device__ inline AttnSmallLayout attn_small_layout(int hd, int ck, int
 constexpr int AT_SMALL_MAXCHUNK = 256;
 
 template <int HD>
-__device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int split, const int kh, const int lb, unsigned char *smraw) {
+__device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int split, const int khq, const int lb, unsigned char *smraw) {
     const int CK = a.chunk;                        // cached keys per CTA: a multiple of 16 up to 256
-    const int G = a.qh / a.kvh, T = a.T, GT = G * T;
+    // khq = KV head + row tile * KV heads; this cluster's query rows are q_lo .. q_lo + GT - 1
+    const int kh = khq % a.kvh, q_lo = khq / a.kvh * 16;
+    const int G = a.qh / a.kvh, T = a.T, GT = min(16, G * T - q_lo);
     const AttnSmallLayout L = attn_small_layout(HD, CK, GT);
     const int KSTR = L.kstr;
     __nv_bfloat16 *K_s = reinterpret_cast<__nv_bfloat16 *>(smraw + L.k_off);         // [keys][KSTR]
@@ -567,7 +570,7 @@ __device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int spl
     const int len = __ldcg(a.kv_len + b) + a.len_off;
     const int nsplit = max(1, (len + CK - 1) / CK);
     if (len < 0 || len + T > a.cap || nsplit > AT_CL) {      // never write past the cache; a cache longer than the host's bound is a host error
-        if (tid == 0 && split == 0 && kh == 0) atomicCAS(a.status, 0, (len >= 0 && len + T > a.cap) ? (int)HS_ERR_CAPACITY : (int)HS_ERR_DEVICE);
+        if (tid == 0 && split == 0 && khq == 0) atomicCAS(a.status, 0, (len >= 0 && len + T > a.cap) ? (int)HS_ERR_CAPACITY : (int)HS_ERR_DEVICE);
         return;
     }
     const int crank = split;                      // the grid has exactly one cluster along x
@@ -631,8 +634,8 @@ __device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int spl
             const int qi = part + u * NH;
             x0[u] = x1[u] = 0.f;
             if (qi < GT) {
-                const int gq = (int)((qi * tinv) >> 16);
-                const float *src = a.zx + (size_t)(rowbase + qi - gq * T) * a.in_ld + a.q_off + (kh * G + gq) * HD;
+                const int gq = (int)(((q_lo + qi) * tinv) >> 16);
+                const float *src = a.zx + (size_t)(rowbase + q_lo + qi - gq * T) * a.in_ld + a.q_off + (kh * G + gq) * HD;
                 x0[u] = __ldcg(src + e); x1[u] = __ldcg(src + e + HP);
             }
         }
@@ -640,7 +643,7 @@ __device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int spl
         for (int u = 0; u < U; ++u) {
             const int qi = part + u * NH;
             if (qi < GT) {
-                const float2 cs = rope_s[(qi - (int)((qi * tinv) >> 16) * T) * HP + e];
+                const float2 cs = rope_s[(q_lo + qi - (int)(((q_lo + qi) * tinv) >> 16) * T) * HP + e];
                 __nv_bfloat16 h, l;
                 split_bf16((x0[u] * cs.x - x1[u] * cs.y) * scale, h, l);
                 Qh_s[qi * KSTR + e] = h; Ql_s[qi * KSTR + e] = l;
@@ -665,6 +668,7 @@ __device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int spl
             const __nv_bfloat16 v1 = __float2bfloat16_rn(kraw[it][3]);
             K_s[(size_t)(rc + i) * KSTR + e] = k0; K_s[(size_t)(rc + i) * KSTR + e + HD / 2] = k1;
             V_s[(size_t)(rc + i) * KSTR + e] = v0; V_s[(size_t)(rc + i) * KSTR + e + HD / 2] = v1;
+            if (q_lo > 0) continue;             // the first row tile's cluster appends
             Kb[(size_t)(len + i) * HD + e] = k0; Kb[(size_t)(len + i) * HD + e + HD / 2] = k1;
             Vb[(size_t)(len + i) * HD + e] = v0; Vb[(size_t)(len + i) * HD + e + HD / 2] = v1;
         }
@@ -685,7 +689,8 @@ __device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int spl
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) { O[nt][0] = O[nt][1] = O[nt][2] = O[nt][3] = 0.f; }
     float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};      // rows g8 and g8 + 8
-    const int ti0 = g8 - (int)((g8 * tinv) >> 16) * T, ti1 = (g8 + 8) - (int)(((g8 + 8) * tinv) >> 16) * T;   // position index of the two rows
+    const int qg0 = q_lo + g8, qg1 = q_lo + g8 + 8;
+    const int ti0 = qg0 - (int)((qg0 * tinv) >> 16) * T, ti1 = qg1 - (int)((qg1 * tinv) >> 16) * T;          // position index of the two rows
 #pragma unroll 1
     for (int kb = warp * 16; kb < nkp; kb += AT_WARPS * 16) {
         // scores: the k steps feed four accumulator sets in turn, so that a chain of dependent MMAs is 4 long, not 16
@@ -816,7 +821,7 @@ __device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int spl
             sum.z += __shfl_xor_sync(0xffffffffu, sum.z, w); sum.w += __shfl_xor_sync(0xffffffffu, sum.w, w);
         }
         if (valid && sub == 0) {
-            const int gq = (int)((qi * tinv) >> 16), i = qi - gq * T;
+            const int q = q_lo + qi, gq = (int)((q * tinv) >> 16), i = q - gq * T;
             const float inv = 1.0f / den;
             *reinterpret_cast<float4 *>(o_base + (size_t)i * (a.qh * HD) + (kh * G + gq) * HD + d) =
                 make_float4(sum.x * inv, sum.y * inv, sum.z * inv, sum.w * inv);
@@ -1299,6 +1304,9 @@ __global__ void __launch_bounds__(AT_THREADS) attn_kernel(const AttnArgs a) {
 // clusters) are attention CTAs, the rest mixer CTAs - and the dependent-launch chain is one kernel shorter.
 struct FusedGeo { int attn_nx, attn_ctas, ssm_nx, ssm_ctas; };
 
+// clusters of 16 query rows per KV head in the latency-lean form
+__host__ __device__ inline int small_tiles(const AttnArgs &a) { return (a.qh / a.kvh * a.T + 15) / 16; }
+
 template <int HD>
 __global__ void __launch_bounds__(AT_THREADS) attn_small_kernel(const AttnArgs a) {
     extern __shared__ __align__(128) unsigned char smraw[];
@@ -1312,7 +1320,7 @@ __global__ void __launch_bounds__(AT_THREADS) ssm_attn_kernel(const SsmArgs sa, 
     const int id = blockIdx.x;
     if (id < g.attn_ctas) {
         const int split = id % g.attn_nx, t = id / g.attn_nx;
-        if (MT == 0) attn_small_body<HD>(aa, split, t % aa.kvh, t / aa.kvh, smraw);
+        if (MT == 0) { const int heads = aa.kvh * small_tiles(aa); attn_small_body<HD>(aa, split, t % heads, t / heads, smraw); }
         else attn_body<HD, MT == 0 ? 1 : MT>(aa, split, t % aa.kvh, t / aa.kvh, smraw);
     } else if (id - g.attn_ctas < g.ssm_ctas) {
         const int j = id - g.attn_ctas, bx = j % g.ssm_nx, t = j / g.ssm_nx;
@@ -1336,19 +1344,19 @@ cudaError_t launch_small_t(const AttnArgs &a, cudaStream_t s) {
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    const size_t smem = attn_small_layout(HD, a.chunk, (a.qh / a.kvh) * a.T).total;
-    return launch_pdl_cluster(attn_small_kernel<HD>, dim3(AT_CL, a.kvh, a.nb), dim3(AT_THREADS), smem, s, AT_CL, a);
+    const size_t smem = attn_small_layout(HD, a.chunk, small_tiles(a) > 1 ? 16 : (a.qh / a.kvh) * a.T).total;
+    return launch_pdl_cluster(attn_small_kernel<HD>, dim3(AT_CL, a.kvh * small_tiles(a), a.nb), dim3(AT_THREADS), smem, s, AT_CL, a);
 }
 
 template <int EPL, int HD, int MT, int TMAX>
 cudaError_t launch_fused_t(const SsmArgs &sa, const AttnArgs &a, cudaStream_t s) {
     FusedGeo g;
     g.attn_nx = MT == 0 ? AT_CL : (a.nch + AT_CL - 1) / AT_CL * AT_CL;
-    g.attn_ctas = g.attn_nx * a.kvh * a.nb;
+    g.attn_ctas = g.attn_nx * a.kvh * (MT == 0 ? small_tiles(a) : 1) * a.nb;
     g.ssm_nx = sa.P / 16;
     g.ssm_ctas = g.ssm_nx * sa.H * sa.nb;
     const int total = (g.attn_ctas + g.ssm_ctas + AT_CL - 1) / AT_CL * AT_CL;
-    const size_t smem = MT == 0 ? attn_small_layout(HD, a.chunk, (a.qh / a.kvh) * a.T).total : attn_layout(HD, a.chunk, (a.qh / a.kvh) * a.T).total;
+    const size_t smem = MT == 0 ? attn_small_layout(HD, a.chunk, small_tiles(a) > 1 ? 16 : (a.qh / a.kvh) * a.T).total : attn_layout(HD, a.chunk, (a.qh / a.kvh) * a.T).total;
     static bool configured = false;
     if (!configured) {
         const size_t most = MT == 0 ? attn_small_layout(HD, AT_SMALL_MAXCHUNK, 16).total : attn_layout(HD, 128, MT * 16).total;
@@ -1382,7 +1390,7 @@ cudaError_t configure_attn() {
 cudaError_t launch_attn(const AttnArgs &a, cudaStream_t s) {
     const int GT = (a.qh / a.kvh) * a.T;
     if (a.small) {
-        if (GT > 16 || a.chunk < 16 || a.chunk > AT_SMALL_MAXCHUNK || (a.chunk & 15)) return cudaErrorInvalidValue;
+        if (GT > HS_MAX_GT || a.chunk < 16 || a.chunk > AT_SMALL_MAXCHUNK || (a.chunk & 15)) return cudaErrorInvalidValue;
         return a.hd == 128 ? launch_small_t<128>(a, s) : a.hd == 64 ? launch_small_t<64>(a, s) : cudaErrorInvalidValue;
     }
     if (a.stream) {          // the streaming form: 128-key tiles, a.tiles of them per CTA, at most 32 query rows
@@ -1413,7 +1421,6 @@ cudaError_t launch_ssm_attn(const SsmArgs &sa, const AttnArgs &a, cudaStream_t s
     // (batch 1) that costs nothing and saves a kernel on the dependent chain; with many (larger batches) it caps the
     // number of resident mixer blocks and with it the state bandwidth: then the two kernels go out separately.
     if ((int64_t)(sa.P / 16) * sa.H * sa.nb > 4 * 148) return cudaSuccess;
-    if (a.small && GT > 16) return cudaErrorInvalidValue;
 #define CASE(n_, e_, hd_, m_) if (sa.N == n_ && a.hd == hd_ && mt == m_) { *fused = true; return a.T <= 3 ? launch_fused_t<e_, hd_, m_, 3>(sa, a, s) : launch_fused_t<e_, hd_, m_, HS_MAX_T>(sa, a, s); }
 #define CASES(n_, e_) CASE(n_, e_, 128, 0) CASE(n_, e_, 64, 0) CASE(n_, e_, 128, 1) CASE(n_, e_, 128, 2) CASE(n_, e_, 128, 3) CASE(n_, e_, 64, 1) CASE(n_, e_, 64, 2) CASE(n_, e_, 64, 3)
     CASES(64, 2) CASES(128, 4) CASES(256, 8)

@@ -201,3 +201,13 @@ def test_cfg5_batch64_two_sequences_128_tokens(env):
     for b in (5, 41):
         kv, _ = eng.get_context(b)
         assert kv == lens[b] + int((np.array(forced[b]) + 1).sum())
+
+
+@pytest.mark.parametrize("name,k,ctx", [("cfg1_tiny", 8, 255), ("cfg1_tiny", 8, 129), ("test_seq", 8, 2000)])
+def test_lean_attention_with_several_row_tiles(env, name, k, ctx):
+    # 17 and more query rows per KV head in the latency-lean form: several clusters of 16 rows each, the last one ragged
+    # (two query heads per KV head x 9 positions = 18 rows), of which only the first appends to the cache
+    s, eng, model, seqs = make(env, name, 1, k, ctx + 64, {0}, [ctx])
+    rep = env["harness"].run_rounds(eng, seqs, s, k, 3, forced=[[8, 3, 0]])
+    print(rep)
+    assert eng.device_status() == 0
