@@ -219,52 +219,60 @@ double gemv_bytes(const GemvArgs &a) {
 //   draft = false: full model M_H (verify);  draft = true: draft model M_S, one position,
 //   reading candidate column `col` and, for step > 0, the scratch state of the previous step.
 // ------------------------------------------------------------------------------------------------
-// Attention geometry of this launch.  Keys per tile: the context is spread over the eight CTAs of one
-// cluster (which combine their partials in shared memory) - 32, 64, 96 or 128 keys each, whichever first
-// covers it - and never below the size the partial buffers were laid out for; longer contexts use 128-key
-// tiles over several clusters.  Tiles per CTA: one, unless the launch would have far more CTAs than the GPU
-// runs at once (long caches at large batch) - then a CTA walks up to sixteen 64-key tiles, so that staging
-// the queries and combining the partials is paid once per 1024 keys.
-// Few query rows (G * T <= 16) over caches that fit one cluster: the latency-lean attention form, keys per CTA in
-// steps of 32 up to 128 (parallel blocks: the mixer CTAs of the fused launch get the same shared memory) or 256.
+// Attention geometry of a launch.  Three forms, in this order:
+//  - lean: the whole cache inside one cluster of eight CTAs, 16 query rows per cluster, up to 288 keys per CTA (128 in a
+//    launch that the mixer shares, whose blocks all carry its shared memory);
+//  - streaming: 128-key tiles, several per CTA, up to 32 query rows, where the caches together fill the GPU;
+//  - general: the rest.  Keys per tile 32, 64, 96 or 128, whichever first covers the cache with the eight CTAs of one
+//    cluster, and never below the size the partial buffers were laid out for; longer caches use 128-key tiles over several
+//    clusters.  One tile per CTA, unless the launch would have far more CTAs than the GPU runs at once - then a CTA walks
+//    up to sixteen 64-key tiles, so that staging the queries and combining the partials is paid once per 1024 keys.
 struct AttnGeom {
     int chunk, tiles, small, stream;
-    int code() const { return stream * 1024 + small * 512 + (chunk / 16 - 1) * 32 + tiles - 1; }   // < 2048, part of the graph key
+    bool fuse;                   // verify pass of a parallel block: mixer and attention in one launch
+    int code() const { return fuse * 4096 + stream * 2048 + small * 1024 + (chunk / 16 - 1) * 32 + tiles - 1; }   // < 8192, part of the graph key
 };
 // Tq: query positions per sequence of the launch; T: rows the pass may append beyond the upper bound of kv_len
 // (the same for a verify pass; a draft that keeps attention appends one row per step, k in all)
 AttnGeom attn_geom(const hs_model *m, int Tq, int T, int b0, int nb) {
-    if (m->att_force_chunk) return AttnGeom{m->att_force_chunk, m->att_force_tiles < 0 ? -m->att_force_tiles : m->att_force_tiles, 0, m->att_force_tiles < 0 ? 1 : 0};
-    const bool have_maps = !m->kmaps.empty();        // the streaming form fetches its tiles with tensor copies
+    const hs_config &c = m->c;
+    // One launch for mixer and attention spares a link of the chain, but every mixer block then carries the attention's
+    // shared memory and two or three fit on an SM.  Verify pass of the 0.5B-class shape, together / apart: 2 sequences
+    // (256 mixer blocks) 1.47 / 1.58 ms, 3 sequences (384) 2.00 / 1.75 ms; 3B-class, 1 sequence (320) 3.38 / 3.04 ms.
+    const bool few = c.arch == HS_ARCH_PARALLEL && (int64_t)(c.P / 16) * c.H * nb <= 2 * 148;
+    if (m->att_force_chunk) return AttnGeom{m->att_force_chunk, m->att_force_tiles < 0 ? -m->att_force_tiles : m->att_force_tiles, 0, m->att_force_tiles < 0 ? 1 : 0, few};
     int maxlen = 0;
     for (int b = b0; b < b0 + nb; ++b) if (m->kv_upper[b] > maxlen) maxlen = m->kv_upper[b];
+    const int groups = c.qh / c.kvh * Tq;            // query rows per KV head
+    const int per_seq = (maxlen + T + 127) / 128;    // 128-key tiles of the longest cache
+    const int64_t tiles128 = (int64_t)nb * c.kvh * per_seq;
+    // The streaming form (its tiles come by tensor copies, hence the maps) pays from about 100 tiles on: 0.5B-class, one
+    // sequence, streaming / general: 4000 keys (64 tiles) 2.49 / 2.24 ms, 9000 keys (142) 1.28 / 1.88, 16000 keys 2.53 / 5.20.
+    const bool streams = g_hs_attn_stream && !m->kmaps.empty() && groups <= 32 && tiles128 >= 100;
     {
-        const int limit = m->c.arch == HS_ARCH_PARALLEL ? 128 : 256;
+        // Lean.  Apart from the mixer from 1025 keys on even where the mixer has few blocks (0.5B-class, one sequence of 2200
+        // keys, k = 0 / 2 / 4: 1.07 / 1.47 / 2.22 ms general -> 0.92 / 1.28 / 1.65).  At more than a CTA per SM the streaming
+        // form is faster where it applies (8 sequences of 1024 keys, k = 4, 256 CTAs, lean / streaming: 2.85 / 2.58 ms; 3 of
+        // 512, 96 CTAs: 1.75 / 1.90); beyond four per SM the general form takes over.
         int ck = 32;
-        while (ck < limit && 8 * ck < maxlen + T) ck += 32;
-        // more than 16 query rows are several clusters per KV head, up to about two thirds of the SMs (verify pass, general form ->
-        // this: sequential hybrid at 5 / 9 rows and 1024 / 2000 keys 0.93 / 1.25 -> 0.80 / 1.02 ms, 0.5B-class at 5 / 9 / 15 rows
-        // 1.50 / 1.74 / 2.05 -> 1.47 / 1.67 / 2.00 ms; with 144 CTAs, 27 rows, 2.50 -> 2.56 ms)
-        const int tiles = ((m->c.qh / m->c.kvh) * Tq + 15) / 16;
-        if (g_hs_attn_small && (tiles == 1 || nb * m->c.kvh * tiles * 8 <= 96) && 8 * ck >= maxlen + T) return AttnGeom{ck, 1, 1, 0};
+        while (ck < 288 && 8 * ck < maxlen + T) ck += 32;
+        const bool fuse = few && ck <= 128;
+        const int ctas = nb * c.kvh * ((groups + 15) / 16) * 8;
+        if (g_hs_attn_small && ctas <= (streams || fuse ? 148 : 4 * 148) && 8 * ck >= maxlen + T) return AttnGeom{ck, 1, 1, 0, fuse};
+    }
+    if (streams) {
+        // 128-key tiles per CTA.  A whole cache in one CTA spares the merge of ranges; otherwise about one CTA per SM, half
+        // that where there is work for several tiles each (staging the queries and merging the ranges is paid per CTA: 544
+        // tiles of work run best as 8 per CTA)
+        const int half = (int)((tiles128 + 73) / 74);
+        int tiles = per_seq <= half ? per_seq : tiles128 <= 2 * 148 ? (int)((tiles128 + 147) / 148) : half;
+        tiles = tiles < 1 ? 1 : tiles > 16 ? 16 : tiles;
+        return AttnGeom{128, tiles, 0, 1, false};
     }
     int want = 32;
     while (want < 128 && 8 * want < maxlen + T) want += 32;
-    // Long caches at a batch that fills the GPU several times over, in a launch of its own (not fused with the mixer):
-    // the streaming form - 128-key tiles, up to 16 per CTA.
-    {
-        const bool own_launch = m->c.arch == HS_ARCH_SEQUENTIAL || (int64_t)(m->c.P / 16) * m->c.H * nb > 4 * 148;
-        const int64_t ctas128 = (int64_t)nb * m->c.kvh * ((maxlen + T + 127) / 128);
-        if (g_hs_attn_stream && have_maps && own_launch && (m->c.qh / m->c.kvh) * Tq <= 32 && ctas128 >= 2 * 148) {
-            // tiles per CTA: up to 16, fewer only while that still leaves about half an SM count of CTAs (measured: 544 tiles
-            // of work run best as 8 per CTA - staging the queries and merging the ranges is paid per CTA)
-            int tiles = (int)((ctas128 + 73) / 74);
-            tiles = tiles < 1 ? 1 : tiles > 16 ? 16 : tiles;
-            return AttnGeom{128, tiles, 0, 1};
-        }
-    }
-    AttnGeom g{want > m->att_chunk ? want : m->att_chunk, 1, 0, 0};
-    const int64_t ctas64 = (int64_t)nb * m->c.kvh * ((maxlen + T + 63) / 64);
+    AttnGeom g{want > m->att_chunk ? want : m->att_chunk, 1, 0, 0, few};
+    const int64_t ctas64 = (int64_t)nb * c.kvh * ((maxlen + T + 63) / 64);
     const int64_t fill = 148 * 8;             // CTAs that keep every SM busy for several rounds
     if (g.chunk == 128 && ctas64 >= 4 * fill) {
         g.chunk = 64;
@@ -406,7 +414,7 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
             bool fused = false;
             if (ssm_deferred) {
                 // a parallel block: mixer and attention are independent of each other - one launch for both
-                if (!ssm_wide(ssm_args)) PROF(HS_PROF_MIXER, 0, launch_ssm_attn(ssm_args, aa, s, &fused), "ssm + attention");
+                if (at_geom.fuse) PROF(HS_PROF_MIXER, 0, launch_ssm_attn(ssm_args, aa, s, &fused), "ssm + attention");
                 if (fused) ++m->launches;
                 else { PROF(HS_PROF_MIXER, 0, launch_ssm(ssm_args, s), "ssm"); ++m->launches; }
             }

@@ -542,7 +542,7 @@ __host__ __device__ inline AttnSmallLayout attn_small_layout(int hd, int ck, int
     L.total = (o + 127) / 128 * 128;
     return L;
 }
-constexpr int AT_SMALL_MAXCHUNK = 256;
+constexpr int AT_SMALL_MAXCHUNK = 288;  // 213 KB of shared memory at a head dimension of 128
 
 template <int HD>
 __device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int split, const int khq, const int lb, unsigned char *smraw) {
@@ -1416,11 +1416,7 @@ cudaError_t launch_attn(const AttnArgs &a, cudaStream_t s) {
 cudaError_t launch_ssm_attn(const SsmArgs &sa, const AttnArgs &a, cudaStream_t s, bool *fused) {
     const int GT = (a.qh / a.kvh) * a.T, mt = a.small ? 0 : (GT + 15) / 16;
     *fused = false;
-    if (ssm_wide(sa) || GT > HS_MAX_GT || a.tiles < 1 || a.chunk < 16 || a.chunk > 128 || (a.chunk & 15) || sa.P % 16) return cudaSuccess;
-    // In the fused launch every mixer block carries the attention's shared-memory allocation.  With a few blocks per SM
-    // (batch 1) that costs nothing and saves a kernel on the dependent chain; with many (larger batches) it caps the
-    // number of resident mixer blocks and with it the state bandwidth: then the two kernels go out separately.
-    if ((int64_t)(sa.P / 16) * sa.H * sa.nb > 4 * 148) return cudaSuccess;
+    if (GT > HS_MAX_GT || a.tiles < 1 || a.chunk < 16 || a.chunk > 128 || (a.chunk & 15) || sa.P % 16) return cudaSuccess;
 #define CASE(n_, e_, hd_, m_) if (sa.N == n_ && a.hd == hd_ && mt == m_) { *fused = true; return a.T <= 3 ? launch_fused_t<e_, hd_, m_, 3>(sa, a, s) : launch_fused_t<e_, hd_, m_, HS_MAX_T>(sa, a, s); }
 #define CASES(n_, e_) CASE(n_, e_, 128, 0) CASE(n_, e_, 64, 0) CASE(n_, e_, 128, 1) CASE(n_, e_, 128, 2) CASE(n_, e_, 128, 3) CASE(n_, e_, 64, 1) CASE(n_, e_, 64, 2) CASE(n_, e_, 64, 3)
     CASES(64, 2) CASES(128, 4) CASES(256, 8)

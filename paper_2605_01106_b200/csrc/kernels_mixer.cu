@@ -284,7 +284,7 @@ cudaError_t launch_replay(const ReplayArgs &a, cudaStream_t s) {
 }
 
 // a whole head per block once blocks of 16 rows would already fill the GPU several times over
-bool ssm_wide(const SsmArgs &a) { return a.P % 64 == 0 && (int64_t)(a.P / 16) * a.H * a.nb >= 148 * 32; }
+static bool ssm_wide(const SsmArgs &a) { return a.P % 64 == 0 && (int64_t)(a.P / 16) * a.H * a.nb >= 148 * 32; }
 
 cudaError_t launch_ssm(const SsmArgs &a, cudaStream_t s) {
     const bool wide = ssm_wide(a);
