@@ -1359,7 +1359,7 @@ cudaError_t launch_fused_t(const SsmArgs &sa, const AttnArgs &a, cudaStream_t s)
     const size_t smem = MT == 0 ? attn_small_layout(HD, a.chunk, small_tiles(a) > 1 ? 16 : (a.qh / a.kvh) * a.T).total : attn_layout(HD, a.chunk, (a.qh / a.kvh) * a.T).total;
     static bool configured = false;
     if (!configured) {
-        const size_t most = MT == 0 ? attn_small_layout(HD, AT_SMALL_MAXCHUNK, 16).total : attn_layout(HD, 128, MT * 16).total;
+        const size_t most = MT == 0 ? attn_small_layout(HD, 128, 16).total : attn_layout(HD, 128, MT * 16).total;
         cudaError_t e = cudaFuncSetAttribute(ssm_attn_kernel<EPL, HD, MT, TMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(ssm_attn_kernel<EPL, HD, MT, TMAX>, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
