@@ -130,14 +130,11 @@ Derived derive(const hs_config &c) {
     return v;
 }
 
-// rows per plane of the packed activation operands
-int64_t tc_rows_max(const Derived &v) { return std::max<int64_t>(gemm_tc_rows(v.R), gemm_tc_rows(v.pf_rows)); }
-
 // layout of the work buffer; base may be null to only measure
 struct WorkLayout {
     int64_t kv_len, slot, cand, g, margin, n_acc, emitted, stage_n, stage_next, status, counters, am_counters, dslot;
     int64_t rope, h, zx, gbuf, obuf, abuf, logits, dlogits, dstat, att_acc, att_ml, am_part, xb, xb_h, xb_a, ssbuf;
-    int64_t pf_rowtab, pf_segtab, pf_list, pf_xbc, pf_dtv, pf_hfin, pf_q, pf_rec, total;
+    int64_t pf_h, pf_zx, pf_gbuf, pf_obuf, pf_xb, pf_xb_h, pf_xb_a, pf_ss, pf_rowtab, pf_segtab, pf_list, pf_xbc, pf_dtv, pf_hfin, pf_q, pf_rec, total;
 };
 
 WorkLayout work_layout(const hs_config &c, const Derived &v) {
@@ -150,30 +147,35 @@ WorkLayout work_layout(const hs_config &c, const Derived &v) {
     w.status = take(4); w.counters = take((int64_t)4 * v.B * c.kvh); w.am_counters = take((int64_t)4 * v.R);
     w.dslot = take(4 * v.B);
     w.rope = take((int64_t)c.kv_capacity * (c.hd / 2) * 8);
-    // activations of a pass: B * (max_k + 1) rows of a verify pass (its residual stream in up to HS_H_PARTS parts), or the
-    // rows of a prompt pass
-    const int64_t pr = std::max<int64_t>(v.R, v.pf_rows);
-    w.h = take((int64_t)4 * 2 * std::max<int64_t>((int64_t)HS_H_PARTS * v.R, v.pf_rows) * c.d);
-    w.zx = take(4 * pr * v.in_rows_max);
-    w.gbuf = take(4 * pr * v.gw);
-    w.obuf = take(4 * pr * c.qh * c.hd);
+    // activations of a draft or verify pass: B * (max_k + 1) rows.  Those of a prompt pass lie behind, apart: spread out to
+    // its row count, they made a one-row verify pass about 1 % slower.
+    w.h = take((int64_t)4 * 2 * HS_H_PARTS * v.R * c.d);
+    w.zx = take((int64_t)4 * v.R * v.in_rows_max);
+    w.gbuf = take((int64_t)4 * v.R * v.gw);
+    w.obuf = take((int64_t)4 * v.R * c.qh * c.hd);
     w.abuf = take((int64_t)4 * v.R * c.ff);
     w.logits = take((int64_t)4 * v.R * c.V);
     w.dlogits = take((int64_t)4 * v.B * std::max(c.max_k, 1) * c.V);
-    w.dstat = take((int64_t)8 * v.B * std::max(c.max_k, 1));
     w.att_acc = take((int64_t)4 * v.B * c.kvh * v.att_nch * HS_MAX_GT * c.hd);
     w.att_ml = take((int64_t)4 * v.B * c.kvh * v.att_nch * HS_MAX_GT * 2);
     w.am_part = take((int64_t)16 * v.R * HS_ARGMAX_CHUNKS);
-    {   // packed bf16 activation operand of the many-row projection kernel: [2][rows][widest reduction]
-        const int64_t kmax = std::max<int64_t>(std::max<int64_t>(c.d, c.ff), (int64_t)v.gw + c.qh * c.hd);
-        const int64_t tr = tc_rows_max(v);
-        w.xb = take((int64_t)2 * 2 * tr * kmax);
+    // packed bf16 activation operand of the many-row projection kernel: [2][rows][widest reduction]
+    const int64_t kmax = std::max<int64_t>(std::max<int64_t>(c.d, c.ff), (int64_t)v.gw + c.qh * c.hd);
+    auto packed = [&](int64_t rows, int64_t &xb, int64_t &xb_h, int64_t &xb_a, int64_t &ss) {
+        xb = take((int64_t)2 * 2 * rows * kmax);
         // the same for the residual stream and the MLP activations, written by the producing projection's epilogue,
         // and the partial sums of squares (one per 128 model dimensions) of the residual stream's rows
-        w.xb_h = take((int64_t)2 * 2 * tr * c.d);
-        w.xb_a = take((int64_t)2 * 2 * tr * c.ff);
-        w.ssbuf = take((int64_t)4 * tr * ((c.d + 127) / 128));
-    }
+        xb_h = take((int64_t)2 * 2 * rows * c.d);
+        xb_a = take((int64_t)2 * 2 * rows * c.ff);
+        ss = take((int64_t)4 * rows * ((c.d + 127) / 128));
+    };
+    packed(gemm_tc_rows(v.R), w.xb, w.xb_h, w.xb_a, w.ssbuf);
+    w.dstat = take((int64_t)8 * v.B * std::max(c.max_k, 1));
+    w.pf_h = take((int64_t)4 * 2 * v.pf_rows * c.d);
+    w.pf_zx = take((int64_t)4 * v.pf_rows * v.in_rows_max);
+    w.pf_gbuf = take((int64_t)4 * v.pf_rows * v.gw);
+    w.pf_obuf = take((int64_t)4 * v.pf_rows * c.qh * c.hd);
+    packed(gemm_tc_rows(v.pf_rows), w.pf_xb, w.pf_xb_h, w.pf_xb_a, w.pf_ss);
     w.pf_rowtab = take((int64_t)16 * v.pf_rows);
     w.pf_segtab = take((int64_t)16 * v.B);
     w.pf_list = take((int64_t)8 * (v.R + v.B));
@@ -533,19 +535,19 @@ int prefill_pass(hs_model *m, int rows, int nseg, int max_seg, int *cur_out) {
     const int64_t q_plane = (int64_t)m->pf_rows * c.qh * c.hd;
     int32_t *st_w = m->ctrl.status;
     int cur = 0;
-    PROF(HS_PROF_EMBED, 0, launch_pf_embed(m->embed, d, c.V, m->pf_rowtab, rows, m->hbuf[0], st_w, s), "prefill embed");
+    PROF(HS_PROF_EMBED, 0, launch_pf_embed(m->embed, d, c.V, m->pf_rowtab, rows, m->pf_h[0], st_w, s), "prefill embed");
     ++m->launches;
     for (int l = 0; l < c.L; ++l) {
         const HsLayer &ly = m->layers[l];
         const bool attn = ly.type != HS_LAYER_GDN, rec = ly.type != HS_LAYER_ATT, par = ly.type == HS_LAYER_PAR;
         GemvArgs ga{};
-        ga.W0 = ly.W_in; ga.ldw0 = d; ga.K0 = d; ga.x0 = m->hbuf[cur]; ga.ldx0 = d; ga.xparts = 1;
-        ga.norm_w = ly.norm1; ga.eps = c.eps; ga.O = ly.in_rows_full; ga.out = m->zx; ga.ldo = m->in_rows_max;
-        ga.nrows = rows; ga.epi = EPI_STORE; ga.early_trigger = 0; ga.xb = m->xb; ga.xb_rows = m->xb_rows;
-        if (l > 0) { ga.pk_in = m->xb_h; ga.ss_in = m->ssbuf; ga.ss_parts = ss_parts; }
+        ga.W0 = ly.W_in; ga.ldw0 = d; ga.K0 = d; ga.x0 = m->pf_h[cur]; ga.ldx0 = d; ga.xparts = 1;
+        ga.norm_w = ly.norm1; ga.eps = c.eps; ga.O = ly.in_rows_full; ga.out = m->pf_zx; ga.ldo = m->in_rows_max;
+        ga.nrows = rows; ga.epi = EPI_STORE; ga.early_trigger = 0; ga.xb = m->pf_xb; ga.xb_rows = m->pf_xb_rows;
+        if (l > 0) { ga.pk_in = m->pf_xb_h; ga.ss_in = m->pf_ss; ga.ss_parts = ss_parts; }
         PROF(HS_PROF_GEMV, gemv_bytes(ga), launch_gemm_tc(ga, st_w, s, &m->launches, nullptr), "prefill in_proj");
         PfPrepArgs pa{};
-        pa.rows = m->pf_rowtab; pa.nrows = rows; pa.zx = m->zx; pa.in_ld = m->in_rows_max; pa.kv_len = m->ctrl.kv_len; pa.cap = c.kv_capacity; pa.status = st_w;
+        pa.rows = m->pf_rowtab; pa.nrows = rows; pa.zx = m->pf_zx; pa.in_ld = m->in_rows_max; pa.kv_len = m->ctrl.kv_len; pa.cap = c.kv_capacity; pa.status = st_w;
         const size_t lrB = rec ? (size_t)ly.rl * m->B : 0;
         float *win = rec ? m->cw + lrB * 3 * m->convd : nullptr;
         if (rec) {
@@ -564,41 +566,41 @@ int prefill_pass(hs_model *m, int rows, int nseg, int max_seg, int *cur_out) {
         ++m->launches;
         if (rec) {
             PfScanArgs sa{};
-            sa.segs = m->pf_segtab; sa.nseg = nseg; sa.max_seg = max_seg; sa.nrows = rows; sa.rec = m->pf_rec; sa.xbc_rw = m->pf_xbc; sa.zx = m->zx; sa.in_ld = m->in_rows_max; sa.conv_off = pa.conv_off;
+            sa.segs = m->pf_segtab; sa.nseg = nseg; sa.max_seg = max_seg; sa.nrows = rows; sa.rec = m->pf_rec; sa.xbc_rw = m->pf_xbc; sa.zx = m->pf_zx; sa.in_ld = m->in_rows_max; sa.conv_off = pa.conv_off;
             sa.xbc = m->pf_xbc; sa.convd = m->convd; sa.di = m->di; sa.dtv = m->pf_dtv; sa.heads = pa.heads;
             sa.P = par ? c.P : c.gdv; sa.N = par ? c.N : c.gdk; sa.D = ly.D; sa.onorm = ly.gnorm; sa.eps = c.eps;
             sa.state = m->snap + lrB * m->nslot * m->state_elems; sa.state_elems = m->state_elems; sa.nslot = m->nslot; sa.slot = m->ctrl.slot;
-            sa.win = win; sa.g = m->gbuf; sa.gw = m->gw; sa.status = st_w;
+            sa.win = win; sa.g = m->pf_gbuf; sa.gw = m->gw; sa.status = st_w;
             PROF(HS_PROF_MIXER, 0, par ? launch_pf_ssm(sa, s, &m->launches) : launch_pf_gdn(sa, s, &m->launches), "prefill scan");
         }
         if (attn) {
             PfAttnArgs aa{};
             aa.segs = m->pf_segtab; aa.nseg = nseg; aa.max_seg = max_seg; aa.q = m->pf_q; aa.q_plane = q_plane;
-            aa.Kc = pa.Kc; aa.Vc = pa.Vc; aa.kv_len = m->ctrl.kv_len; aa.qh = c.qh; aa.kvh = c.kvh; aa.hd = c.hd; aa.cap = c.kv_capacity; aa.o = m->obuf;
+            aa.Kc = pa.Kc; aa.Vc = pa.Vc; aa.kv_len = m->ctrl.kv_len; aa.qh = c.qh; aa.kvh = c.kvh; aa.hd = c.hd; aa.cap = c.kv_capacity; aa.o = m->pf_obuf;
             PROF(HS_PROF_ATTN, 0, launch_pf_attn(aa, s), "prefill attention");
             ++m->launches;
         }
         GemvArgs go{};
-        go.O = d; go.out = m->hbuf[cur ^ 1]; go.ldo = d; go.max_oparts = 1; go.resid = m->hbuf[cur]; go.rparts = 1;
-        go.nrows = rows; go.epi = EPI_RESID; go.xparts = 1; go.early_trigger = 0; go.xb = m->xb; go.xb_rows = m->xb_rows;
+        go.O = d; go.out = m->pf_h[cur ^ 1]; go.ldo = d; go.max_oparts = 1; go.resid = m->pf_h[cur]; go.rparts = 1;
+        go.nrows = rows; go.epi = EPI_RESID; go.xparts = 1; go.early_trigger = 0; go.xb = m->pf_xb; go.xb_rows = m->pf_xb_rows;
         if (rec) {
-            go.W0 = ly.W_out; go.ldw0 = m->gw; go.K0 = m->gw; go.x0 = m->gbuf; go.ldx0 = m->gw;
+            go.W0 = ly.W_out; go.ldw0 = m->gw; go.K0 = m->gw; go.x0 = m->pf_gbuf; go.ldx0 = m->gw;
             if (par) {
                 go.norm_w = ly.gnorm; go.eps = c.eps;
-                go.W1 = ly.W_o; go.ldw1 = c.qh * c.hd; go.K1 = c.qh * c.hd; go.x1 = m->obuf; go.ldx1 = c.qh * c.hd;
+                go.W1 = ly.W_o; go.ldw1 = c.qh * c.hd; go.K1 = c.qh * c.hd; go.x1 = m->pf_obuf; go.ldx1 = c.qh * c.hd;
             }
-        } else { go.W0 = ly.W_o; go.ldw0 = c.qh * c.hd; go.K0 = c.qh * c.hd; go.x0 = m->obuf; go.ldx0 = c.qh * c.hd; }
-        go.pk_out = m->xb_h; go.pk_ld = d; go.pk_nw = ly.norm2; go.ss_out = m->ssbuf;
+        } else { go.W0 = ly.W_o; go.ldw0 = c.qh * c.hd; go.K0 = c.qh * c.hd; go.x0 = m->pf_obuf; go.ldx0 = c.qh * c.hd; }
+        go.pk_out = m->pf_xb_h; go.pk_ld = d; go.pk_nw = ly.norm2; go.ss_out = m->pf_ss;
         PROF(HS_PROF_GEMV, gemv_bytes(go), launch_gemm_tc(go, st_w, s, &m->launches, nullptr), "prefill out_proj");
         cur ^= 1;
         GemvArgs gu{};
         gu.W0 = ly.W_gu; gu.ldw0 = d; gu.K0 = d; gu.O = 2 * c.ff; gu.out = nullptr; gu.ldo = c.ff; gu.nrows = rows; gu.epi = EPI_SWIGLU;
-        gu.eps = c.eps; gu.early_trigger = 0; gu.pk_in = m->xb_h; gu.ss_in = m->ssbuf; gu.ss_parts = ss_parts; gu.pk_out = m->xb_a; gu.pk_ld = c.ff;
+        gu.eps = c.eps; gu.early_trigger = 0; gu.pk_in = m->pf_xb_h; gu.ss_in = m->pf_ss; gu.ss_parts = ss_parts; gu.pk_out = m->pf_xb_a; gu.pk_ld = c.ff;
         PROF(HS_PROF_GEMV, gemv_bytes(gu), launch_gemm_tc(gu, st_w, s, &m->launches, nullptr), "prefill gate_up");
         GemvArgs dn{};
-        dn.W0 = ly.W_down; dn.ldw0 = c.ff; dn.K0 = c.ff; dn.O = d; dn.out = m->hbuf[cur ^ 1]; dn.ldo = d; dn.max_oparts = 1;
-        dn.resid = m->hbuf[cur]; dn.rparts = 1; dn.nrows = rows; dn.epi = EPI_RESID; dn.early_trigger = 0; dn.pk_in = m->xb_a;
-        dn.pk_out = m->xb_h; dn.pk_ld = d; dn.pk_nw = l + 1 < c.L ? m->layers[l + 1].norm1 : m->final_norm; dn.ss_out = m->ssbuf;
+        dn.W0 = ly.W_down; dn.ldw0 = c.ff; dn.K0 = c.ff; dn.O = d; dn.out = m->pf_h[cur ^ 1]; dn.ldo = d; dn.max_oparts = 1;
+        dn.resid = m->pf_h[cur]; dn.rparts = 1; dn.nrows = rows; dn.epi = EPI_RESID; dn.early_trigger = 0; dn.pk_in = m->pf_xb_a;
+        dn.pk_out = m->pf_xb_h; dn.pk_ld = d; dn.pk_nw = l + 1 < c.L ? m->layers[l + 1].norm1 : m->final_norm; dn.ss_out = m->pf_ss;
         PROF(HS_PROF_GEMV, gemv_bytes(dn), launch_gemm_tc(dn, st_w, s, &m->launches, nullptr), "prefill down");
         cur ^= 1;
     }
@@ -666,7 +668,7 @@ int prefill_wide(hs_model *m, const int32_t *tokens_host, const int32_t *lens_ho
         const int rc = prefill_pass(m, (int)rows.size(), (int)segs.size(), max_seg, &cur);
         if (rc) return rc;
         if (!list.empty()) {
-            PROF(HS_PROF_EMBED, 0, launch_pf_gather(m->pf_list, (int)list.size(), m->hbuf[cur], d, m->pf_hfin, s), "prefill gather");
+            PROF(HS_PROF_EMBED, 0, launch_pf_gather(m->pf_list, (int)list.size(), m->pf_h[cur], d, m->pf_hfin, s), "prefill gather");
             ++m->launches;
         }
         tabs.push_back(std::move(rows)); tabs.push_back(std::move(segs)); lists.push_back(std::move(list));
@@ -793,10 +795,14 @@ static int init_model(hs_model *m, const hs_config *cfg, const hs_buffers *bufs,
     m->ctrl.status = (int32_t *)(w + wl.status); m->ctrl.counters = (int32_t *)(w + wl.counters); m->ctrl.am_counters = (int32_t *)(w + wl.am_counters);
     m->ctrl.dslot = (int32_t *)(w + wl.dslot);
     m->rope = (float2 *)(w + wl.rope);
-    m->hbuf[0] = (float *)(w + wl.h); m->hbuf[1] = m->hbuf[0] + std::max<size_t>((size_t)HS_H_PARTS * v.R, v.pf_rows) * c.d; m->zx = (float *)(w + wl.zx); m->gbuf = (float *)(w + wl.gbuf);
+    m->hbuf[0] = (float *)(w + wl.h); m->hbuf[1] = m->hbuf[0] + (size_t)HS_H_PARTS * v.R * c.d; m->zx = (float *)(w + wl.zx); m->gbuf = (float *)(w + wl.gbuf);
     m->obuf = (float *)(w + wl.obuf); m->abuf = (float *)(w + wl.abuf); m->logits = (float *)(w + wl.logits); m->dlogits = (float *)(w + wl.dlogits); m->dstat = (float2 *)(w + wl.dstat);
     m->tau = 0.f; m->u_draft = m->u_accept = m->u_final = nullptr;
-    m->att_acc = (float *)(w + wl.att_acc); m->att_ml = (float *)(w + wl.att_ml); m->am_part = w + wl.am_part; m->xb = (__nv_bfloat16 *)(w + wl.xb); m->xb_rows = tc_rows_max(v);
+    m->att_acc = (float *)(w + wl.att_acc); m->att_ml = (float *)(w + wl.att_ml); m->am_part = w + wl.am_part; m->xb = (__nv_bfloat16 *)(w + wl.xb); m->xb_rows = gemm_tc_rows(v.R);
+    m->pf_h[0] = (float *)(w + wl.pf_h); m->pf_h[1] = m->pf_h[0] + (size_t)v.pf_rows * c.d; m->pf_zx = (float *)(w + wl.pf_zx);
+    m->pf_gbuf = (float *)(w + wl.pf_gbuf); m->pf_obuf = (float *)(w + wl.pf_obuf); m->pf_ss = (float *)(w + wl.pf_ss);
+    m->pf_xb = (__nv_bfloat16 *)(w + wl.pf_xb); m->pf_xb_h = (__nv_bfloat16 *)(w + wl.pf_xb_h); m->pf_xb_a = (__nv_bfloat16 *)(w + wl.pf_xb_a);
+    m->pf_xb_rows = gemm_tc_rows(v.pf_rows);
     m->pf_rows = v.pf_rows; m->pf_rowtab = (int4 *)(w + wl.pf_rowtab); m->pf_segtab = (int4 *)(w + wl.pf_segtab); m->pf_list = (int2 *)(w + wl.pf_list);
     m->pf_xbc = (float *)(w + wl.pf_xbc); m->pf_dtv = (float *)(w + wl.pf_dtv); m->pf_hfin = (float *)(w + wl.pf_hfin); m->pf_rec = (float *)(w + wl.pf_rec); m->pf_q = (__nv_bfloat16 *)(w + wl.pf_q);
     m->xb_h = (__nv_bfloat16 *)(w + wl.xb_h); m->xb_a = (__nv_bfloat16 *)(w + wl.xb_a); m->ssbuf = (float *)(w + wl.ssbuf);

@@ -80,9 +80,10 @@ struct hs_model {
     std::vector<CUtensorMap> kmaps, vmaps;   // per attention layer (streaming attention form)
     int tc_min_rows_auto;                 // the automatic row threshold of the tcgen05 kernel for this model
     __nv_bfloat16 *xb_h, *xb_a; float *ssbuf;   // packed residual stream / MLP activations handed from projection to projection, row statistics
-    // prompt path: activation rows per pass (0: prompts go through verify passes), row / segment / gather tables, conv
-    // outputs, per-head dt and decay, query planes, hidden rows of the prompts' last positions
-    int pf_rows; int4 *pf_rowtab, *pf_segtab; int2 *pf_list; float *pf_xbc, *pf_dtv, *pf_hfin, *pf_rec; __nv_bfloat16 *pf_q;
+    // prompt path: activation rows per pass (0: prompts go through verify passes), the activations of a pass as above,
+    // row / segment / gather tables, conv outputs, per-head dt and decay, query planes, hidden rows of the prompts' last positions
+    int pf_rows; float *pf_h[2], *pf_zx, *pf_gbuf, *pf_obuf, *pf_ss; __nv_bfloat16 *pf_xb, *pf_xb_h, *pf_xb_a; int64_t pf_xb_rows;
+    int4 *pf_rowtab, *pf_segtab; int2 *pf_list; float *pf_xbc, *pf_dtv, *pf_hfin, *pf_rec; __nv_bfloat16 *pf_q;
     void *am_part;             // argmax partials [B*Tm][HS_ARGMAX_CHUNKS] x 16 bytes
     // conv buffers
     float *cw, *hist, *dcw;
