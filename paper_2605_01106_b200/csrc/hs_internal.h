@@ -323,6 +323,7 @@ struct PfAttnArgs {
     const __nv_bfloat16 *q; int64_t q_plane;
     const __nv_bfloat16 *Kc, *Vc; const int32_t *kv_len; int qh, kvh, hd, cap;
     float *o;
+    bool beside;                                                                     // launched behind the scan of the same block, which it does not read
 };
 cudaError_t configure_prefill();
 int64_t pf_record_floats(int rows, int segs, int heads, bool gdn);   // scratch of the scans
