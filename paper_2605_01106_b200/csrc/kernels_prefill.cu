@@ -268,27 +268,28 @@ __global__ void __launch_bounds__(256) pf_gram_kernel(const PfScanArgs a) {
     pdl_trigger();
 }
 
-// The Mamba-2 scan.  grid = (strips of 8 * RW state rows, segments); eight consumer warps and one producer warp.  A warp
+// The Mamba-2 scan.  grid = (strips of NW * RW state rows, segments); NW consumer warps and one producer warp.  A warp
 // owns RW rows of the [heads * P][N] state (they may belong to two heads) for the whole segment, lane l holding N / 32
-// values of each.  RW is the smallest that leaves at most one block per SM (see launch_ssm_n).
-// Bound by latency within a tile at few rows, by the fp32 pipes at many.
-constexpr int SC_WARPS = 8, SC_THREADS = (SC_WARPS + 1) * 32;
-__host__ __device__ constexpr int sc_stage_floats(int N, int RW) { return SC_POS * (2 * N + 2 * SC_WARPS * RW) + 4 * REC_SSM; }
+// values of each.  Bound by latency within a tile at few rows, by reading B and C out of shared memory (every warp reads
+// them all) and the fp32 pipes at many.  Few warps of many rows read less, many warps hide more: up to 24 rows a block four
+// warps are faster (0.5B-class, 512 positions, 16 rows: prompt pass 6.15 ms with eight warps, 5.94 with four), at 40 rows
+// eight (3B-class, 2048 positions: 52.2 ms, 54.7 with four warps of nine).
+__host__ __device__ constexpr int sc_stage_floats(int N, int CR) { return SC_POS * (2 * N + 2 * CR) + 4 * REC_SSM; }
 
-template <int EPL, int RW>
-__global__ void __launch_bounds__(SC_THREADS)
+template <int EPL, int RW, int NW>
+__global__ void __launch_bounds__(NW * 32 + 32)
 pf_ssm_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mBC, const __grid_constant__ CUtensorMap mX,
               const __grid_constant__ CUtensorMap mZ, const int stages) {
     constexpr int N = 32 * EPL, VW = EPL < 4 ? EPL : 4, NVEC = EPL / VW, NP = EPL / 2, PPV = NP / NVEC;
-    constexpr int CR = SC_WARPS * RW, STG = sc_stage_floats(N, RW), RWP = (RW + 1) & ~1;
+    constexpr int CR = NW * RW, STG = sc_stage_floats(N, CR), RWP = (RW + 1) & ~1;
     constexpr int BCW = 2 * N < 256 ? 2 * N : 256;                             // columns of one B | C copy
     extern __shared__ __align__(128) float sm_raw[];
     float *sm = sm_raw + ((128u - (smem_u32(sm_raw) & 127u)) & 127u) / 4;
-    __shared__ __align__(16) float2 es[SC_WARPS][SC_POS + 1][RWP];             // per warp: E_j x_j of its rows, then P_7; each twice
+    __shared__ __align__(16) float2 es[NW][SC_POS + 1][RWP];             // per warp: E_j x_j of its rows, then P_7; each twice
     __shared__ __align__(8) uint64_t full[SC_MAXSTAGES], empty[SC_MAXSTAGES];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int R0 = blockIdx.x * CR, Rw = R0 + warp * RW;                       // first row of the block / of the warp
-    if (tid < stages) { mbar_init(&full[tid], 1); mbar_init(&empty[tid], SC_WARPS); mbar_fence_init(); }
+    if (tid < stages) { mbar_init(&full[tid], 1); mbar_init(&empty[tid], NW); mbar_fence_init(); }
     pdl_wait();
     pdl_trigger();                    // the attention of the same block reads nothing of this kernel and runs beside it
     __syncthreads();
@@ -302,7 +303,7 @@ pf_ssm_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mBC, const
     const int ntile = (n + SC_POS - 1) / SC_POS;
     const int h0 = R0 / a.P, nh = (min(R0 + CR, a.di) - 1) / a.P - h0 + 1;     // heads of the block's rows (at most 4)
     bool ok = true;
-    if (warp == SC_WARPS) {
+    if (warp == NW) {
         // ---- producer.  Rows behind a segment's end belong to the next one or lie outside the tensor (zero): finite
         // values with zero coefficients
         if (lane == 0) {
@@ -339,8 +340,10 @@ pf_ssm_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mBC, const
                 st[r][v * PPV] = pk2(x.x, x.y);
                 if (VW == 4) st[r][v * PPV + PPV - 1] = pk2(x.z, x.w);
             }
-        // rows of the warp are finished in groups of 4, 2 and 1: eight positions x four rows are one transposing reduction
-        constexpr int GA = RW >= 4 ? 4 : RW >= 2 ? 2 : 1, GB = RW - GA;         // GB: 0, 1 or 2
+        // rows of the warp are finished in groups of four (eight positions x four rows are one transposing reduction) and
+        // one of the remaining GR
+        constexpr int G4 = RW / 4, GR = RW % 4, GT = G4 + (GR ? 1 : 0), GRX = GR ? GR : 1;
+        static_assert(GR != 3, "the last group has one or two rows");
         struct Out { int i, col, row, head; float D; bool live; };
         auto outputs = [&](int r_lo, int G) {
             const int lpv = 32 / (SC_POS * G), v = lane / lpv;
@@ -349,7 +352,9 @@ pf_ssm_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mBC, const
             const int hd = min(o.row, a.di - 1) / a.P; o.head = (hd - h0) * REC_SSM; o.D = a.D[hd];
             return o;
         };
-        const Out oa = outputs(0, GA), ob = outputs(GA, GB ? GB : 1);
+        Out og[GT];
+#pragma unroll
+        for (int g = 0; g < GT; ++g) og[g] = outputs(4 * g, g < G4 ? 4 : GRX);
         // coefficient lanes: value (j, r) of the update
         constexpr int NQ = (SC_POS * RW + 31) / 32;
         int e_head[NQ], e_j[NQ], e_r[NQ];
@@ -378,7 +383,7 @@ pf_ssm_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mBC, const
                 }
             if (lane < RW) { const float v = rs[p_head + 71]; es[warp][SC_POS][lane] = make_float2(v, v); }
             // products of the old state with C of every position
-            float va[SC_POS * GA], vb[SC_POS * (GB ? GB : 1)];
+            float va[G4 ? G4 : 1][SC_POS * 4], vb[SC_POS * GRX];
 #pragma unroll
             for (int i = 0; i < SC_POS; ++i) {
                 f2 Cv[NP];
@@ -395,8 +400,8 @@ pf_ssm_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mBC, const
                     for (int e = 1; e < NP; ++e) y = fma2(st[r][e], Cv[e], y);
                     float lo, hi;
                     up2(y, lo, hi);
-                    if (r < GA) va[i * GA + (r < GA ? r : 0)] = lo + hi;
-                    else vb[i * (GB ? GB : 1) + (r >= GA ? r - GA : 0)] = lo + hi;
+                    if (r < 4 * G4) va[G4 ? r / 4 % (G4 ? G4 : 1) : 0][i * 4 + r % 4] = lo + hi;
+                    else vb[i * GRX + (r - 4 * G4) % GRX] = lo + hi;
                 }
             }
             __syncwarp();                 // es complete
@@ -433,8 +438,9 @@ pf_ssm_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mBC, const
                 w = fmaf(mb.x, xc[4 * CR], w); y = fmaf(mb.y, xc[5 * CR], y); w = fmaf(mb.z, xc[6 * CR], w); y = fmaf(mb.w, xc[7 * CR], y);
                 a.g[(size_t)(row0 + t * SC_POS + o.i) * a.gw + o.row] = (y + w) * silu_f(zs[o.i * CR + o.col]);
             };
-            finish(xreduce<SC_POS * GA>(va, lane), oa);
-            if (GB) finish(xreduce<SC_POS * (GB ? GB : 1)>(vb, lane), ob);
+#pragma unroll
+            for (int g = 0; g < G4; ++g) finish(xreduce<SC_POS * 4>(va[g], lane), og[g]);
+            if (GR) finish(xreduce<SC_POS * GRX>(vb, lane), og[GT - 1]);
             __syncwarp();                 // es may be overwritten
             if (lane == 0) mbar_arrive(&empty[s]);
             if (++s == stages) { s = 0; ph ^= 1u; }
@@ -455,7 +461,7 @@ pf_ssm_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mBC, const
     if (!ok && lane == 0) atomicCAS(a.status, 0, (int)HS_ERR_TIMEOUT);          // a copy never landed
     if (tid < CR && R0 + tid < a.di) shift_window(a, b, row0, n, R0 + tid);
     if (blockIdx.x == 0)
-        for (int c = tid; c < 2 * N; c += SC_THREADS) shift_window(a, b, row0, n, a.di + c);
+        for (int c = tid; c < 2 * N; c += NW * 32 + 32) shift_window(a, b, row0, n, a.di + c);
 }
 
 // DeltaNet: q and k of a tile L2-normalised (in place), the tile's record.  grid = (tiles, heads, segments), warp = position
@@ -860,16 +866,16 @@ cudaError_t allow_smem(K kernel, size_t bytes) {
 }
 constexpr size_t pa_smem(int hd) { return (size_t)4 * PA_K * (hd + 8) * 2; }
 
-template <int EPL, int RW>
+template <int EPL, int RW, int NW>
 cudaError_t launch_scan(const PfScanArgs &a, cudaStream_t s) {
-    constexpr size_t stage = (size_t)sc_stage_floats(32 * EPL, RW) * 4, alone = 116 * 1024;
+    constexpr size_t stage = (size_t)sc_stage_floats(32 * EPL, NW * RW) * 4, alone = 116 * 1024;
     static bool configured = false;
     if (!configured) {
-        const cudaError_t e = allow_smem(pf_ssm_kernel<EPL, RW>, 6 * stage + 128 > alone ? 6 * stage + 128 : alone);
+        const cudaError_t e = allow_smem(pf_ssm_kernel<EPL, RW, NW>, 6 * stage + 128 > alone ? 6 * stage + 128 : alone);
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    const dim3 grid((a.di + SC_WARPS * RW - 1) / (SC_WARPS * RW), a.nseg);
+    const dim3 grid((a.di + NW * RW - 1) / (NW * RW), a.nseg);
     // at most one block per SM: ask for more than half of its shared memory, or the scheduler puts two on some SMs while
     // others idle (3B-class, 2048 positions: 780 instead of 530 us with the first form of this kernel)
     const bool spread = (int64_t)grid.x * grid.y <= 148;
@@ -878,21 +884,21 @@ cudaError_t launch_scan(const PfScanArgs &a, cudaStream_t s) {
     constexpr int N = 32 * EPL;
     CUtensorMap mBC, mX, mZ;
     cudaError_t e = hs_make_f32_map(&mBC, a.xbc, a.nrows, a.convd, a.convd, 2 * N < 256 ? 2 * N : 256, SC_POS);
-    if (e == cudaSuccess) e = hs_make_f32_map(&mX, a.xbc, a.nrows, a.convd, a.convd, SC_WARPS * RW, SC_POS);
-    if (e == cudaSuccess) e = hs_make_f32_map(&mZ, a.zx, a.nrows, a.di, a.in_ld, SC_WARPS * RW, SC_POS);
+    if (e == cudaSuccess) e = hs_make_f32_map(&mX, a.xbc, a.nrows, a.convd, a.convd, NW * RW, SC_POS);
+    if (e == cudaSuccess) e = hs_make_f32_map(&mZ, a.zx, a.nrows, a.di, a.in_ld, NW * RW, SC_POS);
     if (e != cudaSuccess) return e;
-    return launch_pdl(pf_ssm_kernel<EPL, RW>, grid, dim3(SC_THREADS), smem, s, a, mBC, mX, mZ, stages);
+    return launch_pdl(pf_ssm_kernel<EPL, RW, NW>, grid, dim3(NW * 32 + 32), smem, s, a, mBC, mX, mZ, stages);
 }
 template <int EPL>
 cudaError_t launch_ssm_n(const PfScanArgs &a, cudaStream_t s) {
     const cudaError_t e = launch_pdl(pf_gram_kernel<EPL>, dim3((a.max_seg + SC_POS - 1) / SC_POS, a.nseg), dim3(256), 0, s, a);
     if (e != cudaSuccess) return e;
-    // rows per warp: the fewest that leave at most one block on each of the 148 SMs (the time of a tile grows with them)
+    // rows per block: the fewest that leave at most one block on each of the 148 SMs (the time of a tile grows with them)
     const int64_t rows = (int64_t)a.di * a.nseg;
-    if (rows <= 148 * 8) return launch_scan<EPL, 1>(a, s);
-    if (rows <= 148 * 16) return launch_scan<EPL, 2>(a, s);
-    if (rows <= 148 * 24) return launch_scan<EPL, 3>(a, s);
-    return launch_scan<EPL, 5>(a, s);
+    if (rows <= 148 * 8) return launch_scan<EPL, 2, 4>(a, s);
+    if (rows <= 148 * 16) return launch_scan<EPL, 4, 4>(a, s);
+    if (rows <= 148 * 24) return launch_scan<EPL, 6, 4>(a, s);
+    return launch_scan<EPL, 5, 8>(a, s);
 }
 
 }  // namespace

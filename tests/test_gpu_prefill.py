@@ -31,6 +31,8 @@ def env():
     ("par64", [1500, 2, 700, 33], 8, 2),          # two passes; rollback by replay
     ("par128", [64, 63, 130], 2, 1),
     ("par256", [17, 50], 4, 0),
+    ("par256", [9], 2, 0), ("par256", [17, 50, 8, 20], 2, 0), ("par256", [17, 50, 8, 20, 11], 2, 1),      # 2, 6 and 5 x 8 rows of the scan per warp
+    ("par128", [17, 9, 8, 20, 11], 2, 0), ("par64", [17, 9, 8, 20, 11, 3, 33], 2, 0),
     ("seq", [72, 3, 9, 128, 40], 4, 0),
     ("seq", [1100, 1100], 8, 2),
     ("seq32", [66, 31], 8, 1),
