@@ -22,7 +22,8 @@ __global__ void __launch_bounds__(SSM_THREADS) ssm_kernel(const SsmArgs a) {
 // ------------------------------------------------------------------------------------------------
 constexpr int GDN_THREADS = 256;   // 8 warps x 8 value rows; key dim 64 = 32 lanes x 2
 
-// TMAX: most positions this instance handles (1 for the draft step, 3 for verify at k <= 2, else the maximum).
+// TMAX: most positions this instance handles (1 for the draft step, 3 for verify at k <= 2, 5 at k <= 4, else the maximum;
+// a verify pass of the sequential hybrid at k = 4 in the instance for 9 positions / for 5: 1.056 / 1.037 ms at 5 sequences).
 // Everything the block needs from the in-projection - the raw conv inputs of a thread's own channel for all
 // positions, the gate inputs, the decay / write-strength inputs - is requested right after the wait, before the
 // first value is used: one trip to L2 for the whole kernel.
@@ -292,6 +293,7 @@ cudaError_t launch_ssm(const SsmArgs &a, cudaStream_t s) {
 #define LAUNCH(e_, pr_, t_) launch_pdl(ssm_kernel<e_, pr_, t_>, grid, dim3(SSM_THREADS), 0, s, a)
 #define CASE(n_, e_) if (a.N == n_) return a.T == 1 ? (wide ? LAUNCH(e_, 64, 1) : LAUNCH(e_, 16, 1))               \
                                          : a.T <= 3 ? (wide ? LAUNCH(e_, 64, 3) : LAUNCH(e_, 16, 3))               \
+                                         : a.T <= 5 ? (wide ? LAUNCH(e_, 64, 5) : LAUNCH(e_, 16, 5))               \
                                                     : (wide ? LAUNCH(e_, 64, HS_MAX_T) : LAUNCH(e_, 16, HS_MAX_T))
     CASE(64, 2); CASE(128, 4); CASE(256, 8);
 #undef CASE
@@ -304,5 +306,6 @@ cudaError_t launch_gdn(const GdnArgs &a, cudaStream_t s) {
     const dim3 grid(a.gh, a.nb), block(GDN_THREADS);
     if (a.T == 1) return launch_pdl(gdn_kernel<1>, grid, block, 0, s, a);
     if (a.T <= 3) return launch_pdl(gdn_kernel<3>, grid, block, 0, s, a);
+    if (a.T <= 5) return launch_pdl(gdn_kernel<5>, grid, block, 0, s, a);
     return launch_pdl(gdn_kernel<HS_MAX_T>, grid, block, 0, s, a);
 }

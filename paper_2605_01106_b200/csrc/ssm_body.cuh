@@ -15,6 +15,9 @@ constexpr int SSM_THREADS = 128; // 4 warps x PR / 4 rows
 // two roles of the fused mixer + attention launch of the verify pass.
 // TMAX: most positions this instance handles (1 for the draft step: a much shorter program, which matters
 // because every launch of a step starts with a cold instruction cache).
+// Instances for 1, 3, 5 and 9 positions: the unrolled loads and shared arrays of unused positions cost (verify pass at
+// k = 4 in the instance for 9 / for 5: 0.5B-class, one sequence 1.447 / 1.386 ms, 8 sequences 2.51 / 2.44; 3B-class, one
+// 3.03 / 2.96, 8 sequences 5.89 / 5.67).
 template <int EPL, int SSM_PR, int TMAX>
 __device__ __forceinline__ void ssm_body(const SsmArgs &a, const int bx, const int by, const int bz) {
     constexpr int N = 32 * EPL;

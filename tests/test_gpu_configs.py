@@ -224,3 +224,14 @@ def test_attention_form_boundaries(env, name, batch, k, ctx):
     rep = env["harness"].run_rounds(eng, seqs, s, k, 1, forced=[hi.forced_accept(k, 1, seq=b) for b in range(batch)])
     print(rep)
     assert eng.device_status() == 0
+
+
+@pytest.mark.parametrize("name", ["cfg1_tiny", "test_seq"])
+def test_mixer_instances_by_positions(env, name):
+    # 4 and 5 positions run in the instance for 5, 6 in the one for 9; two sequences, their rows beside each other
+    s, eng, model, seqs = make(env, name, 2, 5, 160, {0, 1}, [70, 33])
+    rep = None
+    for k in (3, 4, 5):
+        rep = env["harness"].run_rounds(eng, seqs, s, k, 2, forced=[hi.forced_accept(k, 2, seq=b + k) for b in range(2)], rep=rep)
+    print(rep)
+    assert eng.device_status() == 0 and rep.rounds == 6
