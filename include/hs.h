@@ -145,9 +145,9 @@ int hs_reset(hs_model *m);
  * prompts back to back (sequence b starts at sum(lens_host[0..b-1])); lens_host[b] >= 1; every id in [0, V),
  * otherwise HS_ERR_INVALID_ARG before anything is enqueued.  Sets the batch
  * size for the following rounds.  Afterwards kv_len[b] = lens[b] and pending[b] = the greedy choice
- * after the last prompt token (generated token #1).  Runs as verify passes over chunks of max_k+1 prompt
- * positions, all sequences of equal chunk length together, with every candidate accepted; nothing waits on the host
- * between chunks.  Synchronises the stream before returning (tokens_host may be reused afterwards). */
+ * after the last prompt token (generated token #1).  Prompts longer than max_k+1 run as passes of up to 2176
+ * positions, all sequences together; shorter ones, and all with HS_FLAG_LITERAL_DRAFT, as verify passes over chunks of
+ * max_k+1 positions with every candidate accepted.  Nothing waits on the host between passes.  Synchronises the stream before returning (tokens_host may be reused afterwards). */
 int hs_prefill(hs_model *m, const int32_t *tokens_host, const int32_t *lens_host, int batch);
 
 /* Draft phase (paper Sec. 3.3, "Draft phase": M_S generates k tokens autoregressively; M_S is Eq. 4 for a

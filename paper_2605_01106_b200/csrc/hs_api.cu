@@ -884,8 +884,8 @@ int hs_prefill(hs_model *m, const int32_t *tokens_host, const int32_t *lens_host
     // Prompts longer than one verify pass: passes of many positions (their activations do not fit the verify-pass
     // kernels' registers, the projections need the tcgen05 path).  The literal draft state also runs the draft model
     // over the prompt and stays on verify-sized passes.  Measured, chunks of max_k + 1 positions against wide passes: 512
-    // tokens on the 0.5B-class hybrid 103.4 -> 14.0 ms, 2048 tokens on the 3B-class one 1371 -> 80.4 ms, four ragged prompts
-    // (2.3 k tokens) on the sequential one 229 -> 28.6 ms.  A prompt of at most one chunk is one verify pass either way.
+    // tokens on the 0.5B-class hybrid 103.4 -> 5.9 ms, 2048 tokens on the 3B-class one 1371 -> 52 ms, four ragged prompts
+    // (2.3 k tokens) on the sequential one 229 -> 12.6 ms.  A prompt of at most one chunk is one verify pass either way.
     if (longest > m->Tm && g_hs_gemm_tc && !m->literal) return prefill_wide(m, tokens_host, lens_host, batch);
     // Chunk c covers prompt positions [c * Tm, (c + 1) * Tm) of every sequence that reaches that far; neighbouring
     // sequences with the same number of tokens in the chunk go out as one verify pass with every candidate accepted.
