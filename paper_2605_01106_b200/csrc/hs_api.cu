@@ -240,9 +240,11 @@ struct AttnGeom {
 AttnGeom attn_geom(const hs_model *m, int Tq, int T, int b0, int nb) {
     const hs_config &c = m->c;
     // One launch for mixer and attention spares a link of the chain, but every mixer block then carries the attention's
-    // shared memory and two or three fit on an SM.  Verify pass of the 0.5B-class shape, together / apart: 2 sequences
-    // (256 mixer blocks) 1.47 / 1.58 ms, 3 sequences (384) 2.00 / 1.75 ms; 3B-class, 1 sequence (320) 3.38 / 3.04 ms.
-    const bool few = c.arch == HS_ARCH_PARALLEL && (int64_t)(c.P / 16) * c.H * nb <= 2 * 148;
+    // shared memory: while the mixer blocks are at most four per SM and the cache takes at most 128 keys per CTA.  Verify
+    // pass, apart / together: 0.5B-class, 4 sequences (512 mixer blocks) of 50 keys, k = 0 / 1 / 2 / 4: 1.32 / 1.54 / 1.63 /
+    // 1.85 against 1.22 / 1.43 / 1.49 / 1.86 ms; 3 of 400, k = 4: 1.74 / 1.61; 4 of 900, k = 1: 1.64 / 1.54; 3B-class, one
+    // (320 blocks) of 200, k = 4: 2.87 / 2.74, of 900, k = 2: 2.83 / 2.81.
+    const bool few = c.arch == HS_ARCH_PARALLEL && (int64_t)(c.P / 16) * c.H * nb <= 4 * 148;
     if (m->att_force_chunk) return AttnGeom{m->att_force_chunk, m->att_force_tiles < 0 ? -m->att_force_tiles : m->att_force_tiles, 0, m->att_force_tiles < 0 ? 1 : 0, few};
     int maxlen = 0;
     for (int b = b0; b < b0 + nb; ++b) if (m->kv_upper[b] > maxlen) maxlen = m->kv_upper[b];

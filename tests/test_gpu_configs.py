@@ -216,7 +216,7 @@ def test_lean_attention_with_several_row_tiles(env, name, k, ctx):
 @pytest.mark.parametrize("name,batch,k,ctx", [
     ("cfg1_tiny", 1, 4, 1019), ("cfg1_tiny", 1, 4, 1020),       # 1024 keys: lean beside the mixer; 1025: lean, a launch of its own
     ("cfg1_tiny", 1, 4, 2299), ("cfg1_tiny", 1, 4, 2300),       # 2304 keys: the longest lean cache; 2305: general form beside the mixer
-    ("cfg1_tiny", 3, 4, 2300), ("cfg1_tiny", 10, 2, 100),       # 114 tiles of 128 keys: streaming; 320 mixer blocks: apart, lean
+    ("cfg1_tiny", 3, 4, 2300), ("cfg1_tiny", 20, 2, 100),       # 114 tiles of 128 keys: streaming; 640 mixer blocks: apart, lean
     ("cfg1_tiny", 38, 2, 100), ("cfg1_tiny", 26, 4, 200),       # more than 4 lean CTAs per SM: general; 104 tiles, two per cache: streaming
     ("cfg2_0p5b", 1, 2, 2301)])                                 # 288 keys per CTA at a head dimension of 128
 def test_attention_form_boundaries(env, name, batch, k, ctx):
