@@ -243,8 +243,11 @@ AttnGeom attn_geom(const hs_model *m, int Tq, int T, int b0, int nb) {
     // shared memory: while the mixer blocks are at most four per SM and the cache takes at most 128 keys per CTA.  Verify
     // pass, apart / together: 0.5B-class, 4 sequences (512 mixer blocks) of 50 keys, k = 0 / 1 / 2 / 4: 1.32 / 1.54 / 1.63 /
     // 1.85 against 1.22 / 1.43 / 1.49 / 1.86 ms; 3 of 400, k = 4: 1.74 / 1.61; 4 of 900, k = 1: 1.64 / 1.54; 3B-class, one
-    // (320 blocks) of 200, k = 4: 2.87 / 2.74, of 900, k = 2: 2.83 / 2.81.
-    const bool few = c.arch == HS_ARCH_PARALLEL && (int64_t)(c.P / 16) * c.H * nb <= 4 * 148;
+    // (320 blocks) of 200, k = 4: 2.87 / 2.74, of 900, k = 2: 2.83 / 2.81.  Not beside lean blocks of more than 96 keys with
+    // several row tiles, two of which fill an SM, once the mixer blocks are more than two per SM (3 sampled sequences of up to
+    // 901 keys, k = 4, round: 5.06 / 5.17 ms).
+    const int64_t mixers = (int64_t)(c.P / 16) * c.H * nb;
+    const bool few = c.arch == HS_ARCH_PARALLEL && mixers <= 4 * 148;
     if (m->att_force_chunk) return AttnGeom{m->att_force_chunk, m->att_force_tiles < 0 ? -m->att_force_tiles : m->att_force_tiles, 0, m->att_force_tiles < 0 ? 1 : 0, few};
     int maxlen = 0;
     for (int b = b0; b < b0 + nb; ++b) if (m->kv_upper[b] > maxlen) maxlen = m->kv_upper[b];
@@ -261,7 +264,7 @@ AttnGeom attn_geom(const hs_model *m, int Tq, int T, int b0, int nb) {
         // 512, 96 CTAs: 1.75 / 1.90); beyond four per SM the general form takes over.
         int ck = 32;
         while (ck < 288 && 8 * ck < maxlen + T) ck += 32;
-        const bool fuse = few && ck <= 128;
+        const bool fuse = few && ck <= 128 && (ck <= 96 || groups <= 16 || mixers <= 2 * 148);
         const int ctas = nb * c.kvh * ((groups + 15) / 16) * 8;
         if (g_hs_attn_small && ctas <= (streams || fuse ? 148 : 4 * 148) && 8 * ck >= maxlen + T) return AttnGeom{ck, 1, 1, 0, fuse};
     }
