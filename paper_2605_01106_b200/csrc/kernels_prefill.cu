@@ -192,7 +192,9 @@ __device__ __forceinline__ void shift_window(const PfScanArgs &a, int b, int row
 //             MK_ij = beta_i (k_i . k_j) prod_{j<u<=i} alpha_u ,  MQ_ij = (q_i . k_j) prod.. ,  E_j = prod_{j<u<=7} alpha_u
 // Against one position at a time: 17 instead of 24 multiply-adds per state element and tile, no serial chain but the
 // eight-term solve, and one reduction over lanes per (row, position) of which 32 go together.  All of it in fp32.
-// Positions beyond the end of a segment have decay 1 and E_j = 0.
+// Positions beyond the end of a segment have decay 1 and E_j = 0.  The activation rows behind a segment's end belong to the
+// next sequence, and a zero coefficient does not silence an infinity or a NaN: the partial tile a segment may end with is
+// copied row by row, and the rest of it is zeroed.
 // The tiles arrive through a ring of shared-memory stages: a producer thread issues a tile's four or five copies (tensor
 // copies of eight rows; one bulk copy per row and piece, 25 a tile, took 1900 cycles to issue and set the pace), the
 // consumer warps only wait for bytes and hand stages back - no block-wide barrier in the loop.
@@ -211,6 +213,12 @@ __device__ __forceinline__ void tensor_tile(void *dst_smem, const CUtensorMap *m
 }
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(bar)) : "memory");
+}
+// rows cnt .. 7 of a tile of W-float rows, by one warp
+template <int W>
+__device__ __forceinline__ void zero_tail(float *tile, int cnt, int lane) {
+#pragma unroll 1
+    for (int i = cnt * W + 4 * lane; i < SC_POS * W; i += 128) *reinterpret_cast<float4 *>(tile + i) = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // grid = (tiles, segments), eight warps: warp i takes position i of the tile
@@ -273,11 +281,11 @@ __global__ void __launch_bounds__(256) pf_gram_kernel(const PfScanArgs a) {
 // values of each.  Bound by latency within a tile at few rows, by reading B and C out of shared memory (every warp reads
 // them all) and the fp32 pipes at many.  Few warps of many rows read less, many warps hide more: up to 24 rows a block four
 // warps are faster (0.5B-class, 512 positions, 16 rows: prompt pass 6.15 ms with eight warps, 5.94 with four), at 40 rows
-// eight (3B-class, 2048 positions: 52.2 ms, 54.7 with four warps of nine).
+// eight (3B-class, 2048 positions: 52.2 ms, 54.7 with four warps of nine).  (Two blocks of eight warps fit an SM at N = 64.)
 __host__ __device__ constexpr int sc_stage_floats(int N, int CR) { return SC_POS * (2 * N + 2 * CR) + 4 * REC_SSM; }
 
 template <int EPL, int RW, int NW>
-__global__ void __launch_bounds__(NW * 32 + 32)
+__global__ void __launch_bounds__(NW * 32 + 32, EPL == 2 && NW == 8 ? 2 : 1)
 pf_ssm_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mBC, const __grid_constant__ CUtensorMap mX,
               const __grid_constant__ CUtensorMap mZ, const int stages) {
     constexpr int N = 32 * EPL, VW = EPL < 4 ? EPL : 4, NVEC = EPL / VW, NP = EPL / 2, PPV = NP / NVEC;
@@ -304,13 +312,13 @@ pf_ssm_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mBC, const
     const int h0 = R0 / a.P, nh = (min(R0 + CR, a.di) - 1) / a.P - h0 + 1;     // heads of the block's rows (at most 4)
     bool ok = true;
     if (warp == NW) {
-        // ---- producer.  Rows behind a segment's end belong to the next one or lie outside the tensor (zero): finite
-        // values with zero coefficients
+        // ---- producer: the whole tiles, then the partial one
+        const float *rec = a.rec + ((size_t)rec_slot(row0, blockIdx.y, 0) * a.heads + h0) * REC_SSM;
+        const uint32_t rbytes = (uint32_t)nh * REC_SSM * 4;
+        const int whole = n / SC_POS, tail = n % SC_POS;
+        int s = 0; uint32_t ph = 0;
         if (lane == 0) {
-            const float *rec = a.rec + ((size_t)rec_slot(row0, blockIdx.y, 0) * a.heads + h0) * REC_SSM;
-            const uint32_t rbytes = (uint32_t)nh * REC_SSM * 4;
-            int s = 0; uint32_t ph = 0;
-            for (int t = 0; t < ntile; ++t) {
+            for (int t = 0; t < whole; ++t) {
                 if (!mbar_wait_n(&empty[s], ph ^ 1u, 1 << 20)) { ok = false; break; }
                 float *dst = sm + (size_t)s * STG;
                 const int y = row0 + t * SC_POS;
@@ -322,6 +330,28 @@ pf_ssm_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mBC, const
                 bulk_tile(dst + SC_POS * (2 * N + 2 * CR), rec, rbytes, &full[s]);
                 rec += (size_t)a.heads * REC_SSM;
                 if (++s == stages) { s = 0; ph ^= 1u; }
+            }
+        }
+        s = whole % stages; ph = (uint32_t)(whole / stages) & 1u;
+        ok = __all_sync(0xffffffffu, ok);
+        if (ok && tail) ok = __all_sync(0xffffffffu, mbar_wait_n(&empty[s], ph ^ 1u, 1 << 20));
+        if (ok && tail) {
+            float *dst = sm + (size_t)s * STG, *dx = dst + SC_POS * 2 * N, *dz = dx + SC_POS * CR;
+#pragma unroll
+            for (int q = 0; q < 2 * N / BCW; ++q) zero_tail<BCW>(dst + q * SC_POS * BCW, tail, lane);
+            zero_tail<CR>(dx, tail, lane); zero_tail<CR>(dz, tail, lane);
+            __syncwarp();
+            if (lane == 0) {
+                mbar_expect_tx(&full[s], (uint32_t)tail * (2 * N + 2 * CR) * 4 + rbytes);
+                const float *x = a.xbc + (size_t)(row0 + whole * SC_POS) * a.convd, *z = a.zx + (size_t)(row0 + whole * SC_POS) * a.in_ld;
+#pragma unroll 1
+                for (int i = 0; i < tail; ++i) {
+#pragma unroll
+                    for (int q = 0; q < 2 * N / BCW; ++q) bulk_tile(dst + q * SC_POS * BCW + i * BCW, x + (size_t)i * a.convd + a.di + q * BCW, BCW * 4, &full[s]);
+                    bulk_tile(dx + i * CR, x + (size_t)i * a.convd + R0, CR * 4, &full[s]);       // (columns beyond di: B, never live)
+                    bulk_tile(dz + i * CR, z + (size_t)i * a.in_ld + R0, CR * 4, &full[s]);
+                }
+                bulk_tile(dz + SC_POS * CR, a.rec + ((size_t)rec_slot(row0, blockIdx.y, whole) * a.heads + h0) * REC_SSM, rbytes, &full[s]);
             }
         }
     } else {
@@ -512,11 +542,11 @@ __global__ void __launch_bounds__(256) pf_gdn_gram_kernel(const PfScanArgs a) {
 // The delta rule.  grid = (strips of 16 * RT value rows, heads, segments), four consumer warps and one producer warp; eight
 // lanes share RT rows (columns 4 c .. 4 c + 3 and 32 + 4 c .. of lane c), the tile's k vectors stay in registers between
 // the products and the update.  Every lane of a row gathers the eight right-hand sides and solves for the u_i itself:
-// one exchange instead of eight.
+// one exchange instead of eight.  (RT = 2 goes out with more blocks than SMs: registers for three on each.)
 constexpr int GD_STG = (SC_POS * (128 + 32) + REC_GDN + 31) / 32 * 32, GD_STAGES = 4, GD_WARPS = 4, GD_THREADS = (GD_WARPS + 1) * 32;
 
 template <int RT>
-__global__ void __launch_bounds__(GD_THREADS)
+__global__ void __launch_bounds__(GD_THREADS, RT == 2 ? 3 : 1)
 pf_gdn_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mQK, const __grid_constant__ CUtensorMap mV) {
     __shared__ __align__(128) float sm[GD_STAGES * GD_STG];
     __shared__ __align__(8) uint64_t full[GD_STAGES], empty[GD_STAGES];
@@ -535,11 +565,12 @@ pf_gdn_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mQK, const
     const int ntile = (n + SC_POS - 1) / SC_POS;
     bool ok = true;
     if (warp == GD_WARPS) {
-        // ---- producer: stage = q[8][64] k[8][64] v[8][16 RT] record
+        // ---- producer: stage = q[8][64] k[8][64] v[8][16 RT] record; the whole tiles, then the partial one
+        const float *rec = a.rec + ((size_t)rec_slot(row0, blockIdx.z, 0) * a.heads + h) * REC_GDN;
+        const int whole = n / SC_POS, tail = n % SC_POS;
+        int s = 0; uint32_t ph = 0;
         if (lane == 0) {
-            const float *rec = a.rec + ((size_t)rec_slot(row0, blockIdx.z, 0) * a.heads + h) * REC_GDN;
-            int s = 0; uint32_t ph = 0;
-            for (int t = 0; t < ntile; ++t) {
+            for (int t = 0; t < whole; ++t) {
                 if (!mbar_wait_n(&empty[s], ph ^ 1u, 1 << 20)) { ok = false; break; }
                 float *dst = sm + (size_t)s * GD_STG;
                 const int y = row0 + t * SC_POS;
@@ -550,6 +581,25 @@ pf_gdn_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mQK, const
                 bulk_tile(dst + SC_POS * 160, rec, REC_GDN * 4, &full[s]);
                 rec += (size_t)a.heads * REC_GDN;
                 if (++s == GD_STAGES) { s = 0; ph ^= 1u; }
+            }
+        }
+        s = whole % GD_STAGES; ph = (uint32_t)(whole / GD_STAGES) & 1u;
+        ok = __all_sync(0xffffffffu, ok);
+        if (ok && tail) ok = __all_sync(0xffffffffu, mbar_wait_n(&empty[s], ph ^ 1u, 1 << 20));
+        if (ok && tail) {
+            float *dst = sm + (size_t)s * GD_STG;
+            zero_tail<64>(dst, tail, lane); zero_tail<64>(dst + 512, tail, lane); zero_tail<16 * RT>(dst + 1024, tail, lane);
+            __syncwarp();
+            if (lane == 0) {
+                mbar_expect_tx(&full[s], (uint32_t)tail * (128 + 16 * RT) * 4 + REC_GDN * 4);
+#pragma unroll 1
+                for (int i = 0; i < tail; ++i) {
+                    const float *x = a.xbc + (size_t)(row0 + whole * SC_POS + i) * a.convd;
+                    bulk_tile(dst + i * 64, x + h * 64, 256, &full[s]);
+                    bulk_tile(dst + 512 + i * 64, x + nk + h * 64, 256, &full[s]);
+                    bulk_tile(dst + 1024 + i * 16 * RT, x + 2 * nk + h * dv + v0, 64 * RT, &full[s]);
+                }
+                bulk_tile(dst + SC_POS * 160, a.rec + ((size_t)rec_slot(row0, blockIdx.z, whole) * a.heads + h) * REC_GDN, REC_GDN * 4, &full[s]);
             }
         }
     } else {

@@ -73,3 +73,26 @@ def test_logits_after_prefill(env):
         q.prefill(prompt[:45])
         want = q.round(2, cand_in=np.asarray(prompt[45:48], np.int32), forced_n=2, want_logits=True)["logits"][i]
         assert np.abs(got[i] - want).max() <= env["harness"].LOGIT_TOL
+
+
+@pytest.mark.parametrize("name,lens,max_k", [("par64", [13, 9, 20], 4), ("par128", [3, 30, 8, 12], 2), ("par256", [21, 4, 33], 4), ("seq", [13, 9, 20], 4), ("seq32", [31, 6], 4)])
+def test_sequences_of_a_prompt_pass_are_independent(env, name, lens, max_k):
+    # sequence 1 consists of a token whose embedding is not finite; the others, whose last partial scan tile lies in front of
+    # its rows or whose rows lie behind them, are what they are without it
+    s = SHAPES[name]
+    blob, table = hi.make_weights(s, 0, "jitter")
+    prompts = [hi.make_prompt(s.V, n, seq=40 + b) for b, n in enumerate(lens)]
+    bad = next(t for t in range(s.V) if all(t not in p for p in prompts))
+    prompts[1] = np.full(lens[1], bad, np.int32)
+    off = table[(-1, hi.G_EMBED)][0] + 2 * s.d * bad
+    blob[off:off + 2 * s.d].view(np.uint16)[:] = 0x7FC0                # bf16 NaN
+    cap = max(lens) + 32
+    eng = env["hs"].Engine(s, blob, max_batch=len(lens), max_k=max_k, kv_capacity=cap)
+    model = env["oracle"].Model(s, blob, table, cap)
+    seqs = [None if b == 1 else model.new_seq() for b in range(len(lens))]
+    for q, p in zip(seqs, prompts):
+        if q is not None:
+            q.prefill(p)
+    eng.prefill(prompts)
+    env["harness"].compare_states(eng, seqs, s)
+    assert eng.device_status() == 0
