@@ -8,11 +8,17 @@ namespace hsd {
 
 constexpr int TC_BM = 128;          // weight rows per CTA
 constexpr int TC_BK = 64;           // K columns per stage: one 128-byte swizzle atom of bf16
+// tcgen05 truncates when it adds a product to an accumulator.  Measured against exact sums (in-projections of K = 512 .. 8192,
+// 8 .. 1024 MMAs on an accumulator): the finished sum is short by 1.3 .. 1.6e-8 of itself per MMA, 2^-26, and spreads by 0.6
+// of that.  The epilogues put the mean back.
+constexpr float TC_LOST = 1.f / 67108864.f;
 
 struct TcArgs {
     int O, nk0, nk1;            // output rows; 64-column K blocks of segment 0 / 1
     int nrows, rpad, bnh;       // activation rows, rows per plane of the packed operand, rows per plane per CTA
     int ns;                     // shared-memory stages (at most TC_MAXSTAGES)
+    int seg;                    // two-CTA tiles: K blocks per segment
+    float found;                // 1 + what truncation took from a sum; two-CTA tiles in segments: what it takes per K block
     int rb;                     // K split: activation rows of a tile each rank finishes (a power of two >= 4, rb * S >= bnh)
     float *out; int ldo;
     const float *resid; int rparts; int64_t rpstride;

@@ -546,7 +546,7 @@ int prefill_pass(hs_model *m, int rows, int nseg, int max_seg, int *cur_out) {
     for (int l = 0; l < c.L; ++l) {
         const HsLayer &ly = m->layers[l];
         const bool attn = ly.type != HS_LAYER_GDN, rec = ly.type != HS_LAYER_ATT, par = ly.type == HS_LAYER_PAR;
-        GemvArgs ga{};
+        GemvArgs ga{}; ga.prompt = true;
         ga.W0 = ly.W_in; ga.ldw0 = d; ga.K0 = d; ga.x0 = m->pf_h[cur]; ga.ldx0 = d; ga.xparts = 1;
         ga.norm_w = ly.norm1; ga.eps = c.eps; ga.O = ly.in_rows_full; ga.out = m->pf_zx; ga.ldo = m->in_rows_max;
         ga.nrows = rows; ga.epi = EPI_STORE; ga.early_trigger = 0; ga.xb = m->pf_xb; ga.xb_rows = m->pf_xb_rows;
@@ -586,7 +586,7 @@ int prefill_pass(hs_model *m, int rows, int nseg, int max_seg, int *cur_out) {
             PROF(HS_PROF_ATTN, 0, launch_pf_attn(aa, s), "prefill attention");
             ++m->launches;
         }
-        GemvArgs go{};
+        GemvArgs go{}; go.prompt = true;
         go.O = d; go.out = m->pf_h[cur ^ 1]; go.ldo = d; go.max_oparts = 1; go.resid = m->pf_h[cur]; go.rparts = 1;
         go.nrows = rows; go.epi = EPI_RESID; go.xparts = 1; go.early_trigger = 0; go.xb = m->pf_xb; go.xb_rows = m->pf_xb_rows;
         if (rec) {
@@ -599,11 +599,11 @@ int prefill_pass(hs_model *m, int rows, int nseg, int max_seg, int *cur_out) {
         go.pk_out = m->pf_xb_h; go.pk_ld = d; go.pk_nw = ly.norm2; go.ss_out = m->pf_ss;
         PROF(HS_PROF_GEMV, gemv_bytes(go), launch_gemm_tc(go, st_w, s, &m->launches, nullptr), "prefill out_proj");
         cur ^= 1;
-        GemvArgs gu{};
+        GemvArgs gu{}; gu.prompt = true;
         gu.W0 = ly.W_gu; gu.ldw0 = d; gu.K0 = d; gu.O = 2 * c.ff; gu.out = nullptr; gu.ldo = c.ff; gu.nrows = rows; gu.epi = EPI_SWIGLU;
         gu.eps = c.eps; gu.early_trigger = 0; gu.pk_in = m->pf_xb_h; gu.ss_in = m->pf_ss; gu.ss_parts = ss_parts; gu.pk_out = m->pf_xb_a; gu.pk_ld = c.ff;
         PROF(HS_PROF_GEMV, gemv_bytes(gu), launch_gemm_tc(gu, st_w, s, &m->launches, nullptr), "prefill gate_up");
-        GemvArgs dn{};
+        GemvArgs dn{}; dn.prompt = true;
         dn.W0 = ly.W_down; dn.ldw0 = c.ff; dn.K0 = c.ff; dn.O = d; dn.out = m->pf_h[cur ^ 1]; dn.ldo = d; dn.max_oparts = 1;
         dn.resid = m->pf_h[cur]; dn.rparts = 1; dn.nrows = rows; dn.epi = EPI_RESID; dn.early_trigger = 0; dn.pk_in = m->pf_xb_a;
         dn.pk_out = m->pf_xb_h; dn.pk_ld = d; dn.pk_nw = l + 1 < c.L ? m->layers[l + 1].norm1 : m->final_norm; dn.ss_out = m->pf_ss;

@@ -156,6 +156,7 @@ struct GemvArgs {
     int epi;
     const void *pf_ptr; int64_t pf_bytes;   // optional: weights of the next projection, prefetched into L2
     __nv_bfloat16 *xb; int64_t xb_rows;     // scratch for the packed activation operand of the many-row kernel: [2][xb_rows][K0+K1]
+    bool prompt;              // a projection of a prompt pass
     int early_trigger;        // 1: let the next kernel start before this one has waited for its predecessor
                               // (what a prologue may read before its own wait is stated in hs_device.cuh)
     // Many-row kernel only: projections hand the packed operand to each other, so that no packing kernel sits on the
@@ -182,7 +183,7 @@ cudaError_t launch_gemm_tc(const GemvArgs &a, int32_t *status, cudaStream_t s, i
 cudaError_t launch_pack(const GemvArgs &a, int rpad, cudaStream_t s, int64_t *launches);
 cudaError_t hs_make_tile_map(CUtensorMap *map, const void *base, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_rows);
 // hundreds of activation rows: persistent two-CTA tiles (kernels_gemm_wide.cu)
-bool gemm_wide_applies(int nrows, int O);
+bool gemm_wide_applies(int nrows, int O, int range, bool prompt);   // range: K blocks of 64 that a CTA of the many-row kernel would take
 cudaError_t configure_gemm_wide();
 cudaError_t launch_gemm_wide(const GemvArgs &a, int32_t *status, cudaStream_t s, int64_t *launches, int *oparts);
 cudaError_t configure_attn();

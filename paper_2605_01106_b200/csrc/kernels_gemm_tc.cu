@@ -131,7 +131,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
     const uint32_t sbase = (smem_u32(smraw) + 1023u) & ~1023u;            // swizzled tiles need 1024-byte alignment
     unsigned char *stages = smraw + (sbase - smem_u32(smraw));
     float *rx = reinterpret_cast<float *>(stages + a.off_rx);             // [S][128][rb]: partial tiles sent by the cluster's ranks
-    float *rstd_s = reinterpret_cast<float *>(stages + a.off_misc);       // [BNH]
+    float *rstd_s = reinterpret_cast<float *>(stages + a.off_misc);       // [BNH] 1/rms and what truncation took
     float *nw_s = rstd_s + 128;                                           // [128]
     float *ssred = nw_s + 128;                                            // [4][BNH]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -221,7 +221,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
                 for (int p = 0; p < a.ss_parts; ++p) t += __ldcg(a.ss_in + (size_t)p * a.rpad + n0h + i);
                 r = rsqrtf(t * a.inv_k + a.eps);
             }
-            rstd_s[i] = r;
+            rstd_s[i] = r * a.found;
         }
     }
     if (warp < 2 && !(warp == 0 && lane == 0)) pdl_wait();          // the epilogue reads the residual stream
@@ -423,7 +423,6 @@ cudaError_t launch_pack(const GemvArgs &a, int rpad, cudaStream_t s, int64_t *la
 cudaError_t launch_gemm_tc(const GemvArgs &a, int32_t *status, cudaStream_t s, int64_t *launches, int *oparts) {
     if ((!a.xb && !a.pk_in) || (a.K0 & 63) || (a.K1 & 63) || a.nrows < 1) return cudaErrorInvalidValue;
     const int Kt = a.K0 + a.K1;
-    if (gemm_wide_applies(a.nrows, a.O)) return launch_gemm_wide(a, status, s, launches, oparts);
     const int mtiles = (a.O + TC_BM - 1) / TC_BM, nk = Kt / TC_BK;
     // Rows per plane per CTA.  The packed operand is laid out for the largest tile (rpad rows per plane); a small
     // weight matrix is cheap to read again from L2, so its activation rows are cut into more, smaller tiles, which
@@ -463,6 +462,7 @@ cudaError_t launch_gemm_tc(const GemvArgs &a, int32_t *status, cudaStream_t s, i
         S = cand; rb = crb; rx_bytes = crx; budget = pair ? TC_SMEM_PAIR : TC_SMEM_MAX;
     }
     const int nkl = (nk + S - 1) / S;
+    if (gemm_wide_applies(a.nrows, a.O, nkl, a.prompt)) return launch_gemm_wide(a, status, s, launches, oparts);
     int ns = (int)((budget - rx_bytes - TC_MISC_BYTES - 1024) / stage);
     if (ns > TC_MAXSTAGES) ns = TC_MAXSTAGES;
     if (ns > nkl) ns = nkl;
@@ -496,7 +496,7 @@ cudaError_t launch_gemm_tc(const GemvArgs &a, int32_t *status, cudaStream_t s, i
     }
     t.pf_ptr = a.pf_ptr; t.pf_bytes = a.pf_ptr ? (long long)a.pf_bytes : 0;
     t.off_rx = (int)((size_t)ns * stage); t.off_misc = (int)((size_t)ns * stage + rx_bytes);
-    t.early_trigger = a.early_trigger;
+    t.early_trigger = a.early_trigger; t.found = 1.f + (float)(nk * (TC_BK / 16)) / (float)S * TC_LOST;
     if (oparts) *oparts = 1;
     if (launches) ++*launches;
     const dim3 grid(S, mtiles, ntiles);

@@ -96,3 +96,53 @@ def test_sequences_of_a_prompt_pass_are_independent(env, name, lens, max_k):
     eng.prefill(prompts)
     env["harness"].compare_states(eng, seqs, s)
     assert eng.device_status() == 0
+
+
+@pytest.mark.parametrize("d,H,n", [(1024, 32, 70), (1024, 32, 600), (2560, 80, 70), (2560, 80, 300), (2560, 80, 2048), (4096, 64, 1100)])
+def test_prompt_projections_are_as_exact_as_their_operands(env, d, H, n):
+    # Raw conv inputs of the first layer: in-projection sums of d terms, which depend on the last three tokens only.  bf16 head
+    # and remainder hold an activation to at most 2^-18 of itself, 2.45e-6 rms in the sums.  Truncation in tensor memory adds a
+    # spread of at most 0.6 * 64 * 2^-26 = 0.57e-6 (64 MMAs per accumulator; 2.52e-6 together, 10 % on top for the sample of
+    # about 7000 values) and its mean, -2^-26 of a sum per MMA, is put back (what is left: 15 % of 64 * 2^-26, and the
+    # standard error of the slope, 3e-8)
+    s = hi.CONFIGS["cfg2_0p5b"].replace(L=1, V=2048, d=d, H=H, ff=512)
+    blob, table = hi.make_weights(s, 0, "jitter")
+    eng = env["hs"].Engine(s, blob, max_batch=1, max_k=4, kv_capacity=n + 8)
+    p = hi.make_prompt(s.V, n, seq=41)
+    eng.prefill([p])
+    q = env["oracle"].Model(s, blob, table, 8).new_seq()
+    q.prefill(p[-3:])
+    want = np.asarray(q.conv()[0], np.float64)
+    got = eng.export_state(0, 0, env["hs"].STATE_CONV).astype(np.float64)
+    slope = (got * want).sum() / (want * want).sum() - 1
+    err = np.linalg.norm(got - want) / np.linalg.norm(want)
+    print(d, n, "slope %.2e error %.2e" % (slope, err))
+    assert abs(slope) < 0.35e-6 and err < 2.8e-6 and eng.device_status() == 0
+
+
+@pytest.mark.parametrize("name,n,max_k", [
+    ("d512", 200, 4),        # down-projection K = 12288: 256 x 48 tiles in 12 segments, residual epilogue
+    ("d1280", 1900, 4),      # out- and down-projection 256 x 144 tiles, both planes in one accumulator, residual epilogue
+    ("d1024", 700, 8)])      # in-projection 256 x 240 tiles; residual projections 256 x 48, two accumulators
+def test_wide_projection_forms(env, name, n, max_k):
+    base = hi.CONFIGS["cfg1_tiny"].replace(V=512)
+    s = {"d512": base.replace(d=512, ff=12288), "d1280": base.replace(d=1280, H=40, ff=2560, N=128),
+         "d1024": hi.CONFIGS["cfg2_0p5b"].replace(L=2, V=512, ff=4096)}[name]
+    blob, table = hi.make_weights(s, 0, "jitter")
+    eng = env["hs"].Engine(s, blob, max_batch=1, max_k=max_k, kv_capacity=n + 16)
+    model = env["oracle"].Model(s, blob, table, n + 16)
+    p = hi.make_prompt(s.V, n, seq=7)
+    q = model.new_seq()
+    q.prefill(p)
+    eng.prefill([p])
+    env["harness"].compare_states(eng, [q], s, kv_rows=None)
+    # logits of the last position: what the last layer's residual projections left
+    T = max_k + 1
+    row = (n - 1) % T
+    q2 = model.new_seq()
+    q2.prefill(p[:n - 1])
+    want = q2.round(0, cand_in=np.asarray(p[n - 1:], np.int32), forced_n=0, want_logits=True)["logits"][0]
+    got = eng.get_logits(row + 1)[row]
+    err = np.linalg.norm(got - want) / np.linalg.norm(want)
+    print(name, "logits %.2e" % err)
+    assert err < 1e-4 and eng.device_status() == 0
