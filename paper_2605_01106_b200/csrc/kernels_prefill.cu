@@ -737,7 +737,8 @@ __global__ void __launch_bounds__(256) pf_gdn_out_kernel(const PfScanArgs a) {
 // running softmax in registers.  The longest tiles (the last positions) go out first.
 // In a parallel block it starts with the scan (beside), whose blocks are few, hold one SM each and leave the tensor path
 // idle: 0.5B-class, 512 positions, 53 us of scan and 24 of attention per layer; pass one after the other / together
-// 6.86 / 6.16 ms.
+// 6.86 / 6.16 ms.  For that the two have to share an SM's registers: with 255 a thread here beside 128 in the scan they do not
+// (0.5B-class, 1500 positions: 15.0 ms, with 216 registers 12.8).
 constexpr int PA_Q = 64, PA_K = 64, PA_THREADS = 128;
 
 template <int HD>
@@ -771,9 +772,17 @@ __device__ __forceinline__ void pf_attn_body(const PfAttnArgs &a, unsigned char 
         }
         cp_commit();
     };
+    // the queries: heads in registers, remainders in shared memory (for both 255 registers do not suffice)
+    __nv_bfloat16 *Ql_s = V_s + 2 * PA_K * KS;                                                      // [PA_Q][KS]
+    for (int idx = tid; idx < PA_Q * HC; idx += PA_THREADS) {
+        const int j = idx / HC, c = idx - j * HC;
+        if (q0 + j < n) cp16(Ql_s + j * KS + 8 * c, a.q + a.q_plane + (size_t)(row0 + q0 + j) * ld + h * HD + 8 * c);
+        else *reinterpret_cast<uint4 *>(Ql_s + j * KS + 8 * c) = make_uint4(0, 0, 0, 0);
+    }
     fetch(0);
     const int wq = q0 + warp * 16;                    // first position of this warp's rows, within the segment
-    uint32_t qh_[HD / 16][4], ql_[HD / 16][4];
+    const __nv_bfloat16 *ql = Ql_s + (size_t)(warp * 16 + (lane & 15)) * KS + (lane >> 4) * 8;
+    uint32_t qh_[HD / 16][4];
 #pragma unroll
     for (int ks = 0; ks < HD / 16; ++ks)
 #pragma unroll
@@ -781,7 +790,6 @@ __device__ __forceinline__ void pf_attn_body(const PfAttnArgs &a, unsigned char 
             const int i = wq + g8 + (e & 1) * 8, c = ks * 16 + 2 * t4 + (e >> 1) * 8;
             const __nv_bfloat16 *p = a.q + (size_t)(row0 + i) * ld + h * HD + c;
             qh_[ks][e] = i < n ? __ldcg(reinterpret_cast<const uint32_t *>(p)) : 0u;
-            ql_[ks][e] = i < n ? __ldcg(reinterpret_cast<const uint32_t *>(p + a.q_plane)) : 0u;
         }
     float O[NT][4];
 #pragma unroll
@@ -799,14 +807,17 @@ __device__ __forceinline__ void pf_attn_body(const PfAttnArgs &a, unsigned char 
 #pragma unroll
             for (int nt = 0; nt < PA_K / 8; ++nt) S[nt][0] = S[nt][1] = S[nt][2] = S[nt][3] = 0.f;
 #pragma unroll
-            for (int ks = 0; ks < HD / 16; ++ks)
+            for (int ks = 0; ks < HD / 16; ++ks) {
+                uint32_t ql_[4];
+                ldsm_x4(ql_, ql + ks * 16);
 #pragma unroll
                 for (int np = 0; np < PA_K / 16; ++np) {
                     uint32_t bk[4];
                     ldsm_x4(bk, kt + (size_t)(np * 16 + (lane & 7) + (lane >> 4) * 8) * KS + ks * 16 + ((lane >> 3) & 1) * 8);
                     mma_bf16(S[2 * np], qh_[ks], bk[0], bk[1]); mma_bf16(S[2 * np + 1], qh_[ks], bk[2], bk[3]);
-                    mma_bf16(S[2 * np], ql_[ks], bk[0], bk[1]); mma_bf16(S[2 * np + 1], ql_[ks], bk[2], bk[3]);
+                    mma_bf16(S[2 * np], ql_, bk[0], bk[1]); mma_bf16(S[2 * np + 1], ql_, bk[2], bk[3]);
                 }
+            }
             if (k0 + PA_K - 1 > base + wq)            // the diagonal: later positions are masked
 #pragma unroll
                 for (int nt = 0; nt < PA_K / 8; ++nt)
@@ -832,28 +843,38 @@ __device__ __forceinline__ void pf_attn_body(const PfAttnArgs &a, unsigned char 
                 }
                 l_run[r] = fmaf(l_run[r], corr[r], sum);
             }
-            if (__any_sync(0xffffffffu, corr[0] != 1.f || corr[1] != 1.f))
+            uint32_t ph[PA_K / 16][4], pl[PA_K / 16][4];
 #pragma unroll
-                for (int nt = 0; nt < NT; ++nt) { O[nt][0] *= corr[0]; O[nt][1] *= corr[0]; O[nt][2] *= corr[1]; O[nt][3] *= corr[1]; }
-#pragma unroll
-            for (int j = 0; j < PA_K / 16; ++j) {
-                uint32_t ph[4], pl[4];
+            for (int j = 0; j < PA_K / 16; ++j)
 #pragma unroll
                 for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
                     for (int r = 0; r < 2; ++r) {
                         const float p0 = S[2 * j + nt][2 * r], p1 = S[2 * j + nt][2 * r + 1];
                         const uint32_t hh = pack_bf16x2(p0, p1);
-                        ph[r + 2 * nt] = hh;
-                        pl[r + 2 * nt] = pack_bf16x2(p0 - __uint_as_float(hh << 16), p1 - __uint_as_float(hh & 0xffff0000u));
+                        ph[j][r + 2 * nt] = hh;
+                        pl[j][r + 2 * nt] = pack_bf16x2(p0 - __uint_as_float(hh << 16), p1 - __uint_as_float(hh & 0xffff0000u));
+                    }
+            // a tile's products add up in accumulators of their own: the tensor path truncates every sum, and over all keys of
+            // a long prompt on one accumulator that is 2^-26 of the output per MMA.  Four pairs of columns at a time.
+#pragma unroll
+            for (int p0 = 0; p0 < NT / 2; p0 += 4) {
+                float T[8][4];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) T[q][0] = T[q][1] = T[q][2] = T[q][3] = 0.f;
+#pragma unroll
+                for (int j = 0; j < PA_K / 16; ++j)
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                        uint32_t bv[4];
+                        ldsm_x4_t(bv, vt + (size_t)(j * 16 + (lane & 7) + ((lane >> 3) & 1) * 8) * KS + (p0 + p) * 16 + (lane >> 4) * 8);
+                        mma_bf16(T[2 * p], ph[j], bv[0], bv[1]); mma_bf16(T[2 * p + 1], ph[j], bv[2], bv[3]);
+                        mma_bf16(T[2 * p], pl[j], bv[0], bv[1]); mma_bf16(T[2 * p + 1], pl[j], bv[2], bv[3]);
                     }
 #pragma unroll
-                for (int p = 0; p < NT / 2; ++p) {
-                    uint32_t bv[4];
-                    ldsm_x4_t(bv, vt + (size_t)(j * 16 + (lane & 7) + ((lane >> 3) & 1) * 8) * KS + p * 16 + (lane >> 4) * 8);
-                    mma_bf16(O[2 * p], ph, bv[0], bv[1]); mma_bf16(O[2 * p + 1], ph, bv[2], bv[3]);
-                    mma_bf16(O[2 * p], pl, bv[0], bv[1]); mma_bf16(O[2 * p + 1], pl, bv[2], bv[3]);
-                }
+                for (int q = 0; q < 8; ++q)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) O[2 * p0 + q][e] = fmaf(O[2 * p0 + q][e], corr[e >> 1], T[q][e]);
             }
         }
         __syncthreads();                              // everybody is done with this stage: the next fetch refills it
@@ -873,7 +894,7 @@ __device__ __forceinline__ void pf_attn_body(const PfAttnArgs &a, unsigned char 
     }
 }
 template <int HD>
-__global__ void __launch_bounds__(PA_THREADS) pf_attn_kernel(const PfAttnArgs a) {
+__global__ void __maxnreg__(HD == 128 ? 216 : 152) pf_attn_kernel(const PfAttnArgs a) {
     extern __shared__ __align__(16) unsigned char smraw[];
     if (!a.beside) pdl_wait();
     pf_attn_body<HD>(a, smraw);
@@ -914,7 +935,7 @@ cudaError_t allow_smem(K kernel, size_t bytes) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
     return e;
 }
-constexpr size_t pa_smem(int hd) { return (size_t)4 * PA_K * (hd + 8) * 2; }
+constexpr size_t pa_smem(int hd) { return (size_t)(4 * PA_K + PA_Q) * (hd + 8) * 2; }
 
 template <int EPL, int RW, int NW>
 cudaError_t launch_scan(const PfScanArgs &a, cudaStream_t s) {

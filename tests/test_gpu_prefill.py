@@ -120,6 +120,32 @@ def test_prompt_projections_are_as_exact_as_their_operands(env, d, H, n):
     assert abs(slope) < 0.35e-6 and err < 2.8e-6 and eng.device_status() == 0
 
 
+def test_attention_over_a_long_cache_is_as_exact_as_its_operands(env):
+    # A prompt behind 4000 imported keys (the same bits on both sides); the attention of the first layer carries the residual
+    # stream (embedding small, no mixer, no MLP) that the next layer's conv inputs are made of.  Probabilities, the attention's
+    # output and the stream are held as bf16 head and remainder on the way, 2.45e-6 rms each: 4.2e-6 for the three.  One
+    # accumulator over all keys would truncate 500 times: 0.6 * 500 * 2^-26 = 4.5e-6 of spread on top, 6.2e-6
+    s = hi.CONFIGS["cfg1_tiny"]
+    ctx = 4000
+    blob, table = hi.make_weights(s, 0, "unit")
+    bf = lambda l, t: blob[table[(l, t)][0]:table[(l, t)][0] + 2 * int(np.prod(table[(l, t)][1]))].view(np.uint16)
+    bf(0, hi.T_W_OUT)[:] = 0
+    bf(0, hi.T_W_DOWN)[:] = 0
+    e = bf(-1, hi.G_EMBED)
+    e[:] = (hi.bf16_to_f32(e).ravel() * np.float32(2.0 ** -6)).view(np.uint32) >> 16          # an exact shift of the exponent
+    eng = env["hs"].Engine(s, blob, max_batch=1, max_k=4, kv_capacity=ctx + 64)
+    q = env["oracle"].Model(s, blob, table, ctx + 64).new_seq()
+    env["harness"].inject_context(eng, q, s, 0, ctx, 5)
+    p = hi.make_prompt(s.V, 16, seq=41)
+    eng.prefill([p])
+    q.prefill(p)
+    want = np.asarray(q.conv()[1], np.float64)
+    got = eng.export_state(1, 0, env["hs"].STATE_CONV).astype(np.float64)
+    err = np.linalg.norm(got - want) / np.linalg.norm(want)
+    print("error %.2e" % err)
+    assert err < 5e-6 and eng.device_status() == 0
+
+
 @pytest.mark.parametrize("name,n,max_k", [
     ("d512", 200, 4),        # down-projection K = 12288: 256 x 48 tiles in 12 segments, residual epilogue
     ("d1280", 1900, 4),      # out- and down-projection 256 x 144 tiles, both planes in one accumulator, residual epilogue
