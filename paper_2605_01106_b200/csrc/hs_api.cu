@@ -240,12 +240,14 @@ struct AttnGeom {
 AttnGeom attn_geom(const hs_model *m, int Tq, int T, int b0, int nb) {
     const hs_config &c = m->c;
     // One launch for mixer and attention spares a link of the chain, but every mixer block then carries the attention's
-    // shared memory: while the mixer blocks are at most four per SM and the cache takes at most 128 keys per CTA.  Verify
-    // pass, apart / together: 0.5B-class, 4 sequences (512 mixer blocks) of 50 keys, k = 0 / 1 / 2 / 4: 1.32 / 1.54 / 1.63 /
-    // 1.85 against 1.22 / 1.43 / 1.49 / 1.86 ms; 3 of 400, k = 4: 1.74 / 1.61; 4 of 900, k = 1: 1.64 / 1.54; 3B-class, one
-    // (320 blocks) of 200, k = 4: 2.87 / 2.74, of 900, k = 2: 2.83 / 2.81.  Not beside lean blocks of more than 96 keys with
-    // several row tiles, two of which fill an SM, once the mixer blocks are more than two per SM (3 sampled sequences of up to
-    // 901 keys, k = 4, round: 5.06 / 5.17 ms).
+    // shared memory, and fewer run at once.  Lean form: together while all blocks of the launch are at most two rounds of those
+    // that the SMs hold at once by shared memory (1.42 rounds in the mixer's instance for nine positions, which is the slowest
+    // to lose its neighbours).  Verify pass of the 0.5B-class hybrid, apart / together: 1 sequence of 1000 keys, k = 4 (1.1
+    // rounds) 1.511 / 1.381 ms; 3 of 450, k = 4 (1.6) 1.758 / 1.607; 4 of 740, k = 2 (1.95) 1.684 / 1.599; 4 of 300, k = 4 (2.2)
+    // 1.862 / 1.883; 3 of 740, k = 4 (3.2) 1.762 / 1.921; 2 of 450, k = 8 (1.2) 2.029 / 1.844; 3 of 450, k = 8 (1.8) 2.024 /
+    // 2.093; 8 layers of the 3B-class one, 1 sequence, k = 4: 300 keys (1.3) 0.777 / 0.749, 740 (2.6) 0.787 / 0.818.
+    // Otherwise while the mixer blocks are at most four per SM: 0.5B-class, 4 sequences (512 mixer blocks) of 50 keys, k = 0 / 1 /
+    // 2: 1.32 / 1.54 / 1.63 against 1.22 / 1.43 / 1.49 ms.
     const int64_t mixers = (int64_t)(c.P / 16) * c.H * nb;
     const bool few = c.arch == HS_ARCH_PARALLEL && mixers <= 4 * 148;
     if (m->att_force_chunk) return AttnGeom{m->att_force_chunk, m->att_force_tiles < 0 ? -m->att_force_tiles : m->att_force_tiles, 0, m->att_force_tiles < 0 ? 1 : 0, few};
@@ -264,8 +266,9 @@ AttnGeom attn_geom(const hs_model *m, int Tq, int T, int b0, int nb) {
         // 512, 96 CTAs: 1.75 / 1.90); beyond four per SM the general form takes over.
         int ck = 32;
         while (ck < 288 && 8 * ck < maxlen + T) ck += 32;
-        const bool fuse = few && ck <= 128 && (ck <= 96 || groups <= 16 || mixers <= 2 * 148);
         const int ctas = nb * c.kvh * ((groups + 15) / 16) * 8;
+        const int64_t at_once = 148 * (int64_t)ssm_attn_small_per_sm(c.N, c.hd, ck, groups, Tq);
+        const bool fuse = few && ck <= 128 && (Tq <= 5 ? mixers + ctas <= 2 * at_once : 100 * (mixers + ctas) <= 142 * at_once);
         if (g_hs_attn_small && ctas <= (streams || fuse ? 148 : 4 * 148) && 8 * ck >= maxlen + T) return AttnGeom{ck, 1, 1, 0, fuse};
     }
     if (streams) {

@@ -271,6 +271,8 @@ cudaError_t hs_make_f32_map(CUtensorMap *map, const void *base, uint64_t rows, u
 cudaError_t hs_make_kv_tensor_map(CUtensorMap *map, const void *base, uint64_t rows, int hd);
 // mixer + attention of a parallel block in one launch (verify pass); *fused = false: not applicable, nothing launched
 cudaError_t launch_ssm_attn(const SsmArgs &sa, const AttnArgs &a, cudaStream_t s, bool *fused);
+// blocks of that launch in the lean form that an SM holds at once: ck keys per CTA, `rows` query rows per KV head, T positions
+int ssm_attn_small_per_sm(int N, int hd, int ck, int rows, int T);
 
 // part: scratch of HS_ARGMAX_CHUNKS * 16 bytes per logits row (row slot b * Tm + i); counters: one int32 per
 // row slot, zero between launches

@@ -1410,6 +1410,14 @@ cudaError_t launch_attn(const AttnArgs &a, cudaStream_t s) {
     return cudaErrorInvalidValue;
 }
 
+int ssm_attn_small_per_sm(int N, int hd, int ck, int rows, int T) {
+    const size_t pos = T <= 3 ? 3 : T <= 5 ? 5 : HS_MAX_T;
+    const size_t mixer = pos * (2 * N + 34) * 4 + 128;              // the mixer's own (static) shared memory, see ssm_body
+    const size_t block = attn_small_layout(hd, ck, rows > 16 ? 16 : rows).total + mixer + 1024;     // 1 KB per block is the system's
+    const int n = (int)((size_t)228 * 1024 / block);
+    return n < 3 ? n : 3;                                           // up to 168 registers a thread
+}
+
 // Fused launch for a parallel block of the verify pass; `fused` reports whether it applies (mixer blocks of
 // 16 state rows, 128 threads in both roles) - otherwise nothing is launched and the caller issues the two
 // kernels one after the other.

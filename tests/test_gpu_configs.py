@@ -235,3 +235,22 @@ def test_mixer_instances_by_positions(env, name):
         rep = env["harness"].run_rounds(eng, seqs, s, k, 2, forced=[hi.forced_accept(k, 2, seq=b + k) for b in range(2)], rep=rep)
     print(rep)
     assert eng.device_status() == 0 and rep.rounds == 6
+
+
+@pytest.mark.parametrize("name,batch,k,ctx,apart", [
+    ("cfg2_0p5b", 1, 8, 1000, False), ("cfg2_0p5b", 3, 2, 700, False),
+    ("cfg2_0p5b", 3, 4, 700, True),          # 96 keys per CTA and two row tiles: one block fits an SM, 3.2 rounds of them
+    ("cfg2_0p5b", 4, 8, 100, True), ("cfg3_3b", 1, 4, 700, True), ("cfg3_3b", 1, 4, 250, False)])
+def test_mixer_and_attention_share_a_launch_while_blocks_fit(env, name, batch, k, ctx, apart):
+    s = hi.CONFIGS[name].replace(L=1, V=512)
+    eng = env["hs"].Engine(s, np.zeros(hi.blob_layout(s)[1], np.uint8), max_batch=batch, max_k=k, kv_capacity=ctx + 32)
+    for b in range(batch):
+        eng.set_context(b, ctx, 1)
+    eng.set_batch(batch)
+    eng.draft(k)
+    eng.profile(True)
+    eng.verify(k)
+    prof = eng.profile_read()
+    eng.profile(False)
+    eng.accept_rollback()
+    assert (prof["attention"][1] == 1) == apart and eng.device_status() == 0, prof
