@@ -894,7 +894,10 @@ int hs_prefill(hs_model *m, const int32_t *tokens_host, const int32_t *lens_host
     // over the prompt and stays on verify-sized passes.  Measured, chunks of max_k + 1 positions against wide passes: 512
     // tokens on the 0.5B-class hybrid 103.4 -> 5.9 ms, 2048 tokens on the 3B-class one 1371 -> 52 ms, four ragged prompts
     // (2.3 k tokens) on the sequential one 229 -> 12.6 ms.  A prompt of at most one chunk is one verify pass either way.
-    if (longest > m->Tm && g_hs_gemm_tc && !m->literal) return prefill_wide(m, tokens_host, lens_host, batch);
+    // Except two tokens at max_k = 0, one sequence: two one-row passes cost less than a wide one while the matrices are small
+    // (0.5B-class 1.54 / 1.62 ms, sequential 0.94 / 1.03; 3B-class 4.18 / 2.89, eight sequences 3.45 / 2.13).
+    const bool two_steps = longest == 2 && batch == 1 && m->tc_min_rows_auto == 7;
+    if (longest > m->Tm && !two_steps && g_hs_gemm_tc && !m->literal) return prefill_wide(m, tokens_host, lens_host, batch);
     // Chunk c covers prompt positions [c * Tm, (c + 1) * Tm) of every sequence that reaches that far; neighbouring
     // sequences with the same number of tokens in the chunk go out as one verify pass with every candidate accepted.
     // Nothing waits on the host between chunks (the token slices and accept lengths are staged by the copies).

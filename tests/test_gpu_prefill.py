@@ -172,3 +172,25 @@ def test_wide_projection_forms(env, name, n, max_k):
     err = np.linalg.norm(got - want) / np.linalg.norm(want)
     print(name, "logits %.2e" % err)
     assert err < 1e-4 and eng.device_status() == 0
+
+
+@pytest.mark.parametrize("name", ["par64", "seq"])
+def test_two_tokens_at_max_k_0(env, name):
+    # two one-row passes: as many launches as two prompts of one token, and what the oracle has
+    s = SHAPES[name]
+    blob, table = hi.make_weights(s, 0, "jitter")
+    eng = env["hs"].Engine(s, blob, max_batch=1, max_k=0, kv_capacity=16)
+    model = env["oracle"].Model(s, blob, table, 16)
+    p = hi.make_prompt(s.V, 2, seq=3)
+    at = [eng.launch_count()]
+    for prompt in ([p], [p[:1]]):
+        eng.reset()
+        eng.prefill(prompt)
+        at.append(eng.launch_count())
+    assert at[1] - at[0] == 2 * (at[2] - at[1])
+    eng.reset()
+    eng.prefill([p])
+    q = model.new_seq()
+    q.prefill(p)
+    env["harness"].compare_states(eng, [q], s)
+    assert eng.device_status() == 0
