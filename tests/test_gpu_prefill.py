@@ -1,6 +1,7 @@
 """Prompts longer than one verify pass: the wide prefill path against the CPU oracle at the sizes where it can go wrong
 (edges of the 8-position scan tiles, the 16-row conv tiles, the 64-position attention tiles; prompts of one to three
-positions beyond a conv window; a batch that needs more than one pass; a prompt appended to a context)."""
+positions beyond a conv window; a batch that needs more than one pass; a prompt appended to a context; every size class of
+the scans; every form of the two-CTA projections), sequences beside one that is not finite, and the precision of its sums."""
 import numpy as np
 import pytest
 
@@ -14,6 +15,7 @@ SHAPES = {
     "par256": hi.CONFIGS["cfg1_tiny"].replace(N=256, H=12, qh=6, kvh=2, hd=128),
     "seq": hi.CONFIGS["test_seq"],
     "seq32": hi.CONFIGS["test_seq"].replace(gdv=32, gh=8, hd=128),
+    "seq16": hi.CONFIGS["test_seq"].replace(gh=16),
 }
 
 
@@ -36,6 +38,8 @@ def env():
     ("seq", [72, 3, 9, 128, 40], 4, 0),
     ("seq", [1100, 1100], 8, 2),
     ("seq32", [66, 31], 8, 1),
+    ("seq16", [9, 17, 8, 30, 5], 2, 0),           # 320 strips of 16 value rows: two rows per lane group
+    ("par64", [9, 17, 8, 11, 12, 20, 5, 33, 10, 16, 7, 13], 2, 0),        # 6144 state rows: several scan blocks per SM, four stages
 ])
 def test_wide_prefill_matches_oracle(env, name, lens, max_k, flags):
     s = SHAPES[name]

@@ -1,5 +1,5 @@
 """Speculative sampling at vocabularies where its split over eight CTAs can go wrong: shares that are empty, ragged, not a
-multiple of four ids, and more than one sweep per thread (against the CPU oracle, decision margins as in harness.py)."""
+multiple of four ids, more than one sweep per thread, and more than one group of 32 ids per block (against the CPU oracle, decision margins as in harness.py)."""
 import numpy as np
 import pytest
 
@@ -8,7 +8,7 @@ import hs_inputs as hi
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("V,tau", [(31, 0.3), (257, 0.1), (1003, 0.05), (33001, 0.02)])
+@pytest.mark.parametrize("V,tau", [(31, 0.3), (257, 0.1), (1003, 0.05), (33001, 0.02), (262201, 0.01)])
 def test_sampling_vocabulary_sizes(V, tau):
     import oracle
     from paper_2605_01106_b200 import build, binding as hs
