@@ -254,10 +254,11 @@ int hs_set_attn_geometry(hs_model *m, int chunk, int tiles);
  *   HS_OPT_GEMM_TC         projections from HS_OPT_TC_MIN_ROWS activation rows on run on tcgen05 (default on; off: the
  *                          warp-level path, more than 16 rows as several 16-row launches)
  *   HS_OPT_PDL             programmatic dependent launch between the kernels of a pass (default on)
- *   HS_OPT_ATTN_SMALL      verify attention of small batches (few clusters of 16 query rows) over caches of up to 1024 keys
- *                          (2048 in a sequential hybrid) in its latency-lean form (default on; off: the general form)
- *   HS_OPT_ATTN_STREAM     verify attention over long caches at large batch (a launch of its own, at most 32 query rows
- *                          per KV head) in its streaming form (default on; off: the general form)
+ *   HS_OPT_ATTN_SMALL      verify attention of small batches (few clusters of 16 query rows) over caches of up to 2304 keys
+ *                          in its latency-lean form (default on; off: the streaming or the general form)
+ *   HS_OPT_ATTN_STREAM     verify attention over at least 100 tiles of 128 keys, all sequences and KV heads together (a
+ *                          launch of its own, at most 32 query rows per KV head), in its streaming form (default on; off:
+ *                          the general form)
  *   HS_OPT_TC_MIN_ROWS     not a switch: the smallest number of activation rows (2..17) whose projections run on
  *                          tcgen05; 0 restores the automatic choice (7; 4 for models whose weight matrices are large
  *                          enough that the kernel's fixed cost is small beside the time to stream them) */

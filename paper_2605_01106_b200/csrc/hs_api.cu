@@ -892,8 +892,8 @@ int hs_prefill(hs_model *m, const int32_t *tokens_host, const int32_t *lens_host
     // Prompts longer than one verify pass: passes of many positions (their activations do not fit the verify-pass
     // kernels' registers, the projections need the tcgen05 path).  The literal draft state also runs the draft model
     // over the prompt and stays on verify-sized passes.  Measured, chunks of max_k + 1 positions against wide passes: 512
-    // tokens on the 0.5B-class hybrid 103.4 -> 5.9 ms, 2048 tokens on the 3B-class one 1371 -> 52 ms, four ragged prompts
-    // (2.3 k tokens) on the sequential one 229 -> 12.6 ms.  A prompt of at most one chunk is one verify pass either way.
+    // tokens on the 0.5B-class hybrid 103.4 -> 6.0 ms, 2048 tokens on the 3B-class one 1371 -> 54 ms, four ragged prompts
+    // (3225 tokens, two passes) on the sequential one 229 -> 13.1 ms.  A prompt of at most one chunk is one verify pass either way.
     // Except two tokens at max_k = 0, one sequence: two one-row passes cost less than a wide one while the matrices are small
     // (0.5B-class 1.54 / 1.62 ms, sequential 0.94 / 1.03; 3B-class 4.18 / 2.89, eight sequences 3.45 / 2.13).
     const bool two_steps = longest == 2 && batch == 1 && m->tc_min_rows_auto == 7;

@@ -13,7 +13,10 @@
 #define HS_MAX_T (HS_MAX_K + 1)
 #define HS_H_PARTS 4          // a projection may leave the residual stream as up to 4 partial sums
 #define HS_ARGMAX_CHUNKS 32    // CTAs that share one logits row in the argmax
-#define HS_PREFILL_ROWS 2176   // most prompt positions of one pass, all sequences together (17 * 128: a 2048-token prompt in chunks of any size fits)
+// Most prompt positions of one pass, all sequences together.  Every row takes work-buffer space (0.5B-class 96 KB, 3B-class 236
+// KB: 0.21 and 0.51 GB at this limit); a prompt just beyond it pays for a second pass (0.5B-class, one sequence, 2175 tokens
+// 15.9 ms, 2176 19.8 - two passes of 1100 each as well, 9.8 ms apiece).
+#define HS_PREFILL_ROWS 2176
 #define HS_MAX_GT 48          // (q heads per kv head) * (k+1) upper bound of the attention kernel
 
 // ---------------------------------------------------------------------------------------------
@@ -80,7 +83,7 @@ struct hs_model {
     std::vector<CUtensorMap> kmaps, vmaps;   // per attention layer (streaming attention form)
     int tc_min_rows_auto;                 // the automatic row threshold of the tcgen05 kernel for this model
     __nv_bfloat16 *xb_h, *xb_a; float *ssbuf;   // packed residual stream / MLP activations handed from projection to projection, row statistics
-    // prompt path: activation rows per pass (0: prompts go through verify passes), the activations of a pass as above,
+    // prompt path: activation rows per pass, the activations of a pass as above,
     // row / segment / gather tables, conv outputs, per-head dt and decay, query planes, hidden rows of the prompts' last positions
     int pf_rows; float *pf_h[2], *pf_zx, *pf_gbuf, *pf_obuf, *pf_ss; __nv_bfloat16 *pf_xb, *pf_xb_h, *pf_xb_a; int64_t pf_xb_rows;
     int4 *pf_rowtab, *pf_segtab; int2 *pf_list; float *pf_xbc, *pf_dtv, *pf_hfin, *pf_rec; __nv_bfloat16 *pf_q;
