@@ -61,9 +61,9 @@ __device__ __forceinline__ float xreduce(float (&v)[NV], int lane) {
 
 // ---- programmatic dependent launch ---------------------------------------------------------------
 // Every kernel of a pass except the first is launched with the programmatic-stream-serialization
-// attribute: it may begin while its predecessors are still running.  All kernels call pdl_trigger()
-// at their very start, before their own pdl_wait(), so several kernels of the chain can sit in their
-// prologues at once.  Code before pdl_wait() may therefore read only what NO kernel of the same pass
+// attribute: it may begin while its predecessors are still running.  The kernels of a draft or verify
+// pass call pdl_trigger() at their very start, before their own pdl_wait(), so several kernels of the
+// chain can sit in their prologues at once.  Code before pdl_wait() may therefore read only what NO kernel of the same pass
 // writes: weights and parameters, the RoPE table, and what earlier passes left behind - the control
 // words kv_len / slot (written by the accept kernel) and cached KV rows below kv_len.  That is safe in
 // every mode because the first kernel of a pass is launched in plain stream order (a captured graph's
@@ -71,6 +71,13 @@ __device__ __forceinline__ float xreduce(float (&v)[NV], int lane) {
 // pass starts before all earlier work has finished.  Prologues write nothing to global memory.
 // pdl_wait() returns once the preceding kernel has completed and its writes are visible; every grid
 // waits before it completes, so completion is transitive along the chain.
+// Prompt passes keep the same rules with later triggers, and one exception: the attention of a parallel
+// block (pf_attn_kernel, beside = true) reads what pf_prep_kernel wrote, and stores its output, without a
+// wait, while the scan runs.  That holds because (1) pf_ssm_kernel triggers behind its own wait - so the
+// attention starts only when pf_gram_kernel is complete -, (2) pf_gram_kernel waits before it completes,
+// so pf_prep_kernel is complete as well, and nothing in between writes what the attention reads, and
+// (3) one block of the attention waits for the scan before it ends, so that the next kernel's wait covers
+// both.  A trigger moved in front of the wait of either kernel, or a kernel put between them, breaks it.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -108,6 +115,34 @@ __device__ __forceinline__ void bulk_g2s(void *dst_smem, const void *src, uint32
 }
 __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(p), "r"(bytes) : "memory");
+}
+
+// ---- 16-byte asynchronous copies, matrix fragments, the warp-level tensor path --------------------
+__device__ __forceinline__ void cp_async16(void *dst_smem, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem_u32(dst_smem)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_but_one() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
+__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)));
+}
+__device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], const void *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)));
+}
+// D(16x8, fp32) += A(16x16, bf16, row) * B(16x8, bf16, col)
+__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// two floats rounded to bf16 (nearest even) and packed: lo in bits 0-15, hi in bits 16-31
+__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
 }
 
 // ---- thread-block cluster: barrier and distributed shared memory ----------------------------------

@@ -65,32 +65,6 @@ __host__ __device__ inline AttnLayout attn_layout(int hd, int ck, int gt) {
     return L;
 }
 
-__device__ __forceinline__ void cp_async16(void *dst_smem, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem_u32(dst_smem)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_but_one() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
-__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void *p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)));
-}
-__device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], const void *p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)));
-}
-// D(16x8, fp32) += A(16x16, bf16, row) * B(16x8, bf16, col)
-__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// two floats rounded to bf16 (nearest even) and packed: lo in bits 0-15, hi in bits 16-31
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-    uint32_t r;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-    return r;
-}
 // x = head + remainder, both bf16 (round to nearest): exact to 2^-17 relative
 __device__ __forceinline__ void split_bf16(float x, __nv_bfloat16 &h, __nv_bfloat16 &l) {
     h = __float2bfloat16_rn(x);
@@ -520,7 +494,7 @@ __device__ __forceinline__ void attn_body(const AttnArgs &a, const int split, co
 // ------------------------------------------------------------------------------------------------
 // Short caches and few query rows (the whole cache within one cluster of eight CTAs): the latency-lean form.  A cluster takes
 // 16 of the G * T query rows of a KV head; more rows are several clusters, each reading the key range for itself (from L2).
-// A CTA holds its whole key range (up to 256 cached keys plus the new rows) in shared
+// A CTA holds its whole key range (up to 288 cached keys plus the new rows) in shared
 // memory, fetched before the dependency wait.  After the queries are staged there is no block-wide
 // synchronisation any more: every warp takes 16 keys at a time, computes the scores on the tensor cores,
 // keeps the probabilities in registers (the accumulator layout of the score tile is the operand layout of
@@ -546,7 +520,7 @@ constexpr int AT_SMALL_MAXCHUNK = 288;  // 213 KB of shared memory at a head dim
 
 template <int HD>
 __device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int split, const int khq, const int lb, unsigned char *smraw) {
-    const int CK = a.chunk;                        // cached keys per CTA: a multiple of 16 up to 256
+    const int CK = a.chunk;                        // cached keys per CTA: a multiple of 16 up to 288
     // khq = KV head + row tile * KV heads; this cluster's query rows are q_lo .. q_lo + GT - 1
     const int kh = khq % a.kvh, q_lo = khq / a.kvh * 16;
     const int G = a.qh / a.kvh, T = a.T, GT = min(16, G * T - q_lo);

@@ -328,15 +328,6 @@ __global__ void __launch_bounds__(GV_THREADS, 2) gemv_kernel(const GemvArgs a, c
 // the 8 weight rows of a warp's tile, read straight from the streamed bf16 tile (rows padded by 16
 // bytes so that ldmatrix is conflict-free).  Four accumulators per row group take the k steps in turn,
 // which keeps the MMA pipeline full.  NG = groups of 8 activation rows (1 or 2).
-__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void *p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)));
-}
-__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
 
 // EPI / NORMED >= 0 fix the epilogue and the presence of a norm at compile time (shorter program, see above).
 // CL: residual epilogue with the K split reduced inside a thread-block cluster (cluster_reduce_resid).

@@ -1,7 +1,7 @@
 // Kernels of the prompt path: what lies between the projections when a pass carries hundreds of prompt positions.
 //
 // A pass takes up to a few thousand activation rows: the next positions of several sequences, one contiguous piece
-// ("segment") per sequence.  The projections are plain dense contractions at that size (kernels_gemm_tc.cu); here are
+// ("segment") per sequence.  The projections are plain dense contractions at that size (kernels_gemm_wide.cu); here are
 //   pf_prep_kernel   causal conv + SiLU of the recurrent channels, dt / decay of every head, RoPE of q and k, and the
 //                    append of the new K and V rows to the cache - everything that is local to a position
 //   pf_gram_kernel, pf_ssm_kernel                          the Mamba-2 recurrence over the whole segment
@@ -10,8 +10,9 @@
 //   pf_embed_kernel, pf_gather_kernel, pf_advance_kernel, pf_pending_kernel   gathers and control words
 // The verify-pass kernels are built for at most nine positions (one trip to L2, everything in registers); their cost
 // per position is that of streaming all weights once per nine tokens, which is what this path removes.
-// Every kernel of this path lets its successor start when its own work is done, not earlier: blocks that wait hold
-// the registers and shared memory that the blocks still to come need (14.0 -> 9.6 ms for 512 tokens on the 0.5B-class hybrid).
+// The kernels between the projections let their successor start when their own work is done, not earlier: blocks that wait
+// hold the registers and shared memory that the blocks still to come need (14.0 -> 9.6 ms for 512 tokens on the 0.5B-class
+// hybrid).  Except the small gathers and pf_ssm_kernel, which the attention of its block runs beside (hs_device.cuh).
 // fp32 values keep their precision throughout: the recurrences run in fp32, attention splits queries and probabilities
 // into a bf16 head and a bf16 remainder (exact to 2^-17), keys and values enter as the bf16 the cache holds.
 #include "hs_internal.h"
@@ -20,30 +21,6 @@
 namespace {
 using namespace hsd;
 
-__device__ __forceinline__ void cp16(void *dst_smem, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem_u32(dst_smem)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory"); }
-__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void *p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)));
-}
-__device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], const void *p) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)));
-}
-__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-    uint32_t r;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-    return r;
-}
 // two fp32 values in one 64-bit register: one instruction works on both
 typedef unsigned long long f2;
 __device__ __forceinline__ f2 pk2(float x, float y) { f2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y)); return r; }
@@ -299,7 +276,7 @@ pf_ssm_kernel(const PfScanArgs a, const __grid_constant__ CUtensorMap mBC, const
     const int R0 = blockIdx.x * CR, Rw = R0 + warp * RW;                       // first row of the block / of the warp
     if (tid < stages) { mbar_init(&full[tid], 1); mbar_init(&empty[tid], NW); mbar_fence_init(); }
     pdl_wait();
-    pdl_trigger();                    // the attention of the same block reads nothing of this kernel and runs beside it
+    pdl_trigger();                    // behind the wait: the attention of the same block, which runs beside this kernel, counts on it
     __syncthreads();
     const int4 sg = __ldcg(a.segs + blockIdx.y);
     const int b = sg.x, row0 = sg.y, n = sg.z, slot_out = sg.w;
@@ -762,21 +739,21 @@ __device__ __forceinline__ void pf_attn_body(const PfAttnArgs &a, unsigned char 
             for (int idx = tid; idx < PA_K * HC; idx += PA_THREADS) {
                 const int j = idx / HC, c = idx - j * HC;
                 if (j < cnt) {
-                    cp16(kd + j * KS + 8 * c, Kb + (size_t)(t * PA_K + j) * HD + 8 * c);
-                    cp16(vd + j * KS + 8 * c, Vb + (size_t)(t * PA_K + j) * HD + 8 * c);
+                    cp_async16(kd + j * KS + 8 * c, Kb + (size_t)(t * PA_K + j) * HD + 8 * c);
+                    cp_async16(vd + j * KS + 8 * c, Vb + (size_t)(t * PA_K + j) * HD + 8 * c);
                 } else {                              // finite values where the tile ends early
                     *reinterpret_cast<uint4 *>(kd + j * KS + 8 * c) = make_uint4(0, 0, 0, 0);
                     *reinterpret_cast<uint4 *>(vd + j * KS + 8 * c) = make_uint4(0, 0, 0, 0);
                 }
             }
         }
-        cp_commit();
+        cp_async_commit();
     };
     // the queries: heads in registers, remainders in shared memory (for both 255 registers do not suffice)
     __nv_bfloat16 *Ql_s = V_s + 2 * PA_K * KS;                                                      // [PA_Q][KS]
     for (int idx = tid; idx < PA_Q * HC; idx += PA_THREADS) {
         const int j = idx / HC, c = idx - j * HC;
-        if (q0 + j < n) cp16(Ql_s + j * KS + 8 * c, a.q + a.q_plane + (size_t)(row0 + q0 + j) * ld + h * HD + 8 * c);
+        if (q0 + j < n) cp_async16(Ql_s + j * KS + 8 * c, a.q + a.q_plane + (size_t)(row0 + q0 + j) * ld + h * HD + 8 * c);
         else *reinterpret_cast<uint4 *>(Ql_s + j * KS + 8 * c) = make_uint4(0, 0, 0, 0);
     }
     fetch(0);
@@ -798,7 +775,7 @@ __device__ __forceinline__ void pf_attn_body(const PfAttnArgs &a, unsigned char 
 #pragma unroll 1
     for (int t = 0; t < ntile; ++t) {
         fetch(t + 1);
-        cp_wait<1>();
+        cp_async_wait_but_one();
         __syncthreads();
         const __nv_bfloat16 *kt = K_s + (t & 1) * PA_K * KS, *vt = V_s + (t & 1) * PA_K * KS;
         const int k0 = t * PA_K, last = base + wq + 15;            // last key any row of this warp may see
@@ -879,7 +856,7 @@ __device__ __forceinline__ void pf_attn_body(const PfAttnArgs &a, unsigned char 
         }
         __syncthreads();                              // everybody is done with this stage: the next fetch refills it
     }
-    cp_wait<0>();
+    cp_async_wait_all();
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         float l = l_run[r];
