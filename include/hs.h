@@ -146,8 +146,10 @@ int hs_reset(hs_model *m);
  * otherwise HS_ERR_INVALID_ARG before anything is enqueued.  Sets the batch
  * size for the following rounds.  Afterwards kv_len[b] = lens[b] and pending[b] = the greedy choice
  * after the last prompt token (generated token #1).  Prompts longer than max_k+1 run as passes of up to 2176
- * positions, all sequences together; shorter ones, and all with HS_FLAG_LITERAL_DRAFT, as verify passes over chunks of
- * max_k+1 positions with every candidate accepted.  Nothing waits on the host between passes.  Synchronises the stream before returning (tokens_host may be reused afterwards). */
+ * positions, all sequences together (what one sequence holds, finite or not, does not reach another); shorter ones, two
+ * tokens of one sequence at max_k = 0 on models with small matrices, and all with HS_FLAG_LITERAL_DRAFT, as verify passes
+ * over chunks of max_k+1 positions with every candidate accepted.  Nothing waits on the host between passes.  Synchronises
+ * the stream before returning (tokens_host may be reused afterwards). */
 int hs_prefill(hs_model *m, const int32_t *tokens_host, const int32_t *lens_host, int batch);
 
 /* Draft phase (paper Sec. 3.3, "Draft phase": M_S generates k tokens autoregressively; M_S is Eq. 4 for a
