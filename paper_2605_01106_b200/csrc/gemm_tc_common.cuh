@@ -19,7 +19,7 @@ struct TcArgs {
     int ns;                     // shared-memory stages (at most TC_MAXSTAGES)
     int seg;                    // two-CTA tiles: K blocks per segment
     float found;                // 1 + what truncation took from a sum; two-CTA tiles in segments: what it takes per K block
-    int rb;                     // K split: activation rows of a tile each rank finishes (a power of two >= 4, rb * S >= bnh)
+    int rb, rb_inv;             // K split: activation rows of a tile each rank finishes (a multiple of 4, rb * S >= bnh); 65536 / rb rounded up
     float *out; int ldo;
     const float *resid; int rparts; int64_t rpstride;
     int32_t *status;
@@ -29,7 +29,7 @@ struct TcArgs {
     const float *ss_in; int ss_parts; float inv_k, eps;
     // Packed output for the projection that consumes this one's result: bf16 head | remainder planes
     // [2][rpad][pk_ld] of (result * pk_nw[output row]), and (residual epilogue) the partial sums of squares
-    // ss_out[weight-row tile][rpad] of the results.  nullptr: not wanted.
+    // ss_out[tile of weight rows][rpad] of the results.  nullptr: not wanted.
     __nv_bfloat16 *pk_out; int pk_ld; const float *pk_nw; float *ss_out;
     const void *pf_ptr; long long pf_bytes;     // weights of the next projection, pulled into L2 before the wait
     int early_trigger;          // let the next kernel start before this one has waited (else when its accumulators are complete)
@@ -70,27 +70,42 @@ __device__ __forceinline__ void split_bf16(float x, __nv_bfloat16 &h, __nv_bfloa
     l = __float2bfloat16_rn(x - __bfloat162float(h));
 }
 
-// Residual of eight consecutive activation rows r0..r0+7 of weight row `row` (parts added in order); the loads
-// are issued early, so that their trip to L2 hides behind the wait that precedes the epilogue proper.
-__device__ __forceinline__ void tc_load_resid(const TcArgs &a, float (&res)[8], int r0, int nvalid, int row) {
+// 1/rms of an activation row whose partial sums of squares lie `stride` floats apart: sixteen loads at a time, added in order
+__device__ __forceinline__ float tc_rstd(const TcArgs &a, const float *ss, int stride) {
+    float t = 0.f;
+    for (int p0 = 0; p0 < a.ss_parts; p0 += 16) {
+        float x[16];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) res[j] = 0.f;
-    if (row >= a.O) return;
-    const size_t oi = (size_t)r0 * a.ldo + row;
-    for (int p = 0; p < a.rparts; ++p) {
-        const float *rp = a.resid + (size_t)p * a.rpstride + oi;
+        for (int u = 0; u < 16; ++u) x[u] = p0 + u < a.ss_parts ? __ldcg(ss + (size_t)(p0 + u) * stride) : 0.f;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) if (j < nvalid) res[j] += __ldcg(rp + (size_t)j * a.ldo);
+        for (int u = 0; u < 16; ++u) t += x[u];
     }
+    return rsqrtf(t * a.inv_k + a.eps);
 }
 
-// Epilogue for eight consecutive activation rows r0..r0+7 (indices inside the launch) of weight row `row`
+// Residual of NC consecutive activation rows r0 .. of weight row `row` (parts added in order); the loads are issued early, so that
+// their trip to L2 hides behind the wait that precedes the epilogue proper.  (One part, the rule: nothing here touches a loaded
+// value, so the thread does not stall before it has come to that wait.)
+template <int NC>
+__device__ __forceinline__ void tc_load_resid(const TcArgs &a, float (&res)[NC], int r0, int nvalid, int row) {
+#pragma unroll
+    for (int j = 0; j < NC; ++j) res[j] = 0.f;
+    if (row >= a.O) return;
+    const float *rp = a.resid + (size_t)r0 * a.ldo + row;
+#pragma unroll
+    for (int j = 0; j < NC; ++j) if (j < nvalid) res[j] = __ldcg(rp + (size_t)j * a.ldo);
+    for (int p = 1; p < a.rparts; ++p)
+#pragma unroll
+        for (int j = 0; j < NC; ++j) if (j < nvalid) res[j] += __ldcg(rp + (size_t)p * a.rpstride + (size_t)j * a.ldo);
+}
+
+// Epilogue for NC = 4 or 8 consecutive activation rows r0 .. (indices inside the launch) of weight row `row`
 // (v[j] = the finished sum of row r0 + j, 1/rms already applied); nvalid of them exist.  Every lane of the warp
 // calls it (the SwiGLU pairing and the sums of squares shuffle).  res: the residual (tc_load_resid); nw: weight
 // folded into the packed output.  Returns (residual epilogue with statistics) the warp's sum of squares of row
-// r0 + lane / 4.
-template <int EPI>
-__device__ __forceinline__ float tc_finish8(const TcArgs &a, float (&v)[8], const float (&res)[8], int r0, int nvalid, int row, float nw, int lane) {
+// r0 + lane / (32 / NC).
+template <int EPI, int NC>
+__device__ __forceinline__ float tc_finish(const TcArgs &a, float (&v)[NC], const float (&res)[NC], int r0, int nvalid, int row, float nw, int lane) {
     if (EPI == EPI_SWIGLU) {
         // weight rows come in (gate, up) pairs held by neighbouring lanes.  The even lane finishes the even
         // columns of the pair, the odd lane the odd ones, so both lanes work and each evaluates one SiLU per two
@@ -98,7 +113,7 @@ __device__ __forceinline__ float tc_finish8(const TcArgs &a, float (&v)[8], cons
         const bool odd = row & 1;
         const bool st = (row | 1) < a.O;
 #pragma unroll
-        for (int j = 0; j < 8; j += 2) {
+        for (int j = 0; j < NC; j += 2) {
             const float got = __shfl_xor_sync(0xffffffffu, odd ? v[j] : v[j + 1], 1);
             const float gate = odd ? got : v[j], up = odd ? v[j + 1] : got;
             const int jj = j + (odd ? 1 : 0);
@@ -119,16 +134,16 @@ __device__ __forceinline__ float tc_finish8(const TcArgs &a, float (&v)[8], cons
         const bool st = row < a.O;
         if (EPI == EPI_RESID)
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] += res[j];
+            for (int j = 0; j < NC; ++j) v[j] += res[j];
         float *p = a.out + (size_t)r0 * a.ldo + row;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) if (st && j < nvalid) p[(size_t)j * a.ldo] = v[j];
+        for (int j = 0; j < NC; ++j) if (st && j < nvalid) p[(size_t)j * a.ldo] = v[j];
         if (EPI == EPI_RESID && a.pk_out) {
             __nv_bfloat16 *ph = a.pk_out + (size_t)r0 * a.pk_ld + row;
             const size_t plane = (size_t)a.rpad * a.pk_ld;
-            float ssq[8];
+            float ssq[NC];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
+            for (int j = 0; j < NC; ++j) {
                 const bool live = st && j < nvalid;
                 if (live) {
                     __nv_bfloat16 h, l;
@@ -137,7 +152,7 @@ __device__ __forceinline__ float tc_finish8(const TcArgs &a, float (&v)[8], cons
                 }
                 ssq[j] = live ? v[j] * v[j] : 0.f;
             }
-            return xreduce<8>(ssq, lane);           // lanes 4 j .. 4 j + 3 hold the total of row r0 + j
+            return xreduce<NC>(ssq, lane);
         }
         return 0.f;
     }

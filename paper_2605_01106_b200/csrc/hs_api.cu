@@ -165,10 +165,10 @@ WorkLayout work_layout(const hs_config &c, const Derived &v) {
     auto packed = [&](int64_t rows, int64_t &xb, int64_t &xb_h, int64_t &xb_a, int64_t &ss) {
         xb = take((int64_t)2 * 2 * rows * kmax);
         // the same for the residual stream and the MLP activations, written by the producing projection's epilogue,
-        // and the partial sums of squares (one per 128 model dimensions) of the residual stream's rows
+        // and the partial sums of squares (one per 64 model dimensions) of the residual stream's rows
         xb_h = take((int64_t)2 * 2 * rows * c.d);
         xb_a = take((int64_t)2 * 2 * rows * c.ff);
-        ss = take((int64_t)4 * rows * ((c.d + 127) / 128));
+        ss = take((int64_t)4 * rows * ((c.d + 63) / 64));
     };
     packed(gemm_tc_rows(v.R), w.xb, w.xb_h, w.xb_a, w.ssbuf);
     w.dstat = take((int64_t)8 * v.B * std::max(c.max_k, 1));
@@ -322,7 +322,7 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
     // results in the packed form that kernel consumes (only the mixer's output and the embedding are packed by a
     // kernel of their own)
     const bool tc_pass = gemv_uses_tc(rows, m->xb != nullptr);
-    const int ss_parts = (d + 127) / 128;
+    int ss_parts = 0;                       // partial sums of squares per row in ssbuf
     bool h_packed = false;                  // xb_h / ssbuf hold the current residual stream
     PROF(HS_PROF_EMBED, 0, launch_embed(m->embed, d, c.V, m->ctrl.cand, m->Tm, draft ? step : 0, T, b0, nb, m->hbuf[0], st_w, first, s), "embed");
     ++m->launches;
@@ -448,7 +448,7 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
         }
         go.early_trigger = 1; go.pf_ptr = ly.W_gu; go.pf_bytes = 2 * (int64_t)2 * c.ff * d;
         go.xb = m->xb; go.xb_rows = m->xb_rows;
-        if (tc_pass) { go.pk_out = m->xb_h; go.pk_ld = d; go.pk_nw = ly.norm2; go.ss_out = m->ssbuf; }
+        if (tc_pass) { go.pk_out = m->xb_h; go.pk_ld = d; go.pk_nw = ly.norm2; go.ss_out = m->ssbuf; go.ss_parts_out = &ss_parts; }
         PROF(HS_PROF_GEMV, gemv_bytes(go), launch_gemv(go, st_w, s, &m->launches, &hparts), "out_proj");
         cur ^= 1;
         // (5) RMSNorm + gate/up + SwiGLU, (6) down + residual
@@ -474,7 +474,7 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
             }
             else { gdn.pf_ptr = m->lm_head; gdn.pf_bytes = 2 * (int64_t)c.V * d; }
             // the consumer of this layer's output: the next layer that runs (its first norm), else the final norm
-            if (tc_pass) { gdn.pk_out = m->xb_h; gdn.pk_ld = d; gdn.pk_nw = nl < c.L ? m->layers[nl].norm1 : m->final_norm; gdn.ss_out = m->ssbuf; }
+            if (tc_pass) { gdn.pk_out = m->xb_h; gdn.pk_ld = d; gdn.pk_nw = nl < c.L ? m->layers[nl].norm1 : m->final_norm; gdn.ss_out = m->ssbuf; gdn.ss_parts_out = &ss_parts; }
         }
         gdn.xb = m->xb; gdn.xb_rows = m->xb_rows;
         if (tc_pass) gdn.pk_in = m->xb_a;
@@ -540,7 +540,8 @@ int enqueue_accept(hs_model *m, int k, int b0, int nb, const int32_t *fn, const 
 int prefill_pass(hs_model *m, int rows, int nseg, int max_seg, int *cur_out) {
     const hs_config &c = m->c;
     cudaStream_t s = m->stream;
-    const int d = c.d, ss_parts = (d + 127) / 128;
+    const int d = c.d;
+    int ss_parts = 0;
     const int64_t q_plane = (int64_t)m->pf_rows * c.qh * c.hd;
     int32_t *st_w = m->ctrl.status;
     int cur = 0;
@@ -599,7 +600,7 @@ int prefill_pass(hs_model *m, int rows, int nseg, int max_seg, int *cur_out) {
                 go.W1 = ly.W_o; go.ldw1 = c.qh * c.hd; go.K1 = c.qh * c.hd; go.x1 = m->pf_obuf; go.ldx1 = c.qh * c.hd;
             }
         } else { go.W0 = ly.W_o; go.ldw0 = c.qh * c.hd; go.K0 = c.qh * c.hd; go.x0 = m->pf_obuf; go.ldx0 = c.qh * c.hd; }
-        go.pk_out = m->pf_xb_h; go.pk_ld = d; go.pk_nw = ly.norm2; go.ss_out = m->pf_ss;
+        go.pk_out = m->pf_xb_h; go.pk_ld = d; go.pk_nw = ly.norm2; go.ss_out = m->pf_ss; go.ss_parts_out = &ss_parts;
         PROF(HS_PROF_GEMV, gemv_bytes(go), launch_gemm_tc(go, st_w, s, &m->launches, nullptr), "prefill out_proj");
         cur ^= 1;
         GemvArgs gu{}; gu.prompt = true;
@@ -609,7 +610,7 @@ int prefill_pass(hs_model *m, int rows, int nseg, int max_seg, int *cur_out) {
         GemvArgs dn{}; dn.prompt = true;
         dn.W0 = ly.W_down; dn.ldw0 = c.ff; dn.K0 = c.ff; dn.O = d; dn.out = m->pf_h[cur ^ 1]; dn.ldo = d; dn.max_oparts = 1;
         dn.resid = m->pf_h[cur]; dn.rparts = 1; dn.nrows = rows; dn.epi = EPI_RESID; dn.early_trigger = 0; dn.pk_in = m->pf_xb_a;
-        dn.pk_out = m->pf_xb_h; dn.pk_ld = d; dn.pk_nw = l + 1 < c.L ? m->layers[l + 1].norm1 : m->final_norm; dn.ss_out = m->pf_ss;
+        dn.pk_out = m->pf_xb_h; dn.pk_ld = d; dn.pk_nw = l + 1 < c.L ? m->layers[l + 1].norm1 : m->final_norm; dn.ss_out = m->pf_ss; dn.ss_parts_out = &ss_parts;
         PROF(HS_PROF_GEMV, gemv_bytes(dn), launch_gemm_tc(dn, st_w, s, &m->launches, nullptr), "prefill down");
         cur ^= 1;
     }

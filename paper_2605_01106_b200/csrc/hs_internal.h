@@ -167,9 +167,9 @@ struct GemvArgs {
     // ([2][rows per plane][K0], norm weight folded in, WITHOUT 1/rms when ss_in is given: ss_in[p * rows per plane + r],
     // p < ss_parts, are partial sums of squares of row r).  pk_out: where to leave this projection's result in packed
     // form for its consumer (row length pk_ld, times pk_nw[output] if given), with the partial sums of squares of the
-    // residual epilogue's results in ss_out[128-row tile][rows per plane].
+    // residual epilogue's results in ss_out[tile][rows per plane] (tiles of 128 or 64 weight rows; how many: *ss_parts_out).
     const __nv_bfloat16 *pk_in; const float *ss_in; int ss_parts;
-    __nv_bfloat16 *pk_out; int pk_ld; const float *pk_nw; float *ss_out;
+    __nv_bfloat16 *pk_out; int pk_ld; const float *pk_nw; float *ss_out; int *ss_parts_out;
 };
 // does a projection of nrows activation rows run on the many-row kernel?
 bool gemv_uses_tc(int nrows, bool have_xb);

@@ -115,29 +115,30 @@ __global__ void __launch_bounds__(256) pack_kernel(const PackArgs a) {
 }
 
 // ---- the contraction ---------------------------------------------------------------------------------------
-// BN: N of the MMA = 2 * bnh (head columns, then remainder columns).  EPI: the epilogue, fixed at compile time.
-template <int BN, int EPI>
+// BN: N of the MMA = 2 * bnh (head columns, then remainder columns).  BM: weight rows per tile; 64 only with a K split (row r of
+// the tile is then lane r % 16 of tensor-memory quarter r / 16).  EPI: the epilogue, fixed at compile time.
+template <int BN, int BM, int EPI>
 __global__ void __launch_bounds__(TC_THREADS, 2)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
                const __grid_constant__ CUtensorMap mB, const TcArgs a) {
-    constexpr uint32_t A_BYTES = TC_BM * TC_BK * 2, B_BYTES = BN * TC_BK * 2, STAGE = A_BYTES + B_BYTES;
+    constexpr uint32_t A_BYTES = BM * TC_BK * 2, B_BYTES = BN * TC_BK * 2, STAGE = A_BYTES + B_BYTES;
     constexpr uint32_t TCOLS = BN < 32 ? 32 : BN;
-    constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);
-    constexpr int BNH = BN / 2;
+    constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+    constexpr int BNH = BN / 2, RW = BM / 32, CG = 8 / RW;     // finishing a split tile: RW warps side by side, CG groups of four columns at a time
     extern __shared__ unsigned char smraw[];
     __shared__ __align__(8) uint64_t full_bar[TC_MAXSTAGES], empty_bar[TC_MAXSTAGES], done_bar;
     __shared__ uint32_t tmem_base_s;
     __shared__ int failed_s;
     const uint32_t sbase = (smem_u32(smraw) + 1023u) & ~1023u;            // swizzled tiles need 1024-byte alignment
     unsigned char *stages = smraw + (sbase - smem_u32(smraw));
-    float *rx = reinterpret_cast<float *>(stages + a.off_rx);             // [S][128][rb]: partial tiles sent by the cluster's ranks
+    float *rx = reinterpret_cast<float *>(stages + a.off_rx);             // [S][rb / 4][BM][4]: partial tiles sent by the cluster's ranks
     float *rstd_s = reinterpret_cast<float *>(stages + a.off_misc);       // [BNH] 1/rms and what truncation took
     float *nw_s = rstd_s + 128;                                           // [128]
     float *ssred = nw_s + 128;                                            // [4][BNH]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // grid = (K splits = cluster size, weight-row tiles, activation-row tiles)
     const int S = (int)gridDim.x, q = (int)blockIdx.x;
-    const int m0 = blockIdx.y * TC_BM, n0h = blockIdx.z * BNH;
+    const int m0 = blockIdx.y * BM, n0h = blockIdx.z * BNH;
     const int nk = a.nk0 + a.nk1, NS = a.ns;
     const int kb0 = (int)((long long)q * nk / S), kb1 = (int)((long long)(q + 1) * nk / S), nkl = kb1 - kb0;
     if (a.early_trigger) pdl_trigger();
@@ -152,8 +153,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     // parameters (nothing a kernel writes): the weights folded into the packed output
-    if (tid >= 128) {
-        const int i = tid - 128;
+    if (tid >= 256 - BM) {
+        const int i = tid - (256 - BM);
         nw_s[i] = (a.pk_nw && m0 + i < a.O) ? a.pk_nw[m0 + i] : 1.f;
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -215,52 +216,45 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
         pdl_wait();
 #pragma unroll 1
         for (int i = tid - 64; i < BNH; i += TC_THREADS - 64) {
-            float r = 1.f;
-            if (a.ss_in) {
-                float t = 0.f;
-                for (int p = 0; p < a.ss_parts; ++p) t += __ldcg(a.ss_in + (size_t)p * a.rpad + n0h + i);
-                r = rsqrtf(t * a.inv_k + a.eps);
-            }
-            rstd_s[i] = r * a.found;
+            rstd_s[i] = (a.ss_in ? tc_rstd(a, a.ss_in + n0h + i, a.rpad) : 1.f) * a.found;
         }
     }
     if (warp < 2 && !(warp == 0 && lane == 0)) pdl_wait();          // the epilogue reads the residual stream
     __syncwarp();
-    __syncthreads();                                    // rstd_s complete
-    // ---- epilogue: thread = accumulator lane = weight row; warps w and w + 4 share a lane quarter and split
-    //      the columns (activation rows)
-    const int lrow = (warp & 3) * 32 + lane, half = warp >> 2;
-    const int row = m0 + lrow;
-    const float nw = nw_s[lrow];
+    // ---- epilogue.  Whole K range: thread = accumulator lane = weight row, warps w and w + 4 share a lane quarter and split the
+    //      columns (activation rows).  K split: rank p finishes the activation rows [p * rb, (p + 1) * rb) of the tile (the last ranks
+    //      may find none), four columns of a weight row per thread at a time.
     const int nact = a.nrows - n0h;                     // activation rows of this tile that exist
     const bool stats = EPI == EPI_RESID && a.pk_out != nullptr && a.ss_out != nullptr;
-    // K split: rank p finishes the activation rows [p * rb, (p + 1) * rb) of the tile (rb a power of two >= 4; ranks
-    // whose range lies beyond the tile finish nothing)
-    const int rb = a.rb, lg_rb = 31 - __clz(rb);
-    int c_lo = 0, c_n = BNH;                            // the tile's activation rows this CTA finishes
-    if (S > 1) { c_lo = min(q * rb, BNH); c_n = min(rb, BNH - c_lo); }
-    // first group of eight rows this thread finishes: its residual is requested now, the trip to L2 hides behind the
-    // wait for the accumulators (and the exchange)
-    const int first = S == 1 ? half * (BNH / 2) : c_lo + half * 8;
-    float res[8];
-    if (EPI == EPI_RESID) tc_load_resid(a, res, n0h + first, nact - first, row);
+    const int half = warp >> 2, rb = a.rb;
+    const int c_lo = S > 1 ? min(q * rb, BNH) : 0, c_n = S > 1 ? min(rb, BNH - c_lo) : BNH;     // the tile's activation rows this CTA finishes
+    const int frow = S > 1 ? (warp % RW) * 32 + lane : (warp & 3) * 32 + lane, cg = warp / RW;
+    const int row = m0 + frow;
+    // the first columns this thread finishes: their residual is requested now, the trip to L2 hides behind the contraction
+    float res4[4], res[8];
+    if (EPI == EPI_RESID) {
+        if (S > 1) tc_load_resid<4>(a, res4, n0h + c_lo + cg * 4, min(c_n - cg * 4, nact - (c_lo + cg * 4)), row);
+        else if (BM == TC_BM) tc_load_resid<8>(a, res, n0h + half * (BNH / 2), nact - half * (BNH / 2), row);
+    }
+    __syncthreads();                                    // rstd_s complete
+    const float nw = nw_s[frow];
     const bool ok = mbar_wait(&done_bar, 0) && !failed_s;
     if (!a.early_trigger) pdl_trigger();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t taddr = tmem_d + ((uint32_t)((warp & 3) * 32) << 16);
     if (!ok && tid == 0) atomicCAS(a.status, 0, (int)HS_ERR_TIMEOUT);
     if (S == 1) {
-        if (ok) {
+        if (BM == TC_BM && ok) {
             for (int c0 = half * (BNH / 2); c0 < (half + 1) * (BNH / 2); c0 += 8) {
                 uint32_t h[8], l[8];
                 tmem_ld8(taddr + (uint32_t)c0, h);
                 tmem_ld8(taddr + (uint32_t)(BNH + c0), l);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                 float v[8], rnext[8];
-                if (EPI == EPI_RESID && c0 + 8 < (half + 1) * (BNH / 2)) tc_load_resid(a, rnext, n0h + c0 + 8, nact - (c0 + 8), row);
+                if (EPI == EPI_RESID && c0 + 8 < (half + 1) * (BNH / 2)) tc_load_resid<8>(a, rnext, n0h + c0 + 8, nact - (c0 + 8), row);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) v[j] = (__uint_as_float(h[j]) + __uint_as_float(l[j])) * rstd_s[c0 + j];
-                const float sq = tc_finish8<EPI>(a, v, res, n0h + c0, nact - c0, row, nw, lane);
+                const float sq = tc_finish<EPI, 8>(a, v, res, n0h + c0, nact - c0, row, nw, lane);
                 if (stats && (lane & 3) == 0) ssred[(warp & 3) * BNH + c0 + (lane >> 2)] = sq;
                 if (EPI == EPI_RESID)
 #pragma unroll
@@ -269,10 +263,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
         }
     } else {
         // Every rank sends the matching columns of its partial tile straight into rank p's shared memory
-        // ([sender][weight row][rb]: 16-byte remote stores), ONE cluster barrier, then each rank adds the S partials of
-        // its rows in rank order - the result does not depend on timing.
+        // ([sender][four columns][weight row]: remote stores of 16 bytes, side by side for the lanes of a warp), ONE cluster
+        // barrier, then each rank adds the S partials of its rows in rank order - the result does not depend on timing.
+        // (With a weight row's columns side by side the lanes of a store, and of a load, were rb * 4 bytes apart and hit the same
+        // banks: 128 rows of the 0.5B-class model, down-projection at 320 activation rows 3.5 us sending and 4.8 us adding.)
         cluster_wait();                                 // every rank runs: its receive area may be written
-        const uint32_t rx_mine = smem_u32(rx) + (uint32_t)(((q * TC_BM + lrow) * rb) * 4);
+        const int lrow = BM == TC_BM ? (warp & 3) * 32 + lane : (warp & 3) * 16 + (lane & 15);
+        const bool has_row = BM == TC_BM || lane < 16;
+        const uint32_t rx_mine = smem_u32(rx) + (uint32_t)((q * (rb >> 2) * BM + lrow) * 16);
         for (int c0 = half * (BNH / 2); c0 < (half + 1) * (BNH / 2); c0 += 8) {
             uint32_t h[8], l[8];
 #pragma unroll
@@ -282,77 +280,67 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
                 tmem_ld8(taddr + (uint32_t)(BNH + c0), l);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
             }
-            float v[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(h[j]) + __uint_as_float(l[j]);
-            if (rb >= 8) {
-                const uint32_t dst = dsmem_addr(rx_mine + (uint32_t)((c0 & (rb - 1)) * 4), (uint32_t)(c0 >> lg_rb));
-                dsmem_st_v4(dst, v[0], v[1], v[2], v[3]);
-                dsmem_st_v4(dst + 16, v[4], v[5], v[6], v[7]);
-            } else {                                    // rb == 4: the eight columns belong to two ranks
-                const uint32_t p = (uint32_t)(c0 >> 2);
-                dsmem_st_v4(dsmem_addr(rx_mine, p), v[0], v[1], v[2], v[3]);
-                dsmem_st_v4(dsmem_addr(rx_mine, p + 1), v[4], v[5], v[6], v[7]);
+            for (int e = 0; e < 8; e += 4) {
+                const uint32_t p = ((uint32_t)(c0 + e) * (uint32_t)a.rb_inv) >> 16, cl = (uint32_t)(c0 + e) - p * (uint32_t)rb;      // (c0 + e) / rb
+                if (has_row)
+                    dsmem_st_v4(dsmem_addr(rx_mine + (cl >> 2) * (BM * 16), p), __uint_as_float(h[e]) + __uint_as_float(l[e]), __uint_as_float(h[e + 1]) + __uint_as_float(l[e + 1]),
+                                __uint_as_float(h[e + 2]) + __uint_as_float(l[e + 2]), __uint_as_float(h[e + 3]) + __uint_as_float(l[e + 3]));
             }
         }
         cluster_arrive(); cluster_wait();
-        // eight rows at a time, alternating between the two halves of the CTA
-        for (int cl0 = half * 8; cl0 < c_n; cl0 += 16) {
-            const int nr = min(8, c_n - cl0);
-            float v[8], rnext[8];
-            if (EPI == EPI_RESID && cl0 + 16 < c_n) tc_load_resid(a, rnext, n0h + c_lo + cl0 + 16, nact - (c_lo + cl0 + 16), row);
+        for (int cl0 = cg * 4; cl0 < c_n; cl0 += 4 * CG) {
+            float v[4], rnext[4];
+            if (EPI == EPI_RESID && cl0 + 4 * CG < c_n) tc_load_resid<4>(a, rnext, n0h + c_lo + cl0 + 4 * CG, nact - (c_lo + cl0 + 4 * CG), row);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = 0.f;
-            for (int p = 0; p < S; ++p) {
-                const float4 *pr = reinterpret_cast<const float4 *>(rx + ((size_t)(p * TC_BM + lrow) * rb + cl0));
-                const float4 x = pr[0];
-                v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
-                if (nr > 4) { const float4 y = pr[1]; v[4] += y.x; v[5] += y.y; v[6] += y.z; v[7] += y.w; }
-            }
+            for (int j = 0; j < 4; ++j) v[j] = 0.f;
+            const float4 *pr = reinterpret_cast<const float4 *>(rx) + (cl0 >> 2) * BM + frow;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] *= rstd_s[min(c_lo + cl0 + j, BNH - 1)];
-            const int nvalid = min(nr, nact - (c_lo + cl0));
-            const float sq = tc_finish8<EPI>(a, v, res, n0h + c_lo + cl0, nvalid, row, nw, lane);
-            if (stats && (lane & 3) == 0 && (lane >> 2) < nr) ssred[(warp & 3) * BNH + c_lo + cl0 + (lane >> 2)] = sq;
+            for (int p = 0; p < 8; ++p)
+                if (p < S) { const float4 x = pr[p * (rb >> 2) * BM]; v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w; }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] *= rstd_s[c_lo + cl0 + j];
+            const float sq = tc_finish<EPI, 4>(a, v, res4, n0h + c_lo + cl0, nact - (c_lo + cl0), row, nw, lane);
+            if (stats && (lane & 7) == 0) ssred[(warp % RW) * BNH + c_lo + cl0 + (lane >> 3)] = sq;
             if (EPI == EPI_RESID)
 #pragma unroll
-                for (int j = 0; j < 8; ++j) res[j] = rnext[j];
+                for (int j = 0; j < 4; ++j) res4[j] = rnext[j];
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (stats && ok) {
-        // sums of squares of the finished rows over this tile's 128 weight rows: the four lane quarters in order
+        // sums of squares of the finished rows over this tile's weight rows, 32 after 32
         for (int i = tid; i < c_n; i += TC_THREADS) {
             const int c = c_lo + i;
-            if (c < nact) a.ss_out[(size_t)blockIdx.y * a.rpad + n0h + c] = (ssred[c] + ssred[BNH + c]) + (ssred[2 * BNH + c] + ssred[3 * BNH + c]);
+            if (c < nact) a.ss_out[(size_t)blockIdx.y * a.rpad + n0h + c] = BM == TC_BM ? (ssred[c] + ssred[BNH + c]) + (ssred[2 * BNH + c] + ssred[3 * BNH + c]) : ssred[c] + ssred[BNH + c];
         }
     }
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem_d), "r"(TCOLS) : "memory");
 }
 
-constexpr size_t tc_stage_bytes(int bn) { return (size_t)TC_BM * TC_BK * 2 + (size_t)bn * TC_BK * 2; }
+constexpr size_t tc_stage_bytes(int bn, int bm) { return (size_t)bm * TC_BK * 2 + (size_t)bn * TC_BK * 2; }
 constexpr size_t TC_SMEM_MAX = 200 * 1024;
 constexpr size_t TC_SMEM_PAIR = 110 * 1024;   // up to this two CTAs fit on an SM
 constexpr size_t TC_MISC_BYTES = (128 + 128 + 4 * 128) * 4;
 int g_tc_clusters[2][9];     // clusters of S CTAs that run at once with one CTA per SM ([0]; [1]: the same query at the smaller footprint)
 
-template <int BN, int EPI>
+template <int BN, int BM, int EPI>
 cudaError_t launch_tc(const CUtensorMap &mA0, const CUtensorMap &mA1, const CUtensorMap &mB, const TcArgs &t, dim3 grid, size_t smem, cudaStream_t s) {
     static bool configured = false;
     if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_MAX);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI>, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+        cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN, BM, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_MAX);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_tc_kernel<BN, BM, EPI>, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    return launch_pdl_cluster(gemm_tc_kernel<BN, EPI>, grid, dim3(TC_THREADS), smem, s, (int)grid.x, mA0, mA1, mB, t);
+    return launch_pdl_cluster(gemm_tc_kernel<BN, BM, EPI>, grid, dim3(TC_THREADS), smem, s, (int)grid.x, mA0, mA1, mB, t);
 }
 template <int BN>
-cudaError_t launch_tc_epi(int epi, const CUtensorMap &mA0, const CUtensorMap &mA1, const CUtensorMap &mB, const TcArgs &t, dim3 grid, size_t smem, cudaStream_t s) {
-    if (epi == EPI_STORE) return launch_tc<BN, EPI_STORE>(mA0, mA1, mB, t, grid, smem, s);
-    if (epi == EPI_RESID) return launch_tc<BN, EPI_RESID>(mA0, mA1, mB, t, grid, smem, s);
-    return launch_tc<BN, EPI_SWIGLU>(mA0, mA1, mB, t, grid, smem, s);
+cudaError_t launch_tc_epi(int epi, int bm, const CUtensorMap &mA0, const CUtensorMap &mA1, const CUtensorMap &mB, const TcArgs &t, dim3 grid, size_t smem, cudaStream_t s) {
+    if (epi == EPI_STORE) return launch_tc<BN, TC_BM, EPI_STORE>(mA0, mA1, mB, t, grid, smem, s);
+    if (epi == EPI_RESID) return bm == 64 ? launch_tc<BN, 64, EPI_RESID>(mA0, mA1, mB, t, grid, smem, s) : launch_tc<BN, TC_BM, EPI_RESID>(mA0, mA1, mB, t, grid, smem, s);
+    return launch_tc<BN, TC_BM, EPI_SWIGLU>(mA0, mA1, mB, t, grid, smem, s);
 }
 
 }  // namespace
@@ -392,7 +380,7 @@ cudaError_t configure_gemm_tc() {
     g_hs_tensor_maps = true;
     e = cudaFuncSetAttribute(pack_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(gemm_tc_kernel<32, EPI_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_MAX);
+    e = cudaFuncSetAttribute(gemm_tc_kernel<32, TC_BM, EPI_STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_MAX);
     if (e != cudaSuccess) return e;
     for (int pair = 0; pair < 2; ++pair)
         for (int S = 1; S <= 8; ++S) {
@@ -403,7 +391,7 @@ cudaError_t configure_gemm_tc() {
             at[0].val.clusterDim.x = S; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
             cfg.attrs = at; cfg.numAttrs = 1;
             int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, gemm_tc_kernel<32, EPI_STORE>, &cfg) == cudaSuccess && n > 0) g_tc_clusters[pair][S] = n;
+            if (cudaOccupancyMaxActiveClusters(&n, gemm_tc_kernel<32, TC_BM, EPI_STORE>, &cfg) == cudaSuccess && n > 0) g_tc_clusters[pair][S] = n;
             else { g_tc_clusters[pair][S] = S == 1 ? 148 : 0; cudaGetLastError(); }
             if (getenv("HS_VERBOSE")) fprintf(stderr, "libhs: tcgen05 projection, clusters of %d CTAs (%d per SM) resident at once: %d\n", S, pair + 1, g_tc_clusters[pair][S]);
         }
@@ -437,30 +425,41 @@ cudaError_t launch_gemm_tc(const GemvArgs &a, int32_t *status, cudaStream_t s, i
     const int ntiles = (a.nrows + bnh - 1) / bnh;
     // K split (cluster size, 1..8): the weights are the large operand, so the grid is filled by splitting K, as long as
     // all CTAs still run at once, at most one per SM, and every CTA keeps at least two K blocks.  Rank p of a cluster
-    // finishes rb activation rows of the tile (a power of two, at least four).
-    const size_t stage = tc_stage_bytes(2 * bnh);
-    const int tiles = mtiles * ntiles;
+    // finishes rb activation rows of the tile (a multiple of four).  A residual projection of few weight rows cannot fill half of the
+    // GPU that way: it goes out in tiles of 64 weight rows, twice as many.
     // (the CTAs of a cluster share a GPC, so fewer clusters of S CTAs than SMs / S may run at once: g_tc_clusters)
-    int S = 1, rb = 4;
-    size_t rx_bytes = 0, budget = TC_SMEM_MAX;
-    for (int cand = 1; cand <= 8; ++cand) {
-        if (cand > 1 && nk / cand < 2) break;
-        int crb = 4;
-        while (crb * cand < bnh) crb <<= 1;
-        const size_t crx = cand > 1 ? (size_t)cand * crb * TC_BM * 4 : 0;
-        // Stages as deep as shared memory allows: a refill costs a trip to L2 on the critical path (measured: deep
-        // stages with one CTA per SM beat two co-resident CTAs with two or three stages each).  Few activation rows
-        // make the stages small: then two CTAs fit on an SM with four or more stages each, more CTAs than SMs still
-        // run at once and the CTAs of the next projection can stream their weights while this one finishes.
-        // More tiles than SMs would otherwise run in two rounds, the second nearly empty: there three stages are enough
-        // for a pair (measured: 4-6 % per verify pass on the batched workloads; with two stages it loses again).
-        const bool pair = TC_SMEM_PAIR >= 4 * stage + crx + TC_MISC_BYTES + 1024 ||
-                          (tiles * cand > 148 && TC_SMEM_PAIR >= 3 * stage + crx + TC_MISC_BYTES + 1024);
-        // with two CTAs per SM twice as many clusters run at once (the occupancy query is made for one per SM)
-        if (cand > 1 && tiles > g_tc_clusters[0][cand] * (pair ? 2 : 1)) continue;
-        if (cand > 1 && tiles * cand > (pair ? 2 * 148 : 148)) continue;
-        S = cand; rb = crb; rx_bytes = crx; budget = pair ? TC_SMEM_PAIR : TC_SMEM_MAX;
+    struct Split { int S, rb; size_t rx_bytes, budget; };
+    auto split_for = [&](int bm) {
+        const size_t stage = tc_stage_bytes(2 * bnh, bm);
+        const int tiles = (a.O + bm - 1) / bm * ntiles;
+        Split r{1, 4, 0, TC_SMEM_MAX};
+        for (int cand = 1; cand <= 8; ++cand) {
+            if (cand > 1 && nk / cand < 2) break;
+            const int crb = ((bnh + cand - 1) / cand + 3) / 4 * 4;
+            const size_t crx = cand > 1 ? (size_t)cand * crb * bm * 4 : 0;
+            // Stages as deep as shared memory allows: a refill costs a trip to L2 on the critical path (measured: deep
+            // stages with one CTA per SM beat two co-resident CTAs with two or three stages each).  Few activation rows
+            // make the stages small: then two CTAs fit on an SM with four or more stages each, more CTAs than SMs still
+            // run at once and the CTAs of the next projection can stream their weights while this one finishes.
+            // More tiles than SMs would otherwise run in two rounds, the second nearly empty: there three stages are enough
+            // for a pair (measured: 4-6 % per verify pass on the batched workloads; with two stages it loses again).
+            const bool pair = TC_SMEM_PAIR >= 4 * stage + crx + TC_MISC_BYTES + 1024 ||
+                              (tiles * cand > 148 && TC_SMEM_PAIR >= 3 * stage + crx + TC_MISC_BYTES + 1024);
+            // with two CTAs per SM twice as many clusters run at once (the occupancy query is made for one per SM)
+            if (cand > 1 && tiles > g_tc_clusters[0][cand] * (pair ? 2 : 1)) continue;
+            if (cand > 1 && tiles * cand > (pair ? 2 * 148 : 148)) continue;
+            r = Split{cand, crb, crx, pair ? TC_SMEM_PAIR : TC_SMEM_MAX};
+        }
+        return r;
+    };
+    Split sp = split_for(TC_BM);
+    int bm = TC_BM;
+    if (a.epi == EPI_RESID && mtiles * ntiles * sp.S <= 74) {
+        const Split half = split_for(64);
+        if (half.S > 1) { sp = half; bm = 64; }
     }
+    const int S = sp.S, rb = sp.rb;
+    const size_t stage = tc_stage_bytes(2 * bnh, bm), rx_bytes = sp.rx_bytes, budget = sp.budget;
     const int nkl = (nk + S - 1) / S;
     if (gemm_wide_applies(a.nrows, a.O, nkl, a.prompt)) return launch_gemm_wide(a, status, s, launches, oparts);
     int ns = (int)((budget - rx_bytes - TC_MISC_BYTES - 1024) / stage);
@@ -482,12 +481,12 @@ cudaError_t launch_gemm_tc(const GemvArgs &a, int32_t *status, cudaStream_t s, i
         xb = a.xb;
     }
     CUtensorMap mA0, mA1, mB;
-    cudaError_t e = make_map(&mA0, a.W0, a.O, a.K0, a.ldw0, TC_BM);
-    if (e == cudaSuccess) e = a.K1 ? make_map(&mA1, a.W1, a.O, a.K1, a.ldw1, TC_BM) : make_map(&mA1, a.W0, a.O, a.K0, a.ldw0, TC_BM);
+    cudaError_t e = make_map(&mA0, a.W0, a.O, a.K0, a.ldw0, bm);
+    if (e == cudaSuccess) e = a.K1 ? make_map(&mA1, a.W1, a.O, a.K1, a.ldw1, bm) : make_map(&mA1, a.W0, a.O, a.K0, a.ldw0, bm);
     if (e == cudaSuccess) e = make_map(&mB, xb, (uint64_t)2 * rpad, Kt, Kt, bnh);
     if (e != cudaSuccess) return e;
     TcArgs t{};
-    t.O = a.O; t.nk0 = a.K0 / TC_BK; t.nk1 = a.K1 / TC_BK; t.nrows = a.nrows; t.rpad = rpad; t.bnh = bnh; t.ns = ns; t.rb = rb;
+    t.O = a.O; t.nk0 = a.K0 / TC_BK; t.nk1 = a.K1 / TC_BK; t.nrows = a.nrows; t.rpad = rpad; t.bnh = bnh; t.ns = ns; t.rb = rb; t.rb_inv = 65536 / rb + 1;
     t.out = a.out; t.ldo = a.ldo; t.resid = a.resid; t.rparts = a.rparts; t.rpstride = a.rpstride; t.status = status;
     if (a.pk_in && a.ss_in) { t.ss_in = a.ss_in; t.ss_parts = a.ss_parts; t.inv_k = 1.f / (float)a.K0; t.eps = a.eps; }
     if (a.pk_out && a.epi != EPI_STORE) {
@@ -499,11 +498,12 @@ cudaError_t launch_gemm_tc(const GemvArgs &a, int32_t *status, cudaStream_t s, i
     t.early_trigger = a.early_trigger; t.found = 1.f + (float)(nk * (TC_BK / 16)) / (float)S * TC_LOST;
     if (oparts) *oparts = 1;
     if (launches) ++*launches;
-    const dim3 grid(S, mtiles, ntiles);
+    if (a.ss_parts_out && t.ss_out) *a.ss_parts_out = (a.O + bm - 1) / bm;
+    const dim3 grid(S, (a.O + bm - 1) / bm, ntiles);
     switch (2 * bnh) {
-        case 32: return launch_tc_epi<32>(a.epi, mA0, mA1, mB, t, grid, smem, s);
-        case 64: return launch_tc_epi<64>(a.epi, mA0, mA1, mB, t, grid, smem, s);
-        case 128: return launch_tc_epi<128>(a.epi, mA0, mA1, mB, t, grid, smem, s);
-        default: return launch_tc_epi<256>(a.epi, mA0, mA1, mB, t, grid, smem, s);
+        case 32: return launch_tc_epi<32>(a.epi, bm, mA0, mA1, mB, t, grid, smem, s);
+        case 64: return launch_tc_epi<64>(a.epi, bm, mA0, mA1, mB, t, grid, smem, s);
+        case 128: return launch_tc_epi<128>(a.epi, bm, mA0, mA1, mB, t, grid, smem, s);
+        default: return launch_tc_epi<256>(a.epi, bm, mA0, mA1, mB, t, grid, smem, s);
     }
 }

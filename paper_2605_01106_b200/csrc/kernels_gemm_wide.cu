@@ -196,12 +196,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant_
             // contracted
             epi_sync();                               // the previous tile is done with rstd_s / nw_s / ssred
             if (tid < n) {
-                float r = 1.f;
-                if (a.ss_in) {
-                    float t = 0.f;
-                    for (int p = 0; p < a.ss_parts; ++p) t += __ldcg(a.ss_in + (size_t)p * a.rpad + min(n0 + tid, a.rpad - 1));
-                    r = rsqrtf(t * a.inv_k + a.eps);
-                }
+                const float r = a.ss_in ? tc_rstd(a, a.ss_in + min(n0 + tid, a.rpad - 1), a.rpad) : 1.f;
                 rstd_s[tid] = SEG ? r : r * a.found;
             }
             if (tid < TC_BM) nw_s[tid] = (a.pk_nw && m0 + tid < a.O) ? a.pk_nw[m0 + tid] : 1.f;
@@ -234,7 +229,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant_
                     }
 #pragma unroll
                     for (int j = 0; j < 8; ++j) v[j] *= rstd_s[c0 + j];
-                    const float sq = tc_finish8<EPI>(a, v, res, n0 + c0, nact - c0, row, nw, lane);
+                    const float sq = tc_finish<EPI, 8>(a, v, res, n0 + c0, nact - c0, row, nw, lane);
                     if (stats && (lane & 3) == 0) ssred[(warp & 3) * 256 + c0 + (lane >> 2)] = sq;
                     if (EPI == EPI_RESID)
 #pragma unroll
@@ -291,7 +286,7 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant_
                         if (EPI != EPI_RESID)
 #pragma unroll
                             for (int j = 0; j < 8; ++j) acc[u][j] *= rstd_s[c0 + j];
-                        const float sq = tc_finish8<EPI>(a, acc[u], none, n0 + c0, nact - c0, row, nw, lane);
+                        const float sq = tc_finish<EPI, 8>(a, acc[u], none, n0 + c0, nact - c0, row, nw, lane);
                         if (stats && (lane & 3) == 0) ssred[(warp & 3) * 256 + c0 + (lane >> 2)] = sq;
                     }
 #pragma unroll
@@ -397,6 +392,7 @@ cudaError_t launch_gemm_wide(const GemvArgs &a, int32_t *status, cudaStream_t s,
         t.pk_out = a.pk_out; t.pk_ld = a.pk_ld; t.pk_nw = a.pk_nw;
         t.ss_out = a.epi == EPI_RESID ? a.ss_out : nullptr;
     }
+    if (a.ss_parts_out && t.ss_out) *a.ss_parts_out = (a.O + TC_BM - 1) / TC_BM;
     t.off_misc = (int)((size_t)ns * stage);
     // segments of equal length, none with more than GW_CHAIN MMAs on an accumulator
     const int most = GW_CHAIN / (n > 128 ? 8 : 4) * sets, nseg = (nk + most - 1) / most;
