@@ -347,6 +347,12 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
         // (2) recurrent mixer
         SsmArgs ssm_args{};
         bool ssm_deferred = false;
+        // The mixer packs the out-projection's operand itself where that is all of it: a draft step of a Mamba-2 layer without
+        // attention, every DeltaNet layer.  (The partial sums of squares of the gated norm go to the idle gbuf.  From 192 rows on
+        // the two-CTA tiles may take the out-projection; they add the residual in front of the 1/rms factor.)
+        const bool mix_packed = tc_pass && rows < 192 && (ly.type == HS_LAYER_GDN || (ly.type == HS_LAYER_PAR && T == 1 && !with_attn));
+        const int pk_rows = gemm_tc_rows(rows);
+        int mix_parts = 0;
         if (ly.type != HS_LAYER_ATT) {
             const size_t lrB = (size_t)ly.rl * m->B;
             const float *win_in; float *win_out = nullptr, *hist = nullptr;
@@ -391,6 +397,7 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
                 sa.slot = slot_arr; sa.in_add = in_add; sa.out_rel = out_rel; sa.out_add = out_add; sa.slot_mod = slot_mod; sa.g = m->gbuf; sa.T = T; sa.Tm = m->Tm; sa.b0 = b0; sa.nb = nb;
                 sa.log = log_l; sa.log_w = m->log_w;
                 sa.nslot = slot_mod ? slot_mod : (int)ns; sa.status = st_w;
+                if (mix_packed) { sa.pk = m->xb; sa.pk_rows = pk_rows; sa.gnorm = ly.gnorm; sa.pk_ss = m->gbuf; mix_parts = ssm_blocks(sa); }
                 if (with_attn) { ssm_args = sa; ssm_deferred = true; }      // goes out together with the attention
                 else PROF(HS_PROF_MIXER, 0, launch_ssm(sa, s), "ssm");
             } else {
@@ -403,6 +410,7 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
                 gd.slot = slot_arr; gd.in_add = in_add; gd.out_rel = out_rel; gd.out_add = out_add; gd.slot_mod = slot_mod; gd.g = m->gbuf; gd.T = T; gd.Tm = m->Tm; gd.b0 = b0; gd.nb = nb;
                 gd.log = log_l; gd.log_w = m->log_w;
                 gd.nslot = slot_mod ? slot_mod : (int)ns; gd.status = st_w;
+                if (mix_packed) { gd.pk = m->xb; gd.pk_rows = pk_rows; }
                 PROF(HS_PROF_MIXER, 0, launch_gdn(gd, s), "gdn");
             }
             if (!ssm_deferred) ++m->launches;
@@ -448,6 +456,10 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
         }
         go.early_trigger = 1; go.pf_ptr = ly.W_gu; go.pf_bytes = 2 * (int64_t)2 * c.ff * d;
         go.xb = m->xb; go.xb_rows = m->xb_rows;
+        if (mix_packed) {
+            go.pk_in = m->xb;
+            if (mix_parts) { go.ss_in = m->gbuf; go.ss_parts = mix_parts; }
+        }
         if (tc_pass) { go.pk_out = m->xb_h; go.pk_ld = d; go.pk_nw = ly.norm2; go.ss_out = m->ssbuf; go.ss_parts_out = &ss_parts; }
         PROF(HS_PROF_GEMV, gemv_bytes(go), launch_gemv(go, st_w, s, &m->launches, &hparts), "out_proj");
         cur ^= 1;

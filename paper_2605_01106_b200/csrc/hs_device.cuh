@@ -1,6 +1,7 @@
 // Device helpers shared by the kernels of libhs.
 #pragma once
 #include <cuda_runtime.h>
+#include <cuda_bf16.h>
 #include <stdint.h>
 
 namespace hsd {
@@ -143,6 +144,12 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     uint32_t r;
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
+}
+
+// an activation as the tensor-core projections take it: bf16 head and bf16 remainder (exact to 2^-17), in two planes
+__device__ __forceinline__ void store_split(__nv_bfloat16 *p, size_t plane, float x) {
+    const __nv_bfloat16 h = __float2bfloat16_rn(x);
+    p[0] = h; p[plane] = __float2bfloat16_rn(x - __bfloat162float(h));
 }
 
 // ---- thread-block cluster: barrier and distributed shared memory ----------------------------------

@@ -216,8 +216,13 @@ struct SsmArgs {
                                         // no state is stored.  NULL otherwise
     int nslot; int32_t *status;         // slot[b] must lie in [0, nslot): otherwise the block touches no state and
                                         // reports HS_ERR_DEVICE through the status word
+    // One position, no attention beside it: the output goes out as the packed operand of the out-projection (GemvArgs) instead of
+    // g: bf16 head plane [pk_rows][di], remainder plane behind it, times gnorm, and per block the sum of squares of its outputs
+    // in pk_ss[block of the sequence][pk_rows].  NULL: g.
+    __nv_bfloat16 *pk; int pk_rows; const float *gnorm; float *pk_ss;
 };
 cudaError_t launch_ssm(const SsmArgs &a, cudaStream_t s);
+int ssm_blocks(const SsmArgs &a);       // blocks per sequence of that launch (partial sums in pk_ss)
 
 struct GdnArgs {
     int gh, dk, dv, convd, in_ld;
@@ -232,6 +237,7 @@ struct GdnArgs {
     int T, Tm, b0, nb;
     float *log; int log_w;              // rollback by replay: [B][Tm][log_w] (alpha[gh] | beta[gh] | k[gh*dk] | v[gh*dv]); NULL otherwise
     int nslot; int32_t *status;         // as in SsmArgs
+    __nv_bfloat16 *pk; int pk_rows;     // the output as packed operand of the out-projection instead of g: head plane [pk_rows][gh*dv], remainder plane behind it
 };
 cudaError_t launch_gdn(const GdnArgs &a, cudaStream_t s);
 

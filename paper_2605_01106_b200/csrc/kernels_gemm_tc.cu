@@ -214,6 +214,22 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
                 prefetch_l2(reinterpret_cast<const char *>(a.pf_ptr) + o, (uint32_t)min(4096ll, hi - o));
         }
         pdl_wait();
+        if (a.ss_in && a.ss_parts > 32) {
+            // many partial sums (one per block of the mixer): a warp per activation row
+#pragma unroll 1
+            for (int i = warp - 2; i < BNH; i += TC_THREADS / 32 - 2) {
+                const float *ss = a.ss_in + n0h + i;
+                float t = 0.f;
+                for (int p0 = lane; p0 < a.ss_parts; p0 += 128) {
+                    float x[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) x[u] = p0 + 32 * u < a.ss_parts ? __ldcg(ss + (size_t)(p0 + 32 * u) * a.rpad) : 0.f;
+                    t += (x[0] + x[1]) + (x[2] + x[3]);
+                }
+                t = warp_sum(t);
+                if (lane == 0) rstd_s[i] = rsqrtf(t * a.inv_k + a.eps) * a.found;
+            }
+        } else
 #pragma unroll 1
         for (int i = tid - 64; i < BNH; i += TC_THREADS - 64) {
             rstd_s[i] = (a.ss_in ? tc_rstd(a, a.ss_in + n0h + i, a.rpad) : 1.f) * a.found;

@@ -165,7 +165,11 @@ __global__ void __launch_bounds__(GDN_THREADS) gdn_kernel(const GdnArgs a) {
         for (int j = lane; j < dv; j += 32) ss = fmaf(os[i][j], os[i][j], ss);
         const float rstd = rsqrtf(warp_sum(ss) / (float)dv + a.eps);
         for (int j = lane; j < dv; j += 32)
-            a.g[(size_t)(rowbase + i) * nv + h * dv + j] = os[i][j] * rstd * a.onorm[j] * zs[i][j];
+        {
+            const float out = os[i][j] * rstd * a.onorm[j] * zs[i][j];
+            if (a.pk) store_split(a.pk + (size_t)(rowbase + i) * nv + h * dv + j, (size_t)a.pk_rows * nv, out);
+            else a.g[(size_t)(rowbase + i) * nv + h * dv + j] = out;
+        }
     }
 }
 
@@ -287,6 +291,7 @@ cudaError_t launch_replay(const ReplayArgs &a, cudaStream_t s) {
 // a whole head per block once blocks of 16 rows would already fill the GPU several times over
 static bool ssm_wide(const SsmArgs &a) { return a.P % 64 == 0 && (int64_t)(a.P / 16) * a.H * a.nb >= 148 * 32; }
 
+int ssm_blocks(const SsmArgs &a) { return a.P / (ssm_wide(a) ? 64 : 16) * a.H; }
 cudaError_t launch_ssm(const SsmArgs &a, cudaStream_t s) {
     const bool wide = ssm_wide(a);
     const dim3 grid(a.P / (wide ? 64 : 16), a.H, a.nb);

@@ -165,6 +165,7 @@ __device__ __forceinline__ void ssm_body(const SsmArgs &a, const int bx, const i
     }
 
     // ---- recurrence over the T positions
+    float sq = 0.f;                          // packed output: square of this lane's value
     float *sout = a.state_out + (size_t)b * a.out_seq_stride + ((size_t)h * a.P + p0 + warp * RPW) * N;
     for (int i = 0; i < T; ++i) {
         const float dec = a_s[i], dt = dt_s[i];
@@ -193,7 +194,11 @@ __device__ __forceinline__ void ssm_body(const SsmArgs &a, const int bx, const i
         if ((lane & (LPV - 1)) == 0) {
             const int r = lane / LPV, col = h * a.P + p0 + warp * RPW + r;
             const float z = zs[i][warp * RPW + r];
-            a.g[(size_t)(rowbase + i) * a.di + col] = (y + Dh * xs[i][warp * RPW + r]) * silu_f(z);
+            const float out = (y + Dh * xs[i][warp * RPW + r]) * silu_f(z);
+            if (TMAX == 1 && a.pk) {
+                store_split(a.pk + (size_t)lb * a.di + col, (size_t)a.pk_rows * a.di, out * a.gnorm[col]);
+                sq = out * out;
+            } else a.g[(size_t)(rowbase + i) * a.di + col] = out;
         }
         // state after position i (verify: snapshot i; draft: the scratch state; rollback by replay: nothing)
         if (a.log) continue;
@@ -207,6 +212,13 @@ __device__ __forceinline__ void ssm_body(const SsmArgs &a, const int bx, const i
                 if (VW == 4) *reinterpret_cast<float4 *>(p) = make_float4(s[r][v * 4], s[r][v * 4 + 1], s[r][v * 4 + 2], s[r][v * 4 + 3]);
                 else *reinterpret_cast<float2 *>(p) = make_float2(s[r][0], s[r][1]);
             }
+    }
+    if (TMAX == 1 && a.pk) {
+        __shared__ float sq_s[SSM_THREADS / 32];
+        sq = warp_sum(sq);
+        if (lane == 0) sq_s[warp] = sq;
+        __syncthreads();
+        if (threadIdx.x == 0) a.pk_ss[(size_t)(by * (a.P / SSM_PR) + bx) * a.pk_rows + lb] = (sq_s[0] + sq_s[1]) + (sq_s[2] + sq_s[3]);
     }
 }
 

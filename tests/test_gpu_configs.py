@@ -110,6 +110,23 @@ def test_cfg2_projection_kernel_choices(env):
     assert rep.rounds == 7
 
 
+@pytest.mark.parametrize("name,L", [("cfg2_0p5b", 2), ("cfg4_seq", 4)])
+@pytest.mark.parametrize("batch,k", [(7, 1), (16, 2), (17, 3), (33, 4), (40, 4)])
+def test_projections_and_packed_mixers_by_rows(env, monkeypatch, name, L, batch, k):
+    # tcgen05 projections of 7 .. 200 activation rows on the 1024-wide layers: residual ones in tiles of 64 weight rows (up to 17
+    # rows) and of 128, 16 .. 128 rows per tile, K split over clusters whose last rank finishes fewer rows or none; the mixers of
+    # the draft steps (7 .. 40 rows) and the DeltaNet layers (below 192 rows) pack the out-projection's operand themselves
+    s = hi.CONFIGS[name].replace(L=L, V=2048)
+    monkeypatch.setitem(hi.CONFIGS, "small", s)
+    _W.pop(("small", "jitter"), None)
+    _, eng, model, seqs = make(env, "small", batch, k, 96, {0, batch // 2, batch - 1}, [20 + 3 * (b % 9) for b in range(batch)])
+    _W.pop(("small", "jitter"), None)
+    forced = [hi.forced_accept(k, 2, seq=b) for b in range(batch)]
+    rep = env["harness"].run_rounds(eng, seqs, s, k, 2, forced=forced)
+    print(rep)
+    assert rep.rounds == 2 and eng.device_status() == 0
+
+
 def test_streaming_attention_edge_cases(env):
     # the streaming form (128-key tiles walked with two buffers, warp-local running softmax, ranges merged by the last
     # CTA to arrive) on the small sequential stack, where attention is a launch of its own: contexts that end exactly on
