@@ -275,6 +275,8 @@ AttnGeom attn_geom(const hs_model *m, int Tq, int T, int b0, int nb) {
         // 128-key tiles per CTA.  A whole cache in one CTA spares the merge of ranges; otherwise about one CTA per SM, half
         // that where there is work for several tiles each (staging the queries and merging the ranges is paid per CTA: 544
         // tiles of work run best as 8 per CTA)
+        // From several rounds of 16 tiles per CTA on: one CTA per SM, each with an equal share of all tiles (0).
+        if (tiles128 > 148 * 16) return AttnGeom{128, 0, 0, 1, false};
         const int half = (int)((tiles128 + 73) / 74);
         int tiles = per_seq <= half ? per_seq : tiles128 <= 2 * 148 ? (int)((tiles128 + 147) / 148) : half;
         tiles = tiles < 1 ? 1 : tiles > 16 ? 16 : tiles;
@@ -429,7 +431,8 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
             aa.chunk = at_geom.chunk; aa.tiles = at_geom.tiles; aa.small = at_geom.small; aa.stream = at_geom.stream;
             if (!m->kmaps.empty()) { aa.kmap = m->kmaps[ly.al]; aa.vmap = m->vmaps[ly.al]; }
             aa.len_off = draft ? step : 0;
-            aa.nch = (c.kv_capacity + at_geom.chunk * at_geom.tiles - 1) / (at_geom.chunk * at_geom.tiles); aa.T = T; aa.b0 = b0; aa.nb = nb;
+            const int span = at_geom.chunk * std::max(at_geom.tiles, 1);
+            aa.nch = (c.kv_capacity + span - 1) / span; aa.T = T; aa.b0 = b0; aa.nb = nb;
             bool fused = false;
             if (ssm_deferred) {
                 // a parallel block: mixer and attention are independent of each other - one launch for both

@@ -25,6 +25,7 @@
 //    counter, no spinning) merges them in order, so the result is reproducible.
 #include "hs_internal.h"
 #include "hs_device.cuh"
+#include <type_traits>
 #include "ssm_body.cuh"
 #include <cooperative_groups.h>
 
@@ -815,7 +816,11 @@ __device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int spl
 // result, otherwise the CTA publishes its partial and the CTA of the sequence and KV head that arrives last (ticket
 // counter, no spinning) merges the ranges in order, so the result does not depend on timing.  No clusters: every SM
 // takes the next CTA as soon as it is free.
-constexpr int A2_THREADS = 256, A2_WARPS = 8, A2_CK = 128, A2_NBUF = 3;
+// Sixteen warps in two groups of eight.  A warp takes 16 keys of a tile and ONE 16-row query tile: with two query tiles (MT = 2) each
+// group has one of them, with one the groups take the tiles of keys in turn.  (Eight warps with both query tiles held 242
+// registers a thread, two warps on a scheduler, and waited for their own operands most of the time: 178 us per launch on the batch-64
+// workload at k = 4.)
+constexpr int A2_THREADS = 512, A2_KW = 8, A2_CK = 128, A2_NBUF = 3;
 
 // Tile buffers hold 128 keys x HD bf16 without padding; the 16-byte chunk c of row r sits at chunk position
 // c ^ (r & 7), which keeps the eight rows of an ldmatrix 8x8 block on different banks.  Three K and three V buffers:
@@ -830,7 +835,7 @@ __host__ __device__ inline Attn2Layout attn2_layout(int hd, int mt) {
     L.q_off = o; o += (size_t)2 * mt * 16 * L.kstr * 2;            // bf16 head | remainder
     L.new_off = o; o += (size_t)2 * 16 * L.kstr * 2;               // the new K | V rows as they are cached: a 16-key group of their own
     L.rope_off = o; o += (size_t)HS_MAX_T * (hd / 2) * 8;
-    L.ml_off = o; o += (size_t)(A2_WARPS + 1) * mt * 16 * 2 * 4;   // per warp (max, sum) per row, then the merged pair
+    L.ml_off = o; o += (size_t)(2 * A2_KW + mt) * 16 * 2 * 4;      // per warp (max, sum) per row, then the merged pairs
     L.total = (o + 127) / 128 * 128 + 1024;
     return L;
 }
@@ -852,7 +857,7 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     extern __shared__ __align__(1024) unsigned char smraw[];
     constexpr int CK = A2_CK, GTB = MT * 16, NT = HD / 8, RB = HD * 2;       // RB: bytes of a tile row
     constexpr int PB = (MT - 1) * 16;                                        // first row of the packed tile
-    const int split = blockIdx.x, kh = blockIdx.y, lb = blockIdx.z, b = a.b0 + lb;
+    constexpr int NPART = 2 * A2_KW / MT;                                    // partial results per query row
     const int G = a.qh / a.kvh, T = a.T, GT = G * T;
     const Attn2Layout L = attn2_layout(HD, MT);
     const int KSTR = L.kstr;
@@ -865,52 +870,110 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     __nv_bfloat16 *Kn_s = reinterpret_cast<__nv_bfloat16 *>(sm + L.new_off);      // [16][KSTR]
     __nv_bfloat16 *Vn_s = Kn_s + (size_t)16 * KSTR;
     float2 *rope_s = reinterpret_cast<float2 *>(sm + L.rope_off);
-    float *wml_s = reinterpret_cast<float *>(sm + L.ml_off);                      // [A2_WARPS + 1][GTB][2]
+    float *wml_s = reinterpret_cast<float *>(sm + L.ml_off);                      // [NPART][GTB][2], then the merged pairs
     __shared__ int ticket_s;
-    __shared__ __align__(8) uint64_t tile_bar[A2_NBUF];                              // one per tile buffer pair: bytes of K and V landed
+    __shared__ int scan_s[A2_THREADS / 32], at_s[2];
+    // bytes of K and V landed: tile t on barrier t % 6.  (Two per buffer pair: with MT = 1 successive tiles of a pair belong to different
+    // groups, and a warp must not take the phase of a tile that it skips for that of the one it waits for.)
+    __shared__ __align__(8) uint64_t tile_bar[2 * A2_NBUF];
     __shared__ int tile_done[A2_NBUF];                                               // warps that have finished with the pair's current tile
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t tinv = (65536u + T - 1) / T;
     pdl_trigger();
 
-    // ---- before the wait: kv_len, the first two tiles, the RoPE rows
-    const int len = __ldcg(a.kv_len + b) + a.len_off;
-    const int SPAN = CK * a.tiles;
-    const int nsplit = max(1, (len + SPAN - 1) / SPAN);
-    if (split >= nsplit) return;                   // beyond the cache
-    if (len < 0 || len + T > a.cap) {
-        if (tid == 0 && split == 0 && kh == 0) atomicCAS(a.status, 0, len < 0 ? (int)HS_ERR_DEVICE : (int)HS_ERR_CAPACITY);
-        return;
+    // ---- before the wait: this CTA's work.  a.tiles > 0: a.tiles tiles of one cache (grid = ranges, KV heads, sequences).
+    // a.tiles = 0: an equal share of the tiles of all caches, one after the other, for each of the grid's CTAs; a share may start and
+    // end inside a cache.
+    struct Segment { int b, lb, kh, len, c0, rc, ntile, nitem, piece, npiece; bool last; } sg;
+    int u = 0, u_end = 0, n_cache = 0, g0 = 0, ncta = 1, total = 0;     // ranged: next item, end of the share; items of the current cache, number of its first
+    auto cache_len = [&](int lb) { return __ldcg(a.kv_len + a.b0 + lb) + a.len_off; };
+    auto items_of = [&](int len) { return max(1, (min(max(len, 0), a.cap) + CK - 1) / CK); };
+    auto share_start = [&](int c) { return (int)((long long)c * total / ncta); };
+    auto cta_of = [&](int i) {
+        int c = (int)((long long)i * ncta / total);
+        while (c + 1 < ncta && share_start(c + 1) <= i) ++c;
+        while (c > 0 && share_start(c) > i) --c;
+        return c;
+    };
+    auto cut = [&](int tiles_at, int tiles_end) {       // tiles tiles_at .. tiles_end - 1 of the cache
+        sg.c0 = tiles_at * CK; sg.rc = max(0, min(sg.len, tiles_end * CK) - sg.c0);
+        sg.ntile = (sg.rc + CK - 1) / CK;
+        sg.nitem = sg.ntile + (sg.last ? 1 : 0);        // the range that ends the cache also takes the new rows, as one more item
+    };
+    auto ranged_segment = [&]() {
+        const int at = u - g0, end = min(n_cache, at + u_end - u);
+        sg.last = end == n_cache;
+        const int c_lo = cta_of(g0);
+        sg.piece = (int)blockIdx.x - c_lo; sg.npiece = cta_of(g0 + n_cache - 1) - c_lo + 1;
+        cut(at, end);
+        u += end - at;
+    };
+    if (a.tiles > 0) {
+        sg.kh = blockIdx.y; sg.lb = blockIdx.z; sg.b = a.b0 + sg.lb; sg.len = cache_len(sg.lb); sg.piece = blockIdx.x;
+        sg.npiece = max(1, (sg.len + CK * a.tiles - 1) / (CK * a.tiles));
+        if (sg.piece >= sg.npiece) return;             // beyond the cache
+        sg.last = sg.piece == sg.npiece - 1;
+        cut(sg.piece * a.tiles, (sg.piece + 1) * a.tiles);
+    } else {
+        // items before every sequence: a scan over the block, each thread with its part of the sequences
+        const int per = (a.nb + A2_THREADS - 1) / A2_THREADS, lo = min(a.nb, tid * per), hi = min(a.nb, lo + per);
+        int mine = 0;
+        for (int lb = lo; lb < hi; ++lb) mine += items_of(cache_len(lb)) * a.kvh;
+        int inc = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int y = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += y; }
+        if (lane == 31) scan_s[warp] = inc;
+        __syncthreads();
+        int before = inc - mine;
+        for (int w = 0; w < A2_THREADS / 32; ++w) { if (w < warp) before += scan_s[w]; total += scan_s[w]; }
+        ncta = min((int)gridDim.x, total);
+        if ((int)blockIdx.x >= ncta) return;
+        u = share_start(blockIdx.x); u_end = share_start(blockIdx.x + 1);
+        if (u >= before && u < before + mine) {
+            int lb = lo, at = before;
+            for (int n; u >= at + (n = items_of(cache_len(lb)) * a.kvh); ++lb) at += n;
+            at_s[0] = lb; at_s[1] = at;
+        }
+        __syncthreads();
+        sg.lb = at_s[0]; sg.b = a.b0 + sg.lb; sg.len = cache_len(sg.lb); n_cache = items_of(sg.len);
+        sg.kh = (u - at_s[1]) / n_cache; g0 = at_s[1] + sg.kh * n_cache;
+        ranged_segment();
     }
-    const bool last = split == nsplit - 1;
-    const int c0 = split * SPAN, rc = max(0, min(len, c0 + SPAN) - c0);
-    const int ntile = (rc + CK - 1) / CK;
-    const int nitem = ntile + (last ? 1 : 0);      // the range that ends the cache also takes the new rows, as one more item
-    __nv_bfloat16 *Kb = a.Kc + ((size_t)b * a.kvh + kh) * a.cap * HD;
-    __nv_bfloat16 *Vb = a.Vc + ((size_t)b * a.kvh + kh) * a.cap * HD;
-    // Cached rows of tile t into buffer pair t % 3: tensor copies of 64 columns x 128 rows (the two halves of a 128-wide
-    // head dimension land 16 KB apart), issued by one thread, completion counted in bytes on the pair's barrier.  A tile
+    if (tid == 0) {
+#pragma unroll
+        for (int i = 0; i < 2 * A2_NBUF; ++i) { mbar_init(&tile_bar[i], 1); tile_done[i % A2_NBUF] = 0; }
+        mbar_fence_init();
+    }
+    int sq = 0;                             // tiles of the segments before this one
+    constexpr int HALVES = HD / 64, HS_ = CK * 128;      // HS_: bytes between the halves of a tile
+    // Cached rows of tile t into buffer pair (sq + t) % 3: tensor copies of 64 columns x 128 rows (the two halves of a 128-wide
+    // head dimension land 16 KB apart), issued by one thread, completion counted in bytes on the tile's barrier.  A tile
     // is fetched whole: rows beyond the cache length hold earlier contents or belong to the next head - they are masked
     // (K) or cleared (V) below; rows beyond the tensor read as zero.
-    constexpr int HALVES = HD / 64, HS_ = CK * 128;      // HS_: bytes between the halves of a tile
-    const int row00 = (b * a.kvh + kh) * a.cap + c0;
     auto fetch = [&](int t) {              // called by ONE thread
-        if (t >= ntile) return;
-        uint64_t *bar = &tile_bar[t % A2_NBUF];
+        if (t >= sg.ntile) return;
+        uint64_t *bar = &tile_bar[(sq + t) % (2 * A2_NBUF)];
+        const int buf = (sq + t) % A2_NBUF, row00 = (sg.b * a.kvh + sg.kh) * a.cap + sg.c0;
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // the buffer was last touched by ordinary loads / stores
         mbar_expect_tx(bar, 2u * CK * RB);
 #pragma unroll
         for (int hf = 0; hf < HALVES; ++hf) {
-            tma_tile_2d(Kbuf(t % A2_NBUF) + hf * HS_, &a.kmap, hf * 64, row00 + t * CK, bar);
-            tma_tile_2d(Vbuf(t % A2_NBUF) + hf * HS_, &a.vmap, hf * 64, row00 + t * CK, bar);
+            tma_tile_2d(Kbuf(buf) + hf * HS_, &a.kmap, hf * 64, row00 + t * CK, bar);
+            tma_tile_2d(Vbuf(buf) + hf * HS_, &a.vmap, hf * 64, row00 + t * CK, bar);
         }
     };
-    if (tid == 0) {
-#pragma unroll
-        for (int i = 0; i < A2_NBUF; ++i) { mbar_init(&tile_bar[i], 1); tile_done[i] = 0; }
-        mbar_fence_init();
+    for (bool opening = true;; opening = false) {
+    const int b = sg.b, kh = sg.kh, len = sg.len, rc = sg.rc, ntile = sg.ntile, nitem = sg.nitem;
+    const bool last = sg.last;
+    const bool valid = len >= 0 && len + T <= a.cap;
+    if (!valid) {                                  // a control word out of range is never turned into an address
+        if (tid == 0 && last && kh == 0) atomicCAS(a.status, 0, len < 0 ? (int)HS_ERR_DEVICE : (int)HS_ERR_CAPACITY);
+        if (a.tiles > 0) return;
     }
+    __nv_bfloat16 *Kb = a.Kc + ((size_t)b * a.kvh + kh) * a.cap * HD;
+    __nv_bfloat16 *Vb = a.Vc + ((size_t)b * a.kvh + kh) * a.cap * HD;
+    if (valid) {
     if (tid == 0) { fetch(0); fetch(1); fetch(2); }
 #pragma unroll 1
     for (int idx = tid; idx < T * (HD / 2); idx += A2_THREADS) {
@@ -928,11 +991,13 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
         const int r = idx / (HD / 8), c = idx % (HD / 8);
         *reinterpret_cast<uint4 *>(Vn_s + (size_t)r * KSTR + 8 * c) = make_uint4(0, 0, 0, 0);
     }
-    pdl_wait();
+    }
+    if (opening) pdl_wait();
     __syncthreads();                        // rope_s complete, Vn_s cleared
+    if (valid) {
 
     // ---- queries (RoPE, scale, bf16 head + remainder) and, in the last range, the new K / V rows
-    const int rowbase = lb * T;
+    const int rowbase = sg.lb * T;
     const float scale = rsqrtf((float)HD);
     {
         constexpr int HP = HD / 2, NH = A2_THREADS / HP;
@@ -985,38 +1050,39 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     }
     __syncthreads();                        // queries and new rows in place
 
-    const int g8 = lane >> 2, t4 = lane & 3;
-    float O[MT][NT][4];
+    const int g8 = lane >> 2, t4 = lane & 3, grp = warp >> 3, kw = warp & 7;
+    const int q0 = MT == 2 ? grp * 16 : 0;                                   // first row of this warp's query tile
+    float O[NT][4];
 #pragma unroll
-    for (int mt = 0; mt < MT; ++mt)
+    for (int nt = 0; nt < NT; ++nt) { O[nt][0] = O[nt][1] = O[nt][2] = O[nt][3] = 0.f; }
+    float m_run[2], l_run[2];
+    int ti[2];                              // position index of each of this lane's rows among the T new ones
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt) { O[mt][nt][0] = O[mt][nt][1] = O[mt][nt][2] = O[mt][nt][3] = 0.f; }
-    float m_run[MT][2], l_run[MT][2];
-    int ti[MT][2];                          // position index of each of this lane's rows among the T new ones
-#pragma unroll
-    for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            m_run[mt][r] = -INFINITY; l_run[mt][r] = 0.f;
-            const int row = mt * 16 + g8 + 8 * r;
-            ti[mt][r] = row - (int)((row * tinv) >> 16) * T;
-        }
+    for (int r = 0; r < 2; ++r) {
+        m_run[r] = -INFINITY; l_run[r] = 0.f;
+        const int row = q0 + g8 + 8 * r;
+        ti[r] = row - (int)((row * tinv) >> 16) * T;
+    }
 
     // An item is a tile of cached keys (a buffer of the ring, swizzled rows of RB bytes) or, last, the new rows (their own
     // padded buffer): the same code serves both, told apart by base address, row pitch and swizzle mask.
+    auto walk = [&](auto packed_) {
+    constexpr bool packed = decltype(packed_)::value;
 #pragma unroll 1
-    for (int t = 0; t < nitem; ++t) {
+    for (int t = MT == 2 ? 0 : grp ^ (sq & 1); t < nitem; t += MT == 2 ? 1 : 2) {
         const bool newrows = t >= ntile;
+        const int buf = (sq + t) % A2_NBUF;
         const int nkeys = newrows ? T : min(CK, rc - t * CK);
         const int nkp = (nkeys + 15) & ~15;
         if (!newrows) {
             // Tile t has landed (tiles t + 1 and t + 2 may be in flight); a wait that runs out is reported and the pass goes
             // on.  There is no block-wide barrier per tile: a warp works on its 16 keys as soon as the tile is there and
             // hands the buffers back when it is done (below), so the warps drift apart and fill each other's stalls.
-            if (!mbar_wait(&tile_bar[t % A2_NBUF], (uint32_t)(t / A2_NBUF) & 1u) && lane == 0) atomicCAS(a.status, 0, (int)HS_ERR_TIMEOUT);
-            if (nkp != nkeys && warp * 16 <= nkeys && nkeys < warp * 16 + 16) {
-                // a ragged tile (only the last can be): finite V rows for the padding keys of the group that holds them
-                unsigned char *vd = Vbuf(t % A2_NBUF);
+            if (!mbar_wait(&tile_bar[(sq + t) % (2 * A2_NBUF)], (uint32_t)((sq + t) / (2 * A2_NBUF)) & 1u) && lane == 0) atomicCAS(a.status, 0, (int)HS_ERR_TIMEOUT);
+            if (nkp != nkeys && kw * 16 <= nkeys && nkeys < kw * 16 + 16) {
+                // a ragged tile (only the last can be): finite V rows for the padding keys of the group that holds them (two warps
+                // may both write these zeros)
+                unsigned char *vd = Vbuf(buf);
 #pragma unroll 1
                 for (int idx = lane; idx < (nkp - nkeys) * (HD / 8); idx += 32) {
                     const int c = idx % (HD / 8);
@@ -1025,110 +1091,90 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
                 __syncwarp();
             }
         }
-        const unsigned char *K_s = newrows ? reinterpret_cast<const unsigned char *>(Kn_s) : Kbuf(t % A2_NBUF);
-        const unsigned char *V_s = newrows ? reinterpret_cast<const unsigned char *>(Vn_s) : Vbuf(t % A2_NBUF);
+        const unsigned char *K_s = newrows ? reinterpret_cast<const unsigned char *>(Kn_s) : Kbuf(buf);
+        const unsigned char *V_s = newrows ? reinterpret_cast<const unsigned char *>(Vn_s) : Vbuf(buf);
         // a tile: rows of 128 bytes per half, 16-byte chunks XOR-swizzled with the row; the new rows: padded rows, no swizzle
         const int pitch = newrows ? KSTR * 2 : 128, swz = newrows ? 0 : 7, hstr = newrows ? 128 : HS_;
         // 16 keys per warp; the new rows are one group, given to the warp that a ragged last tile leaves idle most often
-#pragma unroll 1
-        for (int kb = (newrows ? (warp == A2_WARPS - 1 ? 0 : nkp) : warp * 16); kb < nkp; kb += A2_WARPS * 16) {
-            // ---- scores of this warp's 16 keys for all query rows (two accumulator sets: head and remainder products)
-            float S[MT][2][4];
+        const int kb = newrows ? (kw == A2_KW - 1 ? 0 : nkp) : kw * 16;
+        if (kb < nkp) {
+            // ---- scores of this warp's 16 keys (two accumulator sets: head and remainder products)
+            float S[2][4];
             {
-                float Sp[2][MT][2][4];
+                float Sp[2][2][4];
 #pragma unroll
                 for (int c = 0; c < 2; ++c)
 #pragma unroll
-                    for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-                        for (int nt = 0; nt < 2; ++nt) { Sp[c][mt][nt][0] = Sp[c][mt][nt][1] = Sp[c][mt][nt][2] = Sp[c][mt][nt][3] = 0.f; }
+                    for (int nt = 0; nt < 2; ++nt) { Sp[c][nt][0] = Sp[c][nt][1] = Sp[c][nt][2] = Sp[c][nt][3] = 0.f; }
                 const int krow = kb + (lane & 7) + (lane >> 4) * 8;
                 const unsigned char *krp = K_s + (size_t)krow * pitch;
                 const int ksw = krow & swz, kc0 = (lane >> 3) & 1;
 #pragma unroll
                 for (int ks = 0; ks < HD / 16; ++ks) {
-                    uint32_t bk[4];
+                    uint32_t bk[4], ah[4];
                     ldsm_x4(bk, krp + ((ks * 2 + kc0) >> 3) * hstr + (((((ks * 2 + kc0) & 7)) ^ ksw) << 4));
-#pragma unroll
-                    for (int mt = 0; mt < MT; ++mt) {
-                        uint32_t ah[4], al[4];
-                        const size_t qo = (size_t)(mt * 16 + (lane & 7) + ((lane >> 3) & 1) * 8) * KSTR + ks * 16 + (lane >> 4) * 8;
-                        ldsm_x4(ah, Qh_s + qo);
-                        mma_bf16(Sp[0][mt][0], ah, bk[0], bk[1]); mma_bf16(Sp[0][mt][1], ah, bk[2], bk[3]);
-                        if (!(PK && mt == MT - 1)) {
-                            ldsm_x4(al, Ql_s + qo);
-                            mma_bf16(Sp[1][mt][0], al, bk[0], bk[1]); mma_bf16(Sp[1][mt][1], al, bk[2], bk[3]);
-                        }
+                    const size_t qo = (size_t)(q0 + (lane & 7) + ((lane >> 3) & 1) * 8) * KSTR + ks * 16 + (lane >> 4) * 8;
+                    ldsm_x4(ah, Qh_s + qo);
+                    // (packed: one accumulator set for even k steps, one for odd ones)
+                    const int c = packed ? ks & 1 : 0;
+                    mma_bf16(Sp[c][0], ah, bk[0], bk[1]); mma_bf16(Sp[c][1], ah, bk[2], bk[3]);
+                    if (!packed) {
+                        uint32_t al[4];
+                        ldsm_x4(al, Ql_s + qo);
+                        mma_bf16(Sp[1][0], al, bk[0], bk[1]); mma_bf16(Sp[1][1], al, bk[2], bk[3]);
                     }
-                }
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-                    for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) S[mt][nt][e] = Sp[0][mt][nt][e] + Sp[1][mt][nt][e];
-                if (PK)                      // packed tile: head product in the registers of row g, remainder product in those of row g + 8
-#pragma unroll
-                    for (int nt = 0; nt < 2; ++nt) { S[MT - 1][nt][0] += S[MT - 1][nt][2]; S[MT - 1][nt][1] += S[MT - 1][nt][3]; }
-            }
-            // ---- masks, running softmax, probabilities as operand fragments
-            const bool edge = newrows || kb + 16 > nkeys;
-            uint32_t ph[MT][4], pl[MT][4];
-            float corr_all[MT][2];
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt) {
-                float mx[2] = {-INFINITY, -INFINITY};
-                if (edge) {                 // only a ragged last group and the new rows have anything to mask
-#pragma unroll
-                    for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int key = kb + nt * 8 + 2 * t4 + (e & 1);
-                            if (key >= nkeys || (newrows && key > ti[mt][e >> 1])) S[mt][nt][e] = -INFINITY;
-                        }
                 }
 #pragma unroll
                 for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) mx[e >> 1] = fmaxf(mx[e >> 1], S[mt][nt][e]);
+                    for (int e = 0; e < 4; ++e) S[nt][e] = Sp[0][nt][e] + Sp[1][nt][e];
+                if (packed)                  // head product in the registers of row g, remainder product in those of row g + 8
 #pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    const bool packed = PK && mt == MT - 1;
-                    if (packed && r == 1) { corr_all[mt][1] = corr_all[mt][0]; continue; }   // rows 8-15 carry remainders, not rows
-                    mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 1));
-                    mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 2));
-                    const float mnew = fmaxf(m_run[mt][r], mx[r]);
-                    const float muse = mnew == -INFINITY ? 0.f : mnew;
-                    const float corr = __expf(m_run[mt][r] - muse);
-                    corr_all[mt][r] = corr;
-                    m_run[mt][r] = mnew;
-                    float sum = 0.f;
+                    for (int nt = 0; nt < 2; ++nt) { S[nt][0] += S[nt][2]; S[nt][1] += S[nt][3]; }
+            }
+            // ---- masks, running softmax, probabilities as operand fragments
+            uint32_t ph[4], pl[4];
+            float corr[2], mx[2] = {-INFINITY, -INFINITY};
+            if (newrows || kb + 16 > nkeys) {   // only a ragged last group and the new rows have anything to mask
 #pragma unroll
-                    for (int nt = 0; nt < 2; ++nt) {
-                        const float p0 = __expf(S[mt][nt][2 * r] - muse), p1 = __expf(S[mt][nt][2 * r + 1] - muse);
-                        sum += p0 + p1;
-                        // two probabilities at a time: bf16 heads packed by one conversion, remainders from the exact differences
-                        const uint32_t hh = pack_bf16x2(p0, p1);
-                        const uint32_t ll = pack_bf16x2(p0 - __uint_as_float(hh << 16), p1 - __uint_as_float(hh & 0xffff0000u));
-                        ph[mt][r + 2 * nt] = hh;
-                        if (packed) ph[mt][1 + 2 * nt] = ll;     // operand rows 8-15 of the packed tile
-                        else pl[mt][r + 2 * nt] = ll;
+                for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int key = kb + nt * 8 + 2 * t4 + (e & 1);
+                        if (key >= nkeys || (newrows && key > ti[e >> 1])) S[nt][e] = -INFINITY;
                     }
-                    l_run[mt][r] = fmaf(l_run[mt][r], corr, sum);
+            }
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) mx[e >> 1] = fmaxf(mx[e >> 1], S[nt][e]);
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                if (packed && r == 1) { corr[1] = corr[0]; continue; }       // rows 8-15 carry remainders, not rows
+                mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 1));
+                mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 2));
+                const float mnew = fmaxf(m_run[r], mx[r]);
+                const float muse = mnew == -INFINITY ? 0.f : mnew;
+                corr[r] = __expf(m_run[r] - muse);
+                m_run[r] = mnew;
+                float sum = 0.f;
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt) {
+                    const float p0 = __expf(S[nt][2 * r] - muse), p1 = __expf(S[nt][2 * r + 1] - muse);
+                    sum += p0 + p1;
+                    // two probabilities at a time: bf16 heads packed by one conversion, remainders from the exact differences
+                    const uint32_t hh = pack_bf16x2(p0, p1);
+                    const uint32_t ll = pack_bf16x2(p0 - __uint_as_float(hh << 16), p1 - __uint_as_float(hh & 0xffff0000u));
+                    ph[r + 2 * nt] = hh;
+                    if (packed) ph[1 + 2 * nt] = ll;             // operand rows 8-15 of the packed tile
+                    else pl[r + 2 * nt] = ll;
                 }
+                l_run[r] = fmaf(l_run[r], corr[r], sum);
             }
             // the accumulators are rescaled only when some row's running maximum moved (rare after the first tiles)
-            bool moved = false;
+            if (__any_sync(0xffffffffu, corr[0] != 1.f || corr[1] != 1.f)) {
 #pragma unroll
-            for (int mt = 0; mt < MT; ++mt) moved = moved || corr_all[mt][0] != 1.f || corr_all[mt][1] != 1.f;
-            if (__any_sync(0xffffffffu, moved)) {
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-                    for (int nt = 0; nt < NT; ++nt) {
-                        O[mt][nt][0] *= corr_all[mt][0]; O[mt][nt][1] *= corr_all[mt][0];
-                        O[mt][nt][2] *= corr_all[mt][1]; O[mt][nt][3] *= corr_all[mt][1];
-                    }
+                for (int nt = 0; nt < NT; ++nt) { O[nt][0] *= corr[0]; O[nt][1] *= corr[0]; O[nt][2] *= corr[1]; O[nt][3] *= corr[1]; }
             }
             // ---- partial output += P V over the whole head dimension
             const int vrow = kb + (lane & 7) + ((lane >> 3) & 1) * 8;
@@ -1138,68 +1184,65 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
             for (int p = 0; p < NT / 2; ++p) {
                 uint32_t bv[4];
                 ldsm_x4_t(bv, vrp + ((p * 2 + vc0) >> 3) * hstr + ((((p * 2 + vc0) & 7) ^ vsw) << 4));
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt) {
-                    mma_bf16(O[mt][2 * p], ph[mt], bv[0], bv[1]); mma_bf16(O[mt][2 * p + 1], ph[mt], bv[2], bv[3]);
-                    if (!(PK && mt == MT - 1)) {
-                        mma_bf16(O[mt][2 * p], pl[mt], bv[0], bv[1]); mma_bf16(O[mt][2 * p + 1], pl[mt], bv[2], bv[3]);
-                    }
-                }
+                mma_bf16(O[2 * p], ph, bv[0], bv[1]); mma_bf16(O[2 * p + 1], ph, bv[2], bv[3]);
+                if (!packed) { mma_bf16(O[2 * p], pl, bv[0], bv[1]); mma_bf16(O[2 * p + 1], pl, bv[2], bv[3]); }
             }
         }
         if (!newrows) {
-            // this warp is done with tile t: the last of the eight to say so refills the buffer pair with tile t + 3
+            // this warp is done with tile t: the last of those that read it refills the buffer pair with tile t + 3
             __syncwarp();
             if (lane == 0) {
                 __threadfence_block();
-                if (atomicAdd(&tile_done[t % A2_NBUF], 1) == A2_WARPS - 1) { tile_done[t % A2_NBUF] = 0; fetch(t + A2_NBUF); }
+                if (atomicAdd(&tile_done[buf], 1) == A2_KW * MT - 1) { tile_done[buf] = 0; fetch(t + A2_NBUF); }
             }
         }
     }
+    };
+    const bool packed = PK && (MT == 1 || grp == 1);
+    if (PK && packed) walk(std::true_type{});
+    else if (!(PK && MT == 1)) walk(std::false_type{});
     __syncthreads();                        // everybody is done with the tile buffers (every requested tile was waited for)
 
-    // ---- merge the eight warp partials through shared memory (the tile buffers are free now)
-    float *wo_s = reinterpret_cast<float *>(sm + L.tile_off);            // [A2_WARPS][GTB][HD]
+    // ---- merge the warp partials through shared memory (the tile buffers are free now)
+    float *wo_s = reinterpret_cast<float *>(sm + L.tile_off);            // [NPART][GTB][HD]
+    const int part = MT == 2 ? kw : warp;
+    if (packed)                             // head and remainder halves of the packed tile's outputs
 #pragma unroll
-    for (int mt = 0; mt < MT; ++mt)
+        for (int nt = 0; nt < NT; ++nt) { O[nt][0] += O[nt][2]; O[nt][1] += O[nt][3]; }
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const bool packed = PK && mt == MT - 1;
-            if (packed && r == 1) continue;
-            if (packed)                       // head and remainder halves of the packed tile's outputs
+    for (int r = 0; r < 2; ++r) {
+        if (packed && r == 1) continue;
+        float l = l_run[r];
+        l += __shfl_xor_sync(0xffffffffu, l, 1);
+        l += __shfl_xor_sync(0xffffffffu, l, 2);
+        const int row = q0 + g8 + 8 * r;
+        if (t4 == 0) { wml_s[((size_t)part * GTB + row) * 2] = m_run[r]; wml_s[((size_t)part * GTB + row) * 2 + 1] = l; }
 #pragma unroll
-                for (int nt = 0; nt < NT; ++nt) { O[mt][nt][0] += O[mt][nt][2]; O[mt][nt][1] += O[mt][nt][3]; }
-            float l = l_run[mt][r];
-            l += __shfl_xor_sync(0xffffffffu, l, 1);
-            l += __shfl_xor_sync(0xffffffffu, l, 2);
-            const int row = mt * 16 + g8 + 8 * r;
-            if (t4 == 0) { wml_s[((size_t)warp * GTB + row) * 2] = m_run[mt][r]; wml_s[((size_t)warp * GTB + row) * 2 + 1] = l; }
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt)
-                *reinterpret_cast<float2 *>(wo_s + ((size_t)warp * GTB + row) * HD + nt * 8 + 2 * t4) = make_float2(O[mt][nt][2 * r], O[mt][nt][2 * r + 1]);
-        }
+        for (int nt = 0; nt < NT; ++nt)
+            *reinterpret_cast<float2 *>(wo_s + ((size_t)part * GTB + row) * HD + nt * 8 + 2 * t4) = make_float2(O[nt][2 * r], O[nt][2 * r + 1]);
+    }
     __syncthreads();
     float *o_base = a.o + (size_t)rowbase * (a.qh * HD);
-    const size_t pslot = ((size_t)b * a.kvh + kh) * a.nch + split;
-    float *mrg_s = wml_s + (size_t)A2_WARPS * GTB * 2;                       // [GTB][2] merged (M, den)
+    const size_t pslot = ((size_t)b * a.kvh + kh) * a.nch + sg.piece;
+    float *mrg_s = wml_s + (size_t)NPART * GTB * 2;                          // [GTB][2] merged (M, den)
     constexpr int DV4 = HD / 4;
 #pragma unroll 1
     for (int idx = tid; idx < GT * DV4; idx += A2_THREADS) {
         const int qi = idx / DV4, d = (idx - qi * DV4) * 4;
         float M = -INFINITY;
 #pragma unroll
-        for (int w = 0; w < A2_WARPS; ++w) M = fmaxf(M, wml_s[((size_t)w * GTB + qi) * 2]);
+        for (int w = 0; w < NPART; ++w) M = fmaxf(M, wml_s[((size_t)w * GTB + qi) * 2]);
         float den = 0.f;
         float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int w = 0; w < A2_WARPS; ++w) {
+        for (int w = 0; w < NPART; ++w) {
             const float mw = wml_s[((size_t)w * GTB + qi) * 2];
             const float wt = mw == -INFINITY ? 0.f : __expf(mw - M);
             den = fmaf(wt, wml_s[((size_t)w * GTB + qi) * 2 + 1], den);
             const float4 v = *reinterpret_cast<const float4 *>(wo_s + ((size_t)w * GTB + qi) * HD + d);
             sum.x = fmaf(wt, v.x, sum.x); sum.y = fmaf(wt, v.y, sum.y); sum.z = fmaf(wt, v.z, sum.z); sum.w = fmaf(wt, v.w, sum.w);
         }
-        if (nsplit == 1) {
+        if (sg.npiece == 1) {
             const int gq = (int)((qi * tinv) >> 16), i = qi - gq * T;
             const float inv = 1.0f / den;
             *reinterpret_cast<float4 *>(o_base + (size_t)i * (a.qh * HD) + (kh * G + gq) * HD + d) =
@@ -1209,7 +1252,7 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
             if (d == 0) { mrg_s[2 * qi] = M; mrg_s[2 * qi + 1] = den; }
         }
     }
-    if (nsplit == 1) return;
+    if (sg.npiece > 1) {
     __syncthreads();
     if (tid < 2 * GT) a.part_ml[pslot * HS_MAX_GT * 2 + tid] = mrg_s[tid];
     // ---- several ranges: the CTA that arrives last merges their partials in order
@@ -1217,13 +1260,14 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     __syncthreads();
     if (tid == 0) ticket_s = atomicAdd(a.counters + b * a.kvh + kh, 1);
     __syncthreads();
-    if (ticket_s != nsplit - 1) return;
+    if (ticket_s == sg.npiece - 1) {
     __threadfence();
+    const int nsplit = sg.npiece;
     if (tid == 0) a.counters[b * a.kvh + kh] = 0;          // ready for the next launch
     const size_t pbase = ((size_t)b * a.kvh + kh) * a.nch;
     const float *pa0 = a.part_acc + pbase * HS_MAX_GT * HD;
     const float *pm0 = a.part_ml + pbase * HS_MAX_GT * 2;
-    for (int qi = warp; qi < GT; qi += A2_WARPS) {
+    for (int qi = warp; qi < GT; qi += A2_THREADS / 32) {
         float M = -INFINITY;
         for (int c = lane; c < nsplit; c += 32) M = fmaxf(M, __ldcg(pm0 + ((size_t)c * HS_MAX_GT + qi) * 2));
         M = warp_max(M);
@@ -1252,6 +1296,17 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
         *reinterpret_cast<float4 *>(o_base + (size_t)i * (a.qh * HD) + (kh * G + gq) * HD + d) =
             make_float4(sum.x * inv, sum.y * inv, sum.z * inv, sum.w * inv);
     }
+    }
+    }
+    }
+    // ---- ranged: on to the next cache of the share
+    if (a.tiles > 0 || u >= u_end) return;
+    __syncthreads();                        // the partial results in the tile buffers have been read
+    sq += valid ? ntile : 0;
+    g0 += n_cache;
+    if (++sg.kh == a.kvh) { sg.kh = 0; ++sg.lb; ++sg.b; sg.len = cache_len(sg.lb); n_cache = items_of(sg.len); }
+    ranged_segment();
+    }
 }
 
 template <int HD, int MT, bool PK>
@@ -1264,7 +1319,7 @@ cudaError_t launch_attn2_t(const AttnArgs &a, cudaStream_t s) {
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    return launch_pdl(attn2_kernel<HD, MT, PK>, dim3(a.nch, a.kvh, a.nb), dim3(A2_THREADS), smem, s, a);
+    return launch_pdl(attn2_kernel<HD, MT, PK>, a.tiles > 0 ? dim3(a.nch, a.kvh, a.nb) : dim3(148), dim3(A2_THREADS), smem, s, a);
 }
 
 template <int HD, int MT>
@@ -1368,7 +1423,7 @@ cudaError_t launch_attn(const AttnArgs &a, cudaStream_t s) {
         return a.hd == 128 ? launch_small_t<128>(a, s) : a.hd == 64 ? launch_small_t<64>(a, s) : cudaErrorInvalidValue;
     }
     if (a.stream) {          // the streaming form: 128-key tiles, a.tiles of them per CTA, at most 32 query rows
-        if (GT > 32 || a.chunk != A2_CK || a.tiles < 1) return cudaErrorInvalidValue;
+        if (GT > 32 || a.chunk != A2_CK || a.tiles < 0) return cudaErrorInvalidValue;
         // at most 8 rows in the last 16-row tile: the packed form of that tile (half its tensor instructions)
 #define A2(hd_) if (a.hd == hd_) return GT <= 8 ? launch_attn2_t<hd_, 1, true>(a, s) : GT <= 16 ? launch_attn2_t<hd_, 1, false>(a, s) \
                                       : GT <= 24 ? launch_attn2_t<hd_, 2, true>(a, s) : launch_attn2_t<hd_, 2, false>(a, s)

@@ -146,6 +146,25 @@ def test_streaming_attention_edge_cases(env):
     assert rep.rounds == 5
 
 
+@pytest.mark.parametrize("qh,ks", [(4, (8, 4, 1)), (8, (7,))])
+def test_streaming_attention_in_equal_shares(env, monkeypatch, qh, ks):
+    # more than 16 rounds' worth of tiles (2600 by the longest of 100 caches): one CTA per SM with an equal share of the tiles of all
+    # caches, which starts and ends inside them; caches of many tiles, of one (full, one key short, one key over) and of a few keys,
+    # one query tile (plain, packed) and two (second one packed, plain)
+    s = hi.CONFIGS["test_seq"].replace(qh=qh)
+    monkeypatch.setitem(hi.CONFIGS, "test_seq_q%d" % qh, s)
+    sizes, batch, checked = (1600, 128, 127, 129, 5, 640, 1599, 1024), 100, {0, 1, 2, 3, 4, 38, 95, 99}
+    lens = [sizes[b % 8] if b % 3 else 1600 - b for b in range(batch)]
+    lens[:5] = [1600, 128, 127, 129, 5]
+    _, eng, model, seqs = make(env, "test_seq_q%d" % qh, batch, max(ks), 1700, checked, lens)
+    rep = None
+    for k in ks:
+        forced = [hi.forced_accept(k, 1, seq=40 + b + k) for b in range(batch)]
+        rep = env["harness"].run_rounds(eng, seqs, s, k, 1, forced=forced, rep=rep)
+        assert eng.device_status() == 0, k
+    assert rep.rounds == len(ks)
+
+
 def test_streaming_attention_batched_parallel_hybrid(env):
     # a batch large enough that the verify attention of the parallel hybrid runs as its own launch in the streaming form
     # (chosen automatically); three sequences carry their context on both sides, the others run beside them
