@@ -305,6 +305,13 @@ inline bool draft_runs(const hs_model *m, int l) {
     return m->plan[l] != HS_DRAFT_SKIP && (m->layers[l].type != HS_LAYER_ATT || m->plan[l] == HS_DRAFT_FULL);
 }
 
+// Activation rows from which a pass runs its projections on tcgen05.  The kernel's fixed cost (set-up, epilogue out of tensor
+// memory) pays from 4 rows on where the weight matrices are large or the mixers pack the out-projection's operand themselves, as in
+// a draft step, else from 6.  1024-wide models, warp-level path / tcgen05: draft step of 4, 5, 6 rows 0.5B-class 1.154 / 1.111,
+// 1.210 / 1.154, 1.350 / 1.126 ms, sequential 0.518 / 0.510, 0.549 / 0.514, 0.609 / 0.513; verify pass of 4, 5, 6 rows 0.5B-class 1.300 /
+// 1.375, 1.370 / 1.403, 1.592 / 1.473, sequential 0.717 / 0.754, 0.758 / 0.778, 0.868 / 0.822.
+inline int tc_rows(const hs_model *m, bool mixers_pack) { return g_hs_tc_min_rows ? g_hs_tc_min_rows : m->large_mats || mixers_pack ? 4 : 6; }
+
 // first = true: this pass opens an API call (its predecessor in the stream may be the accept kernel of the last
 // round): its first kernel goes out in plain stream order, see hs_device.cuh.
 // chunk = true (literal draft state only): the DRAFT model over T positions of every sequence on its own state buffers,
@@ -323,7 +330,8 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
     // many rows: every projection of the pass runs on the tcgen05 kernel, and the projections hand each other their
     // results in the packed form that kernel consumes (only the mixer's output and the embedding are packed by a
     // kernel of their own)
-    const bool tc_pass = gemv_uses_tc(rows, m->xb != nullptr);
+    __nv_bfloat16 *xb = rows > 16 || rows >= tc_rows(m, draft && T == 1) ? m->xb : nullptr;
+    const bool tc_pass = gemv_uses_tc(rows, xb != nullptr);
     int ss_parts = 0;                       // partial sums of squares per row in ssbuf
     bool h_packed = false;                  // xb_h / ssbuf hold the current residual stream
     PROF(HS_PROF_EMBED, 0, launch_embed(m->embed, d, c.V, m->ctrl.cand, m->Tm, draft ? step : 0, T, b0, nb, m->hbuf[0], st_w, first, s), "embed");
@@ -343,7 +351,7 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
         ga.early_trigger = 1;
         ga.pf_ptr = ly.type == HS_LAYER_ATT ? ly.W_o : ly.W_out;
         ga.pf_bytes = 2 * (int64_t)d * (ly.type == HS_LAYER_ATT ? c.qh * c.hd : m->gw);
-        ga.xb = m->xb; ga.xb_rows = m->xb_rows;
+        ga.xb = xb; ga.xb_rows = m->xb_rows;
         if (tc_pass && h_packed) { ga.pk_in = m->xb_h; ga.ss_in = m->ssbuf; ga.ss_parts = ss_parts; }
         PROF(HS_PROF_GEMV, gemv_bytes(ga), launch_gemv(ga, st_w, s, &m->launches, nullptr), "in_proj");
         // (2) recurrent mixer
@@ -458,7 +466,7 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
             go.W0 = ly.W_o; go.ldw0 = c.qh * c.hd; go.K0 = c.qh * c.hd; go.x0 = m->obuf; go.ldx0 = c.qh * c.hd;
         }
         go.early_trigger = 1; go.pf_ptr = ly.W_gu; go.pf_bytes = 2 * (int64_t)2 * c.ff * d;
-        go.xb = m->xb; go.xb_rows = m->xb_rows;
+        go.xb = xb; go.xb_rows = m->xb_rows;
         if (mix_packed) {
             go.pk_in = m->xb;
             if (mix_parts) { go.ss_in = m->gbuf; go.ss_parts = mix_parts; }
@@ -472,7 +480,7 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
         gu.norm_w = ly.norm2; gu.eps = c.eps;
         gu.O = 2 * c.ff; gu.out = m->abuf; gu.ldo = c.ff; gu.nrows = rows; gu.epi = EPI_SWIGLU;
         gu.early_trigger = 1; gu.pf_ptr = ly.W_down; gu.pf_bytes = 2 * (int64_t)d * c.ff;
-        gu.xb = m->xb; gu.xb_rows = m->xb_rows;
+        gu.xb = xb; gu.xb_rows = m->xb_rows;
         if (tc_pass) { gu.pk_in = m->xb_h; gu.ss_in = m->ssbuf; gu.ss_parts = ss_parts; gu.pk_out = m->xb_a; gu.pk_ld = c.ff; }
         PROF(HS_PROF_GEMV, gemv_bytes(gu), launch_gemv(gu, st_w, s, &m->launches, nullptr), "gate_up");
         GemvArgs gdn{};
@@ -491,7 +499,7 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
             // the consumer of this layer's output: the next layer that runs (its first norm), else the final norm
             if (tc_pass) { gdn.pk_out = m->xb_h; gdn.pk_ld = d; gdn.pk_nw = nl < c.L ? m->layers[nl].norm1 : m->final_norm; gdn.ss_out = m->ssbuf; gdn.ss_parts_out = &ss_parts; }
         }
-        gdn.xb = m->xb; gdn.xb_rows = m->xb_rows;
+        gdn.xb = xb; gdn.xb_rows = m->xb_rows;
         if (tc_pass) gdn.pk_in = m->xb_a;
         PROF(HS_PROF_GEMV, gemv_bytes(gdn), launch_gemv(gdn, st_w, s, &m->launches, &hparts), "down");
         cur ^= 1;
@@ -509,7 +517,7 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
     if (sampled) { lm.out = m->dlogits + (size_t)b0 * dstride + (size_t)step * c.V; lm.ldo = (int)dstride; }
     else { lm.out = m->logits; lm.ldo = c.V; }
     lm.early_trigger = 1;
-    lm.xb = m->xb; lm.xb_rows = m->xb_rows;
+    lm.xb = xb; lm.xb_rows = m->xb_rows;
     if (tc_pass && h_packed) { lm.pk_in = m->xb_h; lm.ss_in = m->ssbuf; lm.ss_parts = ss_parts; }
     PROF(HS_PROF_GEMV, gemv_bytes(lm), launch_gemv(lm, st_w, s, &m->launches, nullptr), "lm_head");
     if (sampled) PROF(HS_PROF_ARGMAX, 0, launch_sample(m->dlogits + (size_t)step * c.V, dstride, c.V, m->Tm, b0, nb, m->tau, m->u_draft, c.max_k, step,
@@ -641,7 +649,7 @@ int prefill_head(hs_model *m, const float *x, int T, int b0, int nb) {
     const hs_config &c = m->c;
     GemvArgs lm{};
     lm.W0 = m->lm_head; lm.ldw0 = c.d; lm.K0 = c.d; lm.x0 = x; lm.ldx0 = c.d; lm.xparts = 1; lm.norm_w = m->final_norm; lm.eps = c.eps;
-    lm.O = c.V; lm.out = m->logits; lm.ldo = c.V; lm.nrows = nb * T; lm.epi = EPI_STORE; lm.early_trigger = 1; lm.xb = m->xb; lm.xb_rows = m->xb_rows;
+    lm.O = c.V; lm.out = m->logits; lm.ldo = c.V; lm.nrows = nb * T; lm.epi = EPI_STORE; lm.early_trigger = 1; lm.xb = nb * T > 16 || nb * T >= tc_rows(m, false) ? m->xb : nullptr; lm.xb_rows = m->xb_rows;
     PROF(HS_PROF_GEMV, gemv_bytes(lm), launch_gemv(lm, m->ctrl.status, m->stream, &m->launches, nullptr), "prefill lm_head");
     PROF(HS_PROF_ARGMAX, 0, launch_argmax(m->logits, c.V, T, b0, nb, m->Tm, m->ctrl.g, 0, m->ctrl.margin, m->am_part, m->ctrl.am_counters, m->stream), "prefill argmax");
     PROF(HS_PROF_ARGMAX, 0, launch_pf_pending(m->ctrl.g, m->ctrl.cand, m->Tm, T, b0, nb, m->stream), "prefill pending");
@@ -831,10 +839,7 @@ static int init_model(hs_model *m, const hs_config *cfg, const hs_buffers *bufs,
     m->pf_rows = v.pf_rows; m->pf_rowtab = (int4 *)(w + wl.pf_rowtab); m->pf_segtab = (int4 *)(w + wl.pf_segtab); m->pf_list = (int2 *)(w + wl.pf_list);
     m->pf_xbc = (float *)(w + wl.pf_xbc); m->pf_dtv = (float *)(w + wl.pf_dtv); m->pf_hfin = (float *)(w + wl.pf_hfin); m->pf_rec = (float *)(w + wl.pf_rec); m->pf_q = (__nv_bfloat16 *)(w + wl.pf_q);
     m->xb_h = (__nv_bfloat16 *)(w + wl.xb_h); m->xb_a = (__nv_bfloat16 *)(w + wl.xb_a); m->ssbuf = (float *)(w + wl.ssbuf);
-    // the tcgen05 kernel's fixed cost (operand packing, tensor-memory set-up, epilogue out of tensor memory) pays from
-    // 7 activation rows on, from 4 where the weight matrices are large (measured: model widths 1024 and 2560)
-    m->tc_min_rows_auto = (int64_t)4 * c.ff * c.d >= ((int64_t)64 << 20) ? 4 : 7;
-    g_hs_tc_min_rows = m->tc_min_rows_auto;
+    m->large_mats = (int64_t)4 * c.ff * c.d >= ((int64_t)64 << 20);
     // conv buffer: committed windows | verify history | draft ping-pong
     float *cv = (float *)bufs->conv;
     const size_t win = (size_t)v.n_rl * v.B * 3 * v.convd;
@@ -912,7 +917,7 @@ int hs_prefill(hs_model *m, const int32_t *tokens_host, const int32_t *lens_host
     // (3225 tokens, two passes) on the sequential one 229 -> 13.1 ms.  A prompt of at most one chunk is one verify pass either way.
     // Except two tokens at max_k = 0, one sequence: two one-row passes cost less than a wide one while the matrices are small
     // (0.5B-class 1.54 / 1.62 ms, sequential 0.94 / 1.03; 3B-class 4.18 / 2.89, eight sequences 3.45 / 2.13).
-    const bool two_steps = longest == 2 && batch == 1 && m->tc_min_rows_auto == 7;
+    const bool two_steps = longest == 2 && batch == 1 && !m->large_mats;
     if (longest > m->Tm && !two_steps && g_hs_gemm_tc && !m->literal) return prefill_wide(m, tokens_host, lens_host, batch);
     // Chunk c covers prompt positions [c * Tm, (c + 1) * Tm) of every sequence that reaches that far; neighbouring
     // sequences with the same number of tokens in the chunk go out as one verify pass with every candidate accepted.
@@ -1219,7 +1224,7 @@ int hs_set_option(hs_model *m, int option, int value) {
     if (option == HS_OPT_TC_MIN_ROWS) {
         if (value != 0 && (value < 2 || value > 17)) return fail(m, HS_ERR_INVALID_ARG, "tcgen05 row threshold out of range");
         CK(cudaStreamSynchronize(m->stream), "option sync");
-        g_hs_tc_min_rows = value ? value : m->tc_min_rows_auto;
+        g_hs_tc_min_rows = value;
         for (auto &kv : m->graphs) cudaGraphExecDestroy(kv.second);
         m->graphs.clear(); m->graph_launches.clear();
         return HS_OK;

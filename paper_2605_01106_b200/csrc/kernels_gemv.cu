@@ -643,7 +643,7 @@ cudaError_t configure_gemv() {
 
 // Launches the projection.  a.max_oparts > 1 allows a K split for the residual epilogue; the number
 // of parts written is returned in *oparts (1 for the other epilogues).
-bool gemv_uses_tc(int nrows, bool have_xb) { return (nrows > GV_MAXROWS || nrows >= g_hs_tc_min_rows) && g_hs_gemm_tc && have_xb; }
+bool gemv_uses_tc(int nrows, bool have_xb) { return (nrows > GV_MAXROWS || nrows >= (g_hs_tc_min_rows ? g_hs_tc_min_rows : 4)) && g_hs_gemm_tc && have_xb; }
 
 cudaError_t launch_gemv(const GemvArgs &a_in, int32_t *status, cudaStream_t s, int64_t *launches, int *oparts) {
     GemvArgs a = a_in;

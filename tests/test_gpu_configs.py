@@ -111,11 +111,11 @@ def test_cfg2_projection_kernel_choices(env):
 
 
 @pytest.mark.parametrize("name,L", [("cfg2_0p5b", 2), ("cfg4_seq", 4)])
-@pytest.mark.parametrize("batch,k", [(7, 1), (16, 2), (17, 3), (33, 4), (40, 4)])
+@pytest.mark.parametrize("batch,k", [(4, 1), (7, 1), (16, 2), (17, 3), (33, 4), (40, 4)])
 def test_projections_and_packed_mixers_by_rows(env, monkeypatch, name, L, batch, k):
-    # tcgen05 projections of 7 .. 200 activation rows on the 1024-wide layers: residual ones in tiles of 64 weight rows (up to 17
+    # tcgen05 projections of 4 .. 200 activation rows on the 1024-wide layers: residual ones in tiles of 64 weight rows (up to 17
     # rows) and of 128, 16 .. 128 rows per tile, K split over clusters whose last rank finishes fewer rows or none; the mixers of
-    # the draft steps (7 .. 40 rows) and the DeltaNet layers (below 192 rows) pack the out-projection's operand themselves
+    # the draft steps (4 .. 40 rows) and the DeltaNet layers (below 192 rows) pack the out-projection's operand themselves
     s = hi.CONFIGS[name].replace(L=L, V=2048)
     monkeypatch.setitem(hi.CONFIGS, "small", s)
     _W.pop(("small", "jitter"), None)
