@@ -26,7 +26,7 @@ struct TcArgs {
     // The packed operand may come without the 1/rms factor of its RMSNorm (a projection epilogue wrote it, see
     // pk_out): then ss_in[p * rpad + r], p < ss_parts, are partial sums of squares of activation row r and the
     // factor rsqrt(sum * inv_k + eps) is applied to the finished sums of that row.
-    const float *ss_in; int ss_parts; float inv_k, eps;
+    const float *ss_in; int ss_parts; float inv_k, eps; bool ss_by_row;      // ss_by_row: ss_in[r * ss_parts + p]
     // Packed output for the projection that consumes this one's result: bf16 head | remainder planes
     // [2][rpad][pk_ld] of (result * pk_nw[output row]), and (residual epilogue) the partial sums of squares
     // ss_out[tile of weight rows][rpad] of the results.  nullptr: not wanted.

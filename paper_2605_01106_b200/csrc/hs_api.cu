@@ -469,7 +469,7 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
         go.xb = xb; go.xb_rows = m->xb_rows;
         if (mix_packed) {
             go.pk_in = m->xb;
-            if (mix_parts) { go.ss_in = m->gbuf; go.ss_parts = mix_parts; }
+            if (mix_parts) { go.ss_in = m->gbuf; go.ss_parts = mix_parts; go.ss_by_row = true; }
         }
         if (tc_pass) { go.pk_out = m->xb_h; go.pk_ld = d; go.pk_nw = ly.norm2; go.ss_out = m->ssbuf; go.ss_parts_out = &ss_parts; }
         PROF(HS_PROF_GEMV, gemv_bytes(go), launch_gemv(go, st_w, s, &m->launches, &hparts), "out_proj");

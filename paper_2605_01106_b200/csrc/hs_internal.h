@@ -168,7 +168,7 @@ struct GemvArgs {
     // p < ss_parts, are partial sums of squares of row r).  pk_out: where to leave this projection's result in packed
     // form for its consumer (row length pk_ld, times pk_nw[output] if given), with the partial sums of squares of the
     // residual epilogue's results in ss_out[tile][rows per plane] (tiles of 128 or 64 weight rows; how many: *ss_parts_out).
-    const __nv_bfloat16 *pk_in; const float *ss_in; int ss_parts;
+    const __nv_bfloat16 *pk_in; const float *ss_in; int ss_parts; bool ss_by_row;      // ss_by_row: ss_in[r * ss_parts + p] (the mixers' partial sums)
     __nv_bfloat16 *pk_out; int pk_ld; const float *pk_nw; float *ss_out; int *ss_parts_out;
 };
 // does a projection of nrows activation rows run on the many-row kernel?  (a caller that wants another one passes no xb)
@@ -218,7 +218,7 @@ struct SsmArgs {
                                         // reports HS_ERR_DEVICE through the status word
     // One position, no attention beside it: the output goes out as the packed operand of the out-projection (GemvArgs) instead of
     // g: bf16 head plane [pk_rows][di], remainder plane behind it, times gnorm, and per block the sum of squares of its outputs
-    // in pk_ss[block of the sequence][pk_rows].  NULL: g.
+    // in pk_ss[sequence][block of the sequence].  NULL: g.
     __nv_bfloat16 *pk; int pk_rows; const float *gnorm; float *pk_ss;
 };
 cudaError_t launch_ssm(const SsmArgs &a, cudaStream_t s);

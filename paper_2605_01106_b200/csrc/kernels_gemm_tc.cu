@@ -214,20 +214,27 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ 
                 prefetch_l2(reinterpret_cast<const char *>(a.pf_ptr) + o, (uint32_t)min(4096ll, hi - o));
         }
         pdl_wait();
-        if (a.ss_in && a.ss_parts > 32) {
-            // many partial sums (one per block of the mixer): a warp per activation row
+        if (a.ss_in && a.ss_by_row) {
+            // many partial sums (one per block of the mixer): a warp per activation row, three rows at a time
+            constexpr int W = TC_THREADS / 32 - 2;
 #pragma unroll 1
-            for (int i = warp - 2; i < BNH; i += TC_THREADS / 32 - 2) {
-                const float *ss = a.ss_in + n0h + i;
-                float t = 0.f;
+            for (int i0 = warp - 2; i0 < BNH; i0 += 3 * W) {
+                float t[3] = {0.f, 0.f, 0.f};
                 for (int p0 = lane; p0 < a.ss_parts; p0 += 128) {
-                    float x[4];
+                    float x[3][4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) x[u] = p0 + 32 * u < a.ss_parts ? __ldcg(ss + (size_t)(p0 + 32 * u) * a.rpad) : 0.f;
-                    t += (x[0] + x[1]) + (x[2] + x[3]);
+                    for (int r = 0; r < 3; ++r)
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            x[r][u] = n0h + i0 + r * W < a.nrows && p0 + 32 * u < a.ss_parts ? __ldcg(a.ss_in + (size_t)(n0h + i0 + r * W) * a.ss_parts + p0 + 32 * u) : 0.f;
+#pragma unroll
+                    for (int r = 0; r < 3; ++r) t[r] += (x[r][0] + x[r][1]) + (x[r][2] + x[r][3]);
                 }
-                t = warp_sum(t);
-                if (lane == 0) rstd_s[i] = rsqrtf(t * a.inv_k + a.eps) * a.found;
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    const float tot = warp_sum(t[r]);
+                    if (lane == 0 && i0 + r * W < BNH) rstd_s[i0 + r * W] = rsqrtf(tot * a.inv_k + a.eps) * a.found;
+                }
             }
         } else
 #pragma unroll 1
@@ -504,7 +511,7 @@ cudaError_t launch_gemm_tc(const GemvArgs &a, int32_t *status, cudaStream_t s, i
     TcArgs t{};
     t.O = a.O; t.nk0 = a.K0 / TC_BK; t.nk1 = a.K1 / TC_BK; t.nrows = a.nrows; t.rpad = rpad; t.bnh = bnh; t.ns = ns; t.rb = rb; t.rb_inv = 65536 / rb + 1;
     t.out = a.out; t.ldo = a.ldo; t.resid = a.resid; t.rparts = a.rparts; t.rpstride = a.rpstride; t.status = status;
-    if (a.pk_in && a.ss_in) { t.ss_in = a.ss_in; t.ss_parts = a.ss_parts; t.inv_k = 1.f / (float)a.K0; t.eps = a.eps; }
+    if (a.pk_in && a.ss_in) { t.ss_in = a.ss_in; t.ss_parts = a.ss_parts; t.inv_k = 1.f / (float)a.K0; t.eps = a.eps; t.ss_by_row = a.ss_by_row; }
     if (a.pk_out && a.epi != EPI_STORE) {
         t.pk_out = a.pk_out; t.pk_ld = a.pk_ld; t.pk_nw = a.pk_nw;
         t.ss_out = a.epi == EPI_RESID ? a.ss_out : nullptr;

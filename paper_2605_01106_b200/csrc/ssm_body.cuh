@@ -79,6 +79,7 @@ __device__ __forceinline__ void ssm_body(const SsmArgs &a, const int bx, const i
     }
     const float *dt_p = a.zx + (size_t)(rowbase + threadIdx.x) * a.in_ld + a.di + a.convd + h;
     const float Aexp = expf(a.A_log[h]), dtb = a.dt_bias[h], Dh = a.D[h];
+    const float gn = TMAX == 1 && a.pk ? a.gnorm[h * a.P + p0 + warp * RPW + lane / (32 / RPW)] : 1.f;      // packed output: of this lane's column
     pdl_wait();
 
     // ---- after the wait: the state rows and the conv window (L2 hits), in flight with the sweep below
@@ -196,7 +197,7 @@ __device__ __forceinline__ void ssm_body(const SsmArgs &a, const int bx, const i
             const float z = zs[i][warp * RPW + r];
             const float out = (y + Dh * xs[i][warp * RPW + r]) * silu_f(z);
             if (TMAX == 1 && a.pk) {
-                store_split(a.pk + (size_t)lb * a.di + col, (size_t)a.pk_rows * a.di, out * a.gnorm[col]);
+                store_split(a.pk + (size_t)lb * a.di + col, (size_t)a.pk_rows * a.di, out * gn);
                 sq = out * out;
             } else a.g[(size_t)(rowbase + i) * a.di + col] = out;
         }
@@ -218,7 +219,7 @@ __device__ __forceinline__ void ssm_body(const SsmArgs &a, const int bx, const i
         sq = warp_sum(sq);
         if (lane == 0) sq_s[warp] = sq;
         __syncthreads();
-        if (threadIdx.x == 0) a.pk_ss[(size_t)(by * (a.P / SSM_PR) + bx) * a.pk_rows + lb] = (sq_s[0] + sq_s[1]) + (sq_s[2] + sq_s[3]);
+        if (threadIdx.x == 0) a.pk_ss[(size_t)lb * (a.H * (a.P / SSM_PR)) + by * (a.P / SSM_PR) + bx] = (sq_s[0] + sq_s[1]) + (sq_s[2] + sq_s[3]);
     }
 }
 
