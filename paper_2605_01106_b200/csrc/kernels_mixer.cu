@@ -14,9 +14,9 @@
 namespace {
 using namespace hsd;
 
-template <int EPL, int SSM_PR, int TMAX>
+template <int EPL, int SSM_PR, int TMAX, bool PK = false>
 __global__ void __launch_bounds__(SSM_THREADS) ssm_kernel(const SsmArgs a) {
-    ssm_body<EPL, SSM_PR, TMAX>(a, blockIdx.x, blockIdx.y, blockIdx.z);
+    ssm_body<EPL, SSM_PR, TMAX, PK>(a, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -293,15 +293,18 @@ static bool ssm_wide(const SsmArgs &a) { return a.P % 64 == 0 && (int64_t)(a.P /
 
 int ssm_blocks(const SsmArgs &a) { return a.P / (ssm_wide(a) ? 64 : 16) * a.H; }
 cudaError_t launch_ssm(const SsmArgs &a, cudaStream_t s) {
+    if (a.pk && a.T != 1) return cudaErrorInvalidValue;
     const bool wide = ssm_wide(a);
     const dim3 grid(a.P / (wide ? 64 : 16), a.H, a.nb);
 #define LAUNCH(e_, pr_, t_) launch_pdl(ssm_kernel<e_, pr_, t_>, grid, dim3(SSM_THREADS), 0, s, a)
-#define CASE(n_, e_) if (a.N == n_) return a.T == 1 ? (wide ? LAUNCH(e_, 64, 1) : LAUNCH(e_, 16, 1))               \
+#define PACKED(e_, pr_) launch_pdl(ssm_kernel<e_, pr_, 1, true>, grid, dim3(SSM_THREADS), 0, s, a)
+#define CASE(n_, e_) if (a.N == n_) return a.pk ? (wide ? PACKED(e_, 64) : PACKED(e_, 16)) : a.T == 1 ? (wide ? LAUNCH(e_, 64, 1) : LAUNCH(e_, 16, 1))               \
                                          : a.T <= 3 ? (wide ? LAUNCH(e_, 64, 3) : LAUNCH(e_, 16, 3))               \
                                          : a.T <= 5 ? (wide ? LAUNCH(e_, 64, 5) : LAUNCH(e_, 16, 5))               \
                                                     : (wide ? LAUNCH(e_, 64, HS_MAX_T) : LAUNCH(e_, 16, HS_MAX_T))
     CASE(64, 2); CASE(128, 4); CASE(256, 8);
 #undef CASE
+#undef PACKED
 #undef LAUNCH
     return cudaErrorInvalidValue;
 }

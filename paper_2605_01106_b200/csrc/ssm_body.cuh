@@ -18,7 +18,9 @@ constexpr int SSM_THREADS = 128; // 4 warps x PR / 4 rows
 // Instances for 1, 3, 5 and 9 positions: the unrolled loads and shared arrays of unused positions cost (verify pass at
 // k = 4 in the instance for 9 / for 5: 0.5B-class, one sequence 1.447 / 1.386 ms, 8 sequences 2.51 / 2.44; 3B-class, one
 // 3.03 / 2.96, 8 sequences 5.89 / 5.67).
-template <int EPL, int SSM_PR, int TMAX>
+// PK: the output goes out packed (SsmArgs::pk), one position only; its own instance, because the test alone costs 1 % of a round of one
+// sequence at k = 2 (0.5B-class, 2174 / 2198 us).
+template <int EPL, int SSM_PR, int TMAX, bool PK = false>
 __device__ __forceinline__ void ssm_body(const SsmArgs &a, const int bx, const int by, const int bz) {
     constexpr int N = 32 * EPL;
     constexpr int VW = EPL < 4 ? EPL : 4;       // vector width of the state loads
@@ -79,7 +81,7 @@ __device__ __forceinline__ void ssm_body(const SsmArgs &a, const int bx, const i
     }
     const float *dt_p = a.zx + (size_t)(rowbase + threadIdx.x) * a.in_ld + a.di + a.convd + h;
     const float Aexp = expf(a.A_log[h]), dtb = a.dt_bias[h], Dh = a.D[h];
-    const float gn = TMAX == 1 && a.pk ? a.gnorm[h * a.P + p0 + warp * RPW + lane / (32 / RPW)] : 1.f;      // packed output: of this lane's column
+    const float gn = PK ? a.gnorm[h * a.P + p0 + warp * RPW + lane / (32 / RPW)] : 1.f;      // packed output: of this lane's column
     pdl_wait();
 
     // ---- after the wait: the state rows and the conv window (L2 hits), in flight with the sweep below
@@ -196,7 +198,7 @@ __device__ __forceinline__ void ssm_body(const SsmArgs &a, const int bx, const i
             const int r = lane / LPV, col = h * a.P + p0 + warp * RPW + r;
             const float z = zs[i][warp * RPW + r];
             const float out = (y + Dh * xs[i][warp * RPW + r]) * silu_f(z);
-            if (TMAX == 1 && a.pk) {
+            if (PK) {
                 store_split(a.pk + (size_t)lb * a.di + col, (size_t)a.pk_rows * a.di, out * gn);
                 sq = out * out;
             } else a.g[(size_t)(rowbase + i) * a.di + col] = out;
@@ -214,7 +216,7 @@ __device__ __forceinline__ void ssm_body(const SsmArgs &a, const int bx, const i
                 else *reinterpret_cast<float2 *>(p) = make_float2(s[r][0], s[r][1]);
             }
     }
-    if (TMAX == 1 && a.pk) {
+    if (PK) {
         __shared__ float sq_s[SSM_THREADS / 32];
         sq = warp_sum(sq);
         if (lane == 0) sq_s[warp] = sq;
