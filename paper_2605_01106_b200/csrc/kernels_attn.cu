@@ -911,7 +911,7 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     };
     if (a.tiles > 0) {
         sg.kh = blockIdx.y; sg.lb = blockIdx.z; sg.b = a.b0 + sg.lb; sg.len = cache_len(sg.lb); sg.piece = blockIdx.x;
-        sg.npiece = max(1, (sg.len + CK * a.tiles - 1) / (CK * a.tiles));
+        sg.npiece = (items_of(sg.len) + a.tiles - 1) / a.tiles;
         if (sg.piece >= sg.npiece) return;             // beyond the cache
         sg.last = sg.piece == sg.npiece - 1;
         cut(sg.piece * a.tiles, (sg.piece + 1) * a.tiles);
@@ -968,7 +968,8 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     const bool last = sg.last;
     const bool valid = len >= 0 && len + T <= a.cap;
     if (!valid) {                                  // a control word out of range is never turned into an address
-        if (tid == 0 && last && kh == 0) atomicCAS(a.status, 0, len < 0 ? (int)HS_ERR_DEVICE : (int)HS_ERR_CAPACITY);
+        // reported by piece 0, which every launch has (a length beyond the ranges of the grid has no CTA for its last piece)
+        if (tid == 0 && sg.piece == 0 && kh == 0) atomicCAS(a.status, 0, len < 0 ? (int)HS_ERR_DEVICE : (int)HS_ERR_CAPACITY);
         if (a.tiles > 0) return;
     }
     __nv_bfloat16 *Kb = a.Kc + ((size_t)b * a.kvh + kh) * a.cap * HD;

@@ -165,6 +165,30 @@ def test_streaming_attention_in_equal_shares(env, monkeypatch, qh, ks):
     assert rep.rounds == len(ks)
 
 
+@pytest.mark.parametrize("form", ["fixed tiles", "equal shares"])
+def test_streaming_attention_control_words_out_of_range(env, form):
+    # a bad cache length of one sequence in the streaming form, with a fixed number of tiles per CTA and in equal shares (where a CTA
+    # goes on with the next cache of its share): the status word names the error however far beyond the cache the length lies - the
+    # grid has no CTA for the last range of such a cache -, guard bytes stay intact and the other sequences reproduce the oracle.
+    # (Sequence 0 of many: even an unchecked access would stay inside the cache.)
+    if form == "fixed tiles":
+        cap, lens, checked = 1500, [700, 1151, 640, 77, 1279, 128], {1, 2, 3, 4, 5}
+    else:
+        cap, lens, checked = 1700, [1600 - 53 * (b % 29) for b in range(100)], {1, 2, 50, 99}
+    s, eng, model, seqs = make(env, "test_seq", len(lens), 4, cap, checked, lens)
+    if form == "fixed tiles":
+        eng.set_attn_geometry(128, -2)
+    rep = None
+    for value, want in ((cap - 2, -3), (cap + 1000, -3), (3 * cap, -3), (-5, -7)):
+        eng.poke_control(0, eng.CTRL_KV_LEN, value)
+        forced = [hi.forced_accept(4, 1, seq=b - want) for b in range(len(lens))]
+        rep = env["harness"].run_rounds(eng, seqs, s, 4, 1, forced=forced, rep=rep)
+        assert eng.device_status() == want, value
+        eng.clear_status()
+    print(rep)
+    assert rep.rounds == 4
+
+
 def test_streaming_attention_batched_parallel_hybrid(env):
     # a batch large enough that the verify attention of the parallel hybrid runs as its own launch in the streaming form
     # (chosen automatically); three sequences carry their context on both sides, the others run beside them
