@@ -104,6 +104,10 @@ __device__ __forceinline__ void attn_body(const AttnArgs &a, const int split, co
 
     // ---- before the wait: kv_len, the first cached tile, the RoPE rows
     const int len = __ldcg(a.kv_len + b) + a.len_off;
+    if (len < 0 || len > a.cap - T) {             // never read or write outside the cache; the host reports the status word
+        if (tid == 0 && split == 0 && kh == 0) atomicCAS(a.status, 0, len < 0 ? (int)HS_ERR_DEVICE : (int)HS_ERR_CAPACITY);
+        return;
+    }
     const int SPAN = CK * a.tiles;                // cached keys per CTA
     const int nsplit = max(1, (len + SPAN - 1) / SPAN);
     cg::cluster_group cluster = cg::this_cluster();
@@ -114,10 +118,6 @@ __device__ __forceinline__ void attn_body(const AttnArgs &a, const int split, co
     const bool last = split == nsplit - 1;
     const int c0 = split * SPAN, rc = max(0, min(len, c0 + SPAN) - c0);
     const int ntile = last ? max(1, (rc + CK - 1) / CK) : (rc + CK - 1) / CK;
-    if (len < 0 || len + T > a.cap) {             // never read or write outside the cache; the host reports the status word
-        if (tid == 0 && split == 0 && kh == 0) atomicCAS(a.status, 0, len < 0 ? (int)HS_ERR_DEVICE : (int)HS_ERR_CAPACITY);
-        return;
-    }
     __nv_bfloat16 *Kb = a.Kc + ((size_t)b * a.kvh + kh) * a.cap * HD;
     __nv_bfloat16 *Vb = a.Vc + ((size_t)b * a.kvh + kh) * a.cap * HD;
     // asynchronous copy of the cached rows of tile t (one commit group per call, possibly empty)
@@ -543,9 +543,10 @@ __device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int spl
 
     // ---- before the wait: kv_len, the whole key range of this CTA, the RoPE rows
     const int len = __ldcg(a.kv_len + b) + a.len_off;
-    const int nsplit = max(1, (len + CK - 1) / CK);
-    if (len < 0 || len + T > a.cap || nsplit > AT_CL) {      // never write past the cache; a cache longer than the host's bound is a host error
-        if (tid == 0 && split == 0 && khq == 0) atomicCAS(a.status, 0, (len >= 0 && len + T > a.cap) ? (int)HS_ERR_CAPACITY : (int)HS_ERR_DEVICE);
+    const bool fits = len >= 0 && len <= a.cap - T;
+    const int nsplit = fits ? max(1, (len + CK - 1) / CK) : 0;
+    if (!fits || nsplit > AT_CL) {                // never write past the cache; a cache longer than the host's bound is a host error
+        if (tid == 0 && split == 0 && khq == 0) atomicCAS(a.status, 0, len > a.cap - T ? (int)HS_ERR_CAPACITY : (int)HS_ERR_DEVICE);
         return;
     }
     const int crank = split;                      // the grid has exactly one cluster along x
@@ -966,7 +967,7 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     for (bool opening = true;; opening = false) {
     const int b = sg.b, kh = sg.kh, len = sg.len, rc = sg.rc, ntile = sg.ntile, nitem = sg.nitem;
     const bool last = sg.last;
-    const bool valid = len >= 0 && len + T <= a.cap;
+    const bool valid = len >= 0 && len <= a.cap - T;      // (no sum with a length that may be anything)
     if (!valid) {                                  // a control word out of range is never turned into an address
         // reported by piece 0, which every launch has (a length beyond the ranges of the grid has no CTA for its last piece)
         if (tid == 0 && sg.piece == 0 && kh == 0) atomicCAS(a.status, 0, len < 0 ? (int)HS_ERR_DEVICE : (int)HS_ERR_CAPACITY);

@@ -754,7 +754,7 @@ __device__ __forceinline__ void pf_attn_body(const PfAttnArgs &a, unsigned char 
     const int q0 = qt * PA_Q;
     if (q0 >= n) return;
     const int base = __ldcg(a.kv_len + b);
-    if (base < 0 || base + n > a.cap) return;        // reported by pf_prep_kernel
+    if (base < 0 || base > a.cap - n) return;        // reported by pf_prep_kernel
     const int kh = h / (a.qh / a.kvh), ld = a.qh * HD;
     const __nv_bfloat16 *Kb = a.Kc + ((size_t)b * a.kvh + kh) * a.cap * HD, *Vb = a.Vc + ((size_t)b * a.kvh + kh) * a.cap * HD;
     const int nkeys = base + min(n, q0 + PA_Q), ntile = (nkeys + PA_K - 1) / PA_K;

@@ -179,14 +179,29 @@ def test_streaming_attention_control_words_out_of_range(env, form):
     if form == "fixed tiles":
         eng.set_attn_geometry(128, -2)
     rep = None
-    for value, want in ((cap - 2, -3), (cap + 1000, -3), (3 * cap, -3), (-5, -7)):
+    for value, want in ((cap - 2, -3), (cap + 1000, -3), (3 * cap, -3), (2 ** 31 - 3, -3), (-5, -7)):
         eng.poke_control(0, eng.CTRL_KV_LEN, value)
         forced = [hi.forced_accept(4, 1, seq=b - want) for b in range(len(lens))]
         rep = env["harness"].run_rounds(eng, seqs, s, 4, 1, forced=forced, rep=rep)
         assert eng.device_status() == want, value
         eng.clear_status()
     print(rep)
-    assert rep.rounds == 4
+    assert rep.rounds == 5
+
+
+@pytest.mark.parametrize("name,geometry", [("test_seq", (0, 0)), ("test_seq", (64, 4)), ("cfg1_tiny", (0, 0)), ("cfg1_tiny", (64, 4))])
+def test_control_words_near_the_integer_limit(env, name, geometry):
+    # a cache length to which nothing can be added: reported, not used, in the lean and the general form, alone and beside a mixer
+    lens = [200, 333, 77]
+    s, eng, model, seqs = make(env, name, len(lens), 4, 512, {1, 2}, lens)
+    eng.set_attn_geometry(*geometry)
+    rep = None
+    for value in (2 ** 31 - 1, 2 ** 31 - 4):
+        eng.poke_control(0, eng.CTRL_KV_LEN, value)
+        rep = env["harness"].run_rounds(eng, seqs, s, 4, 1, forced=[hi.forced_accept(4, 1, seq=b) for b in range(len(lens))], rep=rep)
+        assert eng.device_status() == -3, value
+        eng.clear_status()
+    assert rep.rounds == 2
 
 
 def test_streaming_attention_batched_parallel_hybrid(env):
