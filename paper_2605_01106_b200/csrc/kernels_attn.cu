@@ -834,7 +834,7 @@ __host__ __device__ inline Attn2Layout attn2_layout(int hd, int mt) {
     size_t o = 0;                          // offsets from the first 1024-byte boundary of the dynamic shared memory
     L.tile_off = o; o += 2 * A2_NBUF * L.tile_bytes;               // K0 V0 K1 V1 K2 V2; later the warp partials
     L.q_off = o; o += (size_t)2 * mt * 16 * L.kstr * 2;            // bf16 head | remainder
-    L.new_off = o; o += (size_t)2 * 16 * L.kstr * 2;               // the new K | V rows as they are cached: a 16-key group of their own
+    L.new_off = o; o += (size_t)2 * 16 * hd * 2;                   // the new K | V rows as they are cached: a tile of 16 keys of their own
     L.rope_off = o; o += (size_t)HS_MAX_T * (hd / 2) * 8;
     L.ml_off = o; o += (size_t)(2 * A2_KW + mt) * 16 * 2 * 4;      // per warp (max, sum) per row, then the merged pairs
     L.total = (o + 127) / 128 * 128 + 1024;
@@ -868,8 +868,7 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     auto Vbuf = [&](int i) { return tile_s + (size_t)(2 * i + 1) * L.tile_bytes; };
     __nv_bfloat16 *Qh_s = reinterpret_cast<__nv_bfloat16 *>(sm + L.q_off);        // [GTB][KSTR]
     __nv_bfloat16 *Ql_s = Qh_s + (size_t)GTB * KSTR;
-    __nv_bfloat16 *Kn_s = reinterpret_cast<__nv_bfloat16 *>(sm + L.new_off);      // [16][KSTR]
-    __nv_bfloat16 *Vn_s = Kn_s + (size_t)16 * KSTR;
+    unsigned char *new_s = sm + L.new_off;                                        // K, then V: [HD / 64][16][64], chunks swizzled as in a tile
     float2 *rope_s = reinterpret_cast<float2 *>(sm + L.rope_off);
     float *wml_s = reinterpret_cast<float *>(sm + L.ml_off);                      // [NPART][GTB][2], then the merged pairs
     __shared__ int ticket_s;
@@ -989,13 +988,11 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
         *reinterpret_cast<uint4 *>(Ql_s + (size_t)r * KSTR + 8 * c) = make_uint4(0, 0, 0, 0);
     }
 #pragma unroll 1
-    for (int idx = tid; idx < 16 * (HD / 8); idx += A2_THREADS) {              // finite V rows behind the new ones
-        const int r = idx / (HD / 8), c = idx % (HD / 8);
-        *reinterpret_cast<uint4 *>(Vn_s + (size_t)r * KSTR + 8 * c) = make_uint4(0, 0, 0, 0);
-    }
+    for (int idx = tid; idx < 16 * (HD / 8); idx += A2_THREADS)                // finite V rows behind the new ones
+        *reinterpret_cast<uint4 *>(new_s + 16 * RB + idx * 16) = make_uint4(0, 0, 0, 0);
     }
     if (opening) pdl_wait();
-    __syncthreads();                        // rope_s complete, Vn_s cleared
+    __syncthreads();                        // rope_s complete, new V rows cleared
     if (valid) {
 
     // ---- queries (RoPE, scale, bf16 head + remainder) and, in the last range, the new K / V rows
@@ -1044,8 +1041,10 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
             const __nv_bfloat16 k1 = __float2bfloat16_rn(x1 * cs.x + x0 * cs.y);
             const __nv_bfloat16 v0 = __float2bfloat16_rn(__ldcg(row + a.v_off + kh * HD + e));
             const __nv_bfloat16 v1 = __float2bfloat16_rn(__ldcg(row + a.v_off + kh * HD + e + HD / 2));
-            Kn_s[i * KSTR + e] = k0; Kn_s[i * KSTR + e + HD / 2] = k1;
-            Vn_s[i * KSTR + e] = v0; Vn_s[i * KSTR + e + HD / 2] = v1;
+            auto at = [&](int col) { return new_s + (col >> 6) * (16 * 128) + i * 128 + ((((col >> 3) & 7) ^ (i & 7)) << 4) + (col & 7) * 2; };
+            unsigned char *lo = at(e), *hi = at(e + HD / 2);
+            *reinterpret_cast<__nv_bfloat16 *>(lo) = k0; *reinterpret_cast<__nv_bfloat16 *>(hi) = k1;
+            *reinterpret_cast<__nv_bfloat16 *>(lo + 16 * RB) = v0; *reinterpret_cast<__nv_bfloat16 *>(hi + 16 * RB) = v1;
             Kb[(size_t)(len + i) * HD + e] = k0; Kb[(size_t)(len + i) * HD + e + HD / 2] = k1;
             Vb[(size_t)(len + i) * HD + e] = v0; Vb[(size_t)(len + i) * HD + e + HD / 2] = v1;
         }
@@ -1054,9 +1053,9 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
 
     const int g8 = lane >> 2, t4 = lane & 3, grp = warp >> 3, kw = warp & 7;
     const int q0 = MT == 2 ? grp * 16 : 0;                                   // first row of this warp's query tile
-    float O[NT][4];
+    float O[NT][4];                         // pairs of columns of rows g8 and g8 + 8 (packed: row g8 only)
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt) { O[nt][0] = O[nt][1] = O[nt][2] = O[nt][3] = 0.f; }
+    for (int nt = 0; nt < NT; ++nt) O[nt][0] = O[nt][1] = O[nt][2] = O[nt][3] = 0.f;
     float m_run[2], l_run[2];
     int ti[2];                              // position index of each of this lane's rows among the T new ones
 #pragma unroll
@@ -1066,8 +1065,12 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
         ti[r] = row - (int)((row * tinv) >> 16) * T;
     }
 
-    // An item is a tile of cached keys (a buffer of the ring, swizzled rows of RB bytes) or, last, the new rows (their own
-    // padded buffer): the same code serves both, told apart by base address, row pitch and swizzle mask.
+    // An item is a tile of cached keys (a buffer of the ring) or, last, the new rows (a tile of 16 keys): the same code serves both,
+    // told apart by base address and distance of the halves.  This lane's address in a row of 128 bytes, chunk c of it being
+    // address ^ 16 c: shared-space addresses of 32 bits, because registers are what this loop is short of.
+    const uint32_t q_at = smem_u32(Qh_s) + (uint32_t)((q0 + (lane & 7) + ((lane >> 3) & 1) * 8) * KSTR * 2 + (lane >> 4) * 16);
+    const uint32_t k_at = (uint32_t)(((lane & 7) + (lane >> 4) * 8) * 128 + ((((lane >> 3) & 1) ^ (lane & 7)) << 4));
+    const uint32_t v_at = (uint32_t)(((lane & 7) + ((lane >> 3) & 1) * 8) * 128 + (((lane >> 4) ^ (lane & 7)) << 4));
     auto walk = [&](auto packed_) {
     constexpr bool packed = decltype(packed_)::value;
 #pragma unroll 1
@@ -1093,13 +1096,10 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
                 __syncwarp();
             }
         }
-        const unsigned char *K_s = newrows ? reinterpret_cast<const unsigned char *>(Kn_s) : Kbuf(buf);
-        const unsigned char *V_s = newrows ? reinterpret_cast<const unsigned char *>(Vn_s) : Vbuf(buf);
-        // a tile: rows of 128 bytes per half, 16-byte chunks XOR-swizzled with the row; the new rows: padded rows, no swizzle
-        const int pitch = newrows ? KSTR * 2 : 128, swz = newrows ? 0 : 7, hstr = newrows ? 128 : HS_;
         // 16 keys per warp; the new rows are one group, given to the warp that a ragged last tile leaves idle most often
         const int kb = newrows ? (kw == A2_KW - 1 ? 0 : nkp) : kw * 16;
         if (kb < nkp) {
+            const uint32_t keys = (newrows ? smem_u32(new_s) : smem_u32(Kbuf(buf))) + (uint32_t)kb * 128, hstr = newrows ? 16 * 128 : HS_;
             // ---- scores of this warp's 16 keys (two accumulator sets: head and remainder products)
             float S[2][4];
             {
@@ -1108,21 +1108,17 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
                 for (int c = 0; c < 2; ++c)
 #pragma unroll
                     for (int nt = 0; nt < 2; ++nt) { Sp[c][nt][0] = Sp[c][nt][1] = Sp[c][nt][2] = Sp[c][nt][3] = 0.f; }
-                const int krow = kb + (lane & 7) + (lane >> 4) * 8;
-                const unsigned char *krp = K_s + (size_t)krow * pitch;
-                const int ksw = krow & swz, kc0 = (lane >> 3) & 1;
 #pragma unroll
                 for (int ks = 0; ks < HD / 16; ++ks) {
                     uint32_t bk[4], ah[4];
-                    ldsm_x4(bk, krp + ((ks * 2 + kc0) >> 3) * hstr + (((((ks * 2 + kc0) & 7)) ^ ksw) << 4));
-                    const size_t qo = (size_t)(q0 + (lane & 7) + ((lane >> 3) & 1) * 8) * KSTR + ks * 16 + (lane >> 4) * 8;
-                    ldsm_x4(ah, Qh_s + qo);
+                    ldsm_x4(bk, ((keys + k_at) ^ (uint32_t)((ks & 3) * 32)) + (ks >> 2) * hstr);
+                    ldsm_x4(ah, q_at + ks * 32);
                     // (packed: one accumulator set for even k steps, one for odd ones)
                     const int c = packed ? ks & 1 : 0;
                     mma_bf16(Sp[c][0], ah, bk[0], bk[1]); mma_bf16(Sp[c][1], ah, bk[2], bk[3]);
                     if (!packed) {
                         uint32_t al[4];
-                        ldsm_x4(al, Ql_s + qo);
+                        ldsm_x4(al, q_at + (uint32_t)(GTB * (HD + 8) * 2) + ks * 32);
                         mma_bf16(Sp[1][0], al, bk[0], bk[1]); mma_bf16(Sp[1][1], al, bk[2], bk[3]);
                     }
                 }
@@ -1173,22 +1169,33 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
                 }
                 l_run[r] = fmaf(l_run[r], corr[r], sum);
             }
-            // the accumulators are rescaled only when some row's running maximum moved (rare after the first tiles)
-            if (__any_sync(0xffffffffu, corr[0] != 1.f || corr[1] != 1.f)) {
+            // ---- partial output = partial output * correction + P V over the whole head dimension.  A tile's products add up in
+            // accumulators of their own (the tensor path truncates every sum it adds to, and a share may be hundreds of tiles: 250
+            // in one chain left the output short by 1.5e-5 of itself, 16 by 4e-7, so 1e-7).  One pair of column groups is added
+            // while the next one's MMAs run.
+            const uint32_t vals = keys + v_at + (newrows ? 16 * RB : CK * RB);
+            float D[2][2][4];
+            auto add = [&](int p) {
 #pragma unroll
-                for (int nt = 0; nt < NT; ++nt) { O[nt][0] *= corr[0]; O[nt][1] *= corr[0]; O[nt][2] *= corr[1]; O[nt][3] *= corr[1]; }
-            }
-            // ---- partial output += P V over the whole head dimension
-            const int vrow = kb + (lane & 7) + ((lane >> 3) & 1) * 8;
-            const unsigned char *vrp = V_s + (size_t)vrow * pitch;
-            const int vsw = vrow & swz, vc0 = lane >> 4;
+                for (int u = 0; u < 2; ++u) {
+                    float (&o)[4] = O[2 * p + u], (&d)[4] = D[p & 1][u];
+                    if (packed) { o[0] = fmaf(o[0], corr[0], d[0] + d[2]); o[1] = fmaf(o[1], corr[0], d[1] + d[3]); }      // head + remainder
+                    else
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) o[e] = fmaf(o[e], corr[e >> 1], d[e]);
+                }
+            };
 #pragma unroll
             for (int p = 0; p < NT / 2; ++p) {
                 uint32_t bv[4];
-                ldsm_x4_t(bv, vrp + ((p * 2 + vc0) >> 3) * hstr + ((((p * 2 + vc0) & 7) ^ vsw) << 4));
-                mma_bf16(O[2 * p], ph, bv[0], bv[1]); mma_bf16(O[2 * p + 1], ph, bv[2], bv[3]);
-                if (!packed) { mma_bf16(O[2 * p], pl, bv[0], bv[1]); mma_bf16(O[2 * p + 1], pl, bv[2], bv[3]); }
+                ldsm_x4_t(bv, (vals ^ (uint32_t)((p & 3) * 32)) + (p >> 2) * hstr);
+                float (&d0)[4] = D[p & 1][0], (&d1)[4] = D[p & 1][1];
+                d0[0] = d0[1] = d0[2] = d0[3] = d1[0] = d1[1] = d1[2] = d1[3] = 0.f;
+                mma_bf16(d0, ph, bv[0], bv[1]); mma_bf16(d1, ph, bv[2], bv[3]);
+                if (!packed) { mma_bf16(d0, pl, bv[0], bv[1]); mma_bf16(d1, pl, bv[2], bv[3]); }
+                if (p) add(p - 1);
             }
+            add(NT / 2 - 1);
         }
         if (!newrows) {
             // this warp is done with tile t: the last of those that read it refills the buffer pair with tile t + 3
@@ -1208,9 +1215,6 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     // ---- merge the warp partials through shared memory (the tile buffers are free now)
     float *wo_s = reinterpret_cast<float *>(sm + L.tile_off);            // [NPART][GTB][HD]
     const int part = MT == 2 ? kw : warp;
-    if (packed)                             // head and remainder halves of the packed tile's outputs
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) { O[nt][0] += O[nt][2]; O[nt][1] += O[nt][3]; }
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         if (packed && r == 1) continue;

@@ -189,6 +189,61 @@ def test_streaming_attention_control_words_out_of_range(env, form):
     assert rep.rounds == 5
 
 
+@pytest.mark.parametrize("qh,k", [(8, 4), (4, 4), (4, 1)])
+def test_streaming_attention_long_shares_stay_exact(env, qh, k):
+    # 250 tiles of 128 keys per CTA (equal shares), every cached V row of a KV head the same: whatever the probabilities are, the
+    # attention's output is that row.  The tensor path truncates when it adds to an accumulator (2^-26 of the sum per MMA on
+    # average), so a chain over a whole share would leave the output short by 2e-6 to 4e-6.  A tile's products in accumulators of
+    # their own lose at most 2 * 2^-26; the out-projection's factor for its own chain of 8 MMAs adds 8 * 2^-26 here, where a sum has
+    # one term: below 2e-7 together, 5e-7 allowed.  One-layer model: Mamba branch and MLP zero, W_o and the LM head copy, the
+    # last 256 dimensions carry the embedding (1), by which the logits are divided to take the final norm out.
+    torch = env["torch"]
+    hd, kvh, batch, T = 64, 2, 9, k + 1
+    n_o, n = qh * hd, 2056 * 128
+    d = n_o + 256
+    s = hi.CONFIGS["cfg1_tiny"].replace(L=1, d=d, V=d, qh=qh, kvh=kvh, hd=hd, ff=256)
+    table, nbytes = hi.blob_layout(s)
+    blob = np.zeros(nbytes, np.uint8)
+    rng = np.random.default_rng(5)
+
+    def put(layer, tid, a):
+        off, dims, dt = table[(layer, tid)]
+        assert a.shape == tuple(dims)
+        a = torch.from_numpy(np.ascontiguousarray(a, np.float32))
+        a = a.to(torch.bfloat16).view(torch.uint8).numpy() if dt == "bf16" else a.numpy().view(np.uint8)
+        blob[off:off + a.nbytes] = a.reshape(-1)
+
+    c = torch.from_numpy(rng.uniform(0.5, 1.5, (kvh, hd)).astype(np.float32)).to(torch.bfloat16)
+    eye = np.eye(d, dtype=np.float32)
+    put(-1, hi.G_EMBED, np.concatenate([np.zeros((d, n_o)), np.ones((d, 256))], 1))
+    put(-1, hi.G_LM_HEAD, eye)
+    put(-1, hi.G_FINAL_NORM, np.ones(d))
+    put(0, hi.T_NORM1, np.full(d, np.sqrt(256 / d + s.eps)))
+    put(0, hi.T_NORM2, np.ones(d)); put(0, hi.T_GNORM, np.ones(s.d_inner))
+    w = np.zeros(table[(0, hi.T_W_IN)][1], np.float32)
+    q0 = w.shape[0] - (qh + 2 * kvh) * hd
+    w[q0:q0 + n_o, n_o:] = rng.normal(0.0, 0.07, (n_o, 256))
+    w[q0 + n_o + kvh * hd:, n_o] = c.float().numpy().reshape(-1)
+    put(0, hi.T_W_IN, w)
+    put(0, hi.T_W_O, eye[:, :n_o])
+    eng = env["hs"].Engine(s, blob, max_batch=batch, max_k=k, kv_capacity=n + 16)
+    kv = eng.t_kv[:2 * 2 * batch * kvh * (n + 16) * hd].view(torch.bfloat16).view(2, batch, kvh, n + 16, hd)
+    kv[0].normal_(generator=torch.Generator(device=eng.device).manual_seed(7))
+    kv[1].copy_(c.to(eng.device)[None, :, None, :].expand(batch, kvh, n + 16, hd))
+    for b in range(batch):
+        eng.set_context(b, n, 1)
+    eng.set_batch(batch)
+    eng.verify(k, torch.ones((batch, T), dtype=torch.int32, device=eng.device))
+    lg = eng.get_logits(batch * T).astype(np.float64)
+    assert eng.device_status() == 0 and eng.check_guards()
+    o = lg[:, :n_o] / lg[:, n_o:].mean(1, keepdims=True)
+    want = c.double().numpy()[np.arange(qh) // (qh // kvh)].reshape(1, n_o)
+    err = (o / want - 1).reshape(batch, T, qh, hd)
+    print("shortfall of the output: mean %.2e, by head %s" % (-err.mean(), -err.mean((0, 1, 3))))
+    assert abs(err.mean()) <= 5e-7 and np.abs(err.mean((0, 1, 3))).max() <= 5e-7
+    assert np.abs(err).max() <= 2.0 ** -14              # operands as bf16 head and remainder: 2^-17 each
+
+
 @pytest.mark.parametrize("name,geometry", [("test_seq", (0, 0)), ("test_seq", (64, 4)), ("cfg1_tiny", (0, 0)), ("cfg1_tiny", (64, 4))])
 def test_control_words_near_the_integer_limit(env, name, geometry):
     # a cache length to which nothing can be added: reported, not used, in the lean and the general form, alone and beside a mixer
