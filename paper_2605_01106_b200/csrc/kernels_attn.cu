@@ -821,7 +821,11 @@ __device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int spl
 // group has one of them, with one the groups take the tiles of keys in turn.  (Eight warps with both query tiles held 242
 // registers a thread, two warps on a scheduler, and waited for their own operands most of the time: 178 us per launch on the batch-64
 // workload at k = 4.)
-constexpr int A2_THREADS = 512, A2_KW = 8, A2_CK = 128, A2_NBUF = 3;
+constexpr int A2_KW = 8, A2_CK = 128, A2_NBUF = 3;
+// A packed query tile alone (1..8 rows) is served by one group of eight warps: half the instructions a tile, and half as many partial
+// results to merge where a CTA has one or two tiles (0.5B-class, k = 0, sixteen / eight warps: one sequence of 9000 keys 22.4 / 20.5
+// us per launch, three of 2500 at k = 1 16.9 / 14.9, 64 of 4368 .. 16166 124.4 / 123.3).
+__host__ __device__ constexpr int a2_threads(int mt, bool pk) { return mt == 1 && pk ? 256 : 512; }
 
 // Tile buffers hold 128 keys x HD bf16 without padding; the 16-byte chunk c of row r sits at chunk position
 // c ^ (r & 7), which keeps the eight rows of an ldmatrix 8x8 block on different banks.  Three K and three V buffers:
@@ -854,11 +858,12 @@ __device__ __forceinline__ void tma_tile_2d(void *dst_smem, const CUtensorMap *m
 // operand, remainders rows 8-15), so that tile costs half the tensor instructions of a full one.  It serves 1..8 query
 // rows (MT = 1) and 17..24 (MT = 2: 20 rows at four query heads per KV head and k = 4).
 template <int HD, int MT, bool PK>
-__global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_constant__ AttnArgs a) {
+__global__ void __launch_bounds__(a2_threads(MT, PK), 1) attn2_kernel(const __grid_constant__ AttnArgs a) {
     extern __shared__ __align__(1024) unsigned char smraw[];
     constexpr int CK = A2_CK, GTB = MT * 16, NT = HD / 8, RB = HD * 2;       // RB: bytes of a tile row
     constexpr int PB = (MT - 1) * 16;                                        // first row of the packed tile
-    constexpr int NPART = 2 * A2_KW / MT;                                    // partial results per query row
+    constexpr int THREADS = a2_threads(MT, PK), NW = THREADS / 32, TURNS = NW / A2_KW / MT;     // TURNS: groups that take the tiles of keys in turn
+    constexpr int NPART = NW / MT;                                           // partial results per query row
     const int G = a.qh / a.kvh, T = a.T, GT = G * T;
     const Attn2Layout L = attn2_layout(HD, MT);
     const int KSTR = L.kstr;
@@ -872,7 +877,7 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     float2 *rope_s = reinterpret_cast<float2 *>(sm + L.rope_off);
     float *wml_s = reinterpret_cast<float *>(sm + L.ml_off);                      // [NPART][GTB][2], then the merged pairs
     __shared__ int ticket_s;
-    __shared__ int scan_s[A2_THREADS / 32], at_s[2];
+    __shared__ int scan_s[NW], at_s[2];
     // bytes of K and V landed: tile t on barrier t % 6.  (Two per buffer pair: with MT = 1 successive tiles of a pair belong to different
     // groups, and a warp must not take the phase of a tile that it skips for that of the one it waits for.)
     __shared__ __align__(8) uint64_t tile_bar[2 * A2_NBUF];
@@ -917,7 +922,7 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
         cut(sg.piece * a.tiles, (sg.piece + 1) * a.tiles);
     } else {
         // items before every sequence: a scan over the block, each thread with its part of the sequences
-        const int per = (a.nb + A2_THREADS - 1) / A2_THREADS, lo = min(a.nb, tid * per), hi = min(a.nb, lo + per);
+        const int per = (a.nb + THREADS - 1) / THREADS, lo = min(a.nb, tid * per), hi = min(a.nb, lo + per);
         int mine = 0;
         for (int lb = lo; lb < hi; ++lb) mine += items_of(cache_len(lb)) * a.kvh;
         int inc = mine;
@@ -926,7 +931,7 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
         if (lane == 31) scan_s[warp] = inc;
         __syncthreads();
         int before = inc - mine;
-        for (int w = 0; w < A2_THREADS / 32; ++w) { if (w < warp) before += scan_s[w]; total += scan_s[w]; }
+        for (int w = 0; w < NW; ++w) { if (w < warp) before += scan_s[w]; total += scan_s[w]; }
         ncta = min((int)gridDim.x, total);
         if ((int)blockIdx.x >= ncta) return;
         u = share_start(blockIdx.x); u_end = share_start(blockIdx.x + 1);
@@ -977,18 +982,18 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     if (valid) {
     if (tid == 0) { fetch(0); fetch(1); fetch(2); }
 #pragma unroll 1
-    for (int idx = tid; idx < T * (HD / 2); idx += A2_THREADS) {
+    for (int idx = tid; idx < T * (HD / 2); idx += THREADS) {
         const int i = idx / (HD / 2), e = idx - i * (HD / 2);
         rope_s[idx] = a.rope[(size_t)(len + i) * (HD / 2) + e];
     }
 #pragma unroll 1
-    for (int idx = tid; idx < (GTB - GT) * (HD / 8); idx += A2_THREADS) {      // query rows that do not exist are zero
+    for (int idx = tid; idx < (GTB - GT) * (HD / 8); idx += THREADS) {      // query rows that do not exist are zero
         const int r = GT + idx / (HD / 8), c = idx % (HD / 8);
         *reinterpret_cast<uint4 *>(Qh_s + (size_t)r * KSTR + 8 * c) = make_uint4(0, 0, 0, 0);
         *reinterpret_cast<uint4 *>(Ql_s + (size_t)r * KSTR + 8 * c) = make_uint4(0, 0, 0, 0);
     }
 #pragma unroll 1
-    for (int idx = tid; idx < 16 * (HD / 8); idx += A2_THREADS)                // finite V rows behind the new ones
+    for (int idx = tid; idx < 16 * (HD / 8); idx += THREADS)                // finite V rows behind the new ones
         *reinterpret_cast<uint4 *>(new_s + 16 * RB + idx * 16) = make_uint4(0, 0, 0, 0);
     }
     if (opening) pdl_wait();
@@ -999,7 +1004,7 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     const int rowbase = sg.lb * T;
     const float scale = rsqrtf((float)HD);
     {
-        constexpr int HP = HD / 2, NH = A2_THREADS / HP;
+        constexpr int HP = HD / 2, NH = THREADS / HP;
         const int e = tid % HP, part = tid / HP;
 #pragma unroll 1
         for (int q0 = part; q0 < GT; q0 += 4 * NH) {
@@ -1032,7 +1037,7 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     }
     if (last) {
 #pragma unroll 1
-        for (int idx = tid; idx < T * (HD / 2); idx += A2_THREADS) {
+        for (int idx = tid; idx < T * (HD / 2); idx += THREADS) {
             const int i = idx / (HD / 2), e = idx - i * (HD / 2);
             const float *row = a.zx + (size_t)(rowbase + i) * a.in_ld;
             const float2 cs = rope_s[idx];
@@ -1074,7 +1079,7 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     auto walk = [&](auto packed_) {
     constexpr bool packed = decltype(packed_)::value;
 #pragma unroll 1
-    for (int t = MT == 2 ? 0 : grp ^ (sq & 1); t < nitem; t += MT == 2 ? 1 : 2) {
+    for (int t = TURNS == 1 ? 0 : grp ^ (sq & 1); t < nitem; t += TURNS) {
         const bool newrows = t >= ntile;
         const int buf = (sq + t) % A2_NBUF;
         const int nkeys = newrows ? T : min(CK, rc - t * CK);
@@ -1233,7 +1238,7 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     float *mrg_s = wml_s + (size_t)NPART * GTB * 2;                          // [GTB][2] merged (M, den)
     constexpr int DV4 = HD / 4;
 #pragma unroll 1
-    for (int idx = tid; idx < GT * DV4; idx += A2_THREADS) {
+    for (int idx = tid; idx < GT * DV4; idx += THREADS) {
         const int qi = idx / DV4, d = (idx - qi * DV4) * 4;
         float M = -INFINITY;
 #pragma unroll
@@ -1273,7 +1278,7 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     const size_t pbase = ((size_t)b * a.kvh + kh) * a.nch;
     const float *pa0 = a.part_acc + pbase * HS_MAX_GT * HD;
     const float *pm0 = a.part_ml + pbase * HS_MAX_GT * 2;
-    for (int qi = warp; qi < GT; qi += A2_THREADS / 32) {
+    for (int qi = warp; qi < GT; qi += NW) {
         float M = -INFINITY;
         for (int c = lane; c < nsplit; c += 32) M = fmaxf(M, __ldcg(pm0 + ((size_t)c * HS_MAX_GT + qi) * 2));
         M = warp_max(M);
@@ -1287,7 +1292,7 @@ __global__ void __launch_bounds__(A2_THREADS, 1) attn2_kernel(const __grid_const
     }
     __syncthreads();
 #pragma unroll 1
-    for (int idx = tid; idx < GT * DV4; idx += A2_THREADS) {
+    for (int idx = tid; idx < GT * DV4; idx += THREADS) {
         const int qi = idx / DV4, d = (idx - qi * DV4) * 4;
         const float M = mrg_s[2 * qi];
         float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1325,7 +1330,7 @@ cudaError_t launch_attn2_t(const AttnArgs &a, cudaStream_t s) {
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    return launch_pdl(attn2_kernel<HD, MT, PK>, a.tiles > 0 ? dim3(a.nch, a.kvh, a.nb) : dim3(148), dim3(A2_THREADS), smem, s, a);
+    return launch_pdl(attn2_kernel<HD, MT, PK>, a.tiles > 0 ? dim3(a.nch, a.kvh, a.nb) : dim3(148), dim3(a2_threads(MT, PK)), smem, s, a);
 }
 
 template <int HD, int MT>
