@@ -233,7 +233,8 @@ double gemv_bytes(const GemvArgs &a) {
 struct AttnGeom {
     int chunk, tiles, small, stream;
     bool fuse;                   // verify pass of a parallel block: mixer and attention in one launch
-    int code() const { return fuse * 4096 + stream * 2048 + small * 1024 + (chunk / 16 - 1) * 32 + tiles - 1; }   // < 8192, part of the graph key
+    int warps = 16;              // streaming form, one tile of query rows: warps per CTA
+    int code() const { return (warps == 16) * 8192 + fuse * 4096 + stream * 2048 + small * 1024 + (chunk / 16 - 1) * 32 + tiles - 1; }   // < 16384, part of the graph key
 };
 // Tq: query positions per sequence of the launch; T: rows the pass may append beyond the upper bound of kv_len
 // (the same for a verify pass; a draft that keeps attention appends one row per step, k in all)
@@ -250,10 +251,26 @@ AttnGeom attn_geom(const hs_model *m, int Tq, int T, int b0, int nb) {
     // 2: 1.32 / 1.54 / 1.63 against 1.22 / 1.43 / 1.49 ms.
     const int64_t mixers = (int64_t)(c.P / 16) * c.H * nb;
     const bool few = c.arch == HS_ARCH_PARALLEL && mixers <= 4 * 148;
-    if (m->att_force_chunk) return AttnGeom{m->att_force_chunk, m->att_force_tiles < 0 ? -m->att_force_tiles : m->att_force_tiles, 0, m->att_force_tiles < 0 ? 1 : 0, few};
     int maxlen = 0;
     for (int b = b0; b < b0 + nb; ++b) if (m->kv_upper[b] > maxlen) maxlen = m->kv_upper[b];
     const int groups = c.qh / c.kvh * Tq;            // query rows per KV head
+    // Warps of a streaming CTA that has one tile of query rows (two tiles: sixteen, eight for each).  Eight: a second group of eight
+    // runs short of registers with a full tile (9 .. 16 rows), and adds partial results to merge.  It pays with a packed tile (up to
+    // 8 rows) in equal shares and where 64-wide heads leave a CTA with a whole cache waiting for its own instructions; with a full tile
+    // where a cache is cut into many ranges, whose merge more threads finish sooner.  Verify pass, us per layer, 8 / 16 warps: packed
+    // 0.5B-class 64 sequences of 4368 .. 16166 keys 186.2 / 185.2, 8 of 8000 56.9 / 58.3, 40 of 1200 72.0 / 72.9, one of 9000 32.5 / 33.4,
+    // 64-wide 40 of 1500 41.3 / 38.9, 60 of 700 38.6 / 37.8, 80 of 500 41.8 / 45.4; full 64 of 4368 .. 16166 228.9 / 233.5, 30 of 700 ..
+    // 9400 122.5 / 129.9, 10 of 2500 61.2 / 63.5, one of 9000 (71 ranges) 51.0 / 46.5, two of 9000 (36) 134.5 / 132.2, two of 16000
+    // (21 ranges) 57.4 / 57.7.
+    auto stream_warps = [&](int tiles) {
+        const int ranges = tiles ? ((maxlen + 127) / 128 + tiles - 1) / tiles : 0;
+        const bool packed = groups <= 8;
+        return groups > 16 || (packed ? tiles == 0 || (c.hd == 64 && ranges == 1 && tiles >= 6) : ranges > 24) ? 16 : 8;
+    };
+    if (m->att_force_chunk) {
+        const int tiles = m->att_force_tiles < 0 ? -m->att_force_tiles : m->att_force_tiles;
+        return AttnGeom{m->att_force_chunk, tiles, 0, m->att_force_tiles < 0 ? 1 : 0, few, stream_warps(tiles)};
+    }
     const int per_seq = (maxlen + T + 127) / 128;    // 128-key tiles of the longest cache
     const int64_t tiles128 = (int64_t)nb * c.kvh * per_seq;
     // The streaming form (its tiles come by tensor copies, hence the maps) pays from about 100 tiles on: 0.5B-class, one
@@ -276,11 +293,11 @@ AttnGeom attn_geom(const hs_model *m, int Tq, int T, int b0, int nb) {
         // that where there is work for several tiles each (staging the queries and merging the ranges is paid per CTA: 544
         // tiles of work run best as 8 per CTA)
         // From several rounds of 16 tiles per CTA on: one CTA per SM, each with an equal share of all tiles (0).
-        if (tiles128 > 148 * 16) return AttnGeom{128, 0, 0, 1, false};
+        if (tiles128 > 148 * 16) return AttnGeom{128, 0, 0, 1, false, stream_warps(0)};
         const int half = (int)((tiles128 + 73) / 74);
         int tiles = per_seq <= half ? per_seq : tiles128 <= 2 * 148 ? (int)((tiles128 + 147) / 148) : half;
         tiles = tiles < 1 ? 1 : tiles > 16 ? 16 : tiles;
-        return AttnGeom{128, tiles, 0, 1, false};
+        return AttnGeom{128, tiles, 0, 1, false, stream_warps(tiles)};
     }
     int want = 32;
     while (want < 128 && 8 * want < maxlen + T) want += 32;
@@ -436,7 +453,7 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
             aa.Kc = m->Kc + ly.al * per_layer; aa.Vc = m->Vc + ly.al * per_layer; aa.cap = c.kv_capacity;
             aa.kv_len = m->ctrl.kv_len; aa.o = m->obuf;
             aa.part_acc = m->att_acc; aa.part_ml = m->att_ml; aa.counters = m->ctrl.counters; aa.status = m->ctrl.status;
-            aa.chunk = at_geom.chunk; aa.tiles = at_geom.tiles; aa.small = at_geom.small; aa.stream = at_geom.stream;
+            aa.chunk = at_geom.chunk; aa.tiles = at_geom.tiles; aa.small = at_geom.small; aa.stream = at_geom.stream; aa.warps = at_geom.warps;
             if (!m->kmaps.empty()) { aa.kmap = m->kmaps[ly.al]; aa.vmap = m->vmaps[ly.al]; }
             aa.len_off = draft ? step : 0;
             const int span = at_geom.chunk * std::max(at_geom.tiles, 1);

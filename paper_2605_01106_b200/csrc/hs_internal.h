@@ -267,6 +267,7 @@ struct AttnArgs {
     int chunk, tiles, nch;              // keys per tile, tiles per CTA (streaming form, 0: an equal share of all tiles), key ranges that cover the cache capacity
     int len_off;                        // the new rows start at kv_len[b] + len_off (draft step i of a plan that keeps attention: i)
     int stream;                         // 1: the streaming form for long caches (stand-alone launches: chunk = 128, at most 32 query rows)
+    int warps;                          // of a streaming CTA with one tile of query rows: 8 or 16
     int small;                          // 1: the latency-lean form (G*T <= 16 rows, every cache within one cluster of 8 CTAs x chunk keys)
     int T, b0, nb;
     // streaming form: this layer's K and V cache as 2-D tensors [B * kvh * cap rows][hd] for tiled bulk copies

@@ -822,10 +822,6 @@ __device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int spl
 // registers a thread, two warps on a scheduler, and waited for their own operands most of the time: 178 us per launch on the batch-64
 // workload at k = 4.)
 constexpr int A2_KW = 8, A2_CK = 128, A2_NBUF = 3;
-// A packed query tile alone (1..8 rows) is served by one group of eight warps: half the instructions a tile, and half as many partial
-// results to merge where a CTA has one or two tiles (0.5B-class, k = 0, sixteen / eight warps: one sequence of 9000 keys 22.4 / 20.5
-// us per launch, three of 2500 at k = 1 16.9 / 14.9, 64 of 4368 .. 16166 124.4 / 123.3).
-__host__ __device__ constexpr int a2_threads(int mt, bool pk) { return mt == 1 && pk ? 256 : 512; }
 
 // Tile buffers hold 128 keys x HD bf16 without padding; the 16-byte chunk c of row r sits at chunk position
 // c ^ (r & 7), which keeps the eight rows of an ldmatrix 8x8 block on different banks.  Three K and three V buffers:
@@ -857,12 +853,12 @@ __device__ __forceinline__ void tma_tile_2d(void *dst_smem, const CUtensorMap *m
 // accumulator registers of rows g and g + 8), for the scores and again for P V (probability heads feed rows 0-7 of the
 // operand, remainders rows 8-15), so that tile costs half the tensor instructions of a full one.  It serves 1..8 query
 // rows (MT = 1) and 17..24 (MT = 2: 20 rows at four query heads per KV head and k = 4).
-template <int HD, int MT, bool PK>
-__global__ void __launch_bounds__(a2_threads(MT, PK), 1) attn2_kernel(const __grid_constant__ AttnArgs a) {
+template <int HD, int MT, bool PK, int NW>
+__global__ void __launch_bounds__(NW * 32, 1) attn2_kernel(const __grid_constant__ AttnArgs a) {
     extern __shared__ __align__(1024) unsigned char smraw[];
     constexpr int CK = A2_CK, GTB = MT * 16, NT = HD / 8, RB = HD * 2;       // RB: bytes of a tile row
     constexpr int PB = (MT - 1) * 16;                                        // first row of the packed tile
-    constexpr int THREADS = a2_threads(MT, PK), NW = THREADS / 32, TURNS = NW / A2_KW / MT;     // TURNS: groups that take the tiles of keys in turn
+    constexpr int THREADS = NW * 32, TURNS = NW / A2_KW / MT;                // TURNS: groups that take the tiles of keys in turn
     constexpr int NPART = NW / MT;                                           // partial results per query row
     const int G = a.qh / a.kvh, T = a.T, GT = G * T;
     const Attn2Layout L = attn2_layout(HD, MT);
@@ -1320,17 +1316,17 @@ __global__ void __launch_bounds__(a2_threads(MT, PK), 1) attn2_kernel(const __gr
     }
 }
 
-template <int HD, int MT, bool PK>
+template <int HD, int MT, bool PK, int NW>
 cudaError_t launch_attn2_t(const AttnArgs &a, cudaStream_t s) {
     static bool configured = false;
     const size_t smem = attn2_layout(HD, MT).total;
     if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(attn2_kernel<HD, MT, PK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn2_kernel<HD, MT, PK>, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+        cudaError_t e = cudaFuncSetAttribute(attn2_kernel<HD, MT, PK, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn2_kernel<HD, MT, PK, NW>, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    return launch_pdl(attn2_kernel<HD, MT, PK>, a.tiles > 0 ? dim3(a.nch, a.kvh, a.nb) : dim3(148), dim3(a2_threads(MT, PK)), smem, s, a);
+    return launch_pdl(attn2_kernel<HD, MT, PK, NW>, a.tiles > 0 ? dim3(a.nch, a.kvh, a.nb) : dim3(148), dim3(NW * 32), smem, s, a);
 }
 
 template <int HD, int MT>
@@ -1436,10 +1432,12 @@ cudaError_t launch_attn(const AttnArgs &a, cudaStream_t s) {
     if (a.stream) {          // the streaming form: 128-key tiles, a.tiles of them per CTA, at most 32 query rows
         if (GT > 32 || a.chunk != A2_CK || a.tiles < 0) return cudaErrorInvalidValue;
         // at most 8 rows in the last 16-row tile: the packed form of that tile (half its tensor instructions)
-#define A2(hd_) if (a.hd == hd_) return GT <= 8 ? launch_attn2_t<hd_, 1, true>(a, s) : GT <= 16 ? launch_attn2_t<hd_, 1, false>(a, s) \
-                                      : GT <= 24 ? launch_attn2_t<hd_, 2, true>(a, s) : launch_attn2_t<hd_, 2, false>(a, s)
+#define A2W(hd_, mt_, pk_) (a.warps == 8 ? launch_attn2_t<hd_, mt_, pk_, 8>(a, s) : launch_attn2_t<hd_, mt_, pk_, 16>(a, s))
+#define A2(hd_) if (a.hd == hd_) return GT <= 8 ? A2W(hd_, 1, true) : GT <= 16 ? A2W(hd_, 1, false) \
+                                      : GT <= 24 ? launch_attn2_t<hd_, 2, true, 16>(a, s) : launch_attn2_t<hd_, 2, false, 16>(a, s)
         A2(128); A2(64);
 #undef A2
+#undef A2W
         return cudaErrorInvalidValue;
     }
     if (GT > HS_MAX_GT || a.chunk < 16 || a.chunk > 128 || (a.chunk & 15) || a.tiles < 1) return cudaErrorInvalidValue;

@@ -146,6 +146,19 @@ def test_streaming_attention_edge_cases(env):
     assert rep.rounds == 5
 
 
+@pytest.mark.parametrize("tiles,k,lens", [
+    (-1, 4, [3500, 3201, 3072]),        # a full tile of query rows: more than 24 ranges per cache, sixteen warps in two groups
+    (-2, 4, [3073, 2944, 300]),         # 13 ranges: eight warps
+    (-16, 1, [1279, 900, 700]),         # a packed tile: a whole cache of 6 to 10 tiles, sixteen warps
+    (-2, 1, [1279, 640, 77])])          # several ranges: eight warps
+def test_streaming_attention_by_warps(env, tiles, k, lens):
+    s, eng, model, seqs = make(env, "test_seq", len(lens), k, max(lens) + 64, set(range(len(lens))), lens)
+    eng.set_attn_geometry(128, tiles)
+    rep = env["harness"].run_rounds(eng, seqs, s, k, 2, forced=[hi.forced_accept(k, 2, seq=70 + b) for b in range(len(lens))])
+    print(rep)
+    assert rep.rounds == 2 and eng.device_status() == 0
+
+
 @pytest.mark.parametrize("qh,ks", [(4, (8, 4, 1)), (8, (7,))])
 def test_streaming_attention_in_equal_shares(env, monkeypatch, qh, ks):
     # more than 16 rounds' worth of tiles (2600 by the longest of 100 caches): one CTA per SM with an equal share of the tiles of all
