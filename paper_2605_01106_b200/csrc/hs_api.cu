@@ -324,10 +324,19 @@ inline bool draft_runs(const hs_model *m, int l) {
 
 // Activation rows from which a pass runs its projections on tcgen05.  The kernel's fixed cost (set-up, epilogue out of tensor
 // memory) pays from 4 rows on where the weight matrices are large or the mixers pack the out-projection's operand themselves, as in
-// a draft step, else from 6.  1024-wide models, warp-level path / tcgen05: draft step of 4, 5, 6 rows 0.5B-class 1.154 / 1.111,
-// 1.210 / 1.154, 1.350 / 1.126 ms, sequential 0.518 / 0.510, 0.549 / 0.514, 0.609 / 0.513; verify pass of 4, 5, 6 rows 0.5B-class 1.300 /
-// 1.375, 1.370 / 1.403, 1.592 / 1.473, sequential 0.717 / 0.754, 0.758 / 0.778, 0.868 / 0.822.
-inline int tc_rows(const hs_model *m, bool mixers_pack) { return g_hs_tc_min_rows ? g_hs_tc_min_rows : m->large_mats || mixers_pack ? 4 : 6; }
+// a draft step without attention; a draft step that keeps attention packs it in a kernel of its own like a verify pass (parallel
+// blocks), or does so in its attention layers (sequential).  Warp-level path / tcgen05, ms:
+//   draft step of 4, 5, 6 rows: 0.5B-class 1.165 / 1.049, 1.202 / 1.056, 1.328 / 1.072, with attention 1.223 / 1.318, 1.400 / 1.466,
+//   1.543 / 1.458, layer-skipping 0.823 / 0.886, 0.940 / 0.971, 1.036 / 0.979; 256-wide 0.0467 / 0.0462, 0.0505 / 0.0464, 0.0598 /
+//   0.0466, with attention 0.0530 / 0.0566, 0.0563 / 0.0567, 0.0656 / 0.0574; sequential 0.515 / 0.507, 0.545 / 0.508, with attention
+//   0.676 / 0.690, 0.726 / 0.696, layer-skipping 0.458 / 0.467, 0.486 / 0.468
+//   verify pass of 4, 5, 6 rows: 0.5B-class 1.300 / 1.375, 1.370 / 1.403, 1.592 / 1.473; 256-wide 0.0595 / 0.0632, 0.0620 / 0.0633,
+//   0.0719 / 0.0636; sequential 0.717 / 0.754, 0.758 / 0.778, 0.868 / 0.822
+inline int tc_rows(const hs_model *m, bool draft_step) {
+    if (g_hs_tc_min_rows) return g_hs_tc_min_rows;
+    if (m->large_mats || (draft_step && !m->plan_attn)) return 4;
+    return draft_step && m->c.arch == HS_ARCH_SEQUENTIAL ? 5 : 6;
+}
 
 // first = true: this pass opens an API call (its predecessor in the stream may be the accept kernel of the last
 // round): its first kernel goes out in plain stream order, see hs_device.cuh.

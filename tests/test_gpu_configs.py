@@ -127,6 +127,32 @@ def test_projections_and_packed_mixers_by_rows(env, monkeypatch, name, L, batch,
     assert rep.rounds == 2 and eng.device_status() == 0
 
 
+@pytest.mark.parametrize("name,plan,batch,on_tcgen05", [
+    ("cfg1_tiny", "component", 3, False), ("cfg1_tiny", "component", 4, True),
+    ("cfg1_tiny", "full", 5, False), ("cfg1_tiny", "full", 6, True), ("cfg1_tiny", "layerskip33", 4, False),
+    ("test_seq", "component", 4, True), ("test_seq", "full", 4, False), ("test_seq", "full", 5, True)])
+def test_row_threshold_of_draft_steps(env, name, plan, batch, on_tcgen05):
+    # a draft step runs on tcgen05 from 4 rows on where its mixers pack the out-projection's operand, later where the plan keeps
+    # attention: there is at least one packing kernel more (the embedding's) than with the threshold out of reach
+    s = hi.CONFIGS[name]
+    eng = env["hs"].Engine(s, np.zeros(hi.blob_layout(s)[1], np.uint8), max_batch=batch, max_k=1, kv_capacity=64)
+    eng.set_draft_plan(hi.draft_plan(s, plan))
+    for b in range(batch):
+        eng.set_context(b, 20, 1)
+    eng.set_batch(batch)
+    count = {}
+    try:
+        for threshold in (0, 2, 17):
+            eng.set_option(eng.OPT_TC_MIN_ROWS, threshold)
+            before = eng.launch_count()
+            eng.draft(1)
+            count[threshold] = eng.launch_count() - before
+    finally:
+        eng.set_option(eng.OPT_TC_MIN_ROWS, 0)
+    assert count[2] > count[17] and count[0] == count[2 if on_tcgen05 else 17], count
+    assert eng.device_status() == 0
+
+
 def test_streaming_attention_edge_cases(env):
     # the streaming form (128-key tiles walked with two buffers, warp-local running softmax, ranges merged by the last
     # CTA to arrive) on the small sequential stack, where attention is a launch of its own: contexts that end exactly on
