@@ -247,7 +247,8 @@ int64_t hs_launch_count(const hs_model *m);
  * beyond fp32 summation order. */
 int hs_set_attn_geometry(hs_model *m, int chunk, int tiles);
 /* Tuning / measurement hook: switch a kernel choice on (value != 0) or off.  The choices are process-wide (they
- * apply to every handle); the handle's captured graphs are dropped so that the next step is captured afresh.
+ * apply to every handle) but for HS_OPT_TC_MIN_ROWS, which is the handle's own; the handle's captured graphs are dropped so
+ * that the next step is captured afresh.
  * Results are the same within fp32 summation order.  Synchronises the stream.
  *   HS_OPT_CLUSTER_REDUCE  residual projections with 4..16 activation rows add the partial sums of their K split
  *                          inside a thread-block cluster (default on; off: the consumers add the parts)

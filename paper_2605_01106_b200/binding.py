@@ -337,7 +337,7 @@ class Engine:
     OPT_CLUSTER_REDUCE, OPT_GEMM_MMA, OPT_GEMM_TC, OPT_PDL, OPT_ATTN_SMALL, OPT_ATTN_STREAM, OPT_TC_MIN_ROWS = range(7)
 
     def set_option(self, option, value):
-        """Switch a kernel choice (process-wide) on or off; see hs_set_option."""
+        """Switch a kernel choice on or off; see hs_set_option."""
         self._ck(lib().hs_set_option(self.h, int(option), int(value)))
 
     def profile(self, enable):

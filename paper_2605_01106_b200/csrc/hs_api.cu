@@ -333,7 +333,7 @@ inline bool draft_runs(const hs_model *m, int l) {
 //   verify pass of 4, 5, 6 rows: 0.5B-class 1.300 / 1.375, 1.370 / 1.403, 1.592 / 1.473; 256-wide 0.0595 / 0.0632, 0.0620 / 0.0633,
 //   0.0719 / 0.0636; sequential 0.717 / 0.754, 0.758 / 0.778, 0.868 / 0.822
 inline int tc_rows(const hs_model *m, bool draft_step) {
-    if (g_hs_tc_min_rows) return g_hs_tc_min_rows;
+    if (m->tc_min_rows) return m->tc_min_rows;
     if (m->large_mats || (draft_step && !m->plan_attn)) return 4;
     return draft_step && m->c.arch == HS_ARCH_SEQUENTIAL ? 5 : 6;
 }
@@ -357,7 +357,7 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
     // results in the packed form that kernel consumes (only the mixer's output and the embedding are packed by a
     // kernel of their own)
     __nv_bfloat16 *xb = rows > 16 || rows >= tc_rows(m, draft && T == 1) ? m->xb : nullptr;
-    const bool tc_pass = gemv_uses_tc(rows, xb != nullptr);
+    const bool tc_pass = gemv_uses_tc(xb != nullptr);
     int ss_parts = 0;                       // partial sums of squares per row in ssbuf
     bool h_packed = false;                  // xb_h / ssbuf hold the current residual stream
     PROF(HS_PROF_EMBED, 0, launch_embed(m->embed, d, c.V, m->ctrl.cand, m->Tm, draft ? step : 0, T, b0, nb, m->hbuf[0], st_w, first, s), "embed");
@@ -1250,7 +1250,7 @@ int hs_set_option(hs_model *m, int option, int value) {
     if (option == HS_OPT_TC_MIN_ROWS) {
         if (value != 0 && (value < 2 || value > 17)) return fail(m, HS_ERR_INVALID_ARG, "tcgen05 row threshold out of range");
         CK(cudaStreamSynchronize(m->stream), "option sync");
-        g_hs_tc_min_rows = value;
+        m->tc_min_rows = value;
         for (auto &kv : m->graphs) cudaGraphExecDestroy(kv.second);
         m->graphs.clear(); m->graph_launches.clear();
         return HS_OK;

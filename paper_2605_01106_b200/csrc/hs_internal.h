@@ -81,6 +81,7 @@ struct hs_model {
     float *att_acc, *att_ml;
     __nv_bfloat16 *xb; int64_t xb_rows;   // packed activation operand of the many-row projection kernel
     std::vector<CUtensorMap> kmaps, vmaps;   // per attention layer (streaming attention form)
+    int tc_min_rows;                      // activation rows from which projections run on the tcgen05 kernel; 0: automatic (tc_rows in hs_api.cu)
     bool large_mats;                      // weight matrices large enough that the tcgen05 kernel's fixed cost is small beside the time to stream them
     __nv_bfloat16 *xb_h, *xb_a; float *ssbuf;   // packed residual stream / MLP activations handed from projection to projection, row statistics
     // prompt path: activation rows per pass, the activations of a pass as above,
@@ -171,14 +172,13 @@ struct GemvArgs {
     const __nv_bfloat16 *pk_in; const float *ss_in; int ss_parts; bool ss_by_row;      // ss_by_row: ss_in[r * ss_parts + p] (the mixers' partial sums)
     __nv_bfloat16 *pk_out; int pk_ld; const float *pk_nw; float *ss_out; int *ss_parts_out;
 };
-// does a projection of nrows activation rows run on the many-row kernel?  (a caller that wants another one passes no xb)
-bool gemv_uses_tc(int nrows, bool have_xb);
+// does a projection run on the many-row kernel?  (a caller that wants another one passes no xb)
+bool gemv_uses_tc(bool have_xb);
 // *oparts receives the number of parts written to `out` (1 unless EPI_RESID split the reduction).
 cudaError_t launch_gemv(const GemvArgs &a, int32_t *status, cudaStream_t s, int64_t *launches, int *oparts);
 cudaError_t configure_gemv();   // one-time kernel attributes; call outside stream capture
 // many activation rows (> 16): tcgen05 tensor-core contraction (kernels_gemm_tc.cu)
 extern bool g_hs_gemm_tc;
-extern int g_hs_tc_min_rows;      // projections with at least this many activation rows run on the tcgen05 kernel; 0: automatic (tc_rows in hs_api.cu)
 cudaError_t configure_gemm_tc();
 int gemm_tc_rows(int nrows);
 cudaError_t launch_gemm_tc(const GemvArgs &a, int32_t *status, cudaStream_t s, int64_t *launches, int *oparts);

@@ -391,7 +391,6 @@ cudaError_t hs_make_kv_tensor_map(CUtensorMap *map, const void *base, uint64_t r
     if (hd % 64) return cudaErrorInvalidValue;
     return make_map(map, base, rows, (uint64_t)hd, (uint64_t)hd, 128);
 }
-int g_hs_tc_min_rows = 0;
 
 cudaError_t configure_gemm_tc() {
     void *fn = nullptr;

@@ -105,7 +105,7 @@ def test_cfg2_projection_kernel_choices(env):
                 rep = env["harness"].run_rounds(eng, seqs, s, k, 1, forced=forced, rep=rep)
                 assert eng.device_status() == 0, (thr, k)
     finally:
-        eng.set_option(eng.OPT_TC_MIN_ROWS, 0)          # the choice is process-wide
+        eng.set_option(eng.OPT_TC_MIN_ROWS, 0)
     print(rep)
     assert rep.rounds == 7
 
@@ -151,6 +151,32 @@ def test_row_threshold_of_draft_steps(env, name, plan, batch, on_tcgen05):
         eng.set_option(eng.OPT_TC_MIN_ROWS, 0)
     assert count[2] > count[17] and count[0] == count[2 if on_tcgen05 else 17], count
     assert eng.device_status() == 0
+
+
+def test_row_threshold_belongs_to_the_handle(env):
+    # a threshold set on one handle reaches neither one that is there already nor one that is made afterwards
+    s = hi.CONFIGS["cfg1_tiny"]
+
+    def engine():
+        e = env["hs"].Engine(s, np.zeros(hi.blob_layout(s)[1], np.uint8), max_batch=4, max_k=1, kv_capacity=64)
+        for b in range(4):
+            e.set_context(b, 20, 1)
+        e.set_batch(4)
+        return e
+
+    def launches(e):
+        before = e.launch_count()
+        e.draft(1)
+        return e.launch_count() - before
+
+    first, second = engine(), engine()
+    automatic = launches(first)
+    second.set_option(second.OPT_TC_MIN_ROWS, 17)
+    try:
+        assert launches(second) < automatic and launches(first) == automatic and launches(engine()) == automatic
+    finally:
+        second.set_option(second.OPT_TC_MIN_ROWS, 0)
+    assert launches(second) == automatic
 
 
 def test_streaming_attention_edge_cases(env):
