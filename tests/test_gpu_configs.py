@@ -230,6 +230,33 @@ def test_streaming_attention_in_equal_shares(env, monkeypatch, qh, ks):
     assert rep.rounds == len(ks)
 
 
+def test_streaming_attention_in_equal_shares_of_a_draft(env):
+    # a draft that keeps attention reads its own rows behind the cache (one more per step), here in equal shares: step i starts its
+    # new row at kv_len + i, on both sides of a tile boundary
+    lens = [1600 - 37 * (b % 31) for b in range(100)]
+    lens[:6] = [1535, 1534, 1533, 1536, 127, 128]
+    s, eng, model, seqs = make(env, "test_seq", len(lens), 4, 1700, {0, 1, 2, 3, 4, 5, 57, 99}, lens)
+    plan = hi.draft_plan(s, "full")
+    eng.set_draft_plan(plan)
+    model.set_draft_plan(plan)
+    forced = [hi.forced_accept(4, 2, seq=b) for b in range(len(lens))]
+    rep = env["harness"].run_rounds(eng, seqs, s, 4, 2, forced=forced)
+    print(rep)
+    assert rep.rounds == 2 and eng.device_status() == 0
+
+
+def test_streaming_attention_in_equal_shares_of_many_sequences(env):
+    # more sequences than a block has threads: a thread counts the tiles of several; shares of 16 tiles, most of them over many caches
+    batch, checked = 600, {0, 1, 2, 255, 256, 511, 512, 598, 599}
+    lens = [250 - (7 * b) % 245 for b in range(batch)]
+    lens[:3], lens[598:] = [128, 129, 250], [127, 250]
+    s, eng, model, seqs = make(env, "test_seq", batch, 1, 300, checked, lens)
+    forced = [hi.forced_accept(1, 2, seq=b) for b in range(batch)]
+    rep = env["harness"].run_rounds(eng, seqs, s, 1, 2, forced=forced)
+    print(rep)
+    assert rep.rounds == 2 and eng.device_status() == 0
+
+
 @pytest.mark.parametrize("form", ["fixed tiles", "equal shares"])
 def test_streaming_attention_control_words_out_of_range(env, form):
     # a bad cache length of one sequence in the streaming form, with a fixed number of tiles per CTA and in equal shares (where a CTA
