@@ -244,7 +244,9 @@ int64_t hs_launch_count(const hs_model *m);
  * for small batch * capacity): otherwise HS_ERR_INVALID_ARG and nothing changes.  A negative `tiles` with chunk = 128
  * selects the streaming form (-tiles tiles of 128 keys per CTA, partials merged by the last CTA to arrive) wherever the
  * attention runs as a launch of its own; it needs (qh / kvh) * (max_k + 1) <= 32.  Results do not depend on the setting
- * beyond fp32 summation order. */
+ * beyond fp32 summation order.  The automatic choice depends on the batch and on the longest context, and over more than 2368
+ * tiles of 128 keys each CTA takes an equal share of the tiles of all caches: where a sequence's cache is cut, and with it the
+ * summation order of its attention, then depends on the lengths of the other sequences.  The same contexts give the same bits. */
 int hs_set_attn_geometry(hs_model *m, int chunk, int tiles);
 /* Tuning / measurement hook: switch a kernel choice on (value != 0) or off.  The choices are process-wide (they
  * apply to every handle) but for HS_OPT_TC_MIN_ROWS, which is the handle's own; the handle's captured graphs are dropped so

@@ -289,10 +289,11 @@ AttnGeom attn_geom(const hs_model *m, int Tq, int T, int b0, int nb) {
         if (g_hs_attn_small && ctas <= (streams || fuse ? 148 : 4 * 148) && 8 * ck >= maxlen + T) return AttnGeom{ck, 1, 1, 0, fuse};
     }
     if (streams) {
-        // 128-key tiles per CTA.  A whole cache in one CTA spares the merge of ranges; otherwise about one CTA per SM, half
-        // that where there is work for several tiles each (staging the queries and merging the ranges is paid per CTA: 544
-        // tiles of work run best as 8 per CTA)
         // From several rounds of 16 tiles per CTA on: one CTA per SM, each with an equal share of all tiles (0).
+        // Below, 128-key tiles of one cache per CTA: a whole cache where that leaves half an SM count of CTAs (it spares the merge of
+        // ranges), one CTA per SM up to 296 tiles, else about half an SM count of CTAs.  That half is not the fastest split: as many
+        // ranges as fit the SMs at once take less, a second round of CTAs much more (k = 4, tiles per CTA: us per launch; 16 sequences
+        // of 2048 keys 3: 39.9, 4: 30.8, 8, by this rule: 35.2; 8 of 8000 6: 51.5, 7: 35.3, 14, by this rule: 45.4).
         if (tiles128 > 148 * 16) return AttnGeom{128, 0, 0, 1, false, stream_warps(0)};
         const int half = (int)((tiles128 + 73) / 74);
         int tiles = per_seq <= half ? per_seq : tiles128 <= 2 * 148 ? (int)((tiles128 + 147) / 148) : half;
@@ -354,8 +355,8 @@ int model_pass(hs_model *m, bool draft, int T, int step, int b0, int nb, bool fi
     const int64_t hps = (int64_t)m->B * m->Tm * d;
     int32_t *st_w = m->ctrl.status;
     // many rows: every projection of the pass runs on the tcgen05 kernel, and the projections hand each other their
-    // results in the packed form that kernel consumes (only the mixer's output and the embedding are packed by a
-    // kernel of their own)
+    // results in the packed form that kernel consumes.  The mixers of draft steps and DeltaNet layers write it as well (mix_packed
+    // below); the embedding, and what the mixer and the attention of a verify pass hand on, are packed by a kernel of their own
     __nv_bfloat16 *xb = rows > 16 || rows >= tc_rows(m, draft && T == 1) ? m->xb : nullptr;
     const bool tc_pass = gemv_uses_tc(xb != nullptr);
     int ss_parts = 0;                       // partial sums of squares per row in ssbuf

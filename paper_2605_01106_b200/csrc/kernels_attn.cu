@@ -807,20 +807,23 @@ __device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int spl
 
 
 // ------------------------------------------------------------------------------------------------
-// Long caches (the KV read is the step's largest byte stream): the streaming form.  One CTA of eight warps owns a
-// range of `tiles` tiles of 128 cached keys and walks it with two tile buffers: while the warps work on tile t, the
-// copies of tile t+1 (K and V, 64 KB) are in flight - one block-wide barrier per tile and nothing else.  The work on a
-// tile is warp-local, as in the latency-lean form: warp w takes keys [16 w, 16 w + 16) of the tile, computes their
-// scores for all query rows on the tensor cores, keeps the probabilities in registers, folds them into its own running
-// (max, sum) and accumulates its own partial output over the whole head dimension.  After the last tile the eight warp
-// partials are merged through shared memory (over the tile buffers); a range that is the whole cache writes the
-// result, otherwise the CTA publishes its partial and the CTA of the sequence and KV head that arrives last (ticket
-// counter, no spinning) merges the ranges in order, so the result does not depend on timing.  No clusters: every SM
-// takes the next CTA as soon as it is free.
-// Sixteen warps in two groups of eight.  A warp takes 16 keys of a tile and ONE 16-row query tile: with two query tiles (MT = 2) each
-// group has one of them, with one the groups take the tiles of keys in turn.  (Eight warps with both query tiles held 242
-// registers a thread, two warps on a scheduler, and waited for their own operands most of the time: 178 us per launch on the batch-64
-// workload at k = 4.)
+// Long caches (the KV read is the step's largest byte stream): the streaming form.  A CTA walks tiles of 128 cached keys: `tiles`
+// tiles of one (sequence, KV head) cache, or (tiles = 0) an equal share of the tiles of all caches, one cache after the other,
+// which may start and end inside a cache.  The tiles arrive by tensor copies through a ring of three buffer pairs, two in flight
+// while a third is worked on.  There is no block-wide barrier per tile: a warp waits for a tile's bytes, and the last warp to finish
+// with a pair requests the tile that refills it.
+// The work on a tile is warp-local, as in the latency-lean form: a warp takes 16 of the 128 keys and ONE 16-row tile of queries,
+// computes their scores on the tensor cores, keeps the probabilities in registers, folds them into its own running (max, sum) and
+// adds its product with V - in accumulators of its own for every tile - to its own partial output over the whole head dimension, in
+// fp32.  A group of eight warps covers a tile of keys.  Two query tiles (MT = 2): each of two groups has one of them.  One: one group,
+// or two that take the tiles of keys in turn (NW = 8 or 16, stream_warps in hs_api.cu).
+// At the end of a piece of a cache the partial results of its warps are merged through shared memory (over the tile buffers); a
+// piece that is the whole cache writes the result, otherwise the CTA publishes its partial and the CTA of the sequence and KV
+// head that arrives last (ticket counter, no spinning) merges the pieces in order, so the result does not depend on timing.  No
+// clusters: every SM takes the next CTA as soon as it is free.
+// Bound: HBM up to 8 query rows per KV head, the warps' own instructions beyond (a full query tile runs every product twice, for
+// head and remainder).  64 sequences of 4368 .. 16166 keys, k = 0 / 2 / 4: 124 / 131 / 174 us per launch, the bytes at the copy rate 103;
+// eight warps with both query tiles on ranges of 16 tiles 126 / 147 / 190.
 constexpr int A2_KW = 8, A2_CK = 128, A2_NBUF = 3;
 
 // Tile buffers hold 128 keys x HD bf16 without padding; the 16-byte chunk c of row r sits at chunk position

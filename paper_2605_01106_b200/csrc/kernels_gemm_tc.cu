@@ -1,20 +1,23 @@
-// Projection for many activation rows (batch * (k+1) > 16): a dense contraction, run on the fifth-generation
-// tensor cores.  out[r][o] = sum_j W[o][j] x[r][j] is computed as D = A B^T with
-//   A = a 128-row tile of the weight matrix (bf16, K-major), streamed by TMA tensor copies into 128-byte
-//       swizzled shared-memory stages,
-//   B = the activation rows, packed once per projection by a small kernel into bf16 head and bf16 remainder
-//       planes (x = head + remainder to 2^-17, with the RMSNorm weight and 1/rms folded in); a CTA takes BNH
-//       rows of each plane (all rows when there are at most 128) as the N = 2 * BNH columns of its tile,
-//   D = 128 x N fp32 accumulators in tensor memory; the epilogue reads them back with tcgen05.ld, adds the head
+// Projection for several activation rows (from 4 or 6 on, tc_rows in hs_api.cu): a dense contraction, run on the
+// fifth-generation tensor cores.  out[r][o] = sum_j W[o][j] x[r][j] is computed as D = A B^T with
+//   A = a tile of 128 rows of the weight matrix (bf16, K-major; 64 rows in residual projections whose tiles would leave
+//       half of the GPU idle), streamed by TMA tensor copies into 128-byte swizzled shared-memory stages,
+//   B = the activation rows as bf16 head and bf16 remainder planes (x = head + remainder to 2^-17, the RMSNorm weight
+//       folded in); a CTA takes BNH rows of each plane as the N = 2 * BNH columns of its tile.  The planes are written by the
+//       kernel that produces the rows - the epilogue of the projection before, the mixer of a draft step or a DeltaNet layer -
+//       with partial sums of squares beside them, from which 1/rms is applied to the finished sums; or, where nobody does (the
+//       embedding, what mixer and attention of a verify pass hand on), by pack_kernel with 1/rms folded in,
+//   D = 128 (64) x N fp32 accumulators in tensor memory; the epilogue reads them back with tcgen05.ld, adds the head
 //       and remainder columns and applies the store / residual / SwiGLU epilogue.
 // One elected thread issues the TMA copies, one issues tcgen05.mma (K = 16 per instruction, four per 64-column
-// stage) and releases stages with tcgen05.commit; all eight warps run the epilogue (thread = weight row, two
+// stage) and releases stages with tcgen05.commit; all eight warps run the epilogue (whole K range: thread = weight row, two
 // warps per lane quarter, each half of the columns).  Every wait is bounded.
 // Every CTA fetches its own tiles (no copy is shared between CTAs).
 // The weights are the large operand, so the grid is filled by splitting K, not N: the CTAs of a thread-block
-// cluster (up to 8) take consecutive K ranges of the same tile, leave their fp32 partial tiles in shared
-// memory and add them up, in rank order, through distributed shared memory - every weight byte is fetched
-// once and the result does not depend on timing.
+// cluster (up to 8) take consecutive K ranges of the same tile.  Each finishes an equal share of the tile's activation rows: the
+// others store their partial sums of those rows straight into its shared memory, and after one cluster barrier it adds them
+// in rank order, four columns of a weight row per thread - every weight byte is fetched once and the result does not depend
+// on timing.
 #include "hs_internal.h"
 #include "hs_device.cuh"
 #include "gemm_tc_common.cuh"

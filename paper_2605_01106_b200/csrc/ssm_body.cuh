@@ -18,8 +18,8 @@ constexpr int SSM_THREADS = 128; // 4 warps x PR / 4 rows
 // Instances for 1, 3, 5 and 9 positions: the unrolled loads and shared arrays of unused positions cost (verify pass at
 // k = 4 in the instance for 9 / for 5: 0.5B-class, one sequence 1.447 / 1.386 ms, 8 sequences 2.51 / 2.44; 3B-class, one
 // 3.03 / 2.96, 8 sequences 5.89 / 5.67).
-// PK: the output goes out packed (SsmArgs::pk), one position only; its own instance, because the test alone costs 1 % of a round of one
-// sequence at k = 2 (0.5B-class, 2174 / 2198 us).
+// PK: the output goes out packed (SsmArgs::pk), one position only; its own instance, because the test alone costs 0.3 % of a round of one
+// sequence at k = 2 (0.5B-class, 2191 / 2198 us).
 template <int EPL, int SSM_PR, int TMAX, bool PK = false>
 __device__ __forceinline__ void ssm_body(const SsmArgs &a, const int bx, const int by, const int bz) {
     constexpr int N = 32 * EPL;

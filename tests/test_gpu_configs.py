@@ -180,7 +180,7 @@ def test_row_threshold_belongs_to_the_handle(env):
 
 
 def test_streaming_attention_edge_cases(env):
-    # the streaming form (128-key tiles walked with two buffers, warp-local running softmax, ranges merged by the last
+    # the streaming form (128-key tiles walked through a ring of buffers, warp-local running softmax, ranges merged by the last
     # CTA to arrive) on the small sequential stack, where attention is a launch of its own: contexts that end exactly on
     # a tile boundary (the new rows then form a ninth key group), one key short of and one past it, a single short
     # range, several tiles per CTA, one and two 16-row query tiles (k = 4: 10 rows, k = 8: 18 rows)
