@@ -254,18 +254,17 @@ AttnGeom attn_geom(const hs_model *m, int Tq, int T, int b0, int nb) {
     int maxlen = 0;
     for (int b = b0; b < b0 + nb; ++b) if (m->kv_upper[b] > maxlen) maxlen = m->kv_upper[b];
     const int groups = c.qh / c.kvh * Tq;            // query rows per KV head
-    // Warps of a streaming CTA that has one tile of query rows (two tiles: sixteen, eight for each).  Eight: a second group of eight
-    // runs short of registers with a full tile (9 .. 16 rows), and adds partial results to merge.  It pays with a packed tile (up to
-    // 8 rows) in equal shares and where 64-wide heads leave a CTA with a whole cache waiting for its own instructions; with a full tile
-    // where a cache is cut into many ranges, whose merge more threads finish sooner.  Verify pass, us per layer, 8 / 16 warps: packed
-    // 0.5B-class 64 sequences of 4368 .. 16166 keys 186.2 / 185.2, 8 of 8000 56.9 / 58.3, 40 of 1200 72.0 / 72.9, one of 9000 32.5 / 33.4,
-    // 64-wide 40 of 1500 41.3 / 38.9, 60 of 700 38.6 / 37.8, 80 of 500 41.8 / 45.4; full 64 of 4368 .. 16166 228.9 / 233.5, 30 of 700 ..
-    // 9400 122.5 / 129.9, 10 of 2500 61.2 / 63.5, one of 9000 (71 ranges) 51.0 / 46.5, two of 9000 (36) 134.5 / 132.2, two of 16000
-    // (21 ranges) 57.4 / 57.7.
+    // Warps of a streaming CTA that has one tile of query rows (two tiles: sixteen, eight for each).  Eight: a second group of eight adds
+    // partial results to merge, and with a full tile (9 .. 16 rows) of 128-wide heads runs short of registers.  It pays with a packed tile
+    // (up to 8 rows) in equal shares, and where 64-wide heads leave a CTA waiting for its own instructions: a whole cache per CTA, or
+    // a full tile over many ranges of few tiles.  Verify pass, us per layer, 8 / 16 warps: packed 0.5B-class 64 sequences of 4368 ..
+    // 16166 keys 186.2 / 185.2, 8 of 8000 56.9 / 58.3, 40 of 1200 72.0 / 72.9, one of 9000 32.5 / 33.4, 64-wide 40 of 1500 41.3 / 38.9,
+    // 60 of 700 38.6 / 37.8, 80 of 500 41.8 / 45.4; full 64 of 4368 .. 16166 228.9 / 233.5, 30 of 700 .. 9400 122.5 / 129.9, 10 of 2500
+    // 61.2 / 63.5, two of 16000 55.9 / 58.2, one of 9000 46.6 / 46.5, 64-wide two of 9000 (36 ranges of two tiles) 39.9 / 39.0.
     auto stream_warps = [&](int tiles) {
         const int ranges = tiles ? ((maxlen + 127) / 128 + tiles - 1) / tiles : 0;
         const bool packed = groups <= 8;
-        return groups > 16 || (packed ? tiles == 0 || (c.hd == 64 && ranges == 1 && tiles >= 6) : ranges > 24) ? 16 : 8;
+        return groups > 16 || (packed && tiles == 0) || (c.hd == 64 && (packed ? ranges == 1 && tiles >= 6 : ranges > 10 * tiles)) ? 16 : 8;
     };
     if (m->att_force_chunk) {
         const int tiles = m->att_force_tiles < 0 ? -m->att_force_tiles : m->att_force_tiles;

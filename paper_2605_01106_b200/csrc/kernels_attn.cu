@@ -1290,22 +1290,36 @@ __global__ void __launch_bounds__(NW * 32, 1) attn2_kernel(const __grid_constant
         if (lane == 0) { mrg_s[2 * qi] = M; mrg_s[2 * qi + 1] = den; }
     }
     __syncthreads();
-#pragma unroll 1
-    for (int idx = tid; idx < GT * DV4; idx += THREADS) {
-        const int qi = idx / DV4, d = (idx - qi * DV4) * 4;
-        const float M = mrg_s[2 * qi];
-        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+    // up to two rows per thread, their loads in flight together: as many trips to L2 with eight warps as with sixteen
+    constexpr int STEP = THREADS / DV4;                 // rows between them
+    auto merge = [&](auto rows_, const int qi) {
+        constexpr int NR = decltype(rows_)::value;
+        const int d = tid % DV4 * 4;
+        float M[NR];
+        float4 sum[NR];
+#pragma unroll
+        for (int u = 0; u < NR; ++u) { M[u] = mrg_s[2 * (qi + u * STEP)]; sum[u] = make_float4(0.f, 0.f, 0.f, 0.f); }
 #pragma unroll 4
-        for (int c = 0; c < nsplit; ++c) {
-            const float wt = __expf(__ldcg(pm0 + ((size_t)c * HS_MAX_GT + qi) * 2) - M);
-            const float4 v = __ldcg(reinterpret_cast<const float4 *>(pa0 + ((size_t)c * HS_MAX_GT + qi) * HD + d));
-            sum.x = fmaf(wt, v.x, sum.x); sum.y = fmaf(wt, v.y, sum.y); sum.z = fmaf(wt, v.z, sum.z); sum.w = fmaf(wt, v.w, sum.w);
+        for (int c = 0; c < nsplit; ++c)
+#pragma unroll
+            for (int u = 0; u < NR; ++u) {
+                const size_t row = (size_t)c * HS_MAX_GT + qi + u * STEP;
+                const float wt = __expf(__ldcg(pm0 + row * 2) - M[u]);
+                const float4 v = __ldcg(reinterpret_cast<const float4 *>(pa0 + row * HD + d));
+                sum[u].x = fmaf(wt, v.x, sum[u].x); sum[u].y = fmaf(wt, v.y, sum[u].y); sum[u].z = fmaf(wt, v.z, sum[u].z); sum[u].w = fmaf(wt, v.w, sum[u].w);
+            }
+#pragma unroll
+        for (int u = 0; u < NR; ++u) {
+            const int r = qi + u * STEP, gq = (int)((r * tinv) >> 16), i = r - gq * T;
+            const float inv = 1.0f / mrg_s[2 * r + 1];
+            *reinterpret_cast<float4 *>(o_base + (size_t)i * (a.qh * HD) + (kh * G + gq) * HD + d) =
+                make_float4(sum[u].x * inv, sum[u].y * inv, sum[u].z * inv, sum[u].w * inv);
         }
-        const int gq = (int)((qi * tinv) >> 16), i = qi - gq * T;
-        const float inv = 1.0f / mrg_s[2 * qi + 1];
-        *reinterpret_cast<float4 *>(o_base + (size_t)i * (a.qh * HD) + (kh * G + gq) * HD + d) =
-            make_float4(sum.x * inv, sum.y * inv, sum.z * inv, sum.w * inv);
-    }
+    };
+#pragma unroll 1
+    for (int qi = tid / DV4; qi < GT; qi += 2 * STEP)
+        if (GTB > STEP && qi + STEP < GT) merge(std::integral_constant<int, 2>{}, qi);
+        else merge(std::integral_constant<int, 1>{}, qi);
     }
     }
     }
@@ -1435,7 +1449,7 @@ cudaError_t launch_attn(const AttnArgs &a, cudaStream_t s) {
     if (a.stream) {          // the streaming form: 128-key tiles, a.tiles of them per CTA, at most 32 query rows
         if (GT > 32 || a.chunk != A2_CK || a.tiles < 0) return cudaErrorInvalidValue;
         // at most 8 rows in the last 16-row tile: the packed form of that tile (half its tensor instructions)
-#define A2W(hd_, mt_, pk_) (a.warps == 8 ? launch_attn2_t<hd_, mt_, pk_, 8>(a, s) : launch_attn2_t<hd_, mt_, pk_, 16>(a, s))
+#define A2W(hd_, mt_, pk_) (a.warps == 8 || (hd_ == 128 && !pk_) ? launch_attn2_t<hd_, mt_, pk_, 8>(a, s) : launch_attn2_t<hd_, mt_, pk_, hd_ == 128 && !pk_ ? 8 : 16>(a, s))
 #define A2(hd_) if (a.hd == hd_) return GT <= 8 ? A2W(hd_, 1, true) : GT <= 16 ? A2W(hd_, 1, false) \
                                       : GT <= 24 ? launch_attn2_t<hd_, 2, true, 16>(a, s) : launch_attn2_t<hd_, 2, false, 16>(a, s)
         A2(128); A2(64);

@@ -199,8 +199,8 @@ def test_streaming_attention_edge_cases(env):
 
 
 @pytest.mark.parametrize("tiles,k,lens", [
-    (-1, 4, [3500, 3201, 3072]),        # a full tile of query rows: more than 24 ranges per cache, sixteen warps in two groups
-    (-2, 4, [3073, 2944, 300]),         # 13 ranges: eight warps
+    (-1, 4, [3500, 3201, 3072]),        # a full tile of query rows: 28 ranges of one tile, sixteen warps in two groups
+    (-2, 4, [3073, 2944, 300]),         # 13 ranges of two tiles: eight warps
     (-16, 1, [1279, 900, 700]),         # a packed tile: a whole cache of 6 to 10 tiles, sixteen warps
     (-2, 1, [1279, 640, 77])])          # several ranges: eight warps
 def test_streaming_attention_by_warps(env, tiles, k, lens):
@@ -209,6 +209,25 @@ def test_streaming_attention_by_warps(env, tiles, k, lens):
     rep = env["harness"].run_rounds(eng, seqs, s, k, 2, forced=[hi.forced_accept(k, 2, seq=70 + b) for b in range(len(lens))])
     print(rep)
     assert rep.rounds == 2 and eng.device_status() == 0
+
+
+@pytest.mark.parametrize("lens,checked,ks", [
+    ([7000, 6913], {0, 1}, (4, 3, 2, 1, 0)),                    # 28 ranges of two tiles, merged two rows per thread from 9 rows on
+    ([1600 - 53 * (b % 29) for b in range(100)], {0, 1, 50, 99}, (3, 2, 0))])       # equal shares
+def test_streaming_attention_of_wide_heads(env, monkeypatch, lens, checked, ks):
+    # 128-wide heads, 4 .. 20 query rows per KV head: packed, full, full and packed query tiles
+    s = hi.CONFIGS["cfg2_0p5b"].replace(L=1, V=2048)
+    monkeypatch.setitem(hi.CONFIGS, "wide", s)
+    _W.pop(("wide", "jitter"), None)
+    _, eng, model, seqs = make(env, "wide", len(lens), max(ks), max(lens) + 64, checked, lens)
+    _W.pop(("wide", "jitter"), None)
+    rep = None
+    for k in ks:
+        forced = [hi.forced_accept(k, 1, seq=20 + b + k) for b in range(len(lens))]
+        rep = env["harness"].run_rounds(eng, seqs, s, k, 1, forced=forced, rep=rep)
+        assert eng.device_status() == 0, k
+    print(rep)
+    assert rep.rounds == len(ks)
 
 
 @pytest.mark.parametrize("qh,ks", [(4, (8, 4, 1)), (8, (7,))])
