@@ -822,7 +822,7 @@ __device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int spl
 // head that arrives last (ticket counter, no spinning) merges the pieces in order, so the result does not depend on timing.  No
 // clusters: every SM takes the next CTA as soon as it is free.
 // Bound: HBM up to 8 query rows per KV head, the warps' own instructions beyond (a full query tile runs every product twice, for
-// head and remainder).  64 sequences of 4368 .. 16166 keys, k = 0 / 2 / 4: 124 / 131 / 174 us per launch, the bytes at the copy rate 103;
+// head and remainder).  64 sequences of 4368 .. 16166 keys, k = 0 / 2 / 4: 125 / 130 / 175 us per launch, the bytes at the copy rate 103;
 // eight warps with both query tiles on ranges of 16 tiles 126 / 147 / 190.
 constexpr int A2_KW = 8, A2_CK = 128, A2_NBUF = 3;
 
@@ -1449,6 +1449,7 @@ cudaError_t launch_attn(const AttnArgs &a, cudaStream_t s) {
     if (a.stream) {          // the streaming form: 128-key tiles, a.tiles of them per CTA, at most 32 query rows
         if (GT > 32 || a.chunk != A2_CK || a.tiles < 0) return cudaErrorInvalidValue;
         // at most 8 rows in the last 16-row tile: the packed form of that tile (half its tensor instructions)
+        // (a full tile of 128-wide heads has an instance of eight warps only, see stream_warps)
 #define A2W(hd_, mt_, pk_) (a.warps == 8 || (hd_ == 128 && !pk_) ? launch_attn2_t<hd_, mt_, pk_, 8>(a, s) : launch_attn2_t<hd_, mt_, pk_, hd_ == 128 && !pk_ ? 8 : 16>(a, s))
 #define A2(hd_) if (a.hd == hd_) return GT <= 8 ? A2W(hd_, 1, true) : GT <= 16 ? A2W(hd_, 1, false) \
                                       : GT <= 24 ? launch_attn2_t<hd_, 2, true, 16>(a, s) : launch_attn2_t<hd_, 2, false, 16>(a, s)
