@@ -291,7 +291,7 @@ AttnGeom attn_geom(const hs_model *m, int Tq, int T, int b0, int nb) {
         // From several rounds of 16 tiles per CTA on: one CTA per SM, each with an equal share of all tiles (0).
         // Below, 128-key tiles of one cache per CTA: a whole cache where that leaves half an SM count of CTAs (it spares the merge of
         // ranges), one CTA per SM up to 296 tiles, else about half an SM count of CTAs.  That half is not the fastest split: as many
-        // ranges as fit the SMs at once take less, a second round of CTAs much more (k = 4, tiles per CTA: us per launch; 16 sequences
+        // ranges as fit the SMs at once take less, a second round of CTAs much more (k = 4, accumulators per tile, tiles per CTA: us per launch; 16 sequences
         // of 2048 keys 3: 39.9, 4: 30.8, 8, by this rule: 35.2; 8 of 8000 6: 51.5, 7: 35.3, 14, by this rule: 45.4).
         if (tiles128 > 148 * 16) return AttnGeom{128, 0, 0, 1, false, stream_warps(0)};
         const int half = (int)((tiles128 + 73) / 74);

@@ -814,8 +814,8 @@ __device__ __forceinline__ void attn_small_body(const AttnArgs &a, const int spl
 // with a pair requests the tile that refills it.
 // The work on a tile is warp-local, as in the latency-lean form: a warp takes 16 of the 128 keys and ONE 16-row tile of queries,
 // computes their scores on the tensor cores, keeps the probabilities in registers, folds them into its own running (max, sum) and
-// adds its product with V - in accumulators of its own for every tile - to its own partial output over the whole head dimension, in
-// fp32.  A group of eight warps covers a tile of keys.  Two query tiles (MT = 2): each of two groups has one of them.  One: one group,
+// adds its product with V to its own partial output over the whole head dimension: in accumulators of its own for every tile and
+// then in fp32, or (CHAIN: two query tiles, ranges of at most 16 tiles) in the accumulators that hold the partial output.  A group of eight warps covers a tile of keys.  Two query tiles (MT = 2): each of two groups has one of them.  One: one group,
 // or two that take the tiles of keys in turn (NW = 8 or 16, stream_warps in hs_api.cu).
 // At the end of a piece of a cache the partial results of its warps are merged through shared memory (over the tile buffers); a
 // piece that is the whole cache writes the result, otherwise the CTA publishes its partial and the CTA of the sequence and KV
@@ -856,7 +856,8 @@ __device__ __forceinline__ void tma_tile_2d(void *dst_smem, const CUtensorMap *m
 // accumulator registers of rows g and g + 8), for the scores and again for P V (probability heads feed rows 0-7 of the
 // operand, remainders rows 8-15), so that tile costs half the tensor instructions of a full one.  It serves 1..8 query
 // rows (MT = 1) and 17..24 (MT = 2: 20 rows at four query heads per KV head and k = 4).
-template <int HD, int MT, bool PK, int NW>
+// CHAIN: a tile's products are added to the running output by the tensor path itself (see the key loop).
+template <int HD, int MT, bool PK, int NW, bool CHAIN>
 __global__ void __launch_bounds__(NW * 32, 1) attn2_kernel(const __grid_constant__ AttnArgs a) {
     extern __shared__ __align__(1024) unsigned char smraw[];
     constexpr int CK = A2_CK, GTB = MT * 16, NT = HD / 8, RB = HD * 2;       // RB: bytes of a tile row
@@ -1173,11 +1174,26 @@ __global__ void __launch_bounds__(NW * 32, 1) attn2_kernel(const __grid_constant
                 }
                 l_run[r] = fmaf(l_run[r], corr[r], sum);
             }
-            // ---- partial output = partial output * correction + P V over the whole head dimension.  A tile's products add up in
-            // accumulators of their own (the tensor path truncates every sum it adds to, and a share may be hundreds of tiles: 250
-            // in one chain left the output short by 1.5e-5 of itself, 16 by 4e-7, so 1e-7).  One pair of column groups is added
-            // while the next one's MMAs run.
+            // ---- partial output = partial output * correction + P V over the whole head dimension.
             const uint32_t vals = keys + v_at + (newrows ? 16 * RB : CK * RB);
+            if constexpr (CHAIN) {
+                // At most 16 tiles: the accumulators are the running output, rescaled only
+                // when some row's maximum moved (rare after the first tiles).
+                if (__any_sync(0xffffffffu, corr[0] != 1.f || corr[1] != 1.f)) {
+#pragma unroll
+                    for (int nt = 0; nt < NT; ++nt) { O[nt][0] *= corr[0]; O[nt][1] *= corr[0]; O[nt][2] *= corr[1]; O[nt][3] *= corr[1]; }
+                }
+#pragma unroll
+                for (int p = 0; p < NT / 2; ++p) {
+                    uint32_t bv[4];
+                    ldsm_x4_t(bv, (vals ^ (uint32_t)((p & 3) * 32)) + (p >> 2) * hstr);
+                    mma_bf16(O[2 * p], ph, bv[0], bv[1]); mma_bf16(O[2 * p + 1], ph, bv[2], bv[3]);
+                    if (!packed) { mma_bf16(O[2 * p], pl, bv[0], bv[1]); mma_bf16(O[2 * p + 1], pl, bv[2], bv[3]); }
+                }
+            } else {
+            // A tile's products add up in accumulators of their own (the tensor path truncates every sum it adds to, and a share may be
+            // hundreds of tiles: 250 in one chain left the output short by 1.5e-5 of itself, 16 by 4e-7, so 1e-7).  One pair of
+            // column groups is added while the next one's MMAs run.
             float D[2][2][4];
             auto add = [&](int p) {
 #pragma unroll
@@ -1200,6 +1216,7 @@ __global__ void __launch_bounds__(NW * 32, 1) attn2_kernel(const __grid_constant
                 if (p) add(p - 1);
             }
             add(NT / 2 - 1);
+            }
         }
         if (!newrows) {
             // this warp is done with tile t: the last of those that read it refills the buffer pair with tile t + 3
@@ -1219,6 +1236,9 @@ __global__ void __launch_bounds__(NW * 32, 1) attn2_kernel(const __grid_constant
     // ---- merge the warp partials through shared memory (the tile buffers are free now)
     float *wo_s = reinterpret_cast<float *>(sm + L.tile_off);            // [NPART][GTB][HD]
     const int part = MT == 2 ? kw : warp;
+    if (CHAIN && packed)                    // head and remainder halves of the packed tile's outputs
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) { O[nt][0] += O[nt][2]; O[nt][1] += O[nt][3]; }
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
         if (packed && r == 1) continue;
@@ -1333,17 +1353,17 @@ __global__ void __launch_bounds__(NW * 32, 1) attn2_kernel(const __grid_constant
     }
 }
 
-template <int HD, int MT, bool PK, int NW>
+template <int HD, int MT, bool PK, int NW, bool CHAIN = false>
 cudaError_t launch_attn2_t(const AttnArgs &a, cudaStream_t s) {
     static bool configured = false;
     const size_t smem = attn2_layout(HD, MT).total;
     if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(attn2_kernel<HD, MT, PK, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn2_kernel<HD, MT, PK, NW>, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+        cudaError_t e = cudaFuncSetAttribute(attn2_kernel<HD, MT, PK, NW, CHAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(attn2_kernel<HD, MT, PK, NW, CHAIN>, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    return launch_pdl(attn2_kernel<HD, MT, PK, NW>, a.tiles > 0 ? dim3(a.nch, a.kvh, a.nb) : dim3(148), dim3(NW * 32), smem, s, a);
+    return launch_pdl(attn2_kernel<HD, MT, PK, NW, CHAIN>, a.tiles > 0 ? dim3(a.nch, a.kvh, a.nb) : dim3(148), dim3(NW * 32), smem, s, a);
 }
 
 template <int HD, int MT>
@@ -1451,10 +1471,16 @@ cudaError_t launch_attn(const AttnArgs &a, cudaStream_t s) {
         // at most 8 rows in the last 16-row tile: the packed form of that tile (half its tensor instructions)
         // (a full tile of 128-wide heads has an instance of eight warps only, see stream_warps)
 #define A2W(hd_, mt_, pk_) (a.warps == 8 || (hd_ == 128 && !pk_) ? launch_attn2_t<hd_, mt_, pk_, 8>(a, s) : launch_attn2_t<hd_, mt_, pk_, hd_ == 128 && !pk_ ? 8 : 16>(a, s))
+        // Two tiles of query rows on ranges of at most 16 tiles: one chain per accumulator (a warp there is short of registers: accumulators per
+        // tile spill 88 .. 140 bytes, chains 8 or none; 8 sequences of 2048 keys, k = 4, 8 tiles per CTA: 29.5 us against 29.0, a round of the
+        // 3B-class model 0.6 % longer).  16 tiles in a chain leave the output short by up to 4e-7 of itself; longer ranges, which only
+        // a caller can ask for, and equal shares take the other instance.
+#define A2M(hd_, pk_) (a.tiles > 0 && a.tiles <= 16 ? launch_attn2_t<hd_, 2, pk_, 16, true>(a, s) : launch_attn2_t<hd_, 2, pk_, 16>(a, s))
 #define A2(hd_) if (a.hd == hd_) return GT <= 8 ? A2W(hd_, 1, true) : GT <= 16 ? A2W(hd_, 1, false) \
-                                      : GT <= 24 ? launch_attn2_t<hd_, 2, true, 16>(a, s) : launch_attn2_t<hd_, 2, false, 16>(a, s)
+                                      : GT <= 24 ? A2M(hd_, true) : A2M(hd_, false)
         A2(128); A2(64);
 #undef A2
+#undef A2M
 #undef A2W
         return cudaErrorInvalidValue;
     }

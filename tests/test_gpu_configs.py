@@ -230,6 +230,21 @@ def test_streaming_attention_of_wide_heads(env, monkeypatch, lens, checked, ks):
     assert rep.rounds == len(ks)
 
 
+@pytest.mark.parametrize("hd,qh,k,tiles", [(64, 8, 4, -16), (64, 8, 4, -17), (64, 8, 7, -2), (64, 8, 7, -17), (128, 8, 4, -3), (128, 8, 7, -16)])
+def test_streaming_attention_two_query_tiles(env, monkeypatch, hd, qh, k, tiles):
+    # two tiles of query rows, the second one packed (20 rows) or full (32), with a fixed number of tiles per CTA: up to 16 the products
+    # of a range run on in the same accumulators, beyond that every tile has its own
+    name = "test_seq_h%d_q%d" % (hd, qh)
+    s = hi.CONFIGS["test_seq"].replace(qh=qh, hd=hd)
+    monkeypatch.setitem(hi.CONFIGS, name, s)
+    lens = [2303, 2176, 2049, 5]
+    _, eng, model, seqs = make(env, name, len(lens), k, 2400, set(range(len(lens))), lens)
+    eng.set_attn_geometry(128, tiles)
+    rep = env["harness"].run_rounds(eng, seqs, s, k, 2, forced=[hi.forced_accept(k, 2, seq=30 + b) for b in range(len(lens))])
+    print(rep)
+    assert rep.rounds == 2 and eng.device_status() == 0
+
+
 @pytest.mark.parametrize("qh,ks", [(4, (8, 4, 1)), (8, (7,))])
 def test_streaming_attention_in_equal_shares(env, monkeypatch, qh, ks):
     # more than 16 rounds' worth of tiles (2600 by the longest of 100 caches): one CTA per SM with an equal share of the tiles of all
